@@ -60,6 +60,10 @@ struct TranscodeJob {
 // handed out in this scan (a 64-bit counter, zeroed by the per-scan reset).
 constexpr int TC_POOL_COUNTER = 2;
 
+// Words of the item_counter array of a scan of n_cols output columns.
+PQ_HD constexpr uint32_t SNAP_COUNTER0(uint32_t n_cols) { return 4 + n_cols; }
+PQ_HD constexpr uint32_t SCAN_COUNTERS(uint32_t n_cols) { return SNAP_COUNTER0(n_cols) + 2 * SNAPPY_RUNS * n_cols; }
+
 struct DecodeArgs {
   const ChunkDev* chunks;
   const PageDev* pages;
@@ -68,7 +72,9 @@ struct DecodeArgs {
   Item* items;
   const OutCol* cols;
   DevStatus* st;
-  uint32_t* item_counter;   // [2..3] transcode pool bytes, [4 + c] next work item of output column c
+  uint32_t* item_counter;   // [2..3] transcode pool bytes, [4 + c] next work item of output column c,
+                            // [SNAP_COUNTER0(n) + 2 R c + R d + r] (R = SNAPPY_RUNS) next segment of run r of its split
+                            // data (d = 0) or dictionary (d = 1) pages
   const uint32_t* walk_pps; // plan pages that need the walk, longest chains first
   const uint32_t* delta_pps;// DELTA plan pages (block bases)
   uint32_t* dpos;           // DELTA block positions (stream offsets)
@@ -76,6 +82,8 @@ struct DecodeArgs {
   DeltaRegion* dregs;       // DELTA region summaries
   uint32_t* dreg_lists;     // DELTA region block lists (DELTA_REGION_LIST per region)
   uint32_t* vpos;           // transcoded string pages: value-stream offset of each value (and of the end)
+  uint32_t* snap_state;     // split Snappy pages' state (SnapState), zeroed by the per-scan reset
+  uint64_t snap_words;
   int n_pp;
   int n_items;
   int n_walk;
@@ -119,13 +127,16 @@ void launch_copy_small(void* dst, const void* src, uint32_t bytes, cudaStream_t 
 void launch_make_items(const DecodeArgs& a, int n_pp, cudaStream_t s);
 int expand_blocks_per_sm();
 int walk_blocks_per_sm();
-// coop: one block of 8 warps per page (large pages), else one warp per page;
-// pages with nsub > 1 are skipped (their blocks are separate jobs)
-void launch_snappy(const SnappyJob* jobs, int n_jobs, int n_sms, DevStatus* st, cudaStream_t s, bool coop);
-// The blocks of the pages of jobs [0, n_jobs) that have nsub > 1, written to
-// blocks[sub .. sub + nsub) (SNAPPY_FRAGMENT)
-void launch_snappy_split(const SnappyJob* jobs, int n_jobs, SnappyJob* blocks, int n_sms, DevStatus* st,
-                         cudaStream_t s);
+// One block per page; wide: 16 warps each (large pages), else 4.  Pages with
+// nsub > 1 are skipped: launch_snappy_scan locates their fragments (segments
+// [seg_begin, seg_begin + n_segs) of the list's jobs, handed out through
+// SNAPPY_RUNS counters, zero before the launch) and launch_snappy_fragments decompresses
+// fragments [first, first + n).
+void launch_snappy(const SnappyJob* jobs, int n_jobs, int n_sms, DevStatus* st, cudaStream_t s, bool wide);
+void launch_snappy_scan(const SnappyJob* jobs, int n_jobs, uint32_t seg_begin, uint32_t n_segs, SnapState ss,
+                        uint32_t* tickets, int n_sms, DevStatus* st, cudaStream_t s);
+void launch_snappy_fragments(const SnappyJob* jobs, int first, int n, SnapState ss, int n_sms, DevStatus* st,
+                             cudaStream_t s);
 // Zstandard pages of jobs [0, n_jobs) (the others are skipped)
 void launch_zstd(const SnappyJob* jobs, int n_jobs, int n_sms, DevStatus* st, cudaStream_t s);
 void launch_index_walk(const ChunkDev* chunks, int n_chunks, PageDev* pages, uint32_t* counts, int mode,

@@ -179,6 +179,8 @@ pqi::DecodeArgs decode_args(pq_plan* plan) {
   a.dregs = plan->d_dregs;
   a.dreg_lists = plan->d_dreg_lists;
   a.vpos = plan->d_vpos;
+  a.snap_state = reinterpret_cast<uint32_t*>(plan->d_snap_state);
+  a.snap_words = pqi::snap_state_bytes(plan->snap_blocks, plan->snap_segs) / 4;
   a.n_pp = static_cast<int>(plan->pps.size());
   a.n_items = static_cast<int>(plan->n_items);
   a.n_walk = static_cast<int>(plan->walk_pps.size());
@@ -839,16 +841,21 @@ namespace pqe {
 // Host half of planning: plan pages, work item counts, job lists and the
 // scratch layout for the rows of `segs` (each segment's rows go to output
 // rows starting at its out0), nothing on the device yet.
-// A Snappy page decompressed by fragments (SNAPPY_FRAGMENT): nsub block slots
-// numbered from *counter.  Dictionary and data pages count separately (their
-// blocks sit in two ranges of the block list, like their jobs).
-static void plan_split(pqi::SnappyJob& sj, bool plain, uint32_t* counter) {
-  if (plain || sj.codec != pqi::CODEC_SNAPPY || sj.raw || sj.prefix > sj.dst_len) return;
-  const uint32_t out = sj.dst_len - sj.prefix;
-  if (out <= pqi::SNAPPY_SPLIT_MIN) return;
+// A Snappy page decompressed by fragments (SNAPPY_FRAGMENT): its fragments
+// and input segments are numbered from *frags and *segs.  Dictionary and data
+// pages count separately (theirs sit in two ranges, like their jobs).  Pages
+// longer than any Snappy encoding of their output are left whole (so the
+// state below fits 56 bytes a fragment).
+static void plan_split(pqi::SnappyJob& sj, bool plain, uint32_t* frags, uint32_t* segs) {
+  sj.seg = *segs;
+  if (plain || sj.codec != pqi::CODEC_SNAPPY || sj.raw || sj.prefix > sj.dst_len || sj.prefix > sj.src_len) return;
+  const uint32_t out = sj.dst_len - sj.prefix, in = sj.src_len - sj.prefix;
+  if (out <= pqi::SNAPPY_SPLIT_MIN || in > 32 + out + out / 6) return;
   sj.nsub = (out + pqi::SNAPPY_FRAGMENT - 1) / pqi::SNAPPY_FRAGMENT;
-  sj.sub = *counter;
-  *counter += sj.nsub;
+  sj.sub = *frags;
+  sj.nseg = (in + pqi::SNAPPY_SEGMENT - 1) / pqi::SNAPPY_SEGMENT;
+  *frags += sj.nsub;
+  *segs += sj.nseg;
 }
 
 pq_status plan_build(pq_ctx* ctx, pq_index* idx, const std::vector<int32_t>& cols, const std::vector<RowSeg>& segs,
@@ -871,7 +878,8 @@ pq_status plan_build(pq_ctx* ctx, pq_index* idx, const std::vector<int32_t>& col
   std::vector<int64_t> data_job_off;  // scratch offset per data snappy job
   std::vector<int64_t> walk_cost;     // estimated chain steps per walked page
   std::vector<int32_t> dict_job_of_chunk(idx->chunks.size(), -1);
-  uint32_t blk_data = 0, blk_dict = 0;  // block slots of split data / dictionary pages
+  uint32_t blk_data = 0, blk_dict = 0;  // fragments of split data / dictionary pages
+  uint32_t seg_data = 0, seg_dict = 0;  // and their input segments
   {
     // at most every indexed page of the requested columns, once per row segment
     size_t np = 0;
@@ -899,6 +907,8 @@ pq_status plan_build(pq_ctx* ctx, pq_index* idx, const std::vector<int32_t>& col
     cw.tc_begin = static_cast<int>(plan->tc_jobs.size());
     cw.blk_data_begin = blk_data;
     cw.blk_dict_begin = blk_dict;
+    cw.seg_data_begin = seg_data;
+    cw.seg_dict_begin = seg_dict;
     cw.copy_only = cm.repetition != 1 && cm.type != pqi::T_BYTE_ARRAY;
     const int max_fixed_before = plan->max_fixed_dict_bytes;
     plan->max_fixed_dict_bytes = 0;
@@ -948,7 +958,7 @@ pq_status plan_build(pq_ctx* ctx, pq_index* idx, const std::vector<int32_t>& col
             sj.dst_len = static_cast<uint32_t>(dp.uncompressed);
             sj.page = cd.dict_page;
             sj.codec = cd.codec;
-            plan_split(sj, plain, &blk_dict);
+            plan_split(sj, plain, &blk_dict, &seg_dict);
             if (cd.codec == pqi::CODEC_ZSTD) plan->zstd_jobs++;
             plan->snappy_dict.push_back(sj);
             dj.body = idx->dict_body[ch];
@@ -1020,11 +1030,11 @@ pq_status plan_build(pq_ctx* ctx, pq_index* idx, const std::vector<int32_t>& col
           sj.prefix = pg.page_type == pqi::PAGE_DATA_V2 ? static_cast<uint32_t>(pg.def_len + pg.rep_len) : 0u;
           sj.page = static_cast<int32_t>(pid);
           sj.codec = cd.codec;
-          plan_split(sj, plain, &blk_data);
+          plan_split(sj, plain, &blk_data, &seg_data);
           if (cd.codec == pqi::CODEC_ZSTD) plan->zstd_jobs++;
           data_job_off.push_back(static_cast<int64_t>(scratch));
           plan->snappy_data.push_back(sj);
-          if (sj.nsub == 0) {  // (split pages are decompressed by blocks)
+          if (sj.nsub == 0) {  // (split pages are decompressed by fragments)
             cw.snap_data_max = std::max<uint32_t>(cw.snap_data_max, sj.src_len);
             plan->snap_data_max = std::max<uint32_t>(plan->snap_data_max, sj.src_len);
           }
@@ -1131,6 +1141,8 @@ pq_status plan_build(pq_ctx* ctx, pq_index* idx, const std::vector<int32_t>& col
     cw.tc_n = static_cast<int>(plan->tc_jobs.size()) - cw.tc_begin;
     cw.blk_data_n = blk_data - cw.blk_data_begin;
     cw.blk_dict_n = blk_dict - cw.blk_dict_begin;
+    cw.seg_data_n = seg_data - cw.seg_data_begin;
+    cw.seg_dict_n = seg_dict - cw.seg_dict_begin;
     cw.max_fixed_dict = plan->max_fixed_dict_bytes;
     plan->max_fixed_dict_bytes = std::max(max_fixed_before, plan->max_fixed_dict_bytes);
     plan->colwork.push_back(cw);
@@ -1150,11 +1162,17 @@ pq_status plan_build(pq_ctx* ctx, pq_index* idx, const std::vector<int32_t>& col
     for (size_t i = 0; i < order.size(); ++i) sorted[i] = plan->walk_pps[order[i]];
     std::copy(sorted.begin(), sorted.end(), plan->walk_pps.begin() + cw.walk_begin);
   }
-  // the block list: data pages' blocks, then dictionary pages' blocks
-  for (auto& sj : plan->snappy_dict)
-    if (sj.nsub > 1) sj.sub += blk_data;
-  for (auto& cw : plan->colwork) cw.blk_dict_begin += blk_data;
+  // the split pages' numbers: data pages, then dictionary pages
+  for (auto& sj : plan->snappy_dict) {
+    sj.sub += sj.nsub > 1 ? blk_data : 0;
+    sj.seg += seg_data;
+  }
+  for (auto& cw : plan->colwork) {
+    cw.blk_dict_begin += blk_data;
+    cw.seg_dict_begin += seg_data;
+  }
   plan->snap_blocks = blk_data + blk_dict;
+  plan->snap_segs = seg_data + seg_dict;
   plan->tc_pool_off = scratch;
   plan->tc_pool_bytes = tc_pool;
   scratch += tc_pool;
@@ -1187,12 +1205,12 @@ pq_status plan_upload(pq_plan* plan, cudaStream_t s) {
   plan->d_items = plan_alloc(pqi::Item, plan, nit);
   plan->d_cols = plan_alloc(pqi::OutCol, plan, plan->outcols.size());
   plan->d_snappy = plan_alloc(pqi::SnappyJob, plan, plan->snappy_data.size() + plan->snappy_dict.size());
-  plan->d_snap_blocks = plan_alloc(pqi::SnappyJob, plan, plan->snap_blocks);
+  plan->d_snap_state = plan_alloc(uint8_t, plan, pqi::snap_state_bytes(plan->snap_blocks, plan->snap_segs));
   plan->d_vpos = plan_alloc(uint32_t, plan, plan->vpos_rows);
   plan->d_dict_jobs = plan_alloc(pqi::DictJob, plan, plan->dict_jobs.size());
   plan->d_tc_jobs = plan_alloc(pqi::TranscodeJob, plan, plan->tc_jobs.size());
   plan->d_str_cols = plan_alloc(int32_t, plan, plan->str_cols.size());
-  plan->d_counter = plan_alloc(uint32_t, plan, 4 + plan->outcols.size());
+  plan->d_counter = plan_alloc(uint32_t, plan, pqi::SCAN_COUNTERS(static_cast<uint32_t>(plan->outcols.size())));
   plan->d_status = plan_alloc(pqi::DevStatus, plan, 1);
   plan->d_scratch = scratch ? plan_alloc(uint8_t, plan, scratch + 64) : nullptr;
   const uint64_t str_rows = static_cast<uint64_t>(plan->n_rows) * plan->str_cols.size();
@@ -1304,7 +1322,7 @@ pq_status plan_upload(pq_plan* plan, cudaStream_t s) {
       for (size_t oc = 0; oc < plan->colwork.size(); ++oc) {
         const auto& cw = plan->colwork[oc];
         const int dk = plan->zstd_jobs ? 2 : 1;  // decompression kernels per job list
-        // (+2 per job list with split pages: the fragment scan and the blocks)
+        // (+2 per job list with split pages: the element scan and the fragments)
         n += (cw.snap_dict_n ? dk + (cw.blk_dict_n ? 2 : 0) : 0) + (cw.dict_n ? 2 : 0) +
              (cw.snap_data_n ? dk + (cw.blk_data_n ? 2 : 0) : 0) + (cw.walk_n ? 1 : 0) +
              (cw.delta_n ? 4 : 0) + (cw.tc_n ? 1 : 0) + (plan->outcols[oc].item_count ? 1 : 0);
@@ -1392,7 +1410,7 @@ uint64_t plan_device_bytes(const pq_plan* plan, uint64_t scratch) {
   const uint64_t npp = plan->pps.size(), nit = plan->n_items;
   const uint64_t str_rows = static_cast<uint64_t>(plan->n_rows) * plan->str_cols.size();
   return npp * sizeof(pqi::PlanPage) + nit * sizeof(pqi::Item) + plan->outcols.size() * sizeof(pqi::OutCol) +
-         (plan->snappy_data.size() + plan->snappy_dict.size() + plan->snap_blocks) * sizeof(pqi::SnappyJob) +
+         (plan->snappy_data.size() + plan->snappy_dict.size()) * sizeof(pqi::SnappyJob) + 56ull * plan->snap_blocks +
          4 * plan->vpos_rows +
          plan->dict_jobs.size() * sizeof(pqi::DictJob) + plan->tc_jobs.size() * sizeof(pqi::TranscodeJob) +
          4 * (plan->walk_pps.size() + plan->delta_pps.size()) +
@@ -1491,27 +1509,44 @@ static void enqueue_transcode(pq_plan* plan, int begin, int n, const pqi::Decode
                         plan->tc_pool_bytes, plan->d_counter, plan->d_vpos, a.st, s);
 }
 
-// Compressed data pages of at least this many bytes (the tuning's
-// snappy_block_kib) are decompressed by a block of 8 warps each (long
-// literals copied by all of them); smaller ones by one warp each.
-// Dictionary pages always take a block.
-static uint32_t coop_snappy_bytes(const pq_plan* plan) {
+// Columns whose largest compressed data page has at least this many bytes
+// (the tuning's snappy_block_kib) are decompressed by blocks of 16 warps,
+// the others by blocks of 4 (more of them resident).  Dictionary pages
+// always take the wide ones.
+static uint32_t wide_snappy_bytes(const pq_plan* plan) {
   return static_cast<uint32_t>(std::min<int64_t>(int64_t(plan->tuning.snappy_block_kib) * 1024, 0xffffffffll));
 }
 
 // Decompression of jobs [jobs, jobs + n): the Snappy kernel takes the Snappy
 // pages, the Zstandard kernel (launched when the plan has any) the others.
-// Split Snappy pages (blocks [blk_begin, blk_begin + blk_n) of the plan's
-// block list) are scanned for their fragments first; their blocks are then
-// decompressed one warp each.
-static void launch_decompress(pq_plan* plan, const pqi::SnappyJob* jobs, int n, uint32_t blk_begin, uint32_t blk_n,
-                              bool coop, pqi::DevStatus* st, cudaStream_t s) {
+static void launch_decompress(pq_plan* plan, const pqi::SnappyJob* jobs, int n, bool wide, pqi::DevStatus* st,
+                              cudaStream_t s) {
   if (n <= 0) return;
   const int n_sms = plan->ctx->n_sms;
-  if (blk_n) pqi::launch_snappy_split(jobs, n, plan->d_snap_blocks, n_sms, st, s);
-  pqi::launch_snappy(jobs, n, n_sms, st, s, coop);
+  pqi::launch_snappy(jobs, n, n_sms, st, s, wide);
   if (plan->zstd_jobs) pqi::launch_zstd(jobs, n, n_sms, st, s);
-  if (blk_n) pqi::launch_snappy(plan->d_snap_blocks + blk_begin, static_cast<int>(blk_n), n_sms, st, s, false);
+}
+
+// The same for the dictionary pages or the data pages of output column oc,
+// whose split Snappy pages are scanned for their fragments first; these are
+// then decompressed by a block each.
+static void launch_column_decompress(pq_plan* plan, size_t oc, bool dicts, pqi::DevStatus* st, cudaStream_t s) {
+  const auto& cw = plan->colwork[oc];
+  const uint32_t n_cols = static_cast<uint32_t>(plan->outcols.size());
+  const pqi::SnappyJob* jobs =
+      plan->d_snappy + (dicts ? plan->snappy_data.size() + cw.snap_dict_begin : static_cast<size_t>(cw.snap_data_begin));
+  const int n = dicts ? cw.snap_dict_n : cw.snap_data_n;
+  const uint32_t blk0 = dicts ? cw.blk_dict_begin : cw.blk_data_begin, nblk = dicts ? cw.blk_dict_n : cw.blk_data_n;
+  const uint32_t seg0 = dicts ? cw.seg_dict_begin : cw.seg_data_begin, nseg = dicts ? cw.seg_dict_n : cw.seg_data_n;
+  if (n <= 0) return;
+  if (nblk) {
+    const int n_sms = plan->ctx->n_sms;
+    const pqi::SnapState ss = pqi::snap_state(plan->d_snap_state, plan->snap_blocks, plan->snap_segs);
+    uint32_t* tickets = plan->d_counter + pqi::SNAP_COUNTER0(n_cols) + pqi::SNAPPY_RUNS * (2 * oc + (dicts ? 1 : 0));
+    pqi::launch_snappy_scan(jobs, n, seg0, nseg, ss, tickets, n_sms, st, s);
+    pqi::launch_snappy_fragments(jobs, static_cast<int>(blk0), static_cast<int>(nblk), ss, n_sms, st, s);
+  }
+  launch_decompress(plan, jobs, n, dicts || cw.snap_data_max >= wide_snappy_bytes(plan), st, s);
 }
 
 // Expansion of one output column: copies (REQUIRED PLAIN fixed width), the
@@ -1545,16 +1580,11 @@ static void launch_column_expand(pq_plan* plan, size_t oc, const pqi::DecodeArgs
 static void enqueue_column(pq_plan* plan, size_t oc, const pqi::DecodeArgs& a, bool with_dicts, cudaStream_t s) {
   pq_ctx* ctx = plan->ctx;
   const auto& cw = plan->colwork[oc];
-  const int n_data_total = static_cast<int>(plan->snappy_data.size());
-  if (with_dicts && cw.snap_dict_n)
-    launch_decompress(plan, plan->d_snappy + n_data_total + cw.snap_dict_begin, cw.snap_dict_n, cw.blk_dict_begin,
-                      cw.blk_dict_n, true, a.st, s);
+  if (with_dicts) launch_column_decompress(plan, oc, true, a.st, s);
   if (with_dicts && cw.dict_n)
     pqi::launch_dict(plan->d_dict_jobs + cw.dict_begin, cw.dict_n, cw.max_fixed_dict, cw.max_str_regions,
                      pqi::DictScratch{plan->d_sregs, plan->d_slists}, plan->idx->d_dicts, ctx->n_sms, a.st, s);
-  if (cw.snap_data_n)
-    launch_decompress(plan, plan->d_snappy + cw.snap_data_begin, cw.snap_data_n, cw.blk_data_begin, cw.blk_data_n,
-                      cw.snap_data_max >= coop_snappy_bytes(plan), a.st, s);
+  launch_column_decompress(plan, oc, false, a.st, s);
   enqueue_transcode(plan, cw.tc_begin, cw.tc_n, a, s);
   const auto& col = plan->outcols[oc];
   pqi::launch_walk(a, cw.walk_begin, cw.walk_n, ctx->n_sms, col.optional != 0, plan->tuning.walk_window, s);
@@ -1587,7 +1617,7 @@ static void enqueue_scan(pq_plan* plan, cudaStream_t s, bool with_dicts, const c
   if (plan->flags & PQ_SCAN_PLAIN) {
     // baseline: per chunk, one launch per stage; one page per thread block
     if (with_dicts && n_dict_jobs)
-      launch_decompress(plan, plan->d_snappy + n_data_jobs, n_dict_jobs, 0, 0, true, a.st, s);
+      launch_decompress(plan, plan->d_snappy + n_data_jobs, n_dict_jobs, true, a.st, s);
     mark(2);
     if (with_dicts && !plan->dict_jobs.empty())
       pqi::launch_dict(plan->d_dict_jobs, static_cast<int>(plan->dict_jobs.size()), plan->max_fixed_dict_bytes,
@@ -1601,7 +1631,7 @@ static void enqueue_scan(pq_plan* plan, cudaStream_t s, bool with_dicts, const c
       for (int p = first; p < first + n; ++p)
         if (job + nj < plan->snappy_data.size() && plan->snappy_data[job + nj].page == static_cast<int32_t>(plan->pps[p].page))
           ++nj;
-      if (nj) launch_decompress(plan, plan->d_snappy + job, nj, 0, 0, plan->snap_data_max >= coop_snappy_bytes(plan), a.st, s);
+      if (nj) launch_decompress(plan, plan->d_snappy + job, nj, plan->snap_data_max >= wide_snappy_bytes(plan), a.st, s);
       job += nj;
       int ntc = 0;
       while (tcj + ntc < plan->tc_jobs.size() && plan->tc_jobs[tcj + ntc].pp < static_cast<uint32_t>(first + n)) ++ntc;
@@ -1616,12 +1646,8 @@ static void enqueue_scan(pq_plan* plan, cudaStream_t s, bool with_dicts, const c
   } else if (timing) {
     for (int oc = 0; oc < ncols; ++oc) {
       const auto& cw = plan->colwork[oc];
-      if (with_dicts && cw.snap_dict_n)
-        launch_decompress(plan, plan->d_snappy + n_data_jobs + cw.snap_dict_begin, cw.snap_dict_n, cw.blk_dict_begin,
-                          cw.blk_dict_n, true, a.st, s);
-      if (cw.snap_data_n)
-        launch_decompress(plan, plan->d_snappy + cw.snap_data_begin, cw.snap_data_n, cw.blk_data_begin, cw.blk_data_n,
-                          cw.snap_data_max >= coop_snappy_bytes(plan), a.st, s);
+      if (with_dicts) launch_column_decompress(plan, oc, true, a.st, s);
+      launch_column_decompress(plan, oc, false, a.st, s);
       enqueue_transcode(plan, cw.tc_begin, cw.tc_n, a, s);
     }
     mark(2);

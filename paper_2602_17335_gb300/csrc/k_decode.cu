@@ -3342,7 +3342,8 @@ __global__ void __launch_bounds__(WALK_THREADS) k_plain_page(DecodeArgs a, int p
 __global__ void k_prepare(DecodeArgs a, int n_cols) {
   const uint64_t tid = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x;
   const uint64_t nthr = static_cast<uint64_t>(gridDim.x) * blockDim.x;
-  if (tid < static_cast<uint64_t>(EXP_COUNTER0 + n_cols)) a.item_counter[tid] = 0;
+  for (uint64_t i = tid; i < static_cast<uint64_t>(SCAN_COUNTERS(n_cols)); i += nthr) a.item_counter[i] = 0;
+  for (uint64_t i = tid; i < a.snap_words; i += nthr) a.snap_state[i] = 0;
   if (tid == 0) {
     a.st->flags = 0;
     a.st->first_page = -1;

@@ -1,4 +1,4 @@
-// K1 — Snappy page decompression, one warp per page.
+// K1 — Snappy page decompression, one thread block per page.
 //
 // Parquet compresses every page body separately with its chunk's codec
 // (paper Section 2; Section 3 "No Unnecessary Compression" weighs its cost).
@@ -6,37 +6,29 @@
 // low two tag bits: a literal (length in the tag, or in 1-4 following
 // bytes) or a copy of `length` bytes from `offset` bytes back in the output
 // (1-, 2- or 4-byte offsets).  Copies are defined byte by byte, so an offset
-// smaller than the length repeats a pattern; output byte i of such a copy is
-// out[start - offset + (i mod offset)], which every lane computes on its own.
+// smaller than the length repeats a pattern.
+//
+// Element headers form a chain: one thread stepping along it takes 250-300
+// cycles an element (64-80 dependent instructions), which used to be the
+// whole cost of element-dense pages.  Here the block computes, for every
+// byte of the staged input window, where the next header would be if a
+// header started there (independent, a dozen instructions a byte), and
+// doubles that map four times; thread 0 then steps 16 elements at a time
+// (one shared load) and the block fills in the rest.  All headers of the
+// batch are decoded together, output positions come from a block scan, and
+// the bytes are produced by lz_run (lz_exec.cuh), which has no order between
+// elements either.  Windows with few elements (literal-heavy pages) are
+// stepped through serially instead: the tables would cost more.  Literals
+// that leave the window go straight from input to output, all warps copying.
 //
 // The compressed page streams through two shared-memory windows filled by
 // the bulk-copy engine (the next window is in flight while the current one
-// is parsed).  Lane 0 parses up to 32 element headers from the window (the
-// tag stream is serial); the warp then executes the batch into a ring of
-// recent output in shared memory -- literals and copies whose source lies
-// before the batch in parallel, one element per lane (long ones by the whole
-// warp), copies that read output of the same batch in order -- and writes
-// the batch's output bytes to global memory with 16-byte stores.  Literals
-// longer than the ring go straight from the input to the output as
-// 16-byte vector copies.  Copy sources older than the ring are read back
-// from the output with coherent loads (this warp wrote them).
+// is decoded).
 #include "dev_util.cuh"
+#include "lz_exec.cuh"
 #include "snappy_job.h"
 
 namespace pqi {
-
-constexpr int kSnappyWarps = 4;     // warps per block
-constexpr uint32_t kRing = 8192;    // recent output kept in shared memory per warp (power of two)
-constexpr uint32_t kWin = 4096;     // input window (two per warp)
-constexpr uint32_t kBatchOut = kRing / 2;  // output bytes of one batch assembled in the ring
-constexpr uint32_t kMidLit = 2048;  // literals up to this long go from the input window through the ring
-
-struct SnWarp {
-  uint64_t bar[2];
-  uint32_t pos[32];      // input offsets of a batch's headers
-  uint8_t win[2][kWin + 16];
-  uint8_t ring[kRing];
-};
 
 // Lane 0's input windows, all scalars (they stay in registers): the current
 // window (*0) and the other one (*1), swapped when the parse moves on.
@@ -162,564 +154,791 @@ __device__ __forceinline__ void sn_bytes5(uint32_t sa, uint32_t* tag, uint32_t* 
   *x = __funnelshift_rc(lo, hi, sh + 8);  // (a shift of 32 gives hi)
 }
 
-// The element whose header sits at input offset p, from its tag and the 4
-// bytes after it, without any check (the element's own decode, or the
-// caller, checks it): the offset of the next header, the output length and
-// the copy offset.  Straight-line code: the header chain is serial, so each
-// step is kept short.
-struct SnStep {
-  uint32_t next, len, arg, kind;
+// A page's block: kThreads threads, kWin bytes per input window.  Two
+// shapes: pages of at least the block threshold take 16 warps and 8 KB
+// windows (a page's latency counts), the many small pages of other files 4
+// warps and 2 KB windows (more of them resident).
+template <int kThreads, uint32_t kWin>
+struct SnShape {
+  static constexpr int kEl = 4 * kThreads < 1024 ? 4 * kThreads : 1024;  // elements of a batch
+  static constexpr int kPer = kEl / kThreads;       // elements a thread decodes
+  static constexpr uint32_t kChunk = kWin > 4096 ? 8192 : 2 * kWin;  // output resolved at a time
+  static constexpr uint32_t kRing = 4 * kChunk;
+  static constexpr uint32_t kOut = 4 * kChunk;      // output of a batch (less its long literal)
 };
-__device__ __forceinline__ SnStep sn_step(uint32_t tag, uint32_t x, uint32_t p) {
-  const uint32_t kind = tag & 3, t6 = tag >> 2;
-  const uint32_t nb = t6 > 59 ? t6 - 59 : 0u;  // literal length bytes after the tag
-  // (a shift by 32 - 8 nb, nb in 1..4: the low nb bytes of x)
-  const uint32_t lv = nb == 0 ? t6 : (x & (0xffffffffu >> ((32 - 8 * nb) & 31)));
-  const uint32_t hl = (0x5320u >> (4 * kind)) & 15u;  // copy header bytes (kind 1, 2, 3: 2, 3, 5)
-  SnStep r;
-  r.kind = kind;
-  r.next = p + (kind == 0 ? 2 + nb + lv : hl);
-  r.len = kind == 0 ? lv + 1 : (kind == 1 ? 4 + (t6 & 7) : t6 + 1);
-  r.arg = kind == 1 ? (((tag >> 5) << 8) | (x & 0xffu)) : (kind == 2 ? (x & 0xffffu) : x);
-  return r;
+// Headers found in a window of kWin bytes, at most kEl of them.
+template <uint32_t kWin, int kEl>
+struct SnHeaders {
+  static constexpr uint32_t kTab = kWin + 16;
+  uint16_t j1[kTab];       // next header after the one at each window byte
+  uint16_t jab[2 * kTab];  // doubled maps
+  uint16_t pos[kEl];       // window offsets of the headers
+  uint16_t hop[kEl / 16];
+  int32_t n, nh;           // headers, hops
+};
+template <int kThreads, uint32_t kWin>
+struct __align__(16) SnBlock {
+  using Sh = SnShape<kThreads, kWin>;
+  uint8_t ring[Sh::kRing];
+  uint8_t win[2][kWin + 32];
+  LzRec rec[Sh::kEl];
+  SnHeaders<kWin, Sh::kEl> h;  // (its doubled maps are lz_run's notes afterwards)
+  uint32_t mask[Sh::kOut / 32 + 2];
+  uint64_t bar[2];
+  uint32_t tmp[32];
+  uint32_t w0, n0, wsel, bad;       // the window of the batch
+  int32_t cut, act;                 // first element not in the batch and why
+  uint32_t total, next;             // output of the batch's elements; input offset after it
+  uint32_t larg, llen;              // the long literal that ends the batch
+  SnIn in;                          // thread 0's window state
+};
+constexpr uint16_t SN_NONE = 0xffffu;  // the next header lies outside the tables
+constexpr uint32_t kAhead = 128 * 1024; // input bytes asked into L2 ahead of a page's position
+constexpr int SN_SERIAL = 64;          // headers per batch on the serial path
+constexpr int SN_DENSE = 24;           // windows with at least this many elements take the tables
+
+// Bytes from a header at a window byte to the next header (its tag and the
+// four bytes after it; nothing is checked: only true headers are, later).
+__device__ __forceinline__ uint32_t sn_advance(uint32_t tag, uint32_t x) {
+  const uint32_t kind = tag & 3;
+  uint32_t adv = kind ? (0x5320u >> (4 * kind)) & 15u : (tag >> 2) + 2;
+  if (kind == 0 && tag >= 240) {  // literal lengths of 1-4 bytes
+    const uint32_t nb = (tag >> 2) - 59;
+    const uint32_t lv = x & (0xffffffffu >> (32 - 8 * nb));
+    adv = (lv < 0xfffffu ? lv : 0xfffffu) + nb + 2;
+  }
+  return adv;
 }
 
-// `n` bytes from ring positions [from, from + n) (positions are output
-// offsets; the ring holds position x at x mod kRing) to global dst, 16-byte
-// stores where the destination allows.
-__device__ __forceinline__ void ring_out(uint8_t* dst, const uint8_t* ring, uint32_t from, uint32_t n, int lane) {
-  constexpr uint32_t RM = kRing - 1;
-  const uint32_t head0 = static_cast<uint32_t>((16 - (reinterpret_cast<uintptr_t>(dst) & 15)) & 15);
-  const uint32_t head = head0 < n ? head0 : n;
-  if (static_cast<uint32_t>(lane) < head) dst[lane] = ring[(from + lane) & RM];
-  const uint32_t nv = (n - head) >> 4;
-  const uint32_t q0 = from + head;
-  if ((q0 & 15) == 0) {
-    // ring slots congruent with the destination: whole 16-byte ring words
-    for (uint32_t v = lane; v < nv; v += 32)
-      *reinterpret_cast<uint4*>(dst + head + 16 * v) = *reinterpret_cast<const uint4*>(ring + ((q0 + 16 * v) & RM));
-  } else {
-    for (uint32_t v = lane; v < nv; v += 32) {
-      const uint32_t q = q0 + 16 * v;
-      uint32_t w4[4];
+// Headers of window bytes [q0, L) from the one at q0 on, into S.pos (at most
+// kEl; the last one found may lead past L).  Block-collective; ends with a
+// barrier.
+template <int kThreads, uint32_t kWin, int kEl>
+__device__ void sn_find_headers(SnHeaders<kWin, kEl>& S, const uint8_t* wb, uint32_t q0, uint32_t L, bool dense) {
+  using H = SnHeaders<kWin, kEl>;
+  if (!dense) {
+    if (threadIdx.x == 0) {
+      int nb = 0;
+      uint32_t q = q0;
+      const uint32_t sb = smem_u32(wb);
+      while (nb < SN_SERIAL) {
+        S.pos[nb++] = static_cast<uint16_t>(q);
+        uint32_t tag, x;
+        sn_bytes5(sb + q, &tag, &x);
+        q += sn_advance(tag, x);
+        if (q >= L) break;
+      }
+      S.n = nb;
+    }
+    __syncthreads();
+    return;
+  }
+  const uint32_t* w32 = reinterpret_cast<const uint32_t*>(wb);
+  constexpr int G = (kWin / 4 + kThreads - 1) / kThreads;  // groups of four window bytes per thread
+  const uint32_t g0 = (q0 >> 2) + threadIdx.x;
+  {
+    uint32_t a[G], b[G];
+#pragma unroll
+    for (int i = 0; i < G; ++i) {
+      const uint32_t g = g0 + i * kThreads;
+      a[i] = 4 * g < L ? w32[g] : 0u;
+      b[i] = 4 * g < L ? w32[g + 1] : 0u;
+    }
+#pragma unroll
+    for (int i = 0; i < G; ++i) {
+      const uint32_t g = g0 + i * kThreads;
+      uint32_t v[4];
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        const uint32_t b = q + 4 * k;
-        w4[k] = static_cast<uint32_t>(ring[b & RM]) | (static_cast<uint32_t>(ring[(b + 1) & RM]) << 8) |
-                (static_cast<uint32_t>(ring[(b + 2) & RM]) << 16) | (static_cast<uint32_t>(ring[(b + 3) & RM]) << 24);
+        const uint32_t tag = (a[i] >> (8 * k)) & 0xffu;
+        const uint32_t x = k == 3 ? b[i] : __funnelshift_r(a[i], b[i], 8 * (k + 1));
+        const uint32_t nx = 4 * g + k + sn_advance(tag, x);
+        v[k] = nx < L ? nx : SN_NONE;
       }
-      *reinterpret_cast<uint4*>(dst + head + 16 * v) = make_uint4(w4[0], w4[1], w4[2], w4[3]);
+      if (4 * g < L) *reinterpret_cast<uint2*>(S.j1 + 4 * g) = make_uint2(v[0] | (v[1] << 16), v[2] | (v[3] << 16));
     }
   }
-  for (uint32_t i = head + (nv << 4) + lane; i < n; i += 32) dst[i] = ring[(from + i) & RM];
+  __syncthreads();
+  const uint16_t* src = S.j1;
+#pragma unroll 1
+  for (int r = 0; r < 4; ++r) {  // 2, 4, 8, 16 elements
+    uint16_t* dst = S.jab + ((r & 1) ? H::kTab : 0u);
+    uint2 m[G];
+#pragma unroll
+    for (int i = 0; i < G; ++i) {
+      const uint32_t g = g0 + i * kThreads;
+      m[i] = 4 * g < L ? *reinterpret_cast<const uint2*>(src + 4 * g) : make_uint2(0xffffffffu, 0xffffffffu);
+    }
+#pragma unroll
+    for (int i = 0; i < G; ++i) {
+      const uint32_t h[4] = {m[i].x & 0xffffu, m[i].x >> 16, m[i].y & 0xffffu, m[i].y >> 16};
+      uint32_t v[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) v[k] = h[k] == SN_NONE ? SN_NONE : src[h[k]];
+      m[i] = make_uint2(v[0] | (v[1] << 16), v[2] | (v[3] << 16));
+    }
+#pragma unroll
+    for (int i = 0; i < G; ++i) {
+      const uint32_t g = g0 + i * kThreads;
+      if (4 * g < L) *reinterpret_cast<uint2*>(dst + 4 * g) = m[i];
+    }
+    __syncthreads();
+    src = dst;
+  }
+  if (threadIdx.x == 0) {
+    int nb = 0, nh = 0;
+    uint32_t q = q0, nx = src[q];
+    while (nb + 16 <= kEl && nx != SN_NONE) {
+      S.hop[nh++] = static_cast<uint16_t>(q);
+      nb += 16;
+      q = nx;
+      nx = src[q];
+    }
+    while (nb < kEl) {
+      nx = S.j1[q];
+      S.pos[nb++] = static_cast<uint16_t>(q);
+      if (nx == SN_NONE) break;
+      q = nx;
+    }
+    S.n = nb;
+    S.nh = nh;
+  }
+  __syncthreads();
+  for (int h = threadIdx.x; h < S.nh; h += kThreads) {
+    uint32_t q = S.hop[h];
+#pragma unroll 4
+    for (int k = 0; k < 16; ++k) {
+      const uint32_t nx = S.j1[q];
+      S.pos[16 * h + k] = static_cast<uint16_t>(q);
+      q = nx;
+    }
+  }
+  __syncthreads();
 }
 
-// A short literal (len <= 64) from global input to the ring: its aligned
-// 16-byte words are loaded together, then placed byte by byte.
-__device__ __forceinline__ void lit_to_ring(uint8_t* ring, uint32_t o0, const uint8_t* src, uint32_t len) {
-  constexpr uint32_t RM = kRing - 1;
-  const uint32_t sh = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(src) & 15);
-  const uint4* sv = reinterpret_cast<const uint4*>(src - sh);
-  const uint32_t nv = (sh + len + 15) >> 4;  // <= 5
-  uint4 v[5];
-#pragma unroll
-  for (int k = 0; k < 5; ++k) v[k] = static_cast<uint32_t>(k) < nv ? __ldg(sv + k) : make_uint4(0, 0, 0, 0);
-  // every byte position of the five words is a constant: registers only
-#pragma unroll
-  for (int k = 0; k < 5; ++k) {
-    const uint32_t wk[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
-#pragma unroll
-    for (int b = 0; b < 16; ++b) {
-      const uint32_t q = 16u * k + b;
-      if (q >= sh && q < sh + len) ring[(o0 + q - sh) & RM] = static_cast<uint8_t>(wk[b >> 2] >> (8 * (b & 3)));
-    }
-  }
-}
-
-// Input bytes src[0, n) to ring positions [pos0, pos0 + n): whole 16-byte
-// ring words built from two aligned source words, the partial words at the
-// two ends byte by byte.
-__device__ __forceinline__ void ring_fill(uint8_t* ring, uint32_t pos0, const uint8_t* src, uint32_t n, int lane) {
-  constexpr uint32_t RM = kRing - 1;
-  const uint32_t head0 = (16 - (pos0 & 15)) & 15;
-  const uint32_t head = head0 < n ? head0 : n;
-  if (static_cast<uint32_t>(lane) < head) ring[(pos0 + lane) & RM] = __ldg(src + lane);
-  const uint32_t nv = (n - head) >> 4;
-  const uint8_t* s1 = src + head;
-  const uint32_t sh = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(s1) & 15);
-  const uint4* sa = reinterpret_cast<const uint4*>(s1 - sh);
-  for (uint32_t v = lane; v < nv; v += 32) {
-    const uint4 A = __ldg(sa + v);
-    const uint4 B = sh ? __ldg(sa + v + 1) : A;
-    *reinterpret_cast<uint4*>(ring + ((pos0 + head + 16 * v) & RM)) = sh ? shift_pair(A, B, sh) : A;
-  }
-  for (uint32_t i = head + (nv << 4) + lane; i < n; i += 32) ring[(pos0 + i) & RM] = __ldg(src + i);
-}
-
-// A cooperative copy request from warp 0 to the other warps of its block.
-struct SnCoop {
-  uint8_t* dst;
-  const uint8_t* src;
-  uint32_t len;  // 0: the page is done
-  uint32_t pad;
-};
-
-__device__ __forceinline__ void coop_bar() { asm volatile("bar.sync 1, %0;" ::"r"(32 * 8) : "memory"); }
-
-// Slice w of 8 of a copy (16-byte aligned destination boundaries).
-__device__ __forceinline__ void coop_slice(const SnCoop& c, int w, int lane) {
-  const uint64_t per = ((static_cast<uint64_t>(c.len) + 8 * 16 - 1) / (8 * 16)) * 16;
-  const uint64_t b = per * w, e = b + per < c.len ? b + per : c.len;
-  if (b < e) warp_copy<true>(c.dst + b, c.src + b, e - b, lane);
-}
-
-// kCoop: one block of 8 warps per page; warp 0 parses and executes, and the
-// literals of at least kCoopLit bytes are copied by all 8 warps.  Otherwise
-// one warp per page.
-constexpr uint32_t kCoopLit = 4096;
-
-template <bool kCoop>
-__global__ void __launch_bounds__(kCoop ? 256 : 32 * kSnappyWarps) k_snappy(const SnappyJob* __restrict__ jobs,
-                                                                            int n_jobs, DevStatus* st) {
-  extern __shared__ __align__(16) uint8_t sn_smem[];
-  const int lane = threadIdx.x & 31;
-  SnWarp& sw = reinterpret_cast<SnWarp*>(sn_smem)[kCoop ? 0 : threadIdx.x >> 5];
-  SnCoop& cq = *reinterpret_cast<SnCoop*>(sn_smem + sizeof(SnWarp) * (kCoop ? 1 : kSnappyWarps));
-  const int wid = kCoop ? blockIdx.x : (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int nwarps = kCoop ? gridDim.x : (gridDim.x * blockDim.x) >> 5;
-  if (kCoop && threadIdx.x >= 32) {
-    // helper warps: slices of warp 0's long literals until it says the page is done
-    for (int j = wid; j < n_jobs; j += nwarps) {
-      for (;;) {
-        coop_bar();
-        const SnCoop c = cq;
-        if (c.len == 0) break;
-        coop_slice(c, threadIdx.x >> 5, lane);
-        coop_bar();
-      }
-    }
-    return;
-  }
-  if (lane == 0) {
-    mbar_init(&sw.bar[0], 1);
-    mbar_init(&sw.bar[1], 1);
-  }
-  fence_mbar_init();
-  __syncwarp();
-  uint32_t par[2] = {0, 0};
-  uint8_t* ring = sw.ring;
-  constexpr uint32_t RM = kRing - 1;
-  auto page_done = [&]() {
-    if (kCoop) {
-      if (lane == 0) cq.len = 0;
-      __syncwarp();
-      coop_bar();
-    }
-  };
-  for (int j = wid; j < n_jobs; j += nwarps) {
-    const SnappyJob jb = jobs[j];
-    if (jb.codec != CODEC_SNAPPY || jb.nsub > 1) {  // another codec's kernel, or the page's blocks, take it
-      page_done();
-      continue;
-    }
-    if (jb.prefix > jb.src_len || jb.prefix > jb.dst_len) {
-      if (lane == 0) report(st, DERR_CORRUPT, jb.page, WHERE_SNAPPY, 1);
-      page_done();
-      continue;
-    }
-    warp_copy<true>(jb.dst, jb.src, jb.prefix, lane);  // V2 level bytes, never compressed
-    if (jb.raw) {
-      if (jb.src_len != jb.dst_len) {
-        if (lane == 0) report(st, DERR_CORRUPT, jb.page, WHERE_SNAPPY, 2);
-        page_done();
-        continue;
-      }
-      warp_copy<true>(jb.dst + jb.prefix, jb.src + jb.prefix, jb.src_len - jb.prefix, lane);
-      __syncwarp();
-      page_done();
-      continue;
-    }
-    const uint8_t* in = jb.src + jb.prefix;
-    const uint32_t in_len = jb.src_len - jb.prefix;
-    uint8_t* out = jb.dst + jb.prefix;
-    const uint32_t out_len = jb.dst_len - jb.prefix;
-    uint64_t declared = out_len;
-    int pl = 0;  // a block of a split page has no length preamble
-    if (!(jb.flags & SJ_BLOCK)) {
-      pl = uleb([&](uint32_t k) { return static_cast<uint32_t>(__ldg(in + k)); }, 0, in_len, &declared);
-      if (pl == 0 || declared != out_len) {
-        if (lane == 0) report(st, DERR_CORRUPT, jb.page, WHERE_SNAPPY, 3);
-        page_done();
-        continue;
-      }
-    }
-    // lane 0's window state
-    SnIn sin{in, in_len, sw.win[0], sw.win[1], &sw.bar[0], &sw.bar[1], 0, 0, 0, 0, par[0], par[1], 0, kWin};
-    int bad = 0;
-    if (lane == 0) {
-      sn_issue(sin, sin.b0, sin.m0, 0, &sin.w0, &sin.n0);
-      if (!mbar_wait(sin.m0, sin.p0)) bad = 2;
-      sin.p0 ^= 1u;
-      if (!bad) sn_prefetch(sin);
-    }
-    uint32_t ip = static_cast<uint32_t>(pl);
-    uint32_t op = 0;
-    bad = __shfl_sync(0xffffffffu, bad, 0);
-    // each element consumes >= 2 input bytes, so in_len bounds the batches
-    for (uint32_t guard = 0; guard <= in_len && ip < in_len && !bad; ++guard) {
-      // the batch's window: switched now when ip has left window 0 (a batch's
-      // headers and window literals all sit in one window)
-      if (lane == 0) {
-        const bool here = ip - sin.w0 < sin.n0 && (ip - sin.w0 + 5 <= sin.n0 || sin.w0 + sin.n0 >= in_len);
-        if (!here && !sn_ensure(sin, ip)) bad = 2;
-      }
-      bad = __shfl_sync(0xffffffffu, bad, 0);
-      if (bad) break;
-      const uint8_t* wbuf = sw.win[__shfl_sync(0xffffffffu, lane == 0 && sin.b0 == sw.win[1] ? 1 : 0, 0)];
-      const uint32_t w0 = __shfl_sync(0xffffffffu, sin.w0, 0), n0 = __shfl_sync(0xffffffffu, sin.n0, 0);
-      // lane 0 follows the header chain to up to 32 headers inside the window;
-      // it stops after an element that ends the batch anyway (a literal that
-      // is long or runs past the window, the output budget) or does not parse
-      // (its own lane reports it)
-      int n_pos = 0;
-      if (lane == 0) {
-        uint32_t p = ip, ob = 0;
-        const uint32_t lim = w0 + n0 >= in_len ? n0 : n0 - 4;  // offsets whose header bytes are all here
-        const uint32_t sb = smem_u32(wbuf) - w0;  // shared address of input offset x: sb + x
-        while (n_pos < 32 && p < in_len) {
-          if (p - w0 >= lim) break;
-          sw.pos[n_pos++] = p;
-          uint32_t tag, x;
-          sn_bytes5(sb + p, &tag, &x);
-          const SnStep e = sn_step(tag, x, p);
-          ob += e.len;
-          if (e.next <= p || e.next > in_len || ob >= kBatchOut - 64 ||
-              (e.kind == 0 && (e.len > kMidLit || e.next - w0 > n0)))
-            break;
-          p = e.next;
-        }
-      }
-      __syncwarp();
-      n_pos = __shfl_sync(0xffffffffu, n_pos, 0);
-      // every lane decodes its header from the window
-      uint32_t kind = 0, len = 0, arg = 0, nextp = 0;
-      bool hok = true;
-      if (lane < n_pos) {
-        const uint32_t mypos = sw.pos[lane];
-        uint32_t tag, x;
-        sn_bytes5(smem_u32(wbuf) + (mypos - w0), &tag, &x);
-        hok = sn_hdr(tag, x, mypos, in_len, &kind, &len, &arg, &nextp);
-      }
-      // output offsets; the batch ends after its first element that fills the
-      // ring's budget or is a literal outside the window (copied directly)
-      const uint32_t plen = lane < n_pos ? len : 0u;
-      uint32_t pinc = plen;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, pinc, o);
-        if (lane >= o) pinc += y;
-      }
-      const bool inwin = kind == 0 && len <= kMidLit && arg - w0 + len <= n0;
-      const bool trig = lane < n_pos && (!hok || pinc >= kBatchOut - 64 || (kind == 0 && !inwin));
-      const uint32_t tm = __ballot_sync(0xffffffffu, trig);
-      const int n_el = tm ? __ffs(tm) : n_pos;
-      const uint32_t o_e = op + pinc - plen;
-      const bool evalid = hok && len <= out_len - o_e && (kind == 0 || (arg != 0 && arg <= o_e));
-      if (n_el == 0 || __any_sync(0xffffffffu, lane < n_el && !evalid)) {
-        bad = 1;
-        break;
-      }
-      ip = __shfl_sync(0xffffffffu, nextp, n_el - 1);
-      int32_t woff = -1;
-      if (lane < n_el && inwin) woff = static_cast<int32_t>(arg - w0);
-      if (lane >= n_el) kind = len = arg = 0;
-      uint32_t incl = len;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += y;
-      }
-      const uint32_t o0 = op + incl - len;  // this lane's element output offset
-      const uint32_t btot = __shfl_sync(0xffffffffu, incl, 31);
-      const uint32_t bend = op + btot;
-      // the ring holds positions [max(0, op - (kRing - btot)), op) before the
-      // batch and gets [op, bend); sources below `rlo` come from global memory
-      const uint32_t keep = btot <= kRing ? kRing - btot : 0u;
-      const uint32_t rlo = op > keep ? op - keep : 0u;
-      const bool valid = lane < n_el;
-      // long literals (the batch's last element): global to global, the
-      // tail into the ring
-      const bool longlit = valid && kind == 0 && woff < 0;
-      const bool indep = valid && !longlit && (kind == 0 || (arg >= len && o0 - arg + len <= op));
-      auto src_byte = [&](uint32_t pos) -> uint8_t {
-        return pos >= rlo ? ring[pos & RM] : ld_src<false>(out + pos);
-      };
-      if (indep) {
-        if (kind == 0 && len <= 32) {
-          for (uint32_t i = 0; i < len; ++i) ring[(o0 + i) & RM] = wbuf[woff + i];
-        } else if (kind == 0) {
-          // longer literals from the window: by the whole warp, below
-        } else {
-          const uint32_t first = o0 - arg;
-          uint32_t i = 0;
-          for (; i + 4 <= len; i += 4) {  // four independent reads in flight
-            const uint8_t c0 = src_byte(first + i), c1 = src_byte(first + i + 1), c2 = src_byte(first + i + 2),
-                          c3 = src_byte(first + i + 3);
-            ring[(o0 + i) & RM] = c0;
-            ring[(o0 + i + 1) & RM] = c1;
-            ring[(o0 + i + 2) & RM] = c2;
-            ring[(o0 + i + 3) & RM] = c3;
+// One Snappy element stream: in[ip, in_len) into out[0, out_len), which no
+// copy reaches out of.  par: thread 0's phase parities of the window barriers.
+template <int kThreads, uint32_t kWin>
+__device__ __forceinline__ void sn_decode(SnBlock<kThreads, kWin>& S, const uint8_t* in, uint32_t ip, uint32_t in_len, uint8_t* out,
+                          uint32_t out_len, uint32_t* par, int page, DevStatus* st) {
+  using Sh = SnShape<kThreads, kWin>;
+  const int tid = threadIdx.x;
+      const uint32_t va = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(out) & 31);
+      uint8_t* vout = out - va;
+      // thread 0's window state
+      SnIn& sin = S.in;
+      if (tid == 0) sin = SnIn{in, in_len, S.win[0], S.win[1], &S.bar[0], &S.bar[1], 0, 0, 0, 0, par[0], par[1], 0, kWin};
+      bool loaded = false, lost = false;  // thread 0's: the first window was asked for; a copy never arrived
+      uint32_t op = 0;
+      int bad = 0;         // 1 malformed, 2 a copy never arrived
+      bool dense = false;  // the last window held many elements
+      uint32_t vfloor = 0; // the ring holds nothing below this position
+      uint32_t fetched = 0;  // input asked into L2 ahead of the windows
+      // each element consumes >= 2 input bytes, so in_len bounds the batches
+      for (uint32_t guard = 0; guard <= in_len && ip < in_len; ++guard) {
+        if (tid == 0) {
+          bool ok = true;
+          if (!loaded) {
+            sn_issue(sin, sin.b0, sin.m0, ip, &sin.w0, &sin.n0);
+            ok = mbar_wait(sin.m0, sin.p0);
+            sin.p0 ^= 1u;
+            if (ok) sn_prefetch(sin);
+            loaded = true;
+          } else {
+            ok = !lost && sn_ensure(sin, ip);
           }
-          for (; i < len; ++i) ring[(o0 + i) & RM] = src_byte(first + i);
+          S.bad = ok ? 0u : 2u;
+          S.w0 = sin.w0;
+          S.n0 = sin.n0;
+          S.wsel = sin.b0 == S.win[1] ? 1u : 0u;
+          S.cut = Sh::kEl;
+          S.act = 0;
+          S.total = 0;
         }
-      }
-      __syncwarp();
-      for (uint32_t m = __ballot_sync(0xffffffffu, indep && kind == 0 && len > 32); m; m &= m - 1) {
-        const int e = __ffs(m) - 1;
-        const uint32_t el = __shfl_sync(0xffffffffu, len, e), eo = __shfl_sync(0xffffffffu, o0, e);
-        const int32_t ew = __shfl_sync(0xffffffffu, woff, e);
-        for (uint32_t i = lane; i < el; i += 32) ring[(eo + i) & RM] = wbuf[ew + i];
-      }
-      __syncwarp();
-      for (uint32_t m = __ballot_sync(0xffffffffu, valid && !indep && !longlit); m; m &= m - 1) {
-        const int e = __ffs(m) - 1;
-        const uint32_t el = __shfl_sync(0xffffffffu, len, e);
-        const uint32_t ea = __shfl_sync(0xffffffffu, arg, e), eo = __shfl_sync(0xffffffffu, o0, e);
-        const uint32_t first = eo - ea;
-        for (uint32_t i0 = 0; i0 < el; i0 += 32) {
-          const uint32_t i = i0 + lane;
-          uint8_t b = 0;
-          if (i < el) b = src_byte(ea >= el ? first + i : first + (i % ea));
-          __syncwarp();
-          if (i < el) ring[(eo + i) & RM] = b;
-          __syncwarp();
+        for (uint32_t w = tid; w < Sh::kOut / 32 + 2; w += kThreads) S.mask[w] = 0;
+        while (fetched < in_len && fetched < ip + kAhead) {
+          if (fetched + 128 * tid < in_len)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(in + fetched + 128 * tid));
+          fetched += 128 * kThreads;
         }
-      }
-      const uint32_t lm = __ballot_sync(0xffffffffu, longlit);
-      // the batch's short output, ring -> global
-      const uint32_t short_end = lm ? __shfl_sync(0xffffffffu, o0, __ffs(lm) - 1) : bend;
-      if (short_end > op) ring_out(out + op, ring, op, short_end - op, lane);
-      __syncwarp();  // the ring's short bytes are out before a long literal's tail overwrites slots
-      if (lm) {
-        const int e = __ffs(lm) - 1;
-        const uint32_t el = __shfl_sync(0xffffffffu, len, e);
-        const uint32_t ea = __shfl_sync(0xffffffffu, arg, e), eo = __shfl_sync(0xffffffffu, o0, e);
-        if (kCoop && el >= kCoopLit) {
-          if (lane == 0) cq = SnCoop{out + eo, in + ea, el, 0};
-          __syncwarp();
-          coop_bar();
-          coop_slice(SnCoop{out + eo, in + ea, el, 0}, 0, lane);
-          coop_bar();
-        } else {
-          warp_copy<true>(out + eo, in + ea, el, lane);
-        }
-        const uint32_t t0 = el > kRing ? el - kRing : 0u;
-        ring_fill(ring, eo + t0, in + ea + t0, el - t0, lane);
-      }
-      __syncwarp();
-      op = bend;
-    }
-    if (lane == 0) {
-      // settle the window copy still in flight before the buffers are reused
-      if (sin.e1) {
-        mbar_wait(sin.m1, sin.p1);
-        sin.p1 ^= 1u;
-        sin.e1 = 0;
-      }
-      if (bad == 2) report(st, DERR_TIMEOUT, jb.page, WHERE_SNAPPY, 5);
-      else if (bad || op != out_len || ip != in_len) report(st, DERR_CORRUPT, jb.page, WHERE_SNAPPY, 4);
-    }
-    // carry the physical buffers' parities to the next page
-    const bool sw0 = sin.b0 == sw.win[0];
-    par[0] = __shfl_sync(0xffffffffu, sw0 ? sin.p0 : sin.p1, 0);
-    par[1] = __shfl_sync(0xffffffffu, sw0 ? sin.p1 : sin.p0, 0);
-    __syncwarp();
-    page_done();
-  }
-}
-
-// Fragment scan of the split pages: lane 0 of a warp follows a page's
-// element headers through two shared-memory windows (as the decoder does,
-// wider) and cuts a block wherever the output reaches a multiple of
-// SNAPPY_FRAGMENT at an element boundary.  A copy whose source lies before
-// its block's start, or anything the decoder would reject, makes the page
-// one job again (decompressed whole, where the decoder reports what is
-// wrong).  The blocks go to the plan's block list at the page's slots; slots
-// the page does not use become no-op jobs.
-constexpr uint32_t kSplitWin = 8192;
-constexpr int kSplitWarps = 4;
-struct SnSplitWarp {
-  uint64_t bar[2];
-  uint8_t win[2][kSplitWin + 16];
-};
-
-__global__ void __launch_bounds__(32 * kSplitWarps) k_snappy_split(const SnappyJob* __restrict__ jobs, int n_jobs,
-                                                                   SnappyJob* blocks, DevStatus* st) {
-  extern __shared__ __align__(16) uint8_t sp_smem[];
-  const int lane = threadIdx.x & 31;
-  SnSplitWarp& sw = reinterpret_cast<SnSplitWarp*>(sp_smem)[threadIdx.x >> 5];
-  const int wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int nwarps = (gridDim.x * blockDim.x) >> 5;
-  if (lane == 0) {
-    mbar_init(&sw.bar[0], 1);
-    mbar_init(&sw.bar[1], 1);
-  }
-  fence_mbar_init();
-  __syncwarp();
-  uint32_t par[2] = {0, 0};
-  for (int j = wid; j < n_jobs; j += nwarps) {
-    const SnappyJob jb = jobs[j];
-    if (jb.codec != CODEC_SNAPPY || jb.nsub <= 1) continue;
-    const bool shape = !jb.raw && jb.prefix <= jb.src_len && jb.prefix <= jb.dst_len;
-    if (shape) warp_copy<true>(jb.dst, jb.src, jb.prefix, lane);  // V2 level bytes, never compressed
-    if (lane == 0) {
-      const uint8_t* in = jb.src + jb.prefix;
-      uint8_t* out = jb.dst + jb.prefix;
-      const uint32_t in_len = shape ? jb.src_len - jb.prefix : 0u;
-      const uint32_t out_len = shape ? jb.dst_len - jb.prefix : 0u;
-      SnappyJob* bl = blocks + jb.sub;
-      auto emit = [&](uint32_t q, uint32_t i0, uint32_t i1, uint32_t o0, uint32_t o1) {
-        SnappyJob b{};
-        b.src = in + i0;
-        b.dst = out + o0;
-        b.src_len = i1 - i0;
-        b.dst_len = o1 - o0;
-        b.page = jb.page;
-        b.codec = CODEC_SNAPPY;
-        b.flags = SJ_BLOCK;
-        bl[q] = b;
-      };
-      auto empty = [&](uint32_t q) {
-        SnappyJob b{};
-        b.page = jb.page;
-        bl[q] = b;  // codec 0: no kernel takes it
-      };
-      uint64_t declared = 0;
-      int pl = 0;
-      bool ok = shape;
-      if (ok) {
-        pl = uleb([&](uint32_t k) { return static_cast<uint32_t>(__ldg(in + k)); }, 0, in_len, &declared);
-        ok = pl != 0 && declared == out_len;
-      }
-      SnIn sin{in, in_len, sw.win[0], sw.win[1], &sw.bar[0], &sw.bar[1], 0, 0, 0, 0, par[0], par[1], 0, kSplitWin};
-      bool loaded = false, timeout = false;
-      if (ok) {
-        sn_issue(sin, sin.b0, sin.m0, 0, &sin.w0, &sin.n0);
-        loaded = true;
-        if (!mbar_wait(sin.m0, sin.p0)) timeout = true;
-        sin.p0 ^= 1u;
-        if (!timeout) sn_prefetch(sin);
-        ok = !timeout;
-      }
-      uint32_t p = static_cast<uint32_t>(pl), o = 0, k = 0, bi = p, bo = 0;
-      uint32_t next_cut = SNAPPY_FRAGMENT;
-      uint32_t sb = smem_u32(sin.b0) - sin.w0;  // shared address of input offset x: sb + x
-      // offsets below plim have all their header bytes in window 0 (the
-      // window test is one compare per element)
-      auto window_end = [&]() {
-        const uint32_t e = sin.w0 + sin.n0;
-        return sin.w0 + sin.n0 >= in_len ? in_len : e - 4;
-      };
-      uint32_t plim = ok ? window_end() : 0u;
-      // each element consumes >= 2 input bytes
-      for (uint32_t guard = 0; ok && p < in_len && guard <= in_len; ++guard) {
-        if (p - sin.w0 >= plim - sin.w0) {
-          if (!sn_ensure(sin, p)) {
-            timeout = true;
-            ok = false;
-            break;
-          }
-          sb = smem_u32(sin.b0) - sin.w0;
-          plim = window_end();
-        }
-        uint32_t tag, x;
-        sn_bytes5(sb + p, &tag, &x);
-        const SnStep e = sn_step(tag, x, p);
-        // the element's bytes are in the input (no wrap, a literal's length
-        // below 2^32); a copy's source lies in its block; the output stays
-        // inside the page
-        if ((e.next - p - 1) >= in_len - p || e.len - 1 >= out_len - o || (e.kind != 0 && e.arg - 1 >= o - bo)) {
-          ok = false;
+        __syncthreads();
+        if (S.bad) {
+          bad = 2;
           break;
         }
-        o += e.len;
-        p = e.next;
-        if (o >= next_cut && o < out_len) {
-          const uint32_t nk = o / SNAPPY_FRAGMENT;
-          if (nk >= jb.nsub) {
-            ok = false;
-            break;
+        const uint32_t w0 = S.w0, n0 = S.n0;
+        const uint8_t* wb = S.win[S.wsel];
+        const uint32_t q0 = ip - w0;
+        const uint32_t L = w0 + n0 >= in_len ? in_len - w0 : n0 - 4;  // headers below L have all their bytes here
+        sn_find_headers<kThreads>(S.h, wb, q0, L, dense);
+        const int n = S.h.n;
+        dense = n >= SN_DENSE;
+        // the warp's elements: `seg` in a row, lane l the (32 u + l)-th (src: a
+        // literal's input offset | LZ_LIT, or a copy's back offset; len 0:
+        // malformed)
+        constexpr int kWarps = kThreads / 32;
+        const int lane = tid & 31, warp = tid >> 5;
+        const int seg = 32 * ((n + 32 * kWarps - 1) / (32 * kWarps));
+        uint32_t len[Sh::kPer], src[Sh::kPer], at[Sh::kPer];
+        uint32_t run = 0;
+  #pragma unroll
+        for (int u = 0; u < Sh::kPer; ++u) {
+          const int e = warp * seg + 32 * u + lane;
+          len[u] = src[u] = 0;
+          if (32 * u < seg && e < n) {
+            uint32_t tag, x, kind, nx;
+            sn_bytes5(smem_u32(wb) + S.h.pos[e], &tag, &x);
+            if (!sn_hdr(tag, x, w0 + S.h.pos[e], in_len, &kind, &len[u], &src[u], &nx)) len[u] = 0;
+            else if (kind == 0) src[u] |= LZ_LIT;
+            else if (src[u] & LZ_LIT) len[u] = 0;  // an offset of 2 GB or more is past any output
           }
-          emit(k, bi, p, bo, o);
-          for (uint32_t e2 = k + 1; e2 < nk; ++e2) empty(e2);
-          k = nk;
-          bi = p;
-          bo = o;
-          next_cut = (k + 1) * SNAPPY_FRAGMENT;
+        }
+  #pragma unroll
+        for (int u = 0; u < Sh::kPer; ++u) {
+          uint32_t incl = len[u];
+  #pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+          }
+          at[u] = run + incl - len[u];
+          run += __shfl_sync(0xffffffffu, incl, 31);
+        }
+        if (lane == 0) S.tmp[warp] = run;
+        __syncthreads();
+        {
+          const uint32_t tv = lane < kWarps ? S.tmp[lane] : 0u;
+          uint32_t incl = tv;
+  #pragma unroll
+          for (int o = 1; o < kWarps; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+          }
+          const uint32_t base = __shfl_sync(0xffffffffu, incl - tv, warp);
+  #pragma unroll
+          for (int u = 0; u < Sh::kPer; ++u) at[u] += base;
+        }
+        // the batch ends before its first element that is malformed, is a
+        // literal reaching past the window, or exceeds the batch's output
+        auto valid = [&](uint32_t o, uint32_t l, uint32_t sr) {
+          const uint32_t p = op + o;
+          return l != 0 && p <= out_len && l <= out_len - p && ((sr & LZ_LIT) || (sr != 0 && sr <= p));
+        };
+        auto longlit = [&](uint32_t l, uint32_t sr) { return (sr & LZ_LIT) && ((sr & ~LZ_LIT) - w0) + l > n0; };
+  #pragma unroll
+        for (int u = 0; u < Sh::kPer; ++u) {
+          const int e = warp * seg + 32 * u + lane;
+          const bool in_list = 32 * u < seg && e < n;
+          const bool stop = in_list && (!valid(at[u], len[u], src[u]) || longlit(len[u], src[u]) ||
+                                        at[u] + len[u] > Sh::kOut - 32);
+          const uint32_t b = __ballot_sync(0xffffffffu, stop);
+          if (b && lane == 0) atomicMin(&S.cut, warp * seg + 32 * u + __ffs(b) - 1);
+        }
+        __syncthreads();
+        const int ne = S.cut < n ? S.cut : n;
+        const uint32_t vb = va + op;
+  #pragma unroll
+        for (int u = 0; u < Sh::kPer; ++u) {
+          const int e = warp * seg + 32 * u + lane;
+          if (32 * u < seg && e < n) {
+            if (e < ne) {
+              const uint32_t a = vb + at[u];
+              S.rec[e] = LzRec{a, (src[u] & LZ_LIT) ? LZ_LIT | ((src[u] & ~LZ_LIT) - w0) : src[u]};
+              atomicOr(S.mask + ((a >> 5) - (vb >> 5)), 1u << (a & 31));
+              if (e == ne - 1) S.total = at[u] + len[u];
+              if (e == n - 1) {
+                uint32_t tag, x;
+                sn_bytes5(smem_u32(wb) + S.h.pos[e], &tag, &x);
+                S.next = w0 + S.h.pos[e] + sn_advance(tag, x);
+              }
+            } else if (e == ne) {  // the element after the batch
+              const bool lit = longlit(len[u], src[u]);
+              S.act = !valid(at[u], len[u], src[u]) ? 1 : (lit ? 2 : 0);
+              S.larg = src[u] & ~LZ_LIT;
+              S.llen = len[u];
+              S.next = lit ? (src[u] & ~LZ_LIT) + len[u] : w0 + S.h.pos[e];
+            }
+          }
+        }
+        __syncthreads();
+        const uint32_t total = S.total, next = S.next;
+        const int act = S.act;
+        if (act == 1) {
+          bad = 1;
+          break;
+        }
+        if (act == 2 && tid == 0 && next < in_len) {
+          // the window behind the long literal, on its way while the batch
+          // and the literal are written
+          if (sin.e1) {
+            lost = !mbar_wait(sin.m1, sin.p1);
+            sin.p1 ^= 1u;
+            sin.e1 = 0;
+          }
+          if (!lost && (next - sin.w1 >= sin.n1 || (next - sin.w1 + 5 > sin.n1 && sin.w1 + sin.n1 < in_len))) {
+            sn_issue(sin, sin.b1, sin.m1, next, &sin.w1, &sin.n1);
+            sin.e1 = 1;
+          }
+        }
+        if (total)
+          lz_run<kThreads, Sh::kChunk, Sh::kRing>(S.rec, ne, S.mask, S.ring, S.h.jab, vout, vb, vb + total, vfloor,
+                                                  [wb](uint32_t i) { return wb + i; });
+        op += total;
+        if (act == 2) {  // straight to the output; the ring starts anew behind it
+          lz_block_copy<kThreads>(out + op, in + S.larg, S.llen);
+          op += S.llen;
+          vfloor = va + op;
+        }
+        ip = next;
+        __syncthreads();
+      }
+      __syncthreads();
+  if (tid == 0) {
+    // settle the window copy still in flight before the buffers are reused
+    if (sin.e1) {
+      mbar_wait(sin.m1, sin.p1);
+      sin.p1 ^= 1u;
+      sin.e1 = 0;
+    }
+    if (bad == 2) report(st, DERR_TIMEOUT, page, WHERE_SNAPPY, 5);
+    else if (bad || op != out_len || ip != in_len) report(st, DERR_CORRUPT, page, WHERE_SNAPPY, 4);
+    // carry the physical buffers' parities to the next stream
+    const bool sw0 = sin.b0 == S.win[0];
+    par[0] = sw0 ? sin.p0 : sin.p1;
+    par[1] = sw0 ? sin.p1 : sin.p0;
+  }
+}
+
+// Length preamble of a page's stream: its bytes, 0 when it does not parse or
+// does not declare out_len bytes.
+__device__ __forceinline__ uint32_t sn_preamble(const uint8_t* in, uint32_t in_len, uint32_t out_len) {
+  uint64_t declared = 0;
+  const int pl = uleb([&](uint32_t k) { return static_cast<uint32_t>(__ldg(in + k)); }, 0, in_len, &declared);
+  return declared == out_len ? static_cast<uint32_t>(pl) : 0u;
+}
+
+// kFragments: the work list is the fragments [first, first + n_work) of split
+// pages, else jobs [0, n_work) (split pages skipped: their fragments are work
+// of their own).
+template <int kThreads, uint32_t kWin, bool kFragments>
+__global__ void __launch_bounds__(kThreads, kThreads == 512 ? 2 : 5)
+    k_snappy(const SnappyJob* __restrict__ jobs, int first, int n_work, SnapState ss, DevStatus* st) {
+  extern __shared__ __align__(16) uint8_t sn_smem[];
+  SnBlock<kThreads, kWin>& S = *reinterpret_cast<SnBlock<kThreads, kWin>*>(sn_smem);
+  const int tid = threadIdx.x;
+  if (tid == 0) {
+    mbar_init(&S.bar[0], 1);
+    mbar_init(&S.bar[1], 1);
+  }
+  fence_mbar_init();
+  __syncthreads();
+  uint32_t par[2] = {0, 0};
+  for (int w = blockIdx.x; w < n_work; w += gridDim.x) {
+    const SnappyJob jb = jobs[kFragments ? ss.owner[first + w] : w];
+    if (jb.codec != CODEC_SNAPPY) continue;  // another codec's kernel takes it
+    const uint8_t* in = jb.src + jb.prefix;
+    uint32_t in_len = jb.src_len - jb.prefix;
+    uint8_t* out = jb.dst + jb.prefix;
+    uint32_t out_len = jb.dst_len - jb.prefix;
+    uint32_t ip = 0;
+    if (kFragments) {
+      const uint32_t k = first + w - jb.sub;
+      if (!ss.bad[jb.sub]) {
+        const uint32_t a = ss.start[jb.sub + k];
+        const uint32_t b = k + 1 < jb.nsub ? ss.start[jb.sub + k + 1] : in_len;
+        in += a;
+        in_len = b - a;
+        out += static_cast<uint64_t>(k) * SNAPPY_FRAGMENT;
+        out_len = k + 1 < jb.nsub ? SNAPPY_FRAGMENT : out_len - k * SNAPPY_FRAGMENT;
+      } else if (k == 0) {  // not framed: the whole page here
+        ip = sn_preamble(in, in_len, out_len);
+        if (ip == 0) {
+          if (tid == 0) report(st, DERR_CORRUPT, jb.page, WHERE_SNAPPY, 3);
+          continue;
+        }
+      } else {
+        continue;
+      }
+    } else {
+      if (jb.nsub > 1) continue;
+      if (jb.prefix > jb.src_len || jb.prefix > jb.dst_len || (jb.raw && jb.src_len != jb.dst_len)) {
+        if (tid == 0) report(st, DERR_CORRUPT, jb.page, WHERE_SNAPPY, jb.raw ? 2 : 1);
+        continue;
+      }
+      lz_block_copy<kThreads>(jb.dst, jb.src, jb.raw ? jb.src_len : jb.prefix);  // V2 levels are never compressed
+      if (jb.raw) continue;
+      ip = sn_preamble(in, in_len, out_len);
+      if (ip == 0) {
+        if (tid == 0) report(st, DERR_CORRUPT, jb.page, WHERE_SNAPPY, 3);
+        continue;
+      }
+    }
+    sn_decode(S, in, ip, in_len, out, out_len, par, jb.page, st);
+  }
+}
+
+// ------------------------------------------------------------------ split pages
+
+// Element scan of the split pages, a thread block per SNAPPY_SEGMENT input
+// bytes.  Which bytes of a segment are headers depends on where the last
+// element before it ends, so the page is one chain; but where the chain
+// leaves the segment can be computed for every possible entry at once: each
+// byte's next header, if one started there, then, right to left, the exit
+// from its 32 bytes (a thread each), from its 1 KB (a warp each) and from the
+// segment, one lookup per byte and level.  (Doubling the map in place until
+// nothing changes took 11 rounds of lookups on literal bytes: 57 us a
+// segment.)  A block then waits only for its
+// predecessor's exit, looks up its own and passes that on (about a
+// microsecond a segment), while all segments' maps are built in parallel.
+// With its entry known, the block lists the segment's elements (window by
+// window, as the decoder does), adds up the output of the segments before it
+// and records which elements start a 64 KiB fragment.  An element that spans
+// two fragments, a copy that reaches out of its fragment, or anything the
+// decoder would reject marks the page: it is then decompressed whole, by one
+// block, which reports what is wrong.
+//
+// The list's pages are cut into up to SNAPPY_RUNS runs of whole pages,
+// each with a ticket counter from which blocks take its segments in order
+// (and go on to the next run when one is used up): the segment a block waits
+// for has always been taken by a block that is running, and the waits of
+// different runs overlap (in one run, 64 pages of 32 segments took 560 us, the
+// chain's 2048 hops).  Waits are bounded all the same.
+constexpr int SC_THREADS = 1024;
+constexpr uint32_t SC_WIN = 4096;
+constexpr int SC_EL = 1024;
+constexpr uint32_t SC_MAX_EL = SNAPPY_SEGMENT / 2;  // an element takes two input bytes or more
+constexpr uint32_t SC_POLLS = 1u << 22;
+struct __align__(16) SnScan {
+  union {
+    uint32_t map[SNAPPY_SEGMENT];  // next header, then the exit, from each byte (at sc_slot)
+    struct {
+      uint32_t at[SC_MAX_EL];      // output offset of each element within the segment's
+      uint16_t pos[SC_MAX_EL];     // its header
+      SnHeaders<SC_WIN, SC_EL> h;
+    } el;
+  };
+  uint8_t stage[SNAPPY_SEGMENT + 64];
+  uint64_t bar;
+  uint32_t tmp[32];
+  uint32_t ticket, entry, next, from, to, done;
+  int32_t job;
+};
+
+// Map slot of a segment byte: its place in its 32 bytes is permuted by the
+// number of the 32 bytes, so that threads at the same place of 32 such runs
+// fall on 32 banks, and so do the 32 bytes of one run.
+__device__ __forceinline__ uint32_t sc_slot(uint32_t p) { return p ^ ((p >> 5) & 31u); }
+
+// One 64-bit word written by another block of this launch: polled until its
+// flag is set.  0 when it never is.
+__device__ __forceinline__ unsigned long long sn_await(const unsigned long long* p) {
+  for (uint32_t i = 0; i < SC_POLLS; ++i) {
+    const unsigned long long v = *reinterpret_cast<const volatile unsigned long long*>(p);
+    if (v & SN_SET) return v;
+  }
+  return 0;
+}
+
+// The job that holds segment g (one warp, 32 ways a step): the last one that
+// starts at or before it.
+__device__ __forceinline__ int sc_job(const SnappyJob* jobs, int n, uint32_t g, int lane) {
+  int lo = 0;
+  while (n > 1) {
+    const int step = (n + 31) / 32;
+    const uint32_t m = __ballot_sync(0xffffffffu, lane * step < n && jobs[lo + lane * step].seg <= g);
+    const int k = 31 - __clz(m | 1u);
+    lo += k * step;
+    n = n - k * step < step ? n - k * step : step;
+  }
+  return lo;
+}
+
+__global__ void __launch_bounds__(SC_THREADS, 1) k_snappy_scan(const SnappyJob* __restrict__ jobs, int n_jobs,
+                                                               uint32_t seg_begin, uint32_t n_segs, SnapState ss,
+                                                               uint32_t* tickets, DevStatus* st) {
+  extern __shared__ __align__(16) uint8_t sn_smem[];
+  SnScan& S = *reinterpret_cast<SnScan*>(sn_smem);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (tid == 0) mbar_init(&S.bar, 1);
+  fence_mbar_init();
+  uint32_t parity = 0;
+  // warp 0: the run it takes segments from, whether its bounds are in S, and
+  // how many runs it has found used up (a used-up run stays so)
+  int run = blockIdx.x % SNAPPY_RUNS, used = 0;
+  bool bounded = false;
+  for (;;) {
+    if (warp == 0) {
+      uint32_t t = 0xffffffffu;
+      while (used < SNAPPY_RUNS) {
+        if (!bounded) {
+          // a run starts after the page that holds the segment before its share
+          uint32_t bound[2];
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            const uint32_t x = static_cast<uint32_t>(static_cast<uint64_t>(n_segs) * (run + i) / SNAPPY_RUNS);
+            bound[i] = seg_begin;
+            if (x > 0) {
+              const SnappyJob& jb = jobs[sc_job(jobs, n_jobs, seg_begin + x - 1, lane)];
+              bound[i] = jb.seg + jb.nseg;
+            }
+          }
+          if (lane == 0) {
+            S.from = bound[0];
+            S.to = bound[1];
+          }
+          __syncwarp();
+          bounded = true;
+        }
+        if (lane == 0 && S.from < S.to) t = S.from + atomicAdd(tickets + run, 1u);
+        t = __shfl_sync(0xffffffffu, t, 0);
+        if (t < S.to) break;
+        t = 0xffffffffu;
+        run = (run + 1) % SNAPPY_RUNS;
+        bounded = false;
+        ++used;
+        __syncwarp();
+      }
+      if (t != 0xffffffffu) {
+        const int j = sc_job(jobs, n_jobs, t, lane);
+        if (lane == 0) S.job = j;
+      }
+      if (lane == 0) S.ticket = t;
+    }
+    __syncthreads();
+    const uint32_t g = S.ticket;
+    if (g == 0xffffffffu) break;
+    const SnappyJob jb = jobs[S.job];
+    const uint32_t k = g - jb.seg;  // segment of the page
+    const uint8_t* in = jb.src + jb.prefix;
+    const uint32_t in_len = jb.src_len - jb.prefix, out_len = jb.dst_len - jb.prefix;
+    const uint32_t s0 = k * SNAPPY_SEGMENT;
+    const uint32_t L = in_len - s0 < SNAPPY_SEGMENT ? in_len - s0 : SNAPPY_SEGMENT;
+    // stage the segment and the header bytes after it, 16-byte aligned, at
+    // most 16 bytes past the input
+    const uintptr_t a0 = reinterpret_cast<uintptr_t>(in + s0) & ~uintptr_t(15);
+    const uint32_t shift = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(in + s0) - a0);
+    if (tid == 0) {
+      const uintptr_t lim = (reinterpret_cast<uintptr_t>(in) + in_len + 16) & ~uintptr_t(15);
+      uint64_t bytes = lim - a0;
+      if (bytes > SNAPPY_SEGMENT + 32) bytes = SNAPPY_SEGMENT + 32;
+      fence_proxy_async_smem();
+      mbar_arrive_expect_tx(&S.bar, static_cast<uint32_t>(bytes));
+      bulk_g2s(S.stage, reinterpret_cast<const void*>(a0), static_cast<uint32_t>(bytes), &S.bar);
+    }
+    if (k == 0) {
+      lz_block_copy<SC_THREADS>(jb.dst, jb.src, jb.prefix);  // V2 level bytes, never compressed
+      for (uint32_t f = tid; f < jb.nsub; f += SC_THREADS) ss.owner[jb.sub + f] = static_cast<uint32_t>(S.job);
+    }
+    bool staged = mbar_wait(&S.bar, parity);
+    if (!staged) staged = mbar_wait(&S.bar, parity) && false;  // (the copy may not outlive its buffer)
+    parity ^= 1u;
+    const bool all_staged = !__syncthreads_or(!staged);
+    if (tid == 0) {
+      // the predecessor's exit is there already, and the chain leaves the
+      // segment within a few elements (literal-heavy pages): no map needed
+      S.done = 0;
+      unsigned long long v = 0;
+      if (k == 0) {
+        const uint32_t pl = all_staged ? sn_preamble(in, in_len, out_len) : 0u;
+        v = SN_SET | (pl ? pl : 0xffffffffu);  // (0xffffffff, passed on: the page is decompressed whole)
+        S.entry = static_cast<uint32_t>(v);
+      } else {
+        v = *reinterpret_cast<const volatile unsigned long long*>(ss.exit + g - 1);
+      }
+      if (v) {
+        const uint32_t e = static_cast<uint32_t>(v);
+        uint32_t x = e;
+        int n = 0;
+        const uint32_t sa = smem_u32(S.stage) + shift;
+        for (; n < SN_SERIAL && all_staged && x < s0 + L; ++n) {
+          uint32_t tag, by;
+          sn_bytes5(sa + (x - s0), &tag, &by);
+          x += sn_advance(tag, by);
+        }
+        if (x >= s0 + L) {
+          *reinterpret_cast<volatile unsigned long long*>(ss.exit + g) = SN_SET | x;
+          S.entry = e;
+          S.next = x;
+          S.done = 1;
         }
       }
-      if (ok && p == in_len && o == out_len) {
-        emit(k, bi, p, bo, o);
-        for (uint32_t e = k + 1; e < jb.nsub; ++e) empty(e);
-      } else {
-        // one job for the whole page (its prefix is copied again there)
-        SnappyJob w = jb;
-        w.nsub = 0;
-        w.sub = 0;
-        bl[0] = w;
-        for (uint32_t e = 1; e < jb.nsub; ++e) empty(e);
-        if (timeout) report(st, DERR_TIMEOUT, jb.page, WHERE_SNAPPY, 6);
-      }
-      if (loaded && sin.e1) {  // settle the window copy still in flight before the buffers are reused
-        mbar_wait(sin.m1, sin.p1);
-        sin.p1 ^= 1u;
-        sin.e1 = 0;
-      }
-      const bool sw0 = sin.b0 == sw.win[0];
-      par[0] = sw0 ? sin.p0 : sin.p1;
-      par[1] = sw0 ? sin.p1 : sin.p0;
     }
-    __syncwarp();
+    __syncthreads();
+    if (!S.done) {
+      // the map: positions relative to the segment's first byte, which is
+      // staged at `shift`; values below L lead on in the segment
+      const uint32_t* w32 = reinterpret_cast<const uint32_t*>(S.stage);
+      const uint32_t sb = 8 * (shift & 3);
+      for (uint32_t p = 4 * tid; p < L; p += 4 * SC_THREADS) {
+        const uint32_t* w = w32 + ((p + shift) >> 2);
+        const uint32_t a = __funnelshift_r(w[0], w[1], sb), b = __funnelshift_r(w[1], w[2], sb);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          S.map[sc_slot(p + i)] =
+              p + i + sn_advance((a >> (8 * i)) & 0xffu, i == 3 ? b : __funnelshift_r(a, b, 8 * (i + 1)));
+      }
+      __syncthreads();
+      // (bytes past L lead past L: every position a level reads is set)
+      static_assert(SNAPPY_SEGMENT == 32 * SC_THREADS && SC_THREADS == 32 * 32, "a run a thread, a block a warp");
+      {
+        const uint32_t end = 32 * tid + 32 < L ? 32 * tid + 32 : L;
+        for (int r = 30; r >= 0; --r) {
+          const uint32_t p = 32 * tid + r;
+          if (p < L) {
+            const uint32_t v = S.map[sc_slot(p)];
+            if (v < end) S.map[sc_slot(p)] = S.map[sc_slot(v)];
+          }
+        }
+        __syncwarp();
+      }
+      {
+        const uint32_t end = 1024 * warp + 1024 < L ? 1024 * warp + 1024 : L;
+        for (int i = 30; i >= 0; --i) {
+          const uint32_t p = 1024 * warp + 32 * i + lane;
+          if (p < L) {
+            const uint32_t v = S.map[sc_slot(p)];
+            if (v < end) S.map[sc_slot(p)] = S.map[sc_slot(v)];
+          }
+          __syncwarp();
+        }
+      }
+      __syncthreads();
+      for (int i = static_cast<int>((L - 1) / 1024) - 1; i >= 0; --i) {
+        const uint32_t p = 1024 * i + tid;
+        const uint32_t v = S.map[sc_slot(p)];
+        if (v < L) S.map[sc_slot(p)] = S.map[sc_slot(v)];
+        __syncthreads();
+      }
+      // the chain: entry from the segment before, exit to the one after
+      if (tid == 0) {
+        uint32_t e = S.entry;  // (k == 0)
+        bool ok = all_staged;
+        if (k > 0) {
+          const unsigned long long v = sn_await(ss.exit + g - 1);
+          e = static_cast<uint32_t>(v);
+          if (!v) {
+            ok = false;
+            report(st, DERR_TIMEOUT, jb.page, WHERE_SNAPPY, 6);
+          }
+        }
+        uint32_t x = e;
+        if (!ok) x = e = 0xffffffffu;  // (passed on: the page is decompressed whole)
+        else if (e < s0 + L) x = S.map[sc_slot(e - s0)] + s0;
+        *reinterpret_cast<volatile unsigned long long*>(ss.exit + g) = SN_SET | x;
+        S.entry = e;
+        S.next = x;
+      }
+    }
+    __syncthreads();
+    const uint32_t entry = S.entry, exit = S.next;
+    bool good = entry <= in_len && exit <= in_len;
+    // the segment's elements and their output (the map is not needed any more)
+    uint32_t n_el = 0, total = 0;
+    if (good && entry < s0 + L) {
+      uint32_t q = entry - s0 + shift;  // staged positions from here on
+      const uint32_t L1 = shift + L;
+      bool dense = false;
+      // a batch ends at the end of its window, at SC_EL or SN_SERIAL headers
+      for (uint32_t guard = 0; guard < SNAPPY_SEGMENT / SN_SERIAL + 2 * SNAPPY_SEGMENT / SC_WIN + 16 && q < L1; ++guard) {
+        const uint32_t wbase = q & ~15u;
+        const uint8_t* wb = S.stage + wbase;
+        const uint32_t wl = L1 - wbase < SC_WIN ? L1 - wbase : SC_WIN;
+        sn_find_headers<SC_THREADS>(S.el.h, wb, q - wbase, wl, dense);
+        const int n = S.el.h.n;
+        dense = n >= SN_DENSE;
+        uint32_t len = 0;
+        if (tid < n) {
+          const uint32_t p = S.el.h.pos[tid];
+          uint32_t tag, x, kind, arg, nx;
+          sn_bytes5(smem_u32(wb) + p, &tag, &x);
+          if (!sn_hdr(tag, x, wbase + p - shift + s0, in_len, &kind, &len, &arg, &nx)) len = 0;
+          if (tid == n - 1) S.next = wbase + p + sn_advance(tag, x);
+        }
+        uint32_t sum;
+        const uint32_t o = block_exclusive_sum(len, S.tmp, &sum);
+        if (tid < n && n_el + tid < SC_MAX_EL) {
+          S.el.at[n_el + tid] = total + o;
+          S.el.pos[n_el + tid] = static_cast<uint16_t>(wbase + S.el.h.pos[tid]);
+          if (len == 0) good = false;
+        }
+        n_el += n;
+        total += sum;
+        q = S.next;
+        if (__syncthreads_or(total > out_len || sum > out_len)) {
+          good = false;
+          break;
+        }
+      }
+      if (q < L1 || n_el > SC_MAX_EL) good = false;
+    }
+    good = !__syncthreads_or(!good);
+    if (tid == 0) *reinterpret_cast<volatile unsigned long long*>(ss.len + g) = SN_SET | (good ? total : 0u);
+    // output of the segments before this one
+    uint64_t mine = 0;
+    for (uint32_t i = tid; i < k; i += SC_THREADS) {
+      const unsigned long long v = sn_await(ss.len + jb.seg + i);
+      if (!v) good = false;
+      mine += static_cast<uint32_t>(v);
+    }
+    uint64_t base;
+    block_exclusive_sum<uint64_t>(mine, reinterpret_cast<uint64_t*>(S.el.h.j1), &base);
+    if (base > out_len || total > out_len - base) good = false;
+    if (good) {
+      for (uint32_t i = tid; i < n_el; i += SC_THREADS) {
+        const uint32_t p = S.el.pos[i], o = static_cast<uint32_t>(base) + S.el.at[i];
+        uint32_t tag, x, kind, len, arg, nx;
+        sn_bytes5(smem_u32(S.stage) + p, &tag, &x);
+        sn_hdr(tag, x, p - shift + s0, in_len, &kind, &len, &arg, &nx);
+        const uint32_t in_frag = o & (SNAPPY_FRAGMENT - 1);
+        if (in_frag + len > SNAPPY_FRAGMENT || (kind != 0 && (arg == 0 || arg > in_frag))) good = false;
+        if (in_frag == 0 && o / SNAPPY_FRAGMENT < jb.nsub) ss.start[jb.sub + o / SNAPPY_FRAGMENT] = p - shift + s0;
+      }
+      if (k + 1 == jb.nseg && (exit != in_len || base + total != out_len)) good = false;
+    }
+    if (__syncthreads_or(!good) && tid == 0) atomicOr(ss.bad + jb.sub, 1u);
   }
 }
 
-void launch_snappy_split(const SnappyJob* jobs, int n_jobs, SnappyJob* blocks, int n_sms, DevStatus* st,
-                         cudaStream_t s) {
-  if (n_jobs <= 0) return;
+void launch_snappy_scan(const SnappyJob* jobs, int n_jobs, uint32_t seg_begin, uint32_t n_segs, SnapState ss,
+                        uint32_t* tickets, int n_sms, DevStatus* st, cudaStream_t s) {
+  if (n_jobs <= 0 || n_segs == 0) return;
   static bool attr = false;
-  constexpr uint32_t smem = kSplitWarps * sizeof(SnSplitWarp);
   if (!attr) {
-    cudaFuncSetAttribute(k_snappy_split, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaFuncSetAttribute(k_snappy_scan, cudaFuncAttributeMaxDynamicSharedMemorySize, sizeof(SnScan));
     attr = true;
   }
-  int blocks_n = (n_jobs + kSplitWarps - 1) / kSplitWarps;
-  if (blocks_n > n_sms * 3) blocks_n = n_sms * 3;
-  k_snappy_split<<<blocks_n, 32 * kSplitWarps, smem, s>>>(jobs, n_jobs, blocks, st);
+  const unsigned blocks = n_segs < static_cast<uint32_t>(n_sms) ? n_segs : n_sms;
+  k_snappy_scan<<<blocks, SC_THREADS, sizeof(SnScan), s>>>(jobs, n_jobs, seg_begin, n_segs, ss, tickets, st);
 }
 
-void launch_snappy(const SnappyJob* jobs, int n_jobs, int n_sms, DevStatus* st, cudaStream_t s, bool coop) {
+template <int kThreads, uint32_t kWin, bool kFragments>
+static void launch_snappy_shape(const SnappyJob* jobs, int first, int n, SnapState ss, int n_sms, DevStatus* st,
+                                cudaStream_t s) {
+  constexpr uint32_t smem = sizeof(SnBlock<kThreads, kWin>);
+  static int bps = 0;
+  if (!bps) {
+    cudaFuncSetAttribute(k_snappy<kThreads, kWin, kFragments>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    int b = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_snappy<kThreads, kWin, kFragments>, kThreads, smem);
+    bps = b < 1 ? 1 : b;
+  }
+  const int blocks = n < n_sms * bps ? n : n_sms * bps;
+  k_snappy<kThreads, kWin, kFragments><<<blocks, kThreads, smem, s>>>(jobs, first, n, ss, st);
+}
+
+void launch_snappy(const SnappyJob* jobs, int n_jobs, int n_sms, DevStatus* st, cudaStream_t s, bool wide) {
   if (n_jobs <= 0) return;
-  static bool attr = false;
-  constexpr uint32_t smem_w = kSnappyWarps * sizeof(SnWarp) + sizeof(SnCoop);
-  constexpr uint32_t smem_c = sizeof(SnWarp) + sizeof(SnCoop);
-  if (!attr) {
-    cudaFuncSetAttribute(k_snappy<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_w);
-    cudaFuncSetAttribute(k_snappy<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_c);
-    attr = true;
-  }
-  int bps = 0;
-  if (coop) {
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_snappy<true>, 256, smem_c);
-    if (bps < 1) bps = 1;
-    const int blocks = n_jobs < n_sms * bps ? n_jobs : n_sms * bps;
-    k_snappy<true><<<blocks, 256, smem_c, s>>>(jobs, n_jobs, st);
-    return;
-  }
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_snappy<false>, 32 * kSnappyWarps, smem_w);
-  if (bps < 1) bps = 1;
-  int blocks = (n_jobs + kSnappyWarps - 1) / kSnappyWarps;
-  if (blocks > n_sms * bps) blocks = n_sms * bps;
-  k_snappy<false><<<blocks, 32 * kSnappyWarps, smem_w, s>>>(jobs, n_jobs, st);
+  // few enough pages for all of them to run at once: the wide shape too
+  // (224 pages of 64 KiB: 414 us in the narrow one)
+  if (wide || n_jobs <= 2 * n_sms)
+    launch_snappy_shape<512, 8192, false>(jobs, 0, n_jobs, SnapState{}, n_sms, st, s);
+  else
+    launch_snappy_shape<128, 2048, false>(jobs, 0, n_jobs, SnapState{}, n_sms, st, s);
+}
+
+void launch_snappy_fragments(const SnappyJob* jobs, int first, int n, SnapState ss, int n_sms, DevStatus* st,
+                             cudaStream_t s) {
+  if (n > 0) launch_snappy_shape<512, 8192, true>(jobs, first, n, ss, n_sms, st, s);
 }
 
 }  // namespace pqi
