@@ -188,12 +188,13 @@ __device__ void lz_run(const LzRec* rec, int n, const uint32_t* mask, uint8_t* r
 
 // src[0, n) to dst by all warps of the block, a slice each.  (Not inlined:
 // a dozen 16-byte values in flight would cost the decoders registers.)
-template <int kThreads>
+// kReadOnly: the source is not written by the running kernel.
+template <int kThreads, bool kReadOnly = true>
 __device__ __noinline__ void lz_block_copy(uint8_t* dst, const uint8_t* src, uint32_t n) {
   constexpr uint32_t kWarps = kThreads / 32;
   const uint64_t per = ((static_cast<uint64_t>(n) + kWarps * 16 - 1) / (kWarps * 16)) * 16;
   const uint64_t b = per * (threadIdx.x >> 5), e = b + per < n ? b + per : n;
-  if (b < e) warp_copy<true>(dst + b, src + b, e - b, threadIdx.x & 31);
+  if (b < e) warp_copy<kReadOnly>(dst + b, src + b, e - b, threadIdx.x & 31);
 }
 
 }  // namespace pqi
