@@ -39,13 +39,13 @@ struct DictScratch {
 };
 
 // A BYTE_STREAM_SPLIT, DELTA_LENGTH_BYTE_ARRAY or DELTA_BYTE_ARRAY data page
-// rewritten into a PLAIN body (level bytes kept in front) before the walk.
+// made readable as a PLAIN page (level bytes kept in front) before the walk.
 struct TranscodeJob {
   const uint8_t* src;   // page body (decompressed): level bytes + encoded values
-  uint8_t* dst;         // BYTE_STREAM_SPLIT, DELTA_LENGTH_BYTE_ARRAY: dst_cap bytes for the PLAIN
-                        // body; DELTA_BYTE_ARRAY: null (a piece of the plan's pool)
+  uint8_t* dst;         // BYTE_STREAM_SPLIT: dst_cap bytes (and 32 more) for the PLAIN body;
+                        // others: null (the page itself; a piece of the plan's pool)
   uint32_t src_len;
-  uint32_t dst_cap;     // src_len (BYTE_STREAM_SPLIT), src_len + 4 * num_values (DELTA_LENGTH_BYTE_ARRAY)
+  uint32_t dst_cap;     // BYTE_STREAM_SPLIT: src_len
   uint32_t pp;          // plan page whose body and body_len the kernel sets
   int32_t page;         // page-table row (errors)
   int32_t enc;          // ENC_BSS, ENC_DELTA_LBA or ENC_DELTA_BA
@@ -81,7 +81,7 @@ struct DecodeArgs {
   int64_t* dbase;           // DELTA value preceding each block
   DeltaRegion* dregs;       // DELTA region summaries
   uint32_t* dreg_lists;     // DELTA region block lists (DELTA_REGION_LIST per region)
-  uint32_t* vpos;           // transcoded string pages: value-stream offset of each value (and of the end)
+  uint64_t* vpos;           // transcoded string pages: an entry per value, (offset into the value bytes << 32) | length
   uint32_t* snap_state;     // split Snappy pages' state (SnapState), zeroed by the per-scan reset
   uint64_t snap_words;
   int n_pp;
@@ -90,11 +90,12 @@ struct DecodeArgs {
   int n_delta;
 };
 
-// One block per job; `counters` is the plan's item_counter array (its pool
-// word); `pool` holds `pool_cap` bytes for DELTA_BYTE_ARRAY bodies; string
-// pages with a value-position table (PlanPage::vtab) get it filled in `vpos`.
-void launch_transcode(const TranscodeJob* jobs, int n, PlanPage* pps, uint8_t* pool, uint64_t pool_cap,
-                      uint32_t* counters, uint32_t* vpos, DevStatus* st, cudaStream_t s);
+// The transcode of jobs [0, n), n_bss of them BYTE_STREAM_SPLIT pages;
+// `counters` is the plan's item_counter array (its pool word); `pool` holds
+// `pool_cap` bytes for DELTA_BYTE_ARRAY bodies; string pages get their entry
+// table (PlanPage::vtab) filled in `vpos`.
+void launch_transcode(const TranscodeJob* jobs, int n, int n_bss, PlanPage* pps, uint8_t* pool, uint64_t pool_cap,
+                      uint32_t* counters, uint64_t* vpos, DevStatus* st, cudaStream_t s);
 void launch_dict(const DictJob* jobs, int n_jobs, int max_fixed_bytes, int max_str_regions, DictScratch ds,
                  DictDev* dicts, int n_sms, DevStatus* st, cudaStream_t s);
 // Launches over sub-ranges (one output column's share of the plan).

@@ -149,6 +149,42 @@ __device__ __forceinline__ int64_t unzigzag(uint64_t u) {
   return static_cast<int64_t>(u >> 1) ^ -static_cast<int64_t>(u & 1);
 }
 
+// DELTA_BINARY_PACKED block header with 4 miniblocks: min delta (zigzag
+// ULEB128, 1-10 bytes) then 4 bit-width bytes, parsed from the 16 bytes at
+// p held in registers (5 aligned 32-bit loads; reads at most 19 bytes past
+// p).  Returns the varint length (0 when longer than 10 bytes); *z the
+// varint, *w4 the widths (byte m = miniblock m).
+template <bool kShared>
+__device__ __forceinline__ int delta_header16(const uint8_t* p, uint64_t* z, uint32_t* w4) {
+  const uintptr_t a = reinterpret_cast<uintptr_t>(p);
+  const uint32_t* q = reinterpret_cast<const uint32_t*>(a & ~uintptr_t(3));
+  const uint32_t sh = static_cast<uint32_t>(a & 3) * 8;
+  uint32_t r[5];
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    if constexpr (kShared)
+      r[k] = q[k];
+    else
+      r[k] = __ldg(q + k);
+  }
+  const uint64_t lo = (static_cast<uint64_t>(__funnelshift_r(r[1], r[2], sh)) << 32) | __funnelshift_r(r[0], r[1], sh);
+  const uint64_t hi = (static_cast<uint64_t>(__funnelshift_r(r[3], r[4], sh)) << 32) | __funnelshift_r(r[2], r[3], sh);
+  // first byte with its high bit clear ends the varint
+  const uint64_t mlo = ~lo & 0x8080808080808080ull;
+  const uint64_t mhi = ~hi & 0x8080ull;
+  const int vl = mlo ? (__ffsll(static_cast<long long>(mlo)) >> 3) : (mhi ? 8 + (__ffsll(static_cast<long long>(mhi)) >> 3) : 0);
+  if (!vl) return 0;
+  uint64_t v = 0;
+  for (int i = 0; i < vl; ++i) {
+    const uint64_t byte = i < 8 ? (lo >> (8 * i)) & 0x7f : (hi >> (8 * (i - 8))) & 0x7f;
+    v |= byte << (7 * i);
+  }
+  *z = v;
+  *w4 = vl < 8 ? static_cast<uint32_t>((lo >> (8 * vl)) | (vl ? hi << (64 - 8 * vl) : 0ull))
+               : static_cast<uint32_t>(hi >> (8 * (vl - 8)));
+  return vl;
+}
+
 // `w` 32-bit little-endian word view of a staged window; bit position `b`
 // relative to the window's first byte.  Extracts `width` <= 32 bits.
 __device__ __forceinline__ uint32_t bits32(const uint32_t* w, uint64_t b, int width) {

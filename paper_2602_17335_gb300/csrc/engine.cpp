@@ -1062,29 +1062,29 @@ pq_status plan_build(pq_ctx* ctx, pq_index* idx, const std::vector<int32_t>& col
           if (enc == pqi::ENC_DELTA_BA && idx->chunk_ba_bytes[ch] < 0)
             return fail(ctx, PQ_ERR_UNSUPPORTED, "DELTA_BYTE_ARRAY chunk without size statistics");
           if (enc == pqi::ENC_DELTA_BA) {
-            // the PLAIN size is known only on the device: the page takes a piece
-            // of a pool that holds its levels, length words and padding, plus
-            // (once per chunk) the chunk's value bytes
+            // the size is known only on the device: the page takes a piece of
+            // a pool that holds its levels and padding, plus (once per chunk)
+            // the chunk's value bytes
             plan->tc_dst_off.push_back(-1);
-            tc_pool += (static_cast<uint64_t>(pg.uncompressed) + 4ull * static_cast<uint64_t>(pg.num_values) + 63) &
-                       ~uint64_t(15);
+            tc_pool += (static_cast<uint64_t>(pg.uncompressed) + 63) & ~uint64_t(15);
             if (!tc_chunk_counted) {
               tc_pool += (static_cast<uint64_t>(idx->chunk_ba_bytes[ch]) + 15) & ~uint64_t(15);
               tc_chunk_counted = true;
             }
+          } else if (enc == pqi::ENC_DELTA_LBA) {
+            plan->tc_dst_off.push_back(-1);  // the strings stay in the page
           } else {
-            const uint64_t cap = static_cast<uint64_t>(pg.uncompressed) +
-                                 (enc == pqi::ENC_DELTA_LBA ? 4ull * static_cast<uint64_t>(pg.num_values) : 0);
-            if (cap > 0x7fffffffull) return fail(ctx, PQ_ERR_UNSUPPORTED, "transcoded page above 2 GiB");
-            j.dst_cap = static_cast<uint32_t>(cap);
+            cw.tc_bss++;
+            j.dst_cap = static_cast<uint32_t>(pg.uncompressed);
             plan->tc_dst_off.push_back(static_cast<int64_t>(scratch));
-            scratch += (cap + 32 + 15) & ~uint64_t(15);
+            scratch += (static_cast<uint64_t>(pg.uncompressed) + 32 + 15) & ~uint64_t(15);
           }
           if (enc != pqi::ENC_BSS) {
-            // the transcoder records where each value starts, so that the
-            // walk need not follow the (length, bytes) chain
+            // the transcoder makes an entry per value
+            if (static_cast<uint64_t>(pg.uncompressed) + 4ull * static_cast<uint64_t>(pg.num_values) > 0x7fffffffull)
+              return fail(ctx, PQ_ERR_UNSUPPORTED, "transcoded page above 2 GiB");
             pp.vtab = static_cast<uint32_t>(1 + plan->vpos_rows);
-            plan->vpos_rows += static_cast<uint64_t>(pg.num_values) + 1;
+            plan->vpos_rows += static_cast<uint64_t>(pg.num_values);
           }
           plan->tc_jobs.push_back(j);
         }
@@ -1206,7 +1206,7 @@ pq_status plan_upload(pq_plan* plan, cudaStream_t s) {
   plan->d_cols = plan_alloc(pqi::OutCol, plan, plan->outcols.size());
   plan->d_snappy = plan_alloc(pqi::SnappyJob, plan, plan->snappy_data.size() + plan->snappy_dict.size());
   plan->d_snap_state = plan_alloc(uint8_t, plan, pqi::snap_state_bytes(plan->snap_blocks, plan->snap_segs));
-  plan->d_vpos = plan_alloc(uint32_t, plan, plan->vpos_rows);
+  plan->d_vpos = plan_alloc(uint64_t, plan, plan->vpos_rows);
   plan->d_dict_jobs = plan_alloc(pqi::DictJob, plan, plan->dict_jobs.size());
   plan->d_tc_jobs = plan_alloc(pqi::TranscodeJob, plan, plan->tc_jobs.size());
   plan->d_str_cols = plan_alloc(int32_t, plan, plan->str_cols.size());
@@ -1238,9 +1238,8 @@ pq_status plan_upload(pq_plan* plan, cudaStream_t s) {
       pp.pad = 0;
     }
   }
-  // transcode jobs: sources and destinations in the scratch; the plan page
-  // reads the PLAIN body (DELTA_BYTE_ARRAY: its source until the kernel
-  // points it at its piece of the pool)
+  // transcode jobs: sources and destinations in the scratch; the kernels
+  // point the plan pages at the bodies to read
   for (size_t i = 0; i < plan->tc_jobs.size(); ++i) {
     auto& j = plan->tc_jobs[i];
     if (plan->tc_src_off[i] >= 0) j.src = plan->d_scratch + plan->tc_src_off[i];
@@ -1311,11 +1310,11 @@ pq_status plan_upload(pq_plan* plan, cudaStream_t s) {
       }
       size_t tcj = 0;
       for (auto& cp : plan->chunk_pp) {
-        int ntc = 0;
+        int ntc = 0, nbss = 0;
         while (tcj + ntc < plan->tc_jobs.size() &&
                plan->tc_jobs[tcj + ntc].pp < static_cast<uint32_t>(cp.first + cp.second))
-          ++ntc;
-        n += ntc ? 1 : 0;
+          nbss += plan->tc_jobs[tcj + ntc++].enc == pqi::ENC_BSS;
+        n += (nbss ? 1 : 0) + (ntc > nbss ? 1 : 0);
         tcj += ntc;
       }
     } else {
@@ -1325,7 +1324,7 @@ pq_status plan_upload(pq_plan* plan, cudaStream_t s) {
         // (+2 per job list with split pages: the element scan and the fragments)
         n += (cw.snap_dict_n ? dk + (cw.blk_dict_n ? 2 : 0) : 0) + (cw.dict_n ? 2 : 0) +
              (cw.snap_data_n ? dk + (cw.blk_data_n ? 2 : 0) : 0) + (cw.walk_n ? 1 : 0) +
-             (cw.delta_n ? 4 : 0) + (cw.tc_n ? 1 : 0) + (plan->outcols[oc].item_count ? 1 : 0);
+             (cw.delta_n ? 4 : 0) + (cw.tc_bss ? 1 : 0) + (cw.tc_n > cw.tc_bss ? 1 : 0) + (plan->outcols[oc].item_count ? 1 : 0);
       }
     }
     for (int32_t sc : plan->str_cols) n += plan->outcols[sc].item_count ? 2 : 0;
@@ -1411,7 +1410,7 @@ uint64_t plan_device_bytes(const pq_plan* plan, uint64_t scratch) {
   const uint64_t str_rows = static_cast<uint64_t>(plan->n_rows) * plan->str_cols.size();
   return npp * sizeof(pqi::PlanPage) + nit * sizeof(pqi::Item) + plan->outcols.size() * sizeof(pqi::OutCol) +
          (plan->snappy_data.size() + plan->snappy_dict.size()) * sizeof(pqi::SnappyJob) + 56ull * plan->snap_blocks +
-         4 * plan->vpos_rows +
+         8 * plan->vpos_rows +
          plan->dict_jobs.size() * sizeof(pqi::DictJob) + plan->tc_jobs.size() * sizeof(pqi::TranscodeJob) +
          4 * (plan->walk_pps.size() + plan->delta_pps.size()) +
          plan->delta_blocks * 12 +
@@ -1503,9 +1502,9 @@ static int max_str_regions_all(const pq_plan* plan) {
   return m;
 }
 
-static void enqueue_transcode(pq_plan* plan, int begin, int n, const pqi::DecodeArgs& a, cudaStream_t s) {
+static void enqueue_transcode(pq_plan* plan, int begin, int n, int n_bss, const pqi::DecodeArgs& a, cudaStream_t s) {
   if (n <= 0) return;
-  pqi::launch_transcode(plan->d_tc_jobs + begin, n, plan->d_pps, plan->d_scratch + plan->tc_pool_off,
+  pqi::launch_transcode(plan->d_tc_jobs + begin, n, n_bss, plan->d_pps, plan->d_scratch + plan->tc_pool_off,
                         plan->tc_pool_bytes, plan->d_counter, plan->d_vpos, a.st, s);
 }
 
@@ -1585,7 +1584,7 @@ static void enqueue_column(pq_plan* plan, size_t oc, const pqi::DecodeArgs& a, b
     pqi::launch_dict(plan->d_dict_jobs + cw.dict_begin, cw.dict_n, cw.max_fixed_dict, cw.max_str_regions,
                      pqi::DictScratch{plan->d_sregs, plan->d_slists}, plan->idx->d_dicts, ctx->n_sms, a.st, s);
   launch_column_decompress(plan, oc, false, a.st, s);
-  enqueue_transcode(plan, cw.tc_begin, cw.tc_n, a, s);
+  enqueue_transcode(plan, cw.tc_begin, cw.tc_n, cw.tc_bss, a, s);
   const auto& col = plan->outcols[oc];
   pqi::launch_walk(a, cw.walk_begin, cw.walk_n, ctx->n_sms, col.optional != 0, plan->tuning.walk_window, s);
   pqi::launch_delta_bases(a, cw.delta_begin, cw.delta_n, cw.max_regions, s);
@@ -1635,7 +1634,9 @@ static void enqueue_scan(pq_plan* plan, cudaStream_t s, bool with_dicts, const c
       job += nj;
       int ntc = 0;
       while (tcj + ntc < plan->tc_jobs.size() && plan->tc_jobs[tcj + ntc].pp < static_cast<uint32_t>(first + n)) ++ntc;
-      enqueue_transcode(plan, static_cast<int>(tcj), ntc, a, s);
+      int nbss = 0;
+      for (int q = 0; q < ntc; ++q) nbss += plan->tc_jobs[tcj + q].enc == pqi::ENC_BSS;
+      enqueue_transcode(plan, static_cast<int>(tcj), ntc, nbss, a, s);
       tcj += ntc;
       pqi::launch_plain_pages(a, first, n, s);
     }
@@ -1648,7 +1649,7 @@ static void enqueue_scan(pq_plan* plan, cudaStream_t s, bool with_dicts, const c
       const auto& cw = plan->colwork[oc];
       if (with_dicts) launch_column_decompress(plan, oc, true, a.st, s);
       launch_column_decompress(plan, oc, false, a.st, s);
-      enqueue_transcode(plan, cw.tc_begin, cw.tc_n, a, s);
+      enqueue_transcode(plan, cw.tc_begin, cw.tc_n, cw.tc_bss, a, s);
     }
     mark(2);
     for (int oc = 0; oc < ncols; ++oc) {

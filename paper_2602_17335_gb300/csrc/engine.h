@@ -150,7 +150,7 @@ struct pq_plan {
   uint64_t delta_blocks = 0;                 // capacity of the DELTA block tables
   uint64_t delta_regions = 0;                // capacity of the DELTA region tables
   uint64_t dict_regions = 0;                 // capacity of the string-dictionary region tables
-  uint64_t vpos_rows = 0;                    // value-position table rows of the transcoded string pages
+  uint64_t vpos_rows = 0;                    // entry table rows of the transcoded string pages
   // per chunk: range of plan pages (plain baseline launches per chunk)
   std::vector<std::pair<int32_t, int32_t>> chunk_pp;  // (first pp, count)
   std::vector<int32_t> chunk_pp_chunk;
@@ -167,7 +167,7 @@ struct pq_plan {
   pqi::OutCol* d_cols = nullptr;
   pqi::SnappyJob* d_snappy = nullptr;        // data jobs then dict jobs
   uint8_t* d_snap_state = nullptr;           // state of the split Snappy pages (pqi::SnapState)
-  uint32_t* d_vpos = nullptr;                // value positions of the transcoded string pages
+  uint64_t* d_vpos = nullptr;                // entries of the transcoded string pages' values
   pqi::DictJob* d_dict_jobs = nullptr;
   pqi::TranscodeJob* d_tc_jobs = nullptr;
   int32_t* d_str_cols = nullptr;
@@ -211,7 +211,7 @@ struct pq_plan {
     int max_fixed_dict = 0;
     int walk_begin = 0, walk_n = 0;            // into walk_pps
     int delta_begin = 0, delta_n = 0;          // into delta_pps
-    int tc_begin = 0, tc_n = 0;                // into tc_jobs
+    int tc_begin = 0, tc_n = 0, tc_bss = 0;    // into tc_jobs; BYTE_STREAM_SPLIT pages among them
     int max_regions = 0;                       // most DELTA regions of one page
     int max_str_regions = 0;                   // most chain regions of one string dictionary
     bool copy_only = false;                    // every page REQUIRED PLAIN fixed-width

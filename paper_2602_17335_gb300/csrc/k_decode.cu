@@ -79,42 +79,6 @@ __device__ __forceinline__ uint64_t gwin64(const uint8_t* base, uint64_t b) {
   return (static_cast<uint64_t>(__funnelshift_r(r1, r2, sh)) << 32) | __funnelshift_r(r0, r1, sh);
 }
 
-// DELTA_BINARY_PACKED block header with 4 miniblocks: min delta (zigzag
-// ULEB128, 1-10 bytes) then 4 bit-width bytes, parsed from the 16 bytes at
-// p held in registers (5 aligned 32-bit loads; reads at most 19 bytes past
-// p).  Returns the varint length (0 when longer than 10 bytes); *z the
-// varint, *w4 the widths (byte m = miniblock m).
-template <bool kShared>
-__device__ __forceinline__ int delta_header16(const uint8_t* p, uint64_t* z, uint32_t* w4) {
-  const uintptr_t a = reinterpret_cast<uintptr_t>(p);
-  const uint32_t* q = reinterpret_cast<const uint32_t*>(a & ~uintptr_t(3));
-  const uint32_t sh = static_cast<uint32_t>(a & 3) * 8;
-  uint32_t r[5];
-#pragma unroll
-  for (int k = 0; k < 5; ++k) {
-    if constexpr (kShared)
-      r[k] = q[k];
-    else
-      r[k] = __ldg(q + k);
-  }
-  const uint64_t lo = (static_cast<uint64_t>(__funnelshift_r(r[1], r[2], sh)) << 32) | __funnelshift_r(r[0], r[1], sh);
-  const uint64_t hi = (static_cast<uint64_t>(__funnelshift_r(r[3], r[4], sh)) << 32) | __funnelshift_r(r[2], r[3], sh);
-  // first byte with its high bit clear ends the varint
-  const uint64_t mlo = ~lo & 0x8080808080808080ull;
-  const uint64_t mhi = ~hi & 0x8080ull;
-  const int vl = mlo ? (__ffsll(static_cast<long long>(mlo)) >> 3) : (mhi ? 8 + (__ffsll(static_cast<long long>(mhi)) >> 3) : 0);
-  if (!vl) return 0;
-  uint64_t v = 0;
-  for (int i = 0; i < vl; ++i) {
-    const uint64_t byte = i < 8 ? (lo >> (8 * i)) & 0x7f : (hi >> (8 * (i - 8))) & 0x7f;
-    v |= byte << (7 * i);
-  }
-  *z = v;
-  *w4 = vl < 8 ? static_cast<uint32_t>((lo >> (8 * vl)) | (vl ? hi << (64 - 8 * vl) : 0ull))
-               : static_cast<uint32_t>(hi >> (8 * (vl - 8)));
-  return vl;
-}
-
 // ------------------------------------------------------------------ K6 dictionaries
 
 // Fixed-width dictionary: an aligned copy of the PLAIN page body.
@@ -1384,28 +1348,18 @@ done:
 // PLAIN BYTE_ARRAY: thread 0 follows the (length, bytes) chain and records
 // for every item the offset of its first value and the chars before it.
 __device__ bool walk_plain_ba(WalkSmem& sm, const uint8_t* sb, uint32_t slen, int32_t total, const PlanPage& pp,
-                              Item* items, int pgid, DevStatus* st, const uint32_t* vp) {
+                              Item* items, int pgid, DevStatus* st, const uint64_t* vp) {
   if (vp) {
-    // a transcoded page: the transcoder recorded where every value starts
-    // (vp[k], and vp[total] = the end of the stream it wrote), so each
-    // item's checkpoint is a lookup; the chars before value k are vp[k] - 4 k
-    int bad = 0;
-    // the table covers exactly `total` values of at least 4 bytes each
-    if (threadIdx.x == 0 && (total < 0 || static_cast<uint64_t>(total) * 4 > slen || vp[total] != slen)) bad = 1;
-    for (uint32_t i = threadIdx.x; i < pp.item_count; i += blockDim.x) {
-      Item& it = items[pp.item_begin + i];
-      if (it.nn <= 0) continue;
-      const int32_t k = it.k0;
-      const uint32_t pos = (k >= 0 && k <= total) ? vp[k] : 0xffffffffu;
-      if (pos > slen || pos < 4u * static_cast<uint32_t>(k)) {
-        bad = 1;
-        continue;
+    // a transcoded page: the transcoder made an entry per value, which the
+    // expansion looks up
+    const bool bad = pp.dblocks != total;
+    if (!bad)
+      for (uint32_t i = threadIdx.x; i < pp.item_count; i += blockDim.x) {
+        Item& it = items[pp.item_begin + i];
+        it.pos = 0;
+        it.run_k0 = it.k0;
+        it.base = 0;
       }
-      it.pos = static_cast<int32_t>(pos);
-      it.run_k0 = k;
-      it.base = static_cast<int64_t>(pos) - 4 * static_cast<int64_t>(k);
-    }
-    bad = __syncthreads_or(bad);
     if (threadIdx.x == 0) {
       if (bad) report(st, DERR_CORRUPT, pgid, WHERE_WALK_VALUES, 8);
       sm.ctl[5] = bad;
@@ -2414,6 +2368,29 @@ __device__ bool warp_plain_ba(const uint8_t* sb, uint32_t slen, uint32_t pos, in
   return __shfl_sync(0xffffffffu, ok, 0) != 0;
 }
 
+// Strings of a transcoded page: values [k0, k1) of its entry table (offsets
+// into the page's slen value bytes), 8 a lane in flight.
+__device__ bool warp_table_ba(const uint64_t* tab, uint32_t slen, int32_t k0, int32_t k1, const Sink& sink,
+                              uint64_t* chars, int lane) {
+  bool bad = false;
+  constexpr int U = 8;
+  for (int32_t j0 = k0; j0 < k1; j0 += 32 * U) {
+    uint64_t e[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) e[u] = j0 + u * 32 + lane < k1 ? tab[j0 + u * 32 + lane] : 0ull;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int32_t k = j0 + u * 32 + lane;
+      if (k < k1) {
+        bad |= (e[u] >> 32) + static_cast<uint32_t>(e[u]) > slen;
+        sink.put(k - k0, e[u]);
+        *chars += static_cast<uint32_t>(e[u]);
+      }
+    }
+  }
+  return !__any_sync(0xffffffffu, bad);
+}
+
 // Bits of the validity bitmap for output rows [r, r + n), n <= 32.
 __device__ __forceinline__ uint32_t bitmap_bits(const uint32_t* v, int64_t r, int n) {
   const int64_t wi = r >> 5;
@@ -2553,6 +2530,8 @@ __device__ void expand_item(const DecodeArgs& a, int it_id, WarpSmem& ws, int la
                                    k0 + nn, dd, isba, sink, &chars, lane);
     } else if (isdelta) {
       ok = warp_delta(sb, pp, a.dpos + pp.dtab, a.dbase + pp.dtab, type_bits, k0, k0 + nn, sink, lane);
+    } else if (isba && pp.vtab) {
+      ok = warp_table_ba(a.vpos + (pp.vtab - 1), slen, k0, k0 + nn, sink, &chars, lane);
     } else if (isba) {
       ok = warp_plain_ba(sb, slen, static_cast<uint32_t>(it.pos), k0, k0 + nn, sink, &chars, lane);
     } else {

@@ -38,20 +38,12 @@ namespace pqi {
 namespace {
 
 constexpr int ZT = 512;                 // threads
-constexpr uint32_t Z_CHUNK = 8192;      // lz_run's
-constexpr uint32_t Z_RING = 32768;
-constexpr uint32_t Z_OUT = 32768;       // output of a batch
-constexpr int Z_EL = 1024;              // elements of a batch
 constexpr int Z_HW = 3;
-constexpr int Z_SEQ = 512;              // sequences decoded at a time, one a thread
-constexpr uint32_t Z_LONG = 4096;       // sequences with a run or a match of this length are written on their own
+constexpr int Z_SEQ = ZT;               // sequences decoded at a time, one a thread
 constexpr uint32_t Z_BITS = (Z_SEQ * 89 + 7) / 8 + 64;  // staged bytes: a sequence takes 89 bits at most
 
 struct __align__(16) ZBlock {
-  uint8_t ring[Z_RING];
-  LzRec rec[Z_EL];
-  uint16_t notes[Z_CHUNK];
-  uint32_t mask[Z_OUT / 32 + 2];
+  LzPairs<ZT, 8192, 32768> lz;
   // sequence tables (literal lengths, offsets, match lengths), by state
   uint32_t step[3][512];       // extra bits | state bits << 8 | next state base << 16
   uint32_t base[3][512];       // value without its extra bits
@@ -74,9 +66,6 @@ struct __align__(16) ZBlock {
   uint32_t used;
   // a group of sequences
   uint32_t at[Z_SEQ], states[Z_SEQ];   // bit position and states each starts with
-  uint32_t ll[Z_SEQ], ml[Z_SEQ], off[Z_SEQ];
-  uint32_t out_at[Z_SEQ + 1], lit_at[Z_SEQ + 1], cnt_at[Z_SEQ + 1];  // sums before each
-  uint64_t tmp64[32];
   uint32_t map[ZT / 32][3];            // the warps' maps of the repeat offsets
   uint32_t rep[3];
   int32_t bad;
@@ -659,38 +648,11 @@ __device__ __forceinline__ uint64_t z_block(ZBlock& S, const uint8_t* src, uint3
   uint8_t* vout = dst - va;
   const auto lit_byte = [=](uint32_t i) { return lit + i * lit_step; };
   uint32_t lits = 0;  // literals used
-  // n literals straight to the output when they do not overlap their place,
-  // else (and repeated bytes) as elements of up to Z_LONG bytes
-  const auto one_element = [&](uint32_t src_word, uint32_t n) {
-    for (uint32_t w = tid; w < Z_LONG / 32 + 2; w += ZT) S.mask[w] = 0;
-    __syncthreads();
-    const uint32_t v = va + static_cast<uint32_t>(out);
-    if (tid == 0) {
-      S.rec[0] = LzRec{v, src_word};
-      S.mask[0] = 1u << (v & 31);
-    }
-    __syncthreads();
-    lz_run<ZT, Z_CHUNK, Z_RING>(S.rec, 1, S.mask, S.ring, S.notes, vout, v, v + n, vfloor, lit_byte);
-    out += n;
-    __syncthreads();
+  // where n literals from the i-th on can be copied from at once
+  const auto plain = [=](uint32_t i, uint32_t n, uint32_t v) -> const uint8_t* {
+    return lit_step && (lit_ro || lit + i >= vout + v + n) ? lit + i : nullptr;
   };
-  const auto literals = [&](uint32_t n) {
-    if (n >= Z_LONG && lit_step && (lit_ro || lit + lits >= dst + out + n)) {
-      if (lit_ro) lz_block_copy<ZT, true>(dst + out, lit + lits, n);
-      else lz_block_copy<ZT, false>(dst + out, lit + lits, n);
-      out += n;
-      lits += n;
-      vfloor = va + static_cast<uint32_t>(out);
-      __syncthreads();
-      return;
-    }
-    while (n) {
-      const uint32_t c = n < Z_LONG ? n : Z_LONG;
-      one_element(LZ_LIT | lits, c);
-      lits += c;
-      n -= c;
-    }
-  };
+  uint32_t v = va + static_cast<uint32_t>(out);
   for (uint32_t done = 0; done < nseq;) {
     const int nb = nseq - done < Z_SEQ ? static_cast<int>(nseq - done) : Z_SEQ;
     const bool final = done + nb == nseq;
@@ -805,23 +767,13 @@ __device__ __forceinline__ uint64_t z_block(ZBlock& S, const uint8_t* src, uint3
     apply(S.map[warp][0], S.map[warp][1], S.map[warp][2]);
     // the sequence's offset is the first of the three after it
     const uint32_t off = m0;
-    // sums before each: output, literals, runs that are not empty, sequences
-    // written on their own
-    uint64_t tot_ol;
+    // output and literals before the sequence
+    uint64_t tot;
     const uint64_t ol = block_exclusive_sum<uint64_t>(static_cast<uint64_t>(ll + ml) | (static_cast<uint64_t>(ll) << 32),
-                                                      S.tmp64, &tot_ol);
-    const bool alone = tid < nb && (ll >= Z_LONG || ml >= Z_LONG);
-    uint32_t tot_c;
-    const uint32_t cn = block_exclusive_sum<uint32_t>((tid < nb && ll ? 1u : 0u) | (alone ? 1u << 16 : 0u), S.tmp, &tot_c);
-    const uint32_t o_at = static_cast<uint32_t>(ol), l_at = static_cast<uint32_t>(ol >> 32);
+                                                      S.lz.tmp64, &tot);
+    const uint32_t l_at = static_cast<uint32_t>(ol >> 32);
     if (tid < nb) {
-      S.ll[tid] = ll;
-      S.ml[tid] = ml;
-      S.off[tid] = off;
-      S.out_at[tid] = o_at;
-      S.lit_at[tid] = l_at;
-      S.cnt_at[tid] = cn;
-      const uint64_t at = out + o_at;  // output before the sequence
+      const uint64_t at = static_cast<uint64_t>(v - va) + static_cast<uint32_t>(ol);
       const uint32_t rest = regen - lits;  // literals before the group
       int e = ZE_OK;
       if (l_at > rest || ll > rest - l_at) e = ZE_SEQ;
@@ -829,57 +781,19 @@ __device__ __forceinline__ uint64_t z_block(ZBlock& S, const uint8_t* src, uint3
       else if (at + ml + (rest - l_at) > dst_len) e = ZE_SIZE;  // (unread literals included)
       if (e) atomicMax(&S.bad, e);
     }
-    if (tid == 0) {
-      S.out_at[nb] = static_cast<uint32_t>(tot_ol);
-      S.lit_at[nb] = static_cast<uint32_t>(tot_ol >> 32);
-      S.cnt_at[nb] = tot_c;
-    }
     __syncthreads();
     if (S.bad) return fail(S.bad);
-    for (int i0 = 0; i0 < nb;) {
-      // as many sequences as fit a batch, up to one that is written on its own
-      const bool fits = tid >= i0 && tid < nb && S.out_at[tid + 1] - S.out_at[i0] <= Z_OUT - 64 &&
-                        (S.cnt_at[tid + 1] >> 16) == (S.cnt_at[i0] >> 16);
-      const int k = __syncthreads_count(fits);
-      if (k == 0) {
-        const uint32_t l1 = S.ll[i0], n1 = S.ml[i0], o1 = S.off[i0];
-        literals(l1);
-        for (uint32_t n = n1; n;) {
-          const uint32_t c = n < Z_LONG ? n : Z_LONG;
-          one_element(o1, c);
-          n -= c;
-        }
-        i0 += 1;
-        continue;
-      }
-      const int i1 = i0 + k;
-      for (uint32_t w = tid; w < Z_OUT / 32 + 2; w += ZT) S.mask[w] = 0;
-      __syncthreads();
-      const uint32_t vb = va + static_cast<uint32_t>(out);
-      if (tid >= i0 && tid < i1) {
-        uint32_t v = vb + S.out_at[tid] - S.out_at[i0];
-        int e = tid - i0 + static_cast<int>((S.cnt_at[tid] - S.cnt_at[i0]) & 0xffffu);
-        if (ll) {
-          S.rec[e++] = LzRec{v, LZ_LIT | (lits + S.lit_at[tid] - S.lit_at[i0])};
-          atomicOr(S.mask + ((v >> 5) - (vb >> 5)), 1u << (v & 31));
-          v += ll;
-        }
-        S.rec[e] = LzRec{v, off};
-        atomicOr(S.mask + ((v >> 5) - (vb >> 5)), 1u << (v & 31));
-      }
-      __syncthreads();
-      const uint32_t total = S.out_at[i1] - S.out_at[i0];
-      const int n = k + static_cast<int>((S.cnt_at[i1] - S.cnt_at[i0]) & 0xffffu);
-      lz_run<ZT, Z_CHUNK, Z_RING>(S.rec, n, S.mask, S.ring, S.notes, vout, vb, vb + total, vfloor, lit_byte);
-      out += total;
-      lits += S.lit_at[i1] - S.lit_at[i0];
-      i0 = i1;
-      __syncthreads();
-    }
+    if (lit_ro)
+      lz_pairs<true>(S.lz, nb, vout, v, vfloor, ll, LZ_LIT | (lits + l_at), ml, off, lit_byte, plain);
+    else
+      lz_pairs<false>(S.lz, nb, vout, v, vfloor, ll, LZ_LIT | (lits + l_at), ml, off, lit_byte, plain);
+    lits += static_cast<uint32_t>(tot >> 32);
     done += static_cast<uint32_t>(nb);
   }
-  literals(regen - lits);
-  return out;
+  // the literals after the last sequence
+  if (lit_ro) lz_one<true>(S.lz, vout, v, vfloor, LZ_LIT | lits, regen - lits, lit_byte, plain);
+  else lz_one<false>(S.lz, vout, v, vfloor, LZ_LIT | lits, regen - lits, lit_byte, plain);
+  return v - va;
 }
 
 // Every frame of src[0, src_len) into dst[0, dst_len); returns 0 or an error.

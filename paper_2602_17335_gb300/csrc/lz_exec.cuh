@@ -197,4 +197,121 @@ __device__ __noinline__ void lz_block_copy(uint8_t* dst, const uint8_t* src, uin
   if (b < e) warp_copy<kReadOnly>(dst + b, src + b, e - b, threadIdx.x & 31);
 }
 
+// ------------------------------------------------------------------ groups of element pairs
+
+// Workspace of lz_pairs: kThreads <= 512 threads, kChunk and kRing as for
+// lz_run; a batch writes up to 4 kChunk bytes.
+template <int kThreads_, uint32_t kChunk_, uint32_t kRing_>
+struct __align__(16) LzPairs {
+  static constexpr int kThreads = kThreads_;
+  static constexpr uint32_t kChunk = kChunk_, kRing = kRing_, kOut = 4 * kChunk_;
+  uint8_t ring[kRing];
+  LzRec rec[2 * kThreads];
+  uint16_t notes[kChunk];
+  uint32_t mask[kOut / 32 + 2];
+  uint32_t out_at[kThreads + 1], cnt_at[kThreads + 1];  // sums before each thread's pair
+  uint32_t len[2][kThreads], src[2][kThreads];
+  uint64_t tmp64[32];
+  uint32_t tmp[32];
+};
+constexpr uint32_t LZ_LONG = 4096;  // pairs with an element of this length are written on their own
+
+// One element of n bytes at output position v; v moves past it.  A long
+// literal is copied straight to the output when plain(i, n, v) gives the
+// address of its bytes (null: they overlap their place, or repeat), others
+// go through lz_run in pieces.  kReadOnly: the literals are not written by the
+// running kernel.
+template <bool kReadOnly, typename W, typename Lit, typename Plain>
+__device__ void lz_one(W& S, uint8_t* vout, uint32_t& v, uint32_t& vfloor, uint32_t src, uint32_t n, Lit lit,
+                       Plain plain) {
+  if (n >= LZ_LONG && (src & LZ_LIT)) {
+    const uint8_t* from = plain(src & ~LZ_LIT, n, v);
+    if (from) {
+      lz_block_copy<W::kThreads, kReadOnly>(vout + v, from, n);
+      v += n;
+      vfloor = v;
+      __syncthreads();
+      return;
+    }
+  }
+  while (n) {
+    const uint32_t c = n < LZ_LONG ? n : LZ_LONG;
+    for (uint32_t w = threadIdx.x; w < LZ_LONG / 32 + 2; w += W::kThreads) S.mask[w] = 0;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      S.rec[0] = LzRec{v, src};
+      S.mask[0] = 1u << (v & 31);
+    }
+    __syncthreads();
+    lz_run<W::kThreads, W::kChunk, W::kRing>(S.rec, 1, S.mask, S.ring, S.notes, vout, v, v + c, vfloor, lit);
+    __syncthreads();
+    v += c;
+    n -= c;
+    if (src & LZ_LIT) src += c;
+  }
+}
+
+// The pairs of threads [0, nb), one after another: element a (len_a bytes
+// from src_a, an LzRec source), then element b; empty ones have length 0.
+// Returns with v past the output.  Block-collective.
+template <bool kReadOnly, typename W, typename Lit, typename Plain>
+__device__ void lz_pairs(W& S, int nb, uint8_t* vout, uint32_t& v, uint32_t& vfloor, uint32_t len_a, uint32_t src_a,
+                         uint32_t len_b, uint32_t src_b, Lit lit, Plain plain) {
+  const int tid = threadIdx.x;
+  if (tid >= nb) len_a = len_b = 0;
+  const bool alone = len_a >= LZ_LONG || len_b >= LZ_LONG;
+  uint32_t total, count;
+  const uint32_t o_at = block_exclusive_sum<uint32_t>(len_a + len_b, S.tmp, &total);
+  const uint32_t c_at = block_exclusive_sum<uint32_t>((len_a ? 1u : 0u) + (len_b ? 1u : 0u) + (alone ? 1u << 16 : 0u),
+                                                      S.tmp, &count);
+  S.out_at[tid] = o_at;
+  S.cnt_at[tid] = c_at;
+  S.len[0][tid] = len_a;
+  S.len[1][tid] = len_b;
+  S.src[0][tid] = src_a;
+  S.src[1][tid] = src_b;
+  if (tid == 0) {
+    S.out_at[W::kThreads] = total;
+    S.cnt_at[W::kThreads] = count;
+  }
+  __syncthreads();
+  for (int i0 = 0; i0 < nb;) {
+    // as many pairs as fit a batch, up to one that is written on its own
+    const bool fits = tid >= i0 && tid < nb && S.out_at[tid + 1] - S.out_at[i0] <= W::kOut - 64 &&
+                      (S.cnt_at[tid + 1] >> 16) == (S.cnt_at[i0] >> 16);
+    const int k = __syncthreads_count(fits);
+    if (k == 0) {
+      lz_one<kReadOnly>(S, vout, v, vfloor, S.src[0][i0], S.len[0][i0], lit, plain);
+      lz_one<kReadOnly>(S, vout, v, vfloor, S.src[1][i0], S.len[1][i0], lit, plain);
+      i0 += 1;
+      continue;
+    }
+    const int i1 = i0 + k;
+    const uint32_t bytes = S.out_at[i1] - S.out_at[i0];
+    if (bytes) {
+      for (uint32_t w = tid; w < (bytes + 31) / 32 + 2 && w < W::kOut / 32 + 2; w += W::kThreads) S.mask[w] = 0;
+      __syncthreads();
+      if (tid >= i0 && tid < i1) {
+        uint32_t a = v + o_at - S.out_at[i0];
+        uint32_t e = (c_at - S.cnt_at[i0]) & 0xffffu;
+        if (len_a) {
+          S.rec[e++] = LzRec{a, src_a};
+          atomicOr(S.mask + ((a >> 5) - (v >> 5)), 1u << (a & 31));
+          a += len_a;
+        }
+        if (len_b) {
+          S.rec[e] = LzRec{a, src_b};
+          atomicOr(S.mask + ((a >> 5) - (v >> 5)), 1u << (a & 31));
+        }
+      }
+      __syncthreads();
+      lz_run<W::kThreads, W::kChunk, W::kRing>(S.rec, static_cast<int>((S.cnt_at[i1] - S.cnt_at[i0]) & 0xffffu), S.mask,
+                                               S.ring, S.notes, vout, v, v + bytes, vfloor, lit);
+      v += bytes;
+      __syncthreads();
+    }
+    i0 = i1;
+  }
+}
+
 }  // namespace pqi

@@ -114,6 +114,7 @@ struct PlanPage {
   int32_t nonnull;         // non-null values on the page; -1 until known [host or walk]
   uint32_t dtab;           // DELTA: first row of the page's block tables
   int32_t dblocks;         // DELTA: blocks found by the walk                [walk]
+                           // transcoded string pages: values             [transcode]
   int32_t dbs;             // DELTA: values per block                        [walk]
   int32_t dvpm;            // DELTA: values per miniblock                    [walk]
   int32_t dmbc;            // DELTA: miniblocks per block                    [walk]
@@ -124,8 +125,8 @@ struct PlanPage {
   int32_t item_rows;       // rows per work item of this page
   int32_t enc;             // encoding the kernels decode: the page's own, or PLAIN once a
                            // BYTE_STREAM_SPLIT / DELTA_(LENGTH_)BYTE_ARRAY page is transcoded
-  uint32_t vtab;           // transcoded string pages: 1 + first row of the page's value-position
-                           // table (DecodeArgs::vpos, written by the transcoder); 0 none
+  uint32_t vtab;           // transcoded string pages: 1 + first row of the page's entry table
+                           // (DecodeArgs::vpos, written by the transcoder); 0 none
 };
 
 // DELTA block-chain region (speculative parallel walk): regions of
