@@ -96,7 +96,8 @@ struct DecodeArgs {
 // table (PlanPage::vtab) filled in `vpos`.
 void launch_transcode(const TranscodeJob* jobs, int n, int n_bss, PlanPage* pps, uint8_t* pool, uint64_t pool_cap,
                       uint32_t* counters, uint64_t* vpos, DevStatus* st, cudaStream_t s);
-void launch_dict(const DictJob* jobs, int n_jobs, int max_fixed_bytes, int max_str_regions, DictScratch ds,
+// fixed: the list has fixed-width dictionaries
+void launch_dict(const DictJob* jobs, int n_jobs, bool fixed, int max_fixed_bytes, int max_str_regions, DictScratch ds,
                  DictDev* dicts, int n_sms, DevStatus* st, cudaStream_t s);
 // Launches over sub-ranges (one output column's share of the plan).
 // levels: the pages have definition levels (their walks use jump tables)

@@ -858,6 +858,15 @@ static void plan_split(pqi::SnappyJob& sj, bool plain, uint32_t* frags, uint32_t
   *segs += sj.nseg;
 }
 
+// Rows per work item: the tuning's, halved down to `least` while a column of
+// n_rows rows has fewer items than the GPU has expansion warps (32 a
+// multiprocessor).  2^20 dictionary rows in 512 items of 2048 occupied 16
+// thread blocks.
+static int64_t plan_item_rows(int64_t rows, int64_t least, int64_t n_rows, int n_sms) {
+  while (rows / 2 >= least && n_rows / rows < 32 * static_cast<int64_t>(n_sms)) rows = rows / 2 / 32 * 32;
+  return rows;
+}
+
 pq_status plan_build(pq_ctx* ctx, pq_index* idx, const std::vector<int32_t>& cols, const std::vector<RowSeg>& segs,
                      int64_t n_rows, uint32_t flags, std::unique_ptr<pq_plan>* out) {
   if ((flags & PQ_SCAN_TIMING) && (flags & PQ_SCAN_GRAPH))
@@ -872,7 +881,9 @@ pq_status plan_build(pq_ctx* ctx, pq_index* idx, const std::vector<int32_t>& col
   const bool plain = (flags & PQ_SCAN_PLAIN) != 0;
   plan->tuning = ctx->tuning;
   plan->staged_expand = plan->tuning.staged_expand && !env_flag("PQ_NO_STAGED_EXPAND");
-  const int64_t item_rows_max = plan->tuning.item_rows;
+  const int64_t item_rows_max = plan_item_rows(plan->tuning.item_rows, 256, n_rows, ctx->n_sms);
+  plan->item_rows = static_cast<int32_t>(item_rows_max);
+  const int64_t item_rows_opt = plan_item_rows(plan->tuning.item_rows_opt, 128, n_rows, ctx->n_sms);
   uint64_t scratch = 0;
   uint64_t tc_pool = 0;               // DELTA_BYTE_ARRAY pool bytes
   std::vector<int64_t> data_job_off;  // scratch offset per data snappy job
@@ -1119,11 +1130,13 @@ pq_status plan_build(pq_ctx* ctx, pq_index* idx, const std::vector<int32_t>& col
         const int64_t span = pp.row_hi - pp.row_lo;
         // pages with definition levels take the short items (their walks and
         // expands carry a bitmap per item; measured faster for PLAIN too)
-        const int64_t per = cd.max_def ? plan->tuning.item_rows_opt : item_rows_max;
+        const int64_t per = cd.max_def ? item_rows_opt : item_rows_max;
+        const int64_t full = cd.max_def ? plan->tuning.item_rows_opt : plan->tuning.item_rows;
         const uint32_t n_it = static_cast<uint32_t>((span + per - 1) / per);
         pp.item_rows = static_cast<int32_t>(per);
         pp.item_count = n_it;
         plan->n_items += n_it;
+        plan->budget_items += static_cast<uint64_t>((span + full - 1) / full);
         plan->pps.push_back(pp);
       }
       const int32_t n_pp = static_cast<int32_t>(plan->pps.size()) - pp_first;
@@ -1406,7 +1419,9 @@ static pq_status plan_size_strings(pq_plan* plan) {
 }
 
 uint64_t plan_device_bytes(const pq_plan* plan, uint64_t scratch) {
-  const uint64_t npp = plan->pps.size(), nit = plan->n_items;
+  // (items counted at the tuning's size: the smaller ones of small scans add
+  // less than the pool's rounding)
+  const uint64_t npp = plan->pps.size(), nit = plan->budget_items;
   const uint64_t str_rows = static_cast<uint64_t>(plan->n_rows) * plan->str_cols.size();
   return npp * sizeof(pqi::PlanPage) + nit * sizeof(pqi::Item) + plan->outcols.size() * sizeof(pqi::OutCol) +
          (plan->snappy_data.size() + plan->snappy_dict.size()) * sizeof(pqi::SnappyJob) + 56ull * plan->snap_blocks +
@@ -1564,7 +1579,7 @@ static void launch_column_expand(pq_plan* plan, size_t oc, const pqi::DecodeArgs
       cw.dict_pages > 0) {
     int bw = 0;
     while (bw < 32 && (int64_t(1) << bw) < cw.max_dict_n) ++bw;
-    const uint32_t stage = pqi::dict_expand_stage_bytes(plan->tuning.item_rows, bw);
+    const uint32_t stage = pqi::dict_expand_stage_bytes(plan->item_rows, bw);
     uint32_t dict_cap = static_cast<uint32_t>((cw.max_dict_bytes + 15) & ~int64_t(15));
     if (cw.max_dict_bytes > (int64_t(1) << 30) || !pqi::dict_expand_fits(stage, dict_cap)) dict_cap = 0;
     if (pqi::dict_expand_fits(stage, dict_cap)) {
@@ -1581,7 +1596,7 @@ static void enqueue_column(pq_plan* plan, size_t oc, const pqi::DecodeArgs& a, b
   const auto& cw = plan->colwork[oc];
   if (with_dicts) launch_column_decompress(plan, oc, true, a.st, s);
   if (with_dicts && cw.dict_n)
-    pqi::launch_dict(plan->d_dict_jobs + cw.dict_begin, cw.dict_n, cw.max_fixed_dict, cw.max_str_regions,
+    pqi::launch_dict(plan->d_dict_jobs + cw.dict_begin, cw.dict_n, plan->outcols[oc].ptype != pqi::T_BYTE_ARRAY, cw.max_fixed_dict, cw.max_str_regions,
                      pqi::DictScratch{plan->d_sregs, plan->d_slists}, plan->idx->d_dicts, ctx->n_sms, a.st, s);
   launch_column_decompress(plan, oc, false, a.st, s);
   enqueue_transcode(plan, cw.tc_begin, cw.tc_n, cw.tc_bss, a, s);
@@ -1619,7 +1634,7 @@ static void enqueue_scan(pq_plan* plan, cudaStream_t s, bool with_dicts, const c
       launch_decompress(plan, plan->d_snappy + n_data_jobs, n_dict_jobs, true, a.st, s);
     mark(2);
     if (with_dicts && !plan->dict_jobs.empty())
-      pqi::launch_dict(plan->d_dict_jobs, static_cast<int>(plan->dict_jobs.size()), plan->max_fixed_dict_bytes,
+      pqi::launch_dict(plan->d_dict_jobs, static_cast<int>(plan->dict_jobs.size()), true, plan->max_fixed_dict_bytes,
                        max_str_regions_all(plan), pqi::DictScratch{plan->d_sregs, plan->d_slists}, plan->idx->d_dicts,
                        ctx->n_sms, a.st, s);
     mark(3);
@@ -1655,7 +1670,7 @@ static void enqueue_scan(pq_plan* plan, cudaStream_t s, bool with_dicts, const c
     for (int oc = 0; oc < ncols; ++oc) {
       const auto& cw = plan->colwork[oc];
       if (with_dicts && cw.dict_n)
-        pqi::launch_dict(plan->d_dict_jobs + cw.dict_begin, cw.dict_n, cw.max_fixed_dict, cw.max_str_regions,
+        pqi::launch_dict(plan->d_dict_jobs + cw.dict_begin, cw.dict_n, plan->outcols[oc].ptype != pqi::T_BYTE_ARRAY, cw.max_fixed_dict, cw.max_str_regions,
                          pqi::DictScratch{plan->d_sregs, plan->d_slists}, plan->idx->d_dicts, ctx->n_sms, a.st, s);
     }
     mark(3);

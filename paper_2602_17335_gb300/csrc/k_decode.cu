@@ -282,9 +282,11 @@ __device__ __forceinline__ int uleb_p(const uint8_t* q, uint64_t* v) {
 constexpr int SREG_LEAD = 1024;
 constexpr int SREG_SMEM = SREG_LEAD + STR_REGION + 64;
 
+// 4 bytes at offset o of a 4-byte aligned buffer (readable for 8 from o
+// rounded down).
 __device__ __forceinline__ uint32_t sle32(const uint8_t* b, uint32_t o) {
-  return static_cast<uint32_t>(b[o]) | (static_cast<uint32_t>(b[o + 1]) << 8) |
-         (static_cast<uint32_t>(b[o + 2]) << 16) | (static_cast<uint32_t>(b[o + 3]) << 24);
+  const uint32_t* w = reinterpret_cast<const uint32_t*>(b) + (o >> 2);
+  return __funnelshift_r(w[0], w[1], 8 * (o & 3));
 }
 
 __global__ void __launch_bounds__(32) k_sreg(const DictJob* __restrict__ jobs, DictScratch ds, DevStatus* st) {
@@ -387,12 +389,13 @@ __global__ void __launch_bounds__(32) k_sreg(const DictJob* __restrict__ jobs, D
 // A region whose found start is not the true entry is walked again from the
 // true entry, in shared memory (the region is staged by one bulk copy), its
 // entries written directly.
-__global__ void __launch_bounds__(256) k_sfix(const DictJob* __restrict__ jobs, DictScratch ds, DictDev* dicts,
+constexpr int SFIX_THREADS = 1024;
+__global__ void __launch_bounds__(SFIX_THREADS) k_sfix(const DictJob* __restrict__ jobs, DictScratch ds, DictDev* dicts,
                                               DevStatus* st) {
   constexpr int MAXR = 2048;
   __shared__ int32_t s_q[MAXR], s_x[MAXR], s_c[MAXR];
   __shared__ int32_t s_skip[MAXR], s_base[MAXR];
-  __shared__ int32_t s_nreg, s_ok;
+  __shared__ int32_t s_nreg, s_ok, s_max;
   __shared__ uint64_t s_bar;
   __shared__ __align__(16) uint8_t s_stage[STR_REGION + 64];
   const DictJob j = jobs[blockIdx.x];
@@ -409,6 +412,7 @@ __global__ void __launch_bounds__(256) k_sfix(const DictJob* __restrict__ jobs, 
       s_c[i] = r.cnt;
     }
   __syncthreads();
+  int32_t walked_max = 0;  // thread 0's: longest entry it walked to
   if (threadIdx.x == 0) {
     mbar_init(&s_bar, 1);
     fence_mbar_init();
@@ -416,6 +420,8 @@ __global__ void __launch_bounds__(256) k_sfix(const DictJob* __restrict__ jobs, 
     bool bad = false;
     uint32_t e = 0;
     int32_t b = 0;
+    s_max = 0;
+    auto walked = [&](uint32_t L) { walked_max = static_cast<int32_t>(L) > walked_max ? static_cast<int32_t>(L) : walked_max; };
     if (!regions) {
       // pages too large for the region tables: one serial walk in global memory
       while (e < blen && b < n) {
@@ -423,6 +429,7 @@ __global__ void __launch_bounds__(256) k_sfix(const DictJob* __restrict__ jobs, 
         const uint32_t L = ld_le32_g(j.body + e);
         if (L > blen - e - 4) { bad = true; break; }
         j.str_ent[b++] = (static_cast<uint64_t>(e + 4) << 32) | L;
+        walked(L);
         e += 4 + L;
       }
       s_nreg = 0;
@@ -464,6 +471,7 @@ __global__ void __launch_bounds__(256) k_sfix(const DictJob* __restrict__ jobs, 
           const uint32_t L = sle32(s_stage, e - e0 + shift);
           if (L > blen - e - 4) { bad = true; break; }
           j.str_ent[b++] = (static_cast<uint64_t>(e + 4) << 32) | L;
+          walked(L);
           e += 4 + L;
         }
       }
@@ -476,23 +484,39 @@ __global__ void __launch_bounds__(256) k_sfix(const DictJob* __restrict__ jobs, 
     if (threadIdx.x == 0) report(st, DERR_CORRUPT, j.page, WHERE_DICT, 2);
     return;
   }
+  // the lists in place, and the longest entry, which picks the padded layout
+  // (copied by k_dict_pad).  Bound by load latency: a region a warp, four
+  // entries a lane in flight (a 10^4-entry page took 65 us with eight warps,
+  // one entry a lane and a second pass for the longest).
   const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  for (int i = threadIdx.x >> 5; i < s_nreg; i += nw) {
-    if (s_skip[i] <= 0) continue;
-    const uint64_t* list = ds.lists + static_cast<uint64_t>(j.sreg + i) * STR_REGION_LIST;
-    for (int k = lane; k < s_skip[i]; k += 32) j.str_ent[s_base[i] + k] = list[k];
-  }
-  __syncthreads();
-  // longest entry: picks the padded layout (copied by k_dict_pad)
-  __shared__ int32_t s_max;
-  if (threadIdx.x == 0) s_max = 0;
-  __syncthreads();
   int32_t mx = 0;
-  for (int32_t i = threadIdx.x; i < n; i += blockDim.x) {
-    const int32_t L = static_cast<int32_t>(static_cast<uint32_t>(j.str_ent[i]));
+  auto longer = [&](uint64_t e) {
+    const int32_t L = static_cast<int32_t>(static_cast<uint32_t>(e));
     mx = L > mx ? L : mx;
+  };
+  for (int i = threadIdx.x >> 5; i < s_nreg; i += nw) {
+    const int32_t c = s_skip[i];
+    const uint64_t* list = ds.lists + static_cast<uint64_t>(j.sreg + i) * STR_REGION_LIST;
+    uint64_t* to = j.str_ent + s_base[i];
+    for (int k0 = 0; k0 < c; k0 += 128) {
+      uint64_t e[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) e[u] = k0 + 32 * u + lane < c ? list[k0 + 32 * u + lane] : 0ull;
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (k0 + 32 * u + lane < c) {
+          to[k0 + 32 * u + lane] = e[u];
+          longer(e[u]);
+        }
+    }
   }
-  atomicMax(&s_max, mx);
+  if (threadIdx.x == 0) mx = mx > walked_max ? mx : walked_max;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const int32_t y = __shfl_xor_sync(0xffffffffu, mx, o);
+    mx = y > mx ? y : mx;
+  }
+  if (lane == 0) atomicMax(&s_max, mx);
   __syncthreads();
   if (threadIdx.x == 0) {
     DictDev d{};
@@ -533,13 +557,14 @@ __global__ void __launch_bounds__(256) k_dict_pad(const DictJob* __restrict__ jo
   }
 }
 
-void launch_dict(const DictJob* jobs, int n_jobs, int max_fixed_bytes, int max_str_regions, DictScratch ds,
+void launch_dict(const DictJob* jobs, int n_jobs, bool fixed, int max_fixed_bytes, int max_str_regions, DictScratch ds,
                  DictDev* dicts, int n_sms, DevStatus* st, cudaStream_t s) {
   if (n_jobs <= 0) return;
   int gx = (max_fixed_bytes / 4 + 256 * 16 - 1) / (256 * 16);
   if (gx < 1) gx = 1;
   if (gx > 4 * n_sms) gx = 4 * n_sms;
-  k_dict_fixed<<<dim3(gx, n_jobs), 256, 0, s>>>(jobs, dicts, st);
+  if (fixed)
+    k_dict_fixed<<<dim3(gx, n_jobs), 256, 0, s>>>(jobs, dicts, st);
   if (max_str_regions > 0) {
     static bool attr = false;
     if (!attr) {
@@ -547,7 +572,7 @@ void launch_dict(const DictJob* jobs, int n_jobs, int max_fixed_bytes, int max_s
       attr = true;
     }
     k_sreg<<<dim3(max_str_regions, n_jobs), 32, SREG_SMEM, s>>>(jobs, ds, st);
-    k_sfix<<<n_jobs, 256, 0, s>>>(jobs, ds, dicts, st);
+    k_sfix<<<n_jobs, SFIX_THREADS, 0, s>>>(jobs, ds, dicts, st);
     k_dict_pad<<<dim3(32, n_jobs), 256, 0, s>>>(jobs, dicts);
   }
 }
@@ -2594,7 +2619,7 @@ __global__ void __launch_bounds__(EXP_THREADS, 4) k_expand(DecodeArgs a, int ibe
 // ------------------------------------------------------------------ staged dictionary expand
 
 // REQUIRED fixed-width columns with dictionary pages.  A thread block claims
-// spans of SX_SPAN consecutive work items; its SX_WARPS warps take every
+// spans of up to SX_SPAN consecutive work items; its SX_WARPS warps take every
 // SX_WARPS-th item of the span.  Each warp stages an item's index bytes
 // (from the checkpoint run header on) into shared memory with one bulk copy,
 // issued one item ahead into the warp's other buffer, so that the next
@@ -2609,7 +2634,7 @@ __global__ void __launch_bounds__(EXP_THREADS, 4) k_expand(DecodeArgs a, int ibe
 // of pages that are not dictionary encoded, take the general warp decode.
 constexpr int SX_WARPS = 8;
 constexpr int SX_THREADS = 32 * SX_WARPS;
-constexpr int SX_SPAN = 32;
+constexpr int SX_SPAN = 32;  // most
 constexpr int SX_MAXRUNS = 96;
 constexpr uint32_t SX_DICT_MAX = 48 * 1024;
 
@@ -2852,7 +2877,7 @@ __device__ bool sx_decode(const DecodeArgs& a, const SxItem& t, const SxPage& g,
 
 template <int kWidth>
 __global__ void __launch_bounds__(SX_THREADS) k_dict_expand(DecodeArgs a, int ibegin, int icount, int cidx,
-                                                            uint32_t stage, uint32_t dict_cap) {
+                                                            uint32_t stage, uint32_t dict_cap, int span_items) {
   extern __shared__ __align__(16) uint8_t sxraw[];
   SxBlock& sm = *reinterpret_cast<SxBlock*>(sxraw);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -2863,7 +2888,7 @@ __global__ void __launch_bounds__(SX_THREADS) k_dict_expand(DecodeArgs a, int ib
   uint8_t* sdict = dict_cap ? bufs + SX_WARPS * 2u * (stage + 16) : nullptr;
   uint32_t* ctr = a.item_counter + EXP_COUNTER0 + cidx;
   uint8_t* const col_values = a.cols[cidx].values;
-  const int nspans = (icount + SX_SPAN - 1) / SX_SPAN;
+  const int nspans = (icount + span_items - 1) / span_items;
   const int iend = ibegin + icount;
   if (threadIdx.x == 0) {
     mbar_init(&sm.dbar, 1);
@@ -2883,8 +2908,8 @@ __global__ void __launch_bounds__(SX_THREADS) k_dict_expand(DecodeArgs a, int ib
     const int span = sm.span;
     if (span >= nspans) break;
     __syncthreads();  // every thread has read sm.span
-    const int first = ibegin + span * SX_SPAN;
-    const int last = first + SX_SPAN < iend ? first + SX_SPAN : iend;
+    const int first = ibegin + span * span_items;
+    const int last = first + span_items < iend ? first + span_items : iend;
     if (threadIdx.x == 0) sm.span = static_cast<int>(atomicAdd(ctr, 1u));
     if (sdict) {
       // the span's dictionary: that of its first item
@@ -3574,13 +3599,18 @@ void launch_dict_expand(const DecodeArgs& a, int ibegin, int n, int cidx, int n_
   else
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_dict_expand<8>, SX_THREADS, smem);
   if (bps < 1) bps = 1;
-  const int spans = (n + SX_SPAN - 1) / SX_SPAN;
+  // long spans overlap the copy of an item with the decode of the one before
+  // it and load a dictionary once; short ones where there would be less than
+  // two for every resident block
+  int span = SX_SPAN;
+  while (span > SX_WARPS && n < 2 * span * n_sms * bps) span /= 2;
+  const int spans = (n + span - 1) / span;
   int blocks = n_sms * bps;
   if (blocks > spans) blocks = spans;
   if (width == 4)
-    k_dict_expand<4><<<blocks, SX_THREADS, smem, s>>>(a, ibegin, n, cidx, stage, dict_cap);
+    k_dict_expand<4><<<blocks, SX_THREADS, smem, s>>>(a, ibegin, n, cidx, stage, dict_cap, span);
   else
-    k_dict_expand<8><<<blocks, SX_THREADS, smem, s>>>(a, ibegin, n, cidx, stage, dict_cap);
+    k_dict_expand<8><<<blocks, SX_THREADS, smem, s>>>(a, ibegin, n, cidx, stage, dict_cap, span);
 }
 
 void launch_expand(const DecodeArgs& a, int ibegin, int n, int cidx, int n_sms, int ctas_per_sm, cudaStream_t s) {
