@@ -62,7 +62,8 @@ constexpr int TC_POOL_COUNTER = 2;
 
 // Words of the item_counter array of a scan of n_cols output columns.
 PQ_HD constexpr uint32_t SNAP_COUNTER0(uint32_t n_cols) { return 4 + n_cols; }
-PQ_HD constexpr uint32_t SCAN_COUNTERS(uint32_t n_cols) { return SNAP_COUNTER0(n_cols) + 2 * SNAPPY_RUNS * n_cols; }
+PQ_HD constexpr uint32_t STR_COUNTER0(uint32_t n_cols) { return SNAP_COUNTER0(n_cols) + 2 * SNAPPY_RUNS * n_cols; }
+PQ_HD constexpr uint32_t SCAN_COUNTERS(uint32_t n_cols) { return STR_COUNTER0(n_cols) + n_cols; }
 
 struct DecodeArgs {
   const ChunkDev* chunks;
@@ -74,7 +75,8 @@ struct DecodeArgs {
   DevStatus* st;
   uint32_t* item_counter;   // [2..3] transcode pool bytes, [4 + c] next work item of output column c,
                             // [SNAP_COUNTER0(n) + 2 R c + R d + r] (R = SNAPPY_RUNS) next segment of run r of its split
-                            // data (d = 0) or dictionary (d = 1) pages
+                            // data (d = 0) or dictionary (d = 1) pages; [STR_COUNTER0(n) + c] strings of c left to
+                            // k_str_copy
   const uint32_t* walk_pps; // plan pages that need the walk, longest chains first
   const uint32_t* delta_pps;// DELTA plan pages (block bases)
   uint32_t* dpos;           // DELTA block positions (stream offsets)
@@ -104,7 +106,9 @@ void launch_dict(const DictJob* jobs, int n_jobs, bool fixed, int max_fixed_byte
 // window: bytes per chain window (0: chosen by page count)
 void launch_walk(const DecodeArgs& a, int wbegin, int n, int n_sms, bool levels, uint32_t window, cudaStream_t s);
 void launch_delta_bases(const DecodeArgs& a, int dbegin, int n, int max_regions, cudaStream_t s);
-void launch_expand(const DecodeArgs& a, int ibegin, int n, int cidx, int n_sms, int ctas_per_sm, cudaStream_t s);
+// delta: the column has DELTA_BINARY_PACKED pages
+void launch_expand(const DecodeArgs& a, int ibegin, int n, int cidx, bool delta, int n_sms, int ctas_per_sm,
+                   cudaStream_t s);
 // REQUIRED fixed-width columns with dictionary pages: items staged in shared
 // memory (`stage` bytes per buffer, dict_expand_stage_bytes), dictionaries of
 // up to `dict_cap` bytes gathered from shared memory (0: from global memory).
@@ -115,8 +119,11 @@ void launch_dict_expand(const DecodeArgs& a, int ibegin, int n, int cidx, int n_
 // Items of a column whose pages are all REQUIRED PLAIN fixed-width: copies.
 void launch_copy_items(const DecodeArgs& a, int ibegin, int n, int cidx, int n_sms, int ctas_per_sm,
                        cudaStream_t s);
-// copy_chars false: only the offsets pass (chars totals), no chars written
-void launch_strings(const DecodeArgs& a, int col, int n_items, int n_sms, bool copy_chars, cudaStream_t s);
+// copy_chars false: only the offsets pass (chars totals), no chars written.
+// left: null when the column has no dictionary pages, else a word (zero
+// before the launch) for what the copy of padded dictionaries leaves.
+void launch_strings(const DecodeArgs& a, int col, int n_items, int n_sms, bool copy_chars, uint32_t* left,
+                    cudaStream_t s);
 // Plain baseline: pages [pp_begin, pp_begin + n) decoded one page per block.
 void launch_plain_pages(const DecodeArgs& a, int pp_begin, int n, cudaStream_t s);
 void launch_prepare(const DecodeArgs& a, int n_cols, int grid, cudaStream_t s);

@@ -1340,7 +1340,8 @@ pq_status plan_upload(pq_plan* plan, cudaStream_t s) {
              (cw.delta_n ? 4 : 0) + (cw.tc_bss ? 1 : 0) + (cw.tc_n > cw.tc_bss ? 1 : 0) + (plan->outcols[oc].item_count ? 1 : 0);
       }
     }
-    for (int32_t sc : plan->str_cols) n += plan->outcols[sc].item_count ? 2 : 0;
+    for (int32_t sc : plan->str_cols)
+      n += plan->outcols[sc].item_count ? (plan->colwork[sc].dict_pages ? 3 : 2) : 0;
     plan->launches = n;
   }
   const int wbps = pqi::walk_blocks_per_sm(), ebps = pqi::expand_blocks_per_sm();
@@ -1587,7 +1588,13 @@ static void launch_column_expand(pq_plan* plan, size_t oc, const pqi::DecodeArgs
       return;
     }
   }
-  pqi::launch_expand(a, ib, n, static_cast<int>(oc), ctx->n_sms, plan->tuning.expand_ctas_per_sm, s);
+  pqi::launch_expand(a, ib, n, static_cast<int>(oc), cw.delta_n > 0, ctx->n_sms, plan->tuning.expand_ctas_per_sm, s);
+}
+
+// The word in which k_str_dict notes strings it leaves (null: no dictionary pages).
+static uint32_t* strings_left(pq_plan* plan, size_t oc) {
+  if (!plan->colwork[oc].dict_pages) return nullptr;
+  return plan->d_counter + pqi::STR_COUNTER0(static_cast<uint32_t>(plan->outcols.size())) + oc;
 }
 
 // Kernels of one output column, in order, on one stream.
@@ -1605,7 +1612,8 @@ static void enqueue_column(pq_plan* plan, size_t oc, const pqi::DecodeArgs& a, b
   pqi::launch_delta_bases(a, cw.delta_begin, cw.delta_n, cw.max_regions, s);
   launch_column_expand(plan, oc, a, s);
   if (col.ptype == pqi::T_BYTE_ARRAY)
-    pqi::launch_strings(a, static_cast<int>(oc), static_cast<int>(col.item_count), ctx->n_sms, !plan->sizing, s);
+    pqi::launch_strings(a, static_cast<int>(oc), static_cast<int>(col.item_count), ctx->n_sms, !plan->sizing,
+                        strings_left(plan, oc), s);
 }
 
 // Enqueues the kernels of one scan (no host synchronisation).  Default:
@@ -1658,7 +1666,8 @@ static void enqueue_scan(pq_plan* plan, cudaStream_t s, bool with_dicts, const c
     mark(4);
     mark(5);
     for (int32_t sc : plan->str_cols)
-      pqi::launch_strings(a, sc, static_cast<int>(plan->outcols[sc].item_count), ctx->n_sms, !plan->sizing, s);
+      pqi::launch_strings(a, sc, static_cast<int>(plan->outcols[sc].item_count), ctx->n_sms, !plan->sizing,
+                          strings_left(plan, sc), s);
   } else if (timing) {
     for (int oc = 0; oc < ncols; ++oc) {
       const auto& cw = plan->colwork[oc];
@@ -1684,7 +1693,8 @@ static void enqueue_scan(pq_plan* plan, cudaStream_t s, bool with_dicts, const c
     for (int oc = 0; oc < ncols; ++oc) launch_column_expand(plan, oc, a, s);
     mark(5);
     for (int32_t sc : plan->str_cols)
-      pqi::launch_strings(a, sc, static_cast<int>(plan->outcols[sc].item_count), ctx->n_sms, !plan->sizing, s);
+      pqi::launch_strings(a, sc, static_cast<int>(plan->outcols[sc].item_count), ctx->n_sms, !plan->sizing,
+                          strings_left(plan, sc), s);
   } else {
     cudaEventRecord(plan->fork, s);
     for (int oc = 0; oc < ncols; ++oc) {

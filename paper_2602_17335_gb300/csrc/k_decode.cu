@@ -523,7 +523,9 @@ __global__ void __launch_bounds__(SFIX_THREADS) k_sfix(const DictJob* __restrict
     d.str_ent = j.str_ent;
     d.n = n;
     d.max_len = s_max;
-    d.chars = j.pad && n > 0 && s_max <= PAD_STRIDE_MAX ? j.pad : j.body;
+    const bool padded = j.pad && n > 0 && s_max <= PAD_STRIDE_MAX;
+    d.chars = padded ? j.pad : j.body;
+    d.width = padded ? (s_max + 15) & ~15 : 0;
     d.valid = 1;
     dicts[j.chunk] = d;
   }
@@ -532,13 +534,13 @@ __global__ void __launch_bounds__(SFIX_THREADS) k_sfix(const DictJob* __restrict
 // Padded copy of the string dictionaries k_sfix marked for it: thread i
 // copies entry i (aligned words, the last one masked) to pad + i * stride
 // and points the entry there.  The bytes after an entry up to the next
-// stride are left as they are (never read as data).
+// stride are zero (k_str_dict ORs whole words of neighbouring strings).
 __global__ void __launch_bounds__(256) k_dict_pad(const DictJob* __restrict__ jobs, const DictDev* dicts) {
   const DictJob j = jobs[blockIdx.y];
   if (j.ptype != T_BYTE_ARRAY || !j.pad) return;
   const DictDev d = dicts[j.chunk];
   if (!d.valid || d.chars != j.pad) return;
-  const uint32_t stride = (static_cast<uint32_t>(d.max_len) + 15u) & ~15u;
+  const uint32_t stride = static_cast<uint32_t>(d.width);
   for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < j.n; i += gridDim.x * blockDim.x) {
     const uint64_t e = j.str_ent[i];
     const uint32_t len = static_cast<uint32_t>(e);
@@ -548,9 +550,10 @@ __global__ void __launch_bounds__(256) k_dict_pad(const DictJob* __restrict__ jo
     const uint32_t sh = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(src) & 3) * 8;
     const uint32_t nw = (len + 3) >> 2;
     uint32_t cur = nw ? q[0] : 0u;
-    for (uint32_t k = 0; k < nw; ++k) {
-      const uint32_t nx = q[k + 1];
-      dst[k] = __funnelshift_r(cur, nx, sh);
+    for (uint32_t k = 0; k < stride / 4; ++k) {
+      const uint32_t nx = k < nw ? q[k + 1] : 0u;
+      const uint32_t w = k < nw ? __funnelshift_r(cur, nx, sh) : 0u;
+      dst[k] = 4 * k + 4 > len && k < nw ? w & (0xffffffffu >> (8 * (4 * k + 4 - len))) : w;
       cur = nx;
     }
     j.str_ent[i] = (static_cast<uint64_t>(static_cast<uint64_t>(i) * stride) << 32) | len;
@@ -2297,6 +2300,73 @@ __device__ bool warp_delta(const uint8_t* sb, const PlanPage& pp, const uint32_t
         const uint32_t offm = 32u * (m == 0 ? 0u : m == 1 ? w0 : m == 2 ? w0 + w1 : w0 + w1 + w2);
         const uint64_t b0 = static_cast<uint64_t>(pos + vl + 4) * 8 + offm + static_cast<uint64_t>(lane & 7) * 4 * w;
         const int v0 = 4 * lane;
+        if (__vcmpgtu4(w4, 0x18181818u) == 0u) {
+          // widths of at most 24 bits: the packed deltas add up in 32 bits
+          // over a block, the min deltas by a product (half the shuffles of
+          // the 64-bit scan)
+          uint32_t r[4];
+          if (w <= 16) {
+            const uint64_t win = v0 < nv ? gwin64(sb, b0) : 0ull;
+            const uint32_t mask = (1u << w) - 1u;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) r[i] = static_cast<uint32_t>(win >> (i * w)) & mask;
+          } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+              r[i] = v0 + i < nv ? gbits32(sb, b0 + static_cast<uint64_t>(i) * w, static_cast<int>(w)) : 0u;
+          }
+          r[1] += r[0];
+          r[2] += r[1];
+          r[3] += r[2];
+          uint32_t incl = r[3];
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+          }
+          uint64_t v[4];
+          const uint64_t from = base + mn * static_cast<uint64_t>(v0) + (incl - r[3]);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) v[i] = from + mn * static_cast<uint64_t>(i + 1) + r[i];
+          if (sink.out && !sink.vbuf && !sink.sidx && nv == 128 && bk >= k0 && bk + 128 <= k1) {
+            // the whole block straight to the output, 16 bytes a store (8-byte
+            // values that start in the middle of 16 bytes pair up with the
+            // next lane's first)
+            const int64_t row = sink.orow0 + (bk - k0) + v0;
+            if (sink.width == 8) {
+              uint64_t* o = reinterpret_cast<uint64_t*>(sink.out) + row;
+              auto put2 = [](uint64_t* p, uint64_t x0, uint64_t x1) {
+                *reinterpret_cast<ulonglong2*>(p) = make_ulonglong2(x0, x1);
+              };
+              if ((reinterpret_cast<uintptr_t>(o) & 15) == 0) {
+                put2(o, v[0], v[1]);
+                put2(o + 2, v[2], v[3]);
+              } else {
+                const uint64_t nx = __shfl_down_sync(0xffffffffu, v[0], 1);
+                if (lane == 0) o[0] = v[0];
+                put2(o + 1, v[1], v[2]);
+                if (lane < 31) put2(o + 3, v[3], nx);
+                else o[3] = v[3];
+              }
+            } else {
+              uint32_t* o = reinterpret_cast<uint32_t*>(sink.out) + row;
+              if ((reinterpret_cast<uintptr_t>(o) & 15) == 0) {
+                *reinterpret_cast<uint4*>(o) = make_uint4(static_cast<uint32_t>(v[0]), static_cast<uint32_t>(v[1]),
+                                                          static_cast<uint32_t>(v[2]), static_cast<uint32_t>(v[3]));
+              } else {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) o[i] = static_cast<uint32_t>(v[i]);
+              }
+            }
+          } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const int64_t dense = bk + v0 + i;
+              if (v0 + i < nv && dense >= k0 && dense < k1) sink.put(static_cast<int32_t>(dense - k0), v[i]);
+            }
+          }
+          continue;
+        }
         uint64_t x[4];
         if (v0 < nv) {
           if (w <= 16) {
@@ -2451,6 +2521,9 @@ __global__ void __launch_bounds__(256) k_copy_items(DecodeArgs a, int ibegin, in
   }
 }
 
+// kDelta false: no page of the item's column is DELTA_BINARY_PACKED (its
+// decode is the one that needs the most registers).
+template <bool kDelta = true>
 __device__ void expand_item(const DecodeArgs& a, int it_id, WarpSmem& ws, int lane) {
   const Item it = a.items[it_id];
   if (it.nrows <= 0) return;
@@ -2553,7 +2626,7 @@ __device__ void expand_item(const DecodeArgs& a, int it_id, WarpSmem& ws, int la
       const int bw = __ldg(sb);
       ok = bw <= 32 && warp_hybrid(sb + 1, slen - 1, bw, pp.nonnull, static_cast<uint32_t>(it.pos), it.run_k0, k0,
                                    k0 + nn, dd, isba, sink, &chars, lane);
-    } else if (isdelta) {
+    } else if (kDelta && isdelta) {
       ok = warp_delta(sb, pp, a.dpos + pp.dtab, a.dbase + pp.dtab, type_bits, k0, k0 + nn, sink, lane);
     } else if (isba && pp.vtab) {
       ok = warp_table_ba(a.vpos + (pp.vtab - 1), slen, k0, k0 + nn, sink, &chars, lane);
@@ -2599,7 +2672,9 @@ __device__ void expand_item(const DecodeArgs& a, int it_id, WarpSmem& ws, int la
 // Items [ibegin, ibegin + icount), handed out one at a time to warps through
 // the column's counter (items differ in cost), over a grid sized to the
 // resident capacity.
-__global__ void __launch_bounds__(EXP_THREADS, 4) k_expand(DecodeArgs a, int ibegin, int icount, int cidx) {
+template <bool kDelta>
+__global__ void __launch_bounds__(EXP_THREADS, 4) k_expand(const __grid_constant__ DecodeArgs a, int ibegin, int icount,
+                                                           int cidx) {
   __shared__ WarpSmem ws[EXP_WARPS];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint32_t* ctr = a.item_counter + EXP_COUNTER0 + cidx;
@@ -2611,16 +2686,23 @@ __global__ void __launch_bounds__(EXP_THREADS, 4) k_expand(DecodeArgs a, int ibe
   while (u < icount) {
     int un = 0;
     if (lane == 0) un = static_cast<int>(atomicAdd(ctr, 1u));
-    expand_item(a, ibegin + u, ws[warp], lane);
+    expand_item<kDelta>(a, ibegin + u, ws[warp], lane);
     u = __shfl_sync(0xffffffffu, un, 0);
   }
 }
 
 // ------------------------------------------------------------------ staged dictionary expand
 
-// REQUIRED fixed-width columns with dictionary pages.  A thread block claims
-// spans of up to SX_SPAN consecutive work items; its SX_WARPS warps take every
-// SX_WARPS-th item of the span.  Each warp stages an item's index bytes
+// REQUIRED fixed-width columns with dictionary pages.  A thread block works
+// on spans of consecutive work items, its SX_WARPS warps taking every
+// SX_WARPS-th item of a span.  Where dictionaries fit shared memory, a block's
+// one span is its equal share of the column, taken in parts where it reaches
+// over several dictionaries (2^25 values of 10^4 distinct ones: 152 us with
+// claimed spans of 32 items, 127 us).  Larger dictionaries are gathered
+// from L2: there blocks claim spans in order, so that all of them are at the
+// same dictionary, SX_SPAN items at most and fewer towards the end (2^25
+// values of 2^20 distinct ones: 238 us in equal shares, 215 us with spans
+// of one size, whose last wave was a third empty, 197 us).  Each warp stages an item's index bytes
 // (from the checkpoint run header on) into shared memory with one bulk copy,
 // issued one item ahead into the warp's other buffer, so that the next
 // item's bytes stream in while the current one is decoded; the item and
@@ -2634,7 +2716,7 @@ __global__ void __launch_bounds__(EXP_THREADS, 4) k_expand(DecodeArgs a, int ibe
 // of pages that are not dictionary encoded, take the general warp decode.
 constexpr int SX_WARPS = 8;
 constexpr int SX_THREADS = 32 * SX_WARPS;
-constexpr int SX_SPAN = 32;  // most
+constexpr int SX_SPAN = 32;
 constexpr int SX_MAXRUNS = 96;
 constexpr uint32_t SX_DICT_MAX = 48 * 1024;
 
@@ -2646,7 +2728,7 @@ struct SxWarp {
 };
 struct SxBlock {
   uint64_t dbar;
-  int32_t span;    // the span claimed for the next round
+  int32_t span, span_n;  // first item (of the column's) and items of the next span
   int32_t dchunk;  // chunk whose dictionary is in shared memory (-1 none)
   SxWarp w[SX_WARPS];
 };
@@ -2875,9 +2957,15 @@ __device__ bool sx_decode(const DecodeArgs& a, const SxItem& t, const SxPage& g,
   return true;
 }
 
+// Chunk whose dictionary the pages of an item index, -1 for other pages.
+__device__ __forceinline__ int32_t sx_dict_of(const DecodeArgs& a, int item) {
+  const PlanPage& pp = a.pps[a.items[item].pp];
+  return (pp.enc == ENC_RLE_DICT || pp.enc == ENC_PLAIN_DICT) && pp.dict >= 0 ? pp.dict : -1;
+}
+
 template <int kWidth>
 __global__ void __launch_bounds__(SX_THREADS) k_dict_expand(DecodeArgs a, int ibegin, int icount, int cidx,
-                                                            uint32_t stage, uint32_t dict_cap, int span_items) {
+                                                            uint32_t stage, uint32_t dict_cap) {
   extern __shared__ __align__(16) uint8_t sxraw[];
   SxBlock& sm = *reinterpret_cast<SxBlock*>(sxraw);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -2888,11 +2976,38 @@ __global__ void __launch_bounds__(SX_THREADS) k_dict_expand(DecodeArgs a, int ib
   uint8_t* sdict = dict_cap ? bufs + SX_WARPS * 2u * (stage + 16) : nullptr;
   uint32_t* ctr = a.item_counter + EXP_COUNTER0 + cidx;
   uint8_t* const col_values = a.cols[cidx].values;
-  const int nspans = (icount + span_items - 1) / span_items;
+  int part = static_cast<int>(static_cast<int64_t>(icount) * blockIdx.x / gridDim.x);
+  const int share_end = static_cast<int>(static_cast<int64_t>(icount) * (blockIdx.x + 1) / gridDim.x);
+  auto claim = [&]() {  // thread 0
+    if (sdict) {
+      // the rest of the share, up to the last item with its first item's dictionary
+      sm.span = part < share_end ? part : icount;
+      int lo = part, hi = share_end - 1;
+      if (part < share_end) {
+        const int32_t want = sx_dict_of(a, ibegin + part);
+        if (sx_dict_of(a, ibegin + hi) == want) {
+          lo = hi;
+        } else {
+          while (lo + 1 < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (sx_dict_of(a, ibegin + mid) == want) lo = mid; else hi = mid;
+          }
+        }
+      }
+      sm.span_n = lo + 1 - part;
+      part = lo + 1;
+      return;
+    }
+    const int left = icount - static_cast<int>(*reinterpret_cast<volatile uint32_t*>(ctr));
+    int n = left / (2 * static_cast<int>(gridDim.x)) / SX_WARPS * SX_WARPS;
+    n = n < SX_WARPS ? SX_WARPS : (n > SX_SPAN ? SX_SPAN : n);
+    sm.span = static_cast<int>(atomicAdd(ctr, static_cast<uint32_t>(n)));
+    sm.span_n = n;
+  };
   const int iend = ibegin + icount;
   if (threadIdx.x == 0) {
     mbar_init(&sm.dbar, 1);
-    sm.span = static_cast<int>(atomicAdd(ctr, 1u));
+    claim();
     sm.dchunk = -1;
   }
   if (lane == 0) {
@@ -2905,19 +3020,16 @@ __global__ void __launch_bounds__(SX_THREADS) k_dict_expand(DecodeArgs a, int ib
   SxPage pg;
   pg.pp = -1;
   for (;;) {
-    const int span = sm.span;
-    if (span >= nspans) break;
+    const int span = sm.span, span_n = sm.span_n;
+    if (span >= icount) break;
     __syncthreads();  // every thread has read sm.span
-    const int first = ibegin + span * span_items;
-    const int last = first + span_items < iend ? first + span_items : iend;
-    if (threadIdx.x == 0) sm.span = static_cast<int>(atomicAdd(ctr, 1u));
+    const int first = ibegin + span;
+    const int last = first + span_n < iend ? first + span_n : iend;
+    if (threadIdx.x == 0) claim();
     if (sdict) {
       // the span's dictionary: that of its first item
       if (threadIdx.x == 0) {
-        const Item& it = a.items[first];
-        const PlanPage& pp = a.pps[it.pp];
-        const bool dict = (pp.enc == ENC_RLE_DICT || pp.enc == ENC_PLAIN_DICT) && pp.dict >= 0;
-        int want = dict ? pp.dict : -1;
+        int want = sx_dict_of(a, first);
         if (want >= 0 && want != sm.dchunk) {
           const DictDev& dd = a.dicts[want];
           const uint64_t db = ((static_cast<uint64_t>(dd.n) * dd.width) + 15) & ~uint64_t(15);
@@ -3113,8 +3225,148 @@ struct StrWarpSmem {
 };
 constexpr int STR_SMEM = 8 * sizeof(StrWarpSmem);
 
-__global__ void __launch_bounds__(256, 4) k_str_copy(DecodeArgs a, int c) {
+// Strings that k_str_dict copies: dictionary entries in a padded layout.
+__device__ __forceinline__ bool str_padded(const DecodeArgs& a, const PlanPage& pp) {
+  // (a transcoded page is never a dictionary page: its own encoding decides)
+  const int32_t enc = a.pages[pp.page].encoding;
+  return (enc == ENC_RLE_DICT || enc == ENC_PLAIN_DICT) && pp.dict >= 0 && a.dicts[pp.dict].width > 0;
+}
+
+// Chars and offsets of an item whose entries sit in a padded dictionary
+// (16-byte aligned, zero past their end, at most 16 NB bytes), one warp, 32
+// strings at a time.  Lane l's string is loaded into registers whole, shifted
+// to its place modulo 4 and stored to the staging words it owns: those from
+// its first byte's word on, the last one together with the next string's
+// first bytes, which come by a shuffle.  Chunks with strings of 1-3 bytes,
+// where a word may belong to three strings, are OR-ed into zeroed words.  The
+// staged chunk, congruent to the output mod 16, leaves as 16-byte stores.
+// The next chunk's entries and the one after that's are in flight meanwhile.
+constexpr int STRD_WORDS = (32 * PAD_STRIDE_MAX + 16 + 48) / 4;
+template <int NB>
+__device__ __forceinline__ void str_dict_item(const DecodeArgs& a, const Item& it, const OutCol& col, int64_t orow0,
+                                              uint64_t base, const uint8_t* chars, uint32_t* stage, int lane) {
+  int64_t* offs = reinterpret_cast<int64_t*>(col.values);
+  auto entry = [&](int r) { return r < it.nrows ? col.str_scratch[orow0 + r] : 0ull; };
+  auto fetch = [&](uint64_t e, uint4 (&v)[NB]) {
+    const uint4* p = reinterpret_cast<const uint4*>(chars + (e >> 32));
+#pragma unroll
+    for (int b = 0; b < NB; ++b)
+      v[b] = static_cast<uint32_t>(e) > 16u * b ? __ldg(p + b) : make_uint4(0, 0, 0, 0);
+  };
+  uint64_t e0 = entry(lane), e1 = entry(32 + lane);
+  uint4 v0[NB];
+  fetch(e0, v0);
+  for (int g0 = 0; g0 < it.nrows; g0 += 32) {
+    uint4 v1[NB];
+    fetch(e1, v1);
+    const uint64_t e2 = entry(g0 + 64 + lane);
+    const uint32_t len = static_cast<uint32_t>(e0);
+    uint32_t incl = len;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += y;
+    }
+    const uint32_t tot = __shfl_sync(0xffffffffu, incl, 31);
+    if (g0 + lane < it.nrows) offs[orow0 + g0 + lane] = static_cast<int64_t>(base + incl - len);
+    if (base + tot <= col.chars_cap) {
+      const uint32_t a0 = static_cast<uint32_t>(base & 15);
+      const uint32_t s = a0 + incl - len, e = s + len, dd = s & 3;
+      uint32_t t[4 * NB + 1];
+      {
+        uint32_t before = 0;
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+          const uint32_t w[4] = {v0[b].x, v0[b].y, v0[b].z, v0[b].w};
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            t[4 * b + i] = __funnelshift_l(before, w[i], 8 * dd);
+            before = w[i];
+          }
+        }
+        t[4 * NB] = __funnelshift_l(before, 0u, 8 * dd);
+      }
+      const uint32_t some = __ballot_sync(0xffffffffu, len > 0);
+      uint32_t* to = stage + (s >> 2);
+      if (!__any_sync(0xffffffffu, len > 0 && len < 4)) {
+        // the next string's bytes in this one's last word
+        const uint32_t after = lane < 31 ? some >> (lane + 1) << (lane + 1) : 0u;
+        const uint32_t head = __shfl_sync(0xffffffffu, dd ? t[0] : 0u, after ? __ffs(after) - 1 : lane);
+        const int i0 = dd && (some & ((1u << lane) - 1u)) ? 1 : 0;
+        const int i1 = static_cast<int>((e + 3) >> 2) - static_cast<int>(s >> 2);  // words the string touches
+        const int il = (e & 3) ? i1 - 1 : -1;
+        if (len > 0) {
+#pragma unroll
+          for (int i = 0; i <= 4 * NB; ++i)
+            if (i >= i0 && i < i1) to[i] = t[i] | (i == il && after ? head : 0u);
+        }
+      } else {
+        for (uint32_t q = lane; q < (a0 + tot + 3) / 4; q += 32) stage[q] = 0;
+        __syncwarp();
+        const int i1 = static_cast<int>((e + 3) >> 2) - static_cast<int>(s >> 2);
+        if (len > 0) {
+#pragma unroll
+          for (int i = 0; i <= 4 * NB; ++i)
+            if (i < i1) atomicOr(to + i, t[i]);
+        }
+      }
+      __syncwarp();
+      const uint8_t* sb = reinterpret_cast<const uint8_t*>(stage);
+      uint8_t* g = col.chars + base;
+      const uint32_t head = a0 ? 16 - a0 : 0;
+      const uint32_t hh = head < tot ? head : tot;
+      if (static_cast<uint32_t>(lane) < hh) g[lane] = sb[a0 + lane];
+      const uint32_t nv = (tot - hh) >> 4;
+      const uint4* sv = reinterpret_cast<const uint4*>(sb + a0 + hh);
+      uint4* gv = reinterpret_cast<uint4*>(g + hh);
+      for (uint32_t q = lane; q < nv; q += 32) gv[q] = sv[q];
+      const uint32_t q = hh + (nv << 4) + lane;
+      if (q < tot) g[q] = sb[a0 + q];
+      __syncwarp();
+    }
+    base += tot;
+    e0 = e1;
+    e1 = e2;
+#pragma unroll
+    for (int b = 0; b < NB; ++b) v0[b] = v1[b];
+  }
+}
+
+// Items of padded dictionaries (others are left to k_str_copy: *left is set).
+// Bound by instruction issue and the L1 data pipe: about half the
+// instructions and a third of the shared-memory traffic a string of the copy
+// through shared-memory source slots that k_str_copy does (2^25 strings of
+// 8-32 bytes: 513 us there).
+__global__ void __launch_bounds__(256, 4) k_str_dict(const __grid_constant__ DecodeArgs a, int c, uint32_t* left) {
+  __shared__ __align__(16) uint32_t stages[8][STRD_WORDS];
+  const int lane = threadIdx.x & 31;
+  uint32_t* stage = stages[threadIdx.x >> 5];
+  const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int nw = (gridDim.x * blockDim.x) >> 5;
+  const OutCol col = a.cols[c];
+  const int ib = static_cast<int>(col.item_begin), ie = ib + static_cast<int>(col.item_count);
+  for (int itx = ib + gw; itx < ie; itx += nw) {
+    const Item it = a.items[itx];
+    const PlanPage& pp = a.pps[it.pp];
+    if (it.nrows <= 0 || pp.nonnull < 0) continue;
+    if (!str_padded(a, pp)) {
+      if (lane == 0) *reinterpret_cast<volatile uint32_t*>(left) = 1;
+      continue;
+    }
+    const DictDev& dd = a.dicts[pp.dict];
+    const int64_t orow0 = pp.out_row + it.row0;
+    const uint64_t base = col.str_item_bytes[itx];
+    if (dd.width <= 32)
+      str_dict_item<2>(a, it, col, orow0, base, dd.chars, stage, lane);
+    else
+      str_dict_item<3>(a, it, col, orow0, base, dd.chars, stage, lane);
+  }
+}
+
+// left: null, or whether k_str_dict left any item of the column.
+__global__ void __launch_bounds__(256, 4) k_str_copy(DecodeArgs a, int c, const uint32_t* left) {
   extern __shared__ __align__(16) uint8_t str_smem[];
+  if (left && *left == 0) return;
   StrWarpSmem& ws = reinterpret_cast<StrWarpSmem*>(str_smem)[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
   uint8_t* sbuf = ws.stage;
@@ -3133,7 +3385,7 @@ __global__ void __launch_bounds__(256, 4) k_str_copy(DecodeArgs a, int c) {
     const PlanPage pp = a.pps[it.pp];
     const OutCol col = a.cols[pp.col];
     if (col.ptype != T_BYTE_ARRAY || pp.nonnull < 0) continue;
-    // (a transcoded page is never a dictionary page: its own encoding decides)
+    if (left && str_padded(a, pp)) continue;
     const PageDev pg = a.pages[pp.page];
     const bool isdict = pg.encoding == ENC_RLE_DICT || pg.encoding == ENC_PLAIN_DICT;
     DictDev dd{};
@@ -3522,7 +3774,7 @@ int walk_blocks_per_sm() {
 
 int expand_blocks_per_sm() {
   if (!g_exp_bps) {
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g_exp_bps, k_expand, EXP_THREADS, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g_exp_bps, k_expand<true>, EXP_THREADS, 0);
     if (g_exp_bps < 1) g_exp_bps = 1;
   }
   return g_exp_bps;
@@ -3599,41 +3851,41 @@ void launch_dict_expand(const DecodeArgs& a, int ibegin, int n, int cidx, int n_
   else
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_dict_expand<8>, SX_THREADS, smem);
   if (bps < 1) bps = 1;
-  // long spans overlap the copy of an item with the decode of the one before
-  // it and load a dictionary once; short ones where there would be less than
-  // two for every resident block
-  int span = SX_SPAN;
-  while (span > SX_WARPS && n < 2 * span * n_sms * bps) span /= 2;
-  const int spans = (n + span - 1) / span;
-  int blocks = n_sms * bps;
-  if (blocks > spans) blocks = spans;
+  int blocks = (n + SX_WARPS - 1) / SX_WARPS;
+  if (blocks > n_sms * bps) blocks = n_sms * bps;
   if (width == 4)
-    k_dict_expand<4><<<blocks, SX_THREADS, smem, s>>>(a, ibegin, n, cidx, stage, dict_cap, span);
+    k_dict_expand<4><<<blocks, SX_THREADS, smem, s>>>(a, ibegin, n, cidx, stage, dict_cap);
   else
-    k_dict_expand<8><<<blocks, SX_THREADS, smem, s>>>(a, ibegin, n, cidx, stage, dict_cap, span);
+    k_dict_expand<8><<<blocks, SX_THREADS, smem, s>>>(a, ibegin, n, cidx, stage, dict_cap);
 }
 
-void launch_expand(const DecodeArgs& a, int ibegin, int n, int cidx, int n_sms, int ctas_per_sm, cudaStream_t s) {
+void launch_expand(const DecodeArgs& a, int ibegin, int n, int cidx, bool delta, int n_sms, int ctas_per_sm,
+                   cudaStream_t s) {
   if (n <= 0) return;
   int blocks = (n + EXP_WARPS - 1) / EXP_WARPS;
   const int bps = expand_blocks_per_sm();
   const int cap = n_sms * (ctas_per_sm > 0 && ctas_per_sm < bps ? ctas_per_sm : bps);
   if (blocks > cap) blocks = cap;
-  k_expand<<<blocks, EXP_THREADS, 0, s>>>(a, ibegin, n, cidx);
+  if (delta)
+    k_expand<true><<<blocks, EXP_THREADS, 0, s>>>(a, ibegin, n, cidx);
+  else
+    k_expand<false><<<blocks, EXP_THREADS, 0, s>>>(a, ibegin, n, cidx);
 }
 
-void launch_strings(const DecodeArgs& a, int col, int n_items, int n_sms, bool copy_chars, cudaStream_t s) {
+void launch_strings(const DecodeArgs& a, int col, int n_items, int n_sms, bool copy_chars, uint32_t* left,
+                    cudaStream_t s) {
   if (n_items <= 0) return;
   k_str_scan<<<1, 1024, 0, s>>>(a, col);
   if (!copy_chars) return;
   int blocks = (n_items + 7) / 8;
   if (blocks > n_sms * 8) blocks = n_sms * 8;
+  if (left) k_str_dict<<<blocks, 256, 0, s>>>(a, col, left);
   static bool attr = false;
   if (!attr) {
     cudaFuncSetAttribute(k_str_copy, cudaFuncAttributeMaxDynamicSharedMemorySize, STR_SMEM);
     attr = true;
   }
-  k_str_copy<<<blocks, 256, STR_SMEM, s>>>(a, col);
+  k_str_copy<<<blocks, 256, STR_SMEM, s>>>(a, col, left);
 }
 
 void launch_plain_pages(const DecodeArgs& a, int pp_begin, int n, cudaStream_t s) {

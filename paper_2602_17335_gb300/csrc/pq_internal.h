@@ -88,9 +88,9 @@ struct DictDev {
   const uint8_t* values;   // fixed width: n * width bytes, 16-byte aligned copy
   const uint64_t* str_ent; // BYTE_ARRAY: n entries; entry i = (offset of its chars in
                            // `chars` << 32) | its length
-  const uint8_t* chars;    // BYTE_ARRAY: the (decompressed) dictionary page body
+  const uint8_t* chars;    // BYTE_ARRAY: the (decompressed) dictionary page body, or its padded copy
   int32_t n;
-  int32_t width;
+  int32_t width;           // BYTE_ARRAY: stride of the padded copy, 0 where `chars` is the body
   int32_t max_len;         // longest entry (BYTE_ARRAY)
   int32_t valid;           // 1 once decoded
 };
