@@ -185,6 +185,23 @@ __device__ __forceinline__ int delta_header16(const uint8_t* p, uint64_t* z, uin
   return vl;
 }
 
+// A full block of the common layout (4 miniblocks of 32 values, one-byte min
+// delta, widths of at most max_width) whose header's first 8 bytes start at w
+// in shared memory: its bytes, 0 for another header; *z the min delta's byte,
+// *w4 the widths.
+__device__ __forceinline__ uint32_t delta_common(const uint8_t* w, uint32_t max_width, uint32_t* z,
+                                                uint32_t* w4) {
+  const uintptr_t a = reinterpret_cast<uintptr_t>(w);
+  const uint32_t* q = reinterpret_cast<const uint32_t*>(a & ~uintptr_t(3));
+  const uint32_t sh = static_cast<uint32_t>(a & 3) * 8;
+  const uint32_t r0 = q[0], r1 = q[1], r2 = q[2];
+  const uint32_t lo = __funnelshift_r(r0, r1, sh), hi = __funnelshift_r(r1, r2, sh);
+  const uint32_t wd = __funnelshift_r(lo, hi, 8);
+  *z = lo & 0xffu;
+  *w4 = wd;
+  return (lo & 0x80u) || __vcmpgtu4(wd, max_width * 0x01010101u) ? 0u : 5u + 4u * __dp4a(wd, 0x01010101u, 0u);
+}
+
 // `w` 32-bit little-endian word view of a staged window; bit position `b`
 // relative to the window's first byte.  Extracts `width` <= 32 bits.
 __device__ __forceinline__ uint32_t bits32(const uint32_t* w, uint64_t b, int width) {

@@ -141,21 +141,6 @@ __device__ int tc_block(const DCursor& c, uint32_t q, uint32_t need, bool header
   return header_only || *size <= have ? 1 : 0;
 }
 
-// A full block of the common layout (4 miniblocks of 32 values, one-byte min
-// delta) whose header's first 8 bytes start at w: its bytes, 0 for another
-// header; *z the min delta's byte, *w4 the widths.
-__device__ __forceinline__ uint32_t tc_common(const uint8_t* w, uint32_t* z, uint32_t* w4) {
-  const uintptr_t a = reinterpret_cast<uintptr_t>(w);
-  const uint32_t* q = reinterpret_cast<const uint32_t*>(a & ~uintptr_t(3));
-  const uint32_t sh = static_cast<uint32_t>(a & 3) * 8;
-  const uint32_t r0 = q[0], r1 = q[1], r2 = q[2];
-  const uint32_t lo = __funnelshift_r(r0, r1, sh), hi = __funnelshift_r(r1, r2, sh);
-  const uint32_t wd = __funnelshift_r(lo, hi, 8);
-  *z = lo & 0xffu;
-  *w4 = wd;
-  return (lo & 0x80u) || __vcmpgtu4(wd, 0x20202020u) ? 0u : 5u + 4u * __dp4a(wd, 0x01010101u, 0u);
-}
-
 // Parses the stream header at `p` and walks the block headers to the stream
 // end (after the last miniblock that holds values).  Records the result in
 // `c`; errors go to sm.  Block-collective.
@@ -200,7 +185,7 @@ __device__ void dstream_open(const uint8_t* b, uint32_t p, uint32_t end, DCursor
       while (left) {
         while (common && left >= 128 && q + 20 <= wend) {
           uint32_t z, w4;
-          const uint32_t size = tc_common(w + q, &z, &w4);
+          const uint32_t size = delta_common(w + q, 32, &z, &w4);
           if (size == 0 || size > end - q) break;
           q += size;
           left -= 128;
@@ -255,7 +240,7 @@ __device__ bool dstream_refill(const uint8_t* b, DCursor& c, TcSmem& sm) {
         while (left && n < TC_MAX_LIST) {
           if (common && left >= 128 && q >= c.w0 && q + 20 <= wend) {
             uint32_t z, w4;
-            const uint32_t size = tc_common(c.win + (wbase + q), &z, &w4);
+            const uint32_t size = delta_common(c.win + (wbase + q), 32, &z, &w4);
             if (size && size <= wend - q && size <= c.end - q) {
               c.minv[n] = unzigzag(z);
               c.wid[n] = wbase + q + 1;
