@@ -1197,6 +1197,15 @@ pq_status plan_build(pq_ctx* ctx, pq_index* idx, const std::vector<int32_t>& col
 
 static pq_status plan_size_strings(pq_plan* plan);
 
+// A scan of several columns with few work items: launching is what it costs
+// (8 columns of 10^4 rows: 33 kernels and 24 event calls, 112 us of host time
+// for 74 us on the device), so each stage is launched once for all columns.
+// The line lies where the items no longer fit the expansion warps at once.
+static bool merged_scan(const pq_plan* plan) {
+  return plan->outcols.size() > 2 && plan->n_items <= 32ull * plan->ctx->n_sms &&
+         !(plan->flags & (PQ_SCAN_PLAIN | PQ_SCAN_TIMING));
+}
+
 // Device half: allocations from the context's pool, uploads, work items,
 // events, pinned staging.  The uploads go on stream `s` (nullptr: the legacy
 // default stream), where the plan's `ready` event is recorded.
@@ -1330,6 +1339,20 @@ pq_status plan_upload(pq_plan* plan, cudaStream_t s) {
         n += (nbss ? 1 : 0) + (ntc > nbss ? 1 : 0);
         tcj += ntc;
       }
+    } else if (merged_scan(plan)) {
+      const int dk = plan->zstd_jobs ? 2 : 1;
+      int split[2] = {0, 0}, strs = 0, fixed = 0, bss = 0;
+      for (size_t oc = 0; oc < plan->colwork.size(); ++oc) {
+        const auto& cw = plan->colwork[oc];
+        split[0] |= cw.blk_data_n != 0;
+        split[1] |= cw.blk_dict_n != 0;
+        strs |= cw.max_str_regions > 0;
+        fixed |= cw.dict_n && plan->outcols[oc].ptype != pqi::T_BYTE_ARRAY;
+        bss += cw.tc_bss;
+      }
+      n += (plan->snappy_data.empty() ? 0 : dk + 2 * split[0]) + (plan->snappy_dict.empty() ? 0 : dk + 2 * split[1]) +
+           fixed + 3 * strs + (bss ? 1 : 0) + (static_cast<int>(plan->tc_jobs.size()) > bss ? 1 : 0) +
+           (plan->walk_pps.empty() ? 0 : 1) + (plan->delta_pps.empty() ? 0 : 4) + (nit ? 1 : 0);
     } else {
       for (size_t oc = 0; oc < plan->colwork.size(); ++oc) {
         const auto& cw = plan->colwork[oc];
@@ -1542,26 +1565,56 @@ static void launch_decompress(pq_plan* plan, const pqi::SnappyJob* jobs, int n, 
   if (plan->zstd_jobs) pqi::launch_zstd(jobs, n, n_sms, st, s);
 }
 
-// The same for the dictionary pages or the data pages of output column oc,
-// whose split Snappy pages are scanned for their fragments first; these are
-// then decompressed by a block each.
-static void launch_column_decompress(pq_plan* plan, size_t oc, bool dicts, pqi::DevStatus* st, cudaStream_t s) {
+// A stretch of one of the plan's decompression job lists: jobs, fragments and
+// segments of its split pages, and the ticket counters of its element scan.
+struct SnapRange {
+  const pqi::SnappyJob* jobs;
+  int n;
+  uint32_t blk0, nblk, seg0, nseg, data_max;
+  uint32_t* tickets;
+};
+
+static uint32_t* snap_tickets(const pq_plan* plan, size_t oc, bool dicts) {
+  return plan->d_counter + pqi::SNAP_COUNTER0(static_cast<uint32_t>(plan->outcols.size())) +
+         pqi::SNAPPY_RUNS * (2 * oc + (dicts ? 1 : 0));
+}
+
+// The dictionary pages or the data pages of output column oc.
+static SnapRange column_range(const pq_plan* plan, size_t oc, bool dicts) {
   const auto& cw = plan->colwork[oc];
-  const uint32_t n_cols = static_cast<uint32_t>(plan->outcols.size());
-  const pqi::SnappyJob* jobs =
-      plan->d_snappy + (dicts ? plan->snappy_data.size() + cw.snap_dict_begin : static_cast<size_t>(cw.snap_data_begin));
-  const int n = dicts ? cw.snap_dict_n : cw.snap_data_n;
-  const uint32_t blk0 = dicts ? cw.blk_dict_begin : cw.blk_data_begin, nblk = dicts ? cw.blk_dict_n : cw.blk_data_n;
-  const uint32_t seg0 = dicts ? cw.seg_dict_begin : cw.seg_data_begin, nseg = dicts ? cw.seg_dict_n : cw.seg_data_n;
-  if (n <= 0) return;
-  if (nblk) {
+  if (dicts)
+    return {plan->d_snappy + plan->snappy_data.size() + cw.snap_dict_begin, cw.snap_dict_n, cw.blk_dict_begin,
+            cw.blk_dict_n, cw.seg_dict_begin, cw.seg_dict_n, ~0u, snap_tickets(plan, oc, true)};
+  return {plan->d_snappy + cw.snap_data_begin, cw.snap_data_n, cw.blk_data_begin, cw.blk_data_n, cw.seg_data_begin,
+          cw.seg_data_n, cw.snap_data_max, snap_tickets(plan, oc, false)};
+}
+
+// Those of all columns (the lists hold them one column after another).
+static SnapRange plan_range(const pq_plan* plan, bool dicts) {
+  uint32_t nblk = 0, nseg = 0;
+  for (const auto& cw : plan->colwork) {
+    nblk += dicts ? cw.blk_dict_n : cw.blk_data_n;
+    nseg += dicts ? cw.seg_dict_n : cw.seg_data_n;
+  }
+  SnapRange r = column_range(plan, 0, dicts);
+  r.n = static_cast<int>(dicts ? plan->snappy_dict.size() : plan->snappy_data.size());
+  r.nblk = nblk;
+  r.nseg = nseg;
+  r.data_max = dicts ? ~0u : plan->snap_data_max;
+  return r;
+}
+
+// Decompression of a range; its split Snappy pages are scanned for their
+// fragments first, which are then decompressed by a block each.
+static void launch_range(pq_plan* plan, const SnapRange& r, pqi::DevStatus* st, cudaStream_t s) {
+  if (r.n <= 0) return;
+  if (r.nblk) {
     const int n_sms = plan->ctx->n_sms;
     const pqi::SnapState ss = pqi::snap_state(plan->d_snap_state, plan->snap_blocks, plan->snap_segs);
-    uint32_t* tickets = plan->d_counter + pqi::SNAP_COUNTER0(n_cols) + pqi::SNAPPY_RUNS * (2 * oc + (dicts ? 1 : 0));
-    pqi::launch_snappy_scan(jobs, n, seg0, nseg, ss, tickets, n_sms, st, s);
-    pqi::launch_snappy_fragments(jobs, static_cast<int>(blk0), static_cast<int>(nblk), ss, n_sms, st, s);
+    pqi::launch_snappy_scan(r.jobs, r.n, r.seg0, r.nseg, ss, r.tickets, n_sms, st, s);
+    pqi::launch_snappy_fragments(r.jobs, static_cast<int>(r.blk0), static_cast<int>(r.nblk), ss, n_sms, st, s);
   }
-  launch_decompress(plan, jobs, n, dicts || cw.snap_data_max >= wide_snappy_bytes(plan), st, s);
+  launch_decompress(plan, r.jobs, r.n, r.data_max >= wide_snappy_bytes(plan), st, s);
 }
 
 // Expansion of one output column: copies (REQUIRED PLAIN fixed width), the
@@ -1601,11 +1654,11 @@ static uint32_t* strings_left(pq_plan* plan, size_t oc) {
 static void enqueue_column(pq_plan* plan, size_t oc, const pqi::DecodeArgs& a, bool with_dicts, cudaStream_t s) {
   pq_ctx* ctx = plan->ctx;
   const auto& cw = plan->colwork[oc];
-  if (with_dicts) launch_column_decompress(plan, oc, true, a.st, s);
+  if (with_dicts) launch_range(plan, column_range(plan, oc, true), a.st, s);
   if (with_dicts && cw.dict_n)
     pqi::launch_dict(plan->d_dict_jobs + cw.dict_begin, cw.dict_n, plan->outcols[oc].ptype != pqi::T_BYTE_ARRAY, cw.max_fixed_dict, cw.max_str_regions,
                      pqi::DictScratch{plan->d_sregs, plan->d_slists}, plan->idx->d_dicts, ctx->n_sms, a.st, s);
-  launch_column_decompress(plan, oc, false, a.st, s);
+  launch_range(plan, column_range(plan, oc, false), a.st, s);
   enqueue_transcode(plan, cw.tc_begin, cw.tc_n, cw.tc_bss, a, s);
   const auto& col = plan->outcols[oc];
   pqi::launch_walk(a, cw.walk_begin, cw.walk_n, ctx->n_sms, col.optional != 0, plan->tuning.walk_window, s);
@@ -1614,6 +1667,41 @@ static void enqueue_column(pq_plan* plan, size_t oc, const pqi::DecodeArgs& a, b
   if (col.ptype == pqi::T_BYTE_ARRAY)
     pqi::launch_strings(a, static_cast<int>(oc), static_cast<int>(col.item_count), ctx->n_sms, !plan->sizing,
                         strings_left(plan, oc), s);
+}
+
+// The stages of all output columns, each launched once: dictionaries beside
+// the walks of the data pages on a branch stream, then expansion and strings.
+static void enqueue_merged(pq_plan* plan, const pqi::DecodeArgs& a, bool with_dicts, cudaStream_t side, cudaStream_t s) {
+  pq_ctx* ctx = plan->ctx;
+  int max_regions = 0, n_bss = 0;
+  bool fixed = false, levels = false;
+  for (size_t oc = 0; oc < plan->colwork.size(); ++oc) {
+    const auto& cw = plan->colwork[oc];
+    max_regions = std::max(max_regions, cw.max_regions);
+    n_bss += cw.tc_bss;
+    fixed |= cw.dict_n && plan->outcols[oc].ptype != pqi::T_BYTE_ARRAY;
+    levels |= plan->outcols[oc].optional != 0;
+  }
+  const bool dicts = with_dicts && !plan->dict_jobs.empty();
+  if (dicts) {
+    cudaEventRecord(plan->fork, s);
+    cudaStreamWaitEvent(side, plan->fork, 0);
+    launch_range(plan, plan_range(plan, true), a.st, side);
+    pqi::launch_dict(plan->d_dict_jobs, static_cast<int>(plan->dict_jobs.size()), fixed, plan->max_fixed_dict_bytes,
+                     max_str_regions_all(plan), pqi::DictScratch{plan->d_sregs, plan->d_slists}, plan->idx->d_dicts,
+                     ctx->n_sms, a.st, side);
+    cudaEventRecord(plan->join[0], side);
+  }
+  launch_range(plan, plan_range(plan, false), a.st, s);
+  enqueue_transcode(plan, 0, static_cast<int>(plan->tc_jobs.size()), n_bss, a, s);
+  pqi::launch_walk(a, 0, static_cast<int>(plan->walk_pps.size()), ctx->n_sms, levels, plan->tuning.walk_window, s);
+  pqi::launch_delta_bases(a, 0, static_cast<int>(plan->delta_pps.size()), max_regions, s);
+  if (dicts) cudaStreamWaitEvent(s, plan->join[0], 0);
+  pqi::launch_expand(a, 0, static_cast<int>(plan->n_items), 0, !plan->delta_pps.empty(), ctx->n_sms,
+                     plan->tuning.expand_ctas_per_sm, s);
+  for (int32_t sc : plan->str_cols)
+    pqi::launch_strings(a, sc, static_cast<int>(plan->outcols[sc].item_count), ctx->n_sms, !plan->sizing,
+                        strings_left(plan, sc), s);
 }
 
 // Enqueues the kernels of one scan (no host synchronisation).  Default:
@@ -1671,8 +1759,8 @@ static void enqueue_scan(pq_plan* plan, cudaStream_t s, bool with_dicts, const c
   } else if (timing) {
     for (int oc = 0; oc < ncols; ++oc) {
       const auto& cw = plan->colwork[oc];
-      if (with_dicts) launch_column_decompress(plan, oc, true, a.st, s);
-      launch_column_decompress(plan, oc, false, a.st, s);
+      if (with_dicts) launch_range(plan, column_range(plan, oc, true), a.st, s);
+      launch_range(plan, column_range(plan, oc, false), a.st, s);
       enqueue_transcode(plan, cw.tc_begin, cw.tc_n, cw.tc_bss, a, s);
     }
     mark(2);
@@ -1695,6 +1783,8 @@ static void enqueue_scan(pq_plan* plan, cudaStream_t s, bool with_dicts, const c
     for (int32_t sc : plan->str_cols)
       pqi::launch_strings(a, sc, static_cast<int>(plan->outcols[sc].item_count), ctx->n_sms, !plan->sizing,
                           strings_left(plan, sc), s);
+  } else if (merged_scan(plan)) {
+    enqueue_merged(plan, a, with_dicts, branches[0], s);
   } else {
     cudaEventRecord(plan->fork, s);
     for (int oc = 0; oc < ncols; ++oc) {
