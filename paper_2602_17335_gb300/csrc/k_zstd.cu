@@ -40,14 +40,18 @@ namespace {
 constexpr int ZT = 512;                 // threads
 constexpr int Z_HW = 3;
 constexpr int Z_SEQ = ZT;               // sequences decoded at a time, one a thread
+constexpr int Z_UNROLL = 8;             // sequences the chain follows between checks of the bit position
+constexpr int Z_PAD = 28;               // words of zeros before the staged bytes: the chain reads up to
+                                        // 8 * 89 + 128 bits below the stream's start before such a check
 constexpr uint32_t Z_BITS = (Z_SEQ * 89 + 7) / 8 + 64;  // staged bytes: a sequence takes 89 bits at most
 
 struct __align__(16) ZBlock {
   LzPairs<ZT, 8192, 32768> lz;
   // sequence tables (literal lengths, offsets, match lengths), by state
-  uint32_t step[3][512];       // extra bits | state bits << 8 | next state base << 16
+  uint32_t step[3][512];       // extra bits | state bits << 8 | next state base << 16, a state
+                               // being the byte offset of its row in `step`
   uint32_t base[3][512];       // value without its extra bits
-  __align__(16) uint32_t bits[4 + (Z_BITS + 16) / 4];  // staged input: four words of zeros, then 16-byte aligned
+  __align__(16) uint32_t bits[Z_PAD + (Z_BITS + 16) / 4];  // staged input: words of zeros, then 16-byte aligned
   uint16_t huf[2048];          // code bits << 8 | symbol, by the next huf_bits bits
   __align__(4) uint8_t weights[256];
   ZFse hw[64];                 // table of the Huffman weights
@@ -116,10 +120,10 @@ __device__ __forceinline__ bool z_open(ZRead& r, const uint8_t* p, uint32_t len)
 __device__ __forceinline__ uint32_t z_stage(ZBlock& S, const uint8_t* from, const uint8_t* to) {
   const uintptr_t a = reinterpret_cast<uintptr_t>(from) & ~uintptr_t(15);
   const uint32_t n = static_cast<uint32_t>(((reinterpret_cast<uintptr_t>(to) + 15) & ~uintptr_t(15)) - a) / 16;
-  uint4* d = reinterpret_cast<uint4*>(S.bits + 4);
-  for (uint32_t i = threadIdx.x; i < n && 16 * i + 16 <= sizeof(S.bits) - 16; i += ZT)
+  uint4* d = reinterpret_cast<uint4*>(S.bits + Z_PAD);
+  for (uint32_t i = threadIdx.x; i < n && 16 * i + 16 <= sizeof(S.bits) - 4 * Z_PAD; i += ZT)
     d[i] = __ldg(reinterpret_cast<const uint4*>(a) + i);
-  return 128 + 8 * static_cast<uint32_t>(reinterpret_cast<uintptr_t>(from) - a);
+  return 32 * Z_PAD + 8 * static_cast<uint32_t>(reinterpret_cast<uintptr_t>(from) - a);
 }
 // The 32 staged bits from bit index b on, and those below bit index b (b >= 32).
 __device__ __forceinline__ uint32_t z_from(const ZBlock& S, uint32_t b) {
@@ -266,7 +270,7 @@ __device__ __forceinline__ void z_entry(ZBlock& S, int which, int state, uint32_
     z_ml(s, &base, &extra);
   }
   S.base[which][state] = base;
-  S.step[which][state] = static_cast<uint32_t>(extra) | (nb << 8) | (next << 16);
+  S.step[which][state] = static_cast<uint32_t>(extra) | (nb << 8) | ((4 * next + 2048 * which) << 16);
 }
 
 // The Huffman tree description at p[0, len): S.huf, S.huf_bits; S.used bytes.
@@ -633,9 +637,9 @@ __device__ __forceinline__ uint64_t z_block(ZBlock& S, const uint8_t* src, uint3
       if (at > plen || !z_open(r, p + at, plen - at)) {
         S.err = ZE_SEQ;
       } else {
-        S.sl = z_bits(r, S.al[0]);
-        S.so = z_bits(r, S.al[1]);
-        S.sm = z_bits(r, S.al[2]);
+        S.sl = 4 * z_bits(r, S.al[0]);
+        S.so = 4 * z_bits(r, S.al[1]) + 2048;
+        S.sm = 4 * z_bits(r, S.al[2]) + 4096;
         if (r.pos < 0) S.err = ZE_STREAM;
         S.pos = static_cast<uint32_t>(r.pos);
       }
@@ -659,33 +663,48 @@ __device__ __forceinline__ uint64_t z_block(ZBlock& S, const uint8_t* src, uint3
     // the chain: states and bit position of each sequence of the group
     const uint32_t pos = S.pos, low = pos > Z_SEQ * 89u ? (pos - Z_SEQ * 89u) / 8 : 0u;
     const uint32_t b0 = z_stage(S, bs + low, bs + (pos + 7) / 8);
-    if (tid < 4) S.bits[tid] = 0;
+    if (tid < Z_PAD) S.bits[tid] = 0;
     __syncthreads();
     if (tid == 0) {
       uint32_t sl = S.sl, so = S.so, sm = S.sm;
       const uint32_t first = b0;  // no sequence of a sound stream starts below it
       uint32_t b = b0 + pos - 8 * low;
       int e = ZE_OK;
-      for (int i = 0; i < nb; ++i) {
-        const uint32_t cl = S.step[0][sl], co = S.step[1][so], cm = S.step[2][sm];
+      const int linked = final ? nb - 1 : nb;  // the stream's last sequence has no state bits
+      // The 96 bits below b are loaded beside the table words, so that once
+      // these give the bit count of the values the state bits are two shifts
+      // away (loading them from there: 185 cycles a sequence, so: 104).
+      const auto row = [&](uint32_t at) {
+        return *reinterpret_cast<const uint32_t*>(reinterpret_cast<const uint8_t*>(S.step) + at);
+      };
+      const auto follow = [&](int i) {
+        const uint32_t cl = row(sl), co = row(so), cm = row(sm);
+        const uint32_t* const q = S.bits + (b >> 5);
+        const uint32_t q0 = q[0], q1 = q[-1], q2 = q[-2], q3 = q[-3];
+        const uint32_t t0 = __funnelshift_r(q1, q0, b), t1 = __funnelshift_r(q2, q1, b), t2 = __funnelshift_r(q3, q2, b);
         S.at[i] = b;
-        S.states[i] = sl | (so << 9) | (sm << 17);
-        const uint32_t sum = cl + co + cm;  // (sums of the two bit counts; the rest overflows upwards)
-        const uint32_t x = sum & 0xffu, nx = (sum >> 8) & 0xffu;
-        const bool more = !final || i + 1 < nb;
-        if (b < first + x + (more ? nx : 0u)) {
-          e = ZE_STREAM;
-          break;
-        }
-        b -= x;
-        if (!more) break;
-        const uint32_t w = z_below(S, b);
-        const uint32_t nl = (cl >> 8) & 0xffu, nm = (cm >> 8) & 0xffu, no = (co >> 8) & 0xffu;
-        sl = (cl >> 16) + z_high(w, nl);
-        sm = (cm >> 16) + z_high(w << nl, nm);
-        so = (co >> 16) + z_high(w << (nl + nm), no);
-        b -= nx;
+        S.states[i] = (sl >> 2) | (so << 7) | (sm << 17);
+        // (sums of the two bit counts, at most 63 and 26; the rest overflows
+        // upwards; shifts take the low five bits)
+        const uint32_t sum = cl + co + cm;
+        const uint32_t w = (sum & 32u) ? __funnelshift_l(t2, t1, sum) : __funnelshift_l(t1, t0, sum);
+        sl = (cl >> 16) + 4 * z_high(w, cl >> 8);
+        sm = (cm >> 16) + 4 * z_high(__funnelshift_l(0u, w, cl >> 8), cm >> 8);
+        so = (co >> 16) + 4 * z_high(__funnelshift_l(0u, w, (cl + cm) >> 8), co >> 8);
+        b -= (sum & 0xffu) + ((sum >> 8) & 0xffu);
+      };
+      int i = 0;
+      for (; i + Z_UNROLL <= linked && b >= first; i += Z_UNROLL) {
+#pragma unroll
+        for (int u = 0; u < Z_UNROLL; ++u) follow(i + u);
       }
+      for (; i < linked && b >= first; ++i) follow(i);
+      if (final && b >= first) {
+        S.at[i] = b;
+        S.states[i] = (sl >> 2) | (so << 7) | (sm << 17);
+        b -= (row(sl) + row(so) + row(sm)) & 0xffu;
+      }
+      if (b < first) e = ZE_STREAM;
       S.sl = sl;
       S.so = so;
       S.sm = sm;
@@ -700,7 +719,7 @@ __device__ __forceinline__ uint64_t z_block(ZBlock& S, const uint8_t* src, uint3
     const int lane = tid & 31, warp = tid >> 5;
     uint32_t ll = 0, ml = 0, ov = 0;
     if (tid < nb) {
-      const uint32_t st = S.states[tid], sl = st & 511u, so = (st >> 9) & 255u, sm = st >> 17;
+      const uint32_t st = S.states[tid], sl = st & 511u, so = ((st >> 9) & 1023u) - 512, sm = (st >> 19) - 1024;
       uint32_t b = S.at[tid];
       const uint32_t xo = S.step[1][so] & 0xffu, xm = S.step[2][sm] & 0xffu, xl = S.step[0][sl] & 0xffu;
       ov = S.base[1][so] + z_high(z_below(S, b), xo);
