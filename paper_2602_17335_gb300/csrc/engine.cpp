@@ -386,10 +386,12 @@ pq_status pq_index_chunks(pq_ctx* ctx, const pq_file* files, int n_files, void* 
   idx->files.assign(files, files + n_files);
   idx->metas.resize(n_files);
   std::vector<uint8_t> big;
+  std::vector<FileTail> tails(n_files);
   for (int f = 0; f < n_files; ++f) {
     const uint8_t* head = ctx->tail.p + toff[f];
     const uint8_t* tail = ctx->tail.p + toff[f] + 16;
     const size_t tl = tlen[f];
+    tails[f] = FileTail{tail, files[f].size - tl};
     if (memcmp(head, "PAR1", 4) || memcmp(tail + tl - 4, "PAR1", 4))
       return fail(ctx, PQ_ERR_CORRUPT, "file " + std::to_string(f) + ": missing PAR1 magic");
     uint32_t flen;
@@ -412,7 +414,7 @@ pq_status pq_index_chunks(pq_ctx* ctx, const pq_file* files, int n_files, void* 
                   "file " + std::to_string(f) + ": " + err);
     idx->metas[f].footer_len = flen;
   }
-  return index_build(ctx, std::move(idx), !env_flag("PQ_NO_OFFSET_INDEX"), s, out);
+  return index_build(ctx, std::move(idx), !env_flag("PQ_NO_OFFSET_INDEX"), s, out, nullptr, tails.data());
 }
 
 }  // extern "C"
@@ -421,9 +423,10 @@ namespace pqe {
 
 // Index from parsed footers: `idx` holds files (device base, size) and
 // metas; chunks at base + chunk offset.  allow_oi: page locations may be
-// read from OffsetIndex structures on the device.
+// read from OffsetIndex structures on the device.  tails (or null): the
+// files' last bytes in ctx->tail.
 pq_status index_build(pq_ctx* ctx, std::unique_ptr<pq_index> idx, bool allow_oi, cudaStream_t s, pq_index** out,
-                      const std::vector<pqi::PageDev>* host_pages) {
+                      const std::vector<pqi::PageDev>* host_pages, const FileTail* tails) {
   const int n_files = static_cast<int>(idx->files.size());
   const pq_file* files = idx->files.data();
   // 2. schema
@@ -522,9 +525,10 @@ pq_status index_build(pq_ctx* ctx, std::unique_ptr<pq_index> idx, bool allow_oi,
     free_index_device(idx.get());
     return fail(ctx, PQ_ERR_OOM, "pinned staging");
   }
+  const void* on_device = nullptr;  // the chunk table as last uploaded
   auto upload_chunks = [&]() -> cudaError_t {
-    return cudaMemcpyAsync(idx->d_chunks, up.put(idx->chunks.data(), chunk_bytes), chunk_bytes,
-                           cudaMemcpyHostToDevice, s);
+    on_device = up.put(idx->chunks.data(), chunk_bytes);
+    return cudaMemcpyAsync(idx->d_chunks, on_device, chunk_bytes, cudaMemcpyHostToDevice, s);
   };
   pqi::DevStatus st0{0, -1, 0, 0};
   CK(cudaMemcpyAsync(idx->d_status, up.put(&st0, sizeof st0), sizeof st0, cudaMemcpyHostToDevice, s));
@@ -560,18 +564,24 @@ pq_status index_build(pq_ctx* ctx, std::unique_ptr<pq_index> idx, bool allow_oi,
       CK(cudaMemcpyAsync(idx->d_pages, up_pages.put(host_pages->data(), bytes), bytes, cudaMemcpyHostToDevice, s));
     idx->pages = *host_pages;
   } else if (all_oi && nch > 0) {
-    // 4a. OffsetIndex: page counts from the list headers (the first 16 bytes
-    // of every chunk's OffsetIndex, fetched in one round trip into the
-    // footer staging, which is free again), then one thread per page
-    // staging: [0, 16 n) the list headers, [16 n, 24 n) their addresses,
-    // [24 n, 28 n) the OffsetIndex lengths; one gather launch between one
-    // upload and one download
+    // 4a. OffsetIndex: page counts from the list headers, then one thread per
+    // page.  The headers are read from the files' tails where these hold all
+    // of them (writers put the OffsetIndex before the footer); else the first
+    // 16 bytes of every chunk's OffsetIndex are fetched in one round trip
+    // (30 us of a small read) into the footer staging, which is free again:
+    // [0, 16 n) the list headers, [16 n, 24 n) their addresses, [24 n, 28 n)
+    // the OffsetIndex lengths; one gather launch between one upload and one
+    // download
     const size_t n16 = 16 * static_cast<size_t>(nch);
-    if (!ctx->tail.reserve(28 * static_cast<size_t>(nch))) {
-      free_index_device(idx.get());
-      return fail(ctx, PQ_ERR_OOM, "pinned staging");
-    }
-    {
+    bool in_tails = tails != nullptr;
+    for (int f = 0; in_tails && f < n_files; ++f)
+      for (const auto& g : idx->metas[f].rgs)
+        for (const auto& cm : g.chunks) in_tails &= static_cast<uint64_t>(cm.oi_offset) >= tails[f].off;
+    if (!in_tails) {
+      if (!ctx->tail.reserve(28 * static_cast<size_t>(nch))) {
+        free_index_device(idx.get());
+        return fail(ctx, PQ_ERR_OOM, "pinned staging");
+      }
       const uint8_t** hp = reinterpret_cast<const uint8_t**>(ctx->tail.p + n16);
       int32_t* hl = reinterpret_cast<int32_t*>(ctx->tail.p + 24 * static_cast<size_t>(nch));
       int ci = 0;
@@ -602,7 +612,9 @@ pq_status index_build(pq_ctx* ctx, std::unique_ptr<pq_index> idx, bool allow_oi,
           const auto& cm = g.chunks[c];
           const uint8_t* base = static_cast<const uint8_t*>(files[f].data);
           int64_t np = 0;
-          if (pqh::offset_index_pages(ctx->tail.p + 16 * ci, std::min<int32_t>(cm.oi_length, 16), &np) !=
+          const uint8_t* head =
+              in_tails ? tails[f].p + (static_cast<uint64_t>(cm.oi_offset) - tails[f].off) : ctx->tail.p + 16 * ci;
+          if (pqh::offset_index_pages(head, std::min<int32_t>(cm.oi_length, 16), &np) !=
                   pqh::META_OK ||
               np < 0) {
             free_index_device(idx.get());
@@ -669,7 +681,6 @@ pq_status index_build(pq_ctx* ctx, std::unique_ptr<pq_index> idx, bool allow_oi,
   }
   // 5. page table back to the host (built on the device)
   if (!host_pages) {
-    idx->pages.resize(n_pages);
     pqi::DevStatus st{};
     if (!ctx->tail.reserve(sizeof st + sizeof(pqi::PageDev) * n_pages)) {
       free_index_device(idx.get());
@@ -680,7 +691,8 @@ pq_status index_build(pq_ctx* ctx, std::unique_ptr<pq_index> idx, bool allow_oi,
     CK(cudaStreamSynchronize(s));
     CK(cudaGetLastError());
     memcpy(&st, ctx->tail.p, sizeof st);
-    if (n_pages) memcpy(idx->pages.data(), ctx->tail.p + sizeof st, sizeof(pqi::PageDev) * n_pages);
+    const auto* pages = reinterpret_cast<const pqi::PageDev*>(ctx->tail.p + sizeof st);
+    idx->pages.assign(pages, pages + n_pages);
     if (st.flags) {
       pq_status r = status_from_device(ctx, st);
       free_index_device(idx.get());
@@ -739,8 +751,11 @@ pq_status index_build(pq_ctx* ctx, std::unique_ptr<pq_index> idx, bool allow_oi,
       }
     }
   }
-  CK(upload_chunks());
-  CK(cudaStreamSynchronize(s));
+  // (the dictionary pages are as uploaded when an OffsetIndex gave the pages)
+  if (!on_device || memcmp(on_device, idx->chunks.data(), chunk_bytes)) {
+    CK(upload_chunks());
+    CK(cudaStreamSynchronize(s));
+  }
   *out = idx.release();
   return PQ_OK;
 }
@@ -1127,16 +1142,17 @@ pq_status plan_build(pq_ctx* ctx, pq_index* idx, const std::vector<int32_t>& col
                               : cd.ptype == pqi::T_BYTE_ARRAY && eff == pqi::ENC_PLAIN ? pg.num_values
                                                                                                  : pg.num_values / 256);
         }
-        const int64_t span = pp.row_hi - pp.row_lo;
+        // (32-bit divisions: two a page)
+        const uint32_t span = pp.row_hi > pp.row_lo ? static_cast<uint32_t>(pp.row_hi - pp.row_lo) : 0u;
         // pages with definition levels take the short items (their walks and
         // expands carry a bitmap per item; measured faster for PLAIN too)
-        const int64_t per = cd.max_def ? item_rows_opt : item_rows_max;
-        const int64_t full = cd.max_def ? plan->tuning.item_rows_opt : plan->tuning.item_rows;
-        const uint32_t n_it = static_cast<uint32_t>((span + per - 1) / per);
+        const uint32_t per = static_cast<uint32_t>(cd.max_def ? item_rows_opt : item_rows_max);
+        const uint32_t full = static_cast<uint32_t>(cd.max_def ? plan->tuning.item_rows_opt : plan->tuning.item_rows);
+        const uint32_t n_it = span / per + (span % per ? 1 : 0);
         pp.item_rows = static_cast<int32_t>(per);
         pp.item_count = n_it;
         plan->n_items += n_it;
-        plan->budget_items += static_cast<uint64_t>((span + full - 1) / full);
+        plan->budget_items += span / full + (span % full ? 1 : 0);
         plan->pps.push_back(pp);
       }
       const int32_t n_pp = static_cast<int32_t>(plan->pps.size()) - pp_first;
@@ -1166,14 +1182,23 @@ pq_status plan_build(pq_ctx* ctx, pq_index* idx, const std::vector<int32_t>& col
     plan->outcols.push_back(col);
     plan->sizes.push_back(sz);
   }
-  // walk list: inside each column, longest header chains first
+  // walk list: inside each column, longest header chains first, in at most
+  // 64 classes of cost (the comparison sort of 10^4 pages took 50 us, this 10)
+  std::vector<uint32_t> sorted;
   for (const auto& cw : plan->colwork) {
-    std::vector<size_t> order(cw.walk_n);
-    for (int i = 0; i < cw.walk_n; ++i) order[i] = cw.walk_begin + i;
-    std::stable_sort(order.begin(), order.end(), [&](size_t x, size_t y) { return walk_cost[x] > walk_cost[y]; });
-    std::vector<uint32_t> sorted(order.size());
-    for (size_t i = 0; i < order.size(); ++i) sorted[i] = plan->walk_pps[order[i]];
-    std::copy(sorted.begin(), sorted.end(), plan->walk_pps.begin() + cw.walk_begin);
+    const int64_t* cost = walk_cost.data() + cw.walk_begin;
+    uint32_t* list = plan->walk_pps.data() + cw.walk_begin;
+    int64_t most = 0;
+    for (int i = 0; i < cw.walk_n; ++i) most = std::max(most, cost[i]);
+    int shift = 0;
+    while ((most >> shift) > 63) ++shift;
+    const auto cls = [&](int i) { return static_cast<size_t>(63 - (std::max<int64_t>(cost[i], 0) >> shift)); };
+    uint32_t at[65] = {};
+    for (int i = 0; i < cw.walk_n; ++i) ++at[cls(i) + 1];
+    for (int k = 0; k < 64; ++k) at[k + 1] += at[k];
+    sorted.resize(static_cast<size_t>(cw.walk_n));
+    for (int i = 0; i < cw.walk_n; ++i) sorted[at[cls(i)]++] = list[i];
+    std::copy(sorted.begin(), sorted.end(), list);
   }
   // the split pages' numbers: data pages, then dictionary pages
   for (auto& sj : plan->snappy_dict) {
@@ -1251,7 +1276,8 @@ pq_status plan_upload(pq_plan* plan, cudaStream_t s) {
                         plan->delta_regions * (sizeof(pqi::DeltaRegion) + 4ull * pqi::DELTA_REGION_LIST);
   // rebase scratch bodies, string scratch per column
   size_t jd = 0;
-  for (auto& pp : plan->pps) {
+  for (size_t i = 0; jd < plan->snappy_data.size() && i < plan->pps.size(); ++i) {
+    auto& pp = plan->pps[i];
     if (pp.pad == 1) {
       uint8_t* b = plan->d_scratch + reinterpret_cast<uintptr_t>(pp.body);
       pp.body = b;
