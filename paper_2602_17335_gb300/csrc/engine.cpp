@@ -868,7 +868,9 @@ static void plan_split(pqi::SnappyJob& sj, bool plain, uint32_t* frags, uint32_t
   if (out <= pqi::SNAPPY_SPLIT_MIN || in > 32 + out + out / 6) return;
   sj.nsub = (out + pqi::SNAPPY_FRAGMENT - 1) / pqi::SNAPPY_FRAGMENT;
   sj.sub = *frags;
-  sj.nseg = (in + pqi::SNAPPY_SEGMENT - 1) / pqi::SNAPPY_SEGMENT;
+  // (segments are cut from the 16-byte boundary at or before the input on)
+  const uint32_t lead = static_cast<uint32_t>((reinterpret_cast<uintptr_t>(sj.src) + sj.prefix) & 15);
+  sj.nseg = static_cast<uint32_t>((uint64_t(in) + lead + pqi::SNAPPY_SEGMENT - 1) / pqi::SNAPPY_SEGMENT);
   *frags += sj.nsub;
   *segs += sj.nseg;
 }

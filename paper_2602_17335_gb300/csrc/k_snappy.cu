@@ -579,23 +579,31 @@ __global__ void __launch_bounds__(kThreads, kThreads == 512 ? 2 : 5)
 
 // ------------------------------------------------------------------ split pages
 
-// Element scan of the split pages, a thread block per SNAPPY_SEGMENT input
-// bytes.  Which bytes of a segment are headers depends on where the last
-// element before it ends, so the page is one chain; but where the chain
-// leaves the segment can be computed for every possible entry at once: each
-// byte's next header, if one started there, then, right to left, the exit
-// from its 32 bytes (a thread each), from its 1 KB (a warp each) and from the
-// segment, one lookup per byte and level.  (Doubling the map in place until
-// nothing changes took 11 rounds of lookups on literal bytes: 57 us a
-// segment.)  A block then waits only for its
+// Element scan of the split pages, a thread block per segment of
+// SNAPPY_SEGMENT input bytes (cut at multiples of it from the input's first
+// 16-byte boundary on).  Which bytes of a segment are headers depends on
+// where the last element before it ends, so the page is one chain; but where
+// the chain leaves the segment can be computed for every possible entry at
+// once, right to left: the exit from each byte's 32 bytes (a thread each,
+// its bytes in registers), from its 1 KB (a warp each), 4 KB and the segment,
+// one lookup per byte and level.  A block then waits only for its
 // predecessor's exit, looks up its own and passes that on (about a
 // microsecond a segment), while all segments' maps are built in parallel.
-// With its entry known, the block lists the segment's elements (window by
-// window, as the decoder does), adds up the output of the segments before it
-// and records which elements start a 64 KiB fragment.  An element that spans
+// With its entry known, one thread hops over the 1 KB blocks, each warp over
+// the 32-byte runs of its block, each lane over the elements of its run: the
+// lanes' outputs are added up, and with the output of the segments before
+// they record which elements start a 64 KiB fragment.  An element that spans
 // two fragments, a copy that reaches out of its fragment, or anything the
 // decoder would reject marks the page: it is then decompressed whole, by one
 // block, which reports what is wrong.
+//
+// Bound by the maps' lookups (issue and shared-memory latency) and, for dense
+// segments, by the lanes' elements (about 80 cycles each, 16 at most).  With
+// the elements listed by the decoder's windowed tables instead of the maps' own
+// levels, and one 32-bit map whose levels replaced one another (a barrier per
+// KB), the scan of an INT64 dictionary column (2^23 rows, 1 MiB pages, 3600
+// elements a segment) took 210 us, now 120, its 1 MiB dictionary pages' 140,
+// now 100.
 //
 // The list's pages are cut into up to SNAPPY_RUNS runs of whole pages,
 // each with a ticket counter from which blocks take its segments in order
@@ -604,30 +612,25 @@ __global__ void __launch_bounds__(kThreads, kThreads == 512 ? 2 : 5)
 // different runs overlap (in one run, 64 pages of 32 segments took 560 us, the
 // chain's 2048 hops).  Waits are bounded all the same.
 constexpr int SC_THREADS = 1024;
-constexpr uint32_t SC_WIN = 4096;
-constexpr int SC_EL = 1024;
-constexpr uint32_t SC_MAX_EL = SNAPPY_SEGMENT / 2;  // an element takes two input bytes or more
 constexpr uint32_t SC_POLLS = 1u << 22;
+constexpr uint32_t SC_NONE = 0xffffffffu;
+// Maps by segment byte (at sc_slot): where the chain from a header there
+// leaves the byte's 32 bytes / 1 KB / (4 KB, then) segment: a byte of the
+// segment, or SC_LAST | the header of the element that leads out of the segment.
+constexpr uint32_t SC_LAST = 0x8000u;
 struct __align__(16) SnScan {
-  union {
-    uint32_t map[SNAPPY_SEGMENT];  // next header, then the exit, from each byte (at sc_slot)
-    struct {
-      uint32_t at[SC_MAX_EL];      // output offset of each element within the segment's
-      uint16_t pos[SC_MAX_EL];     // its header
-      SnHeaders<SC_WIN, SC_EL> h;
-    } el;
-  };
-  uint8_t stage[SNAPPY_SEGMENT + 64];
-  uint64_t bar;
-  uint32_t tmp[32];
+  uint16_t run[SNAPPY_SEGMENT], blk[SNAPPY_SEGMENT], seg[SNAPPY_SEGMENT];
+  uint8_t stage[SNAPPY_SEGMENT + 32];
+  uint64_t bar, tmp[32];
+  uint32_t block_entry[32];  // the first header of each 1 KB
   uint32_t ticket, entry, next, from, to, done;
   int32_t job;
 };
 
 // Map slot of a segment byte: its place in its 32 bytes is permuted by the
-// number of the 32 bytes, so that threads at the same place of 32 such runs
-// fall on 32 banks, and so do the 32 bytes of one run.
-__device__ __forceinline__ uint32_t sc_slot(uint32_t p) { return p ^ ((p >> 5) & 31u); }
+// number of the 64 bytes, so that the same place of 32 successive runs falls
+// on 32 banks.
+__device__ __forceinline__ uint32_t sc_slot(uint32_t p) { return p ^ ((p >> 5) & 30u); }
 
 // One 64-bit word written by another block of this launch: polled until its
 // flag is set.  0 when it never is.
@@ -711,13 +714,15 @@ __global__ void __launch_bounds__(SC_THREADS, 1) k_snappy_scan(const SnappyJob* 
     const uint32_t k = g - jb.seg;  // segment of the page
     const uint8_t* in = jb.src + jb.prefix;
     const uint32_t in_len = jb.src_len - jb.prefix, out_len = jb.dst_len - jb.prefix;
-    const uint32_t s0 = k * SNAPPY_SEGMENT;
-    const uint32_t L = in_len - s0 < SNAPPY_SEGMENT ? in_len - s0 : SNAPPY_SEGMENT;
-    // stage the segment and the header bytes after it, 16-byte aligned, at
-    // most 16 bytes past the input
-    const uintptr_t a0 = reinterpret_cast<uintptr_t>(in + s0) & ~uintptr_t(15);
-    const uint32_t shift = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(in + s0) - a0);
+    // segment byte p is input byte org + p (the first segment starts at the
+    // 16-byte boundary before the input)
+    const uint32_t lead = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(in) & 15);
+    const uint32_t org = k * SNAPPY_SEGMENT - lead;  // (modulo 2^32)
+    const uint32_t left = in_len - org, L = left < SNAPPY_SEGMENT ? left : SNAPPY_SEGMENT;
+    // stage the segment and the header bytes after it, at most 16 bytes past
+    // the input
     if (tid == 0) {
+      const uintptr_t a0 = reinterpret_cast<uintptr_t>(in) - lead + static_cast<uint64_t>(k) * SNAPPY_SEGMENT;
       const uintptr_t lim = (reinterpret_cast<uintptr_t>(in) + in_len + 16) & ~uintptr_t(15);
       uint64_t bytes = lim - a0;
       if (bytes > SNAPPY_SEGMENT + 32) bytes = SNAPPY_SEGMENT + 32;
@@ -749,13 +754,12 @@ __global__ void __launch_bounds__(SC_THREADS, 1) k_snappy_scan(const SnappyJob* 
         const uint32_t e = static_cast<uint32_t>(v);
         uint32_t x = e;
         int n = 0;
-        const uint32_t sa = smem_u32(S.stage) + shift;
-        for (; n < SN_SERIAL && all_staged && x < s0 + L; ++n) {
+        for (; n < SN_SERIAL && all_staged && x - org < L; ++n) {
           uint32_t tag, by;
-          sn_bytes5(sa + (x - s0), &tag, &by);
+          sn_bytes5(smem_u32(S.stage) + (x - org), &tag, &by);
           x += sn_advance(tag, by);
         }
-        if (x >= s0 + L) {
+        if (x - org >= L) {
           *reinterpret_cast<volatile unsigned long long*>(ss.exit + g) = SN_SET | x;
           S.entry = e;
           S.next = x;
@@ -763,50 +767,62 @@ __global__ void __launch_bounds__(SC_THREADS, 1) k_snappy_scan(const SnappyJob* 
         }
       }
     }
+    if (tid < 32) S.block_entry[tid] = SC_NONE;
     __syncthreads();
-    if (!S.done) {
-      // the map: positions relative to the segment's first byte, which is
-      // staged at `shift`; values below L lead on in the segment
-      const uint32_t* w32 = reinterpret_cast<const uint32_t*>(S.stage);
-      const uint32_t sb = 8 * (shift & 3);
-      for (uint32_t p = 4 * tid; p < L; p += 4 * SC_THREADS) {
-        const uint32_t* w = w32 + ((p + shift) >> 2);
-        const uint32_t a = __funnelshift_r(w[0], w[1], sb), b = __funnelshift_r(w[1], w[2], sb);
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-          S.map[sc_slot(p + i)] =
-              p + i + sn_advance((a >> (8 * i)) & 0xffu, i == 3 ? b : __funnelshift_r(a, b, 8 * (i + 1)));
-      }
-      __syncthreads();
+    static_assert(SNAPPY_SEGMENT == 32 * SC_THREADS && SC_THREADS == 32 * 32 && SNAPPY_SEGMENT == SC_LAST,
+                  "a run a thread, a block a warp");
+    const bool listed = S.done != 0;  // (few elements: thread 0 steps along them, without maps)
+    if (!listed) {
       // (bytes past L lead past L: every position a level reads is set)
-      static_assert(SNAPPY_SEGMENT == 32 * SC_THREADS && SC_THREADS == 32 * 32, "a run a thread, a block a warp");
       {
-        const uint32_t end = 32 * tid + 32 < L ? 32 * tid + 32 : L;
-        for (int r = 30; r >= 0; --r) {
-          const uint32_t p = 32 * tid + r;
-          if (p < L) {
-            const uint32_t v = S.map[sc_slot(p)];
-            if (v < end) S.map[sc_slot(p)] = S.map[sc_slot(v)];
-          }
+        const uint4* s4 = reinterpret_cast<const uint4*>(S.stage) + 2 * tid;
+        const uint4 lo = s4[0], hi = s4[1];
+        const uint32_t w[9] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w,
+                               reinterpret_cast<const uint32_t*>(S.stage)[8 * tid + 8]};
+        const uint32_t p0 = 32 * tid;
+#pragma unroll
+        for (int r = 31; r >= 0; --r) {
+          const uint32_t a = w[r / 4], b = w[r / 4 + 1];
+          const uint32_t tag = (a >> (8 * (r & 3))) & 0xffu;
+          const uint32_t by = (r & 3) == 3 ? b : __funnelshift_r(a, b, 8 * ((r & 3) + 1));
+          const uint32_t nx = p0 + r + sn_advance(tag, by);
+          uint32_t v = nx < L ? nx : SC_LAST | (p0 + r);
+          if (v < p0 + 32) v = S.run[sc_slot(v)];
+          S.run[sc_slot(p0 + r)] = static_cast<uint16_t>(v);
         }
         __syncwarp();
       }
-      {
-        const uint32_t end = 1024 * warp + 1024 < L ? 1024 * warp + 1024 : L;
-        for (int i = 30; i >= 0; --i) {
-          const uint32_t p = 1024 * warp + 32 * i + lane;
-          if (p < L) {
-            const uint32_t v = S.map[sc_slot(p)];
-            if (v < end) S.map[sc_slot(p)] = S.map[sc_slot(v)];
-          }
-          __syncwarp();
+      for (int i = 31; i >= 0; --i) {
+        const uint32_t p = 1024 * warp + 32 * i + lane;
+        if (p < L) {
+          uint32_t v = S.run[sc_slot(p)];
+          if (v < 1024u * warp + 1024u) v = S.blk[sc_slot(v)];
+          S.blk[sc_slot(p)] = static_cast<uint16_t>(v);
         }
+        __syncwarp();
       }
       __syncthreads();
-      for (int i = static_cast<int>((L - 1) / 1024) - 1; i >= 0; --i) {
-        const uint32_t p = 1024 * i + tid;
-        const uint32_t v = S.map[sc_slot(p)];
-        if (v < L) S.map[sc_slot(p)] = S.map[sc_slot(v)];
+      for (int j = 3; j >= 0; --j) {  // block j of every 4 KB
+#pragma unroll
+        for (uint32_t q = 0; q < 8; ++q) {
+          const uint32_t p = 4096 * q + 1024 * j + tid;
+          if (p < L) {
+            uint32_t v = S.blk[sc_slot(p)];
+            if (v < 4096 * q + 4096) v = S.seg[sc_slot(v)];
+            S.seg[sc_slot(p)] = static_cast<uint16_t>(v);
+          }
+        }
+        __syncthreads();
+      }
+      for (int q = 6; q >= 0; --q) {
+#pragma unroll
+        for (uint32_t j = 0; j < 4; ++j) {
+          const uint32_t p = 4096 * q + 1024 * j + tid;
+          if (p < L) {
+            const uint32_t v = S.seg[sc_slot(p)];
+            if (v < SC_LAST) S.seg[sc_slot(p)] = S.seg[sc_slot(v)];
+          }
+        }
         __syncthreads();
       }
       // the chain: entry from the segment before, exit to the one after
@@ -823,75 +839,76 @@ __global__ void __launch_bounds__(SC_THREADS, 1) k_snappy_scan(const SnappyJob* 
         }
         uint32_t x = e;
         if (!ok) x = e = 0xffffffffu;  // (passed on: the page is decompressed whole)
-        else if (e < s0 + L) x = S.map[sc_slot(e - s0)] + s0;
+        else if (e - org < L) {
+          const uint32_t h = S.seg[sc_slot(e - org)] & (SC_LAST - 1);
+          uint32_t tag, by;
+          sn_bytes5(smem_u32(S.stage) + h, &tag, &by);
+          x = org + h + sn_advance(tag, by);
+        }
         *reinterpret_cast<volatile unsigned long long*>(ss.exit + g) = SN_SET | x;
         S.entry = e;
         S.next = x;
+        if (x <= in_len)  // (not after a failed wait, nor past a literal that overruns the input)
+          for (uint32_t q = e - org; q < L;) {
+            S.block_entry[q >> 10] = q;
+            q = S.blk[sc_slot(q)];
+          }
       }
     }
     __syncthreads();
     const uint32_t entry = S.entry, exit = S.next;
     bool good = entry <= in_len && exit <= in_len;
-    // the segment's elements and their output (the map is not needed any more)
-    uint32_t n_el = 0, total = 0;
-    if (good && entry < s0 + L) {
-      uint32_t q = entry - s0 + shift;  // staged positions from here on
-      const uint32_t L1 = shift + L;
-      bool dense = false;
-      // a batch ends at the end of its window, at SC_EL or SN_SERIAL headers
-      for (uint32_t guard = 0; guard < SNAPPY_SEGMENT / SN_SERIAL + 2 * SNAPPY_SEGMENT / SC_WIN + 16 && q < L1; ++guard) {
-        const uint32_t wbase = q & ~15u;
-        const uint8_t* wb = S.stage + wbase;
-        const uint32_t wl = L1 - wbase < SC_WIN ? L1 - wbase : SC_WIN;
-        sn_find_headers<SC_THREADS>(S.el.h, wb, q - wbase, wl, dense);
-        const int n = S.el.h.n;
-        dense = n >= SN_DENSE;
-        uint32_t len = 0;
-        if (tid < n) {
-          const uint32_t p = S.el.h.pos[tid];
-          uint32_t tag, x, kind, arg, nx;
-          sn_bytes5(smem_u32(wb) + p, &tag, &x);
-          if (!sn_hdr(tag, x, wbase + p - shift + s0, in_len, &kind, &len, &arg, &nx)) len = 0;
-          if (tid == n - 1) S.next = wbase + p + sn_advance(tag, x);
-        }
-        uint32_t sum;
-        const uint32_t o = block_exclusive_sum(len, S.tmp, &sum);
-        if (tid < n && n_el + tid < SC_MAX_EL) {
-          S.el.at[n_el + tid] = total + o;
-          S.el.pos[n_el + tid] = static_cast<uint16_t>(wbase + S.el.h.pos[tid]);
-          if (len == 0) good = false;
-        }
-        n_el += n;
-        total += sum;
-        q = S.next;
-        if (__syncthreads_or(total > out_len || sum > out_len)) {
-          good = false;
-          break;
-        }
+    // the thread's elements: those of its 32 bytes, all of the segment's for
+    // thread 0 where it has stepped along them
+    uint32_t first = SC_NONE, end = 32 * tid + 32;
+    if (listed) {
+      end = L;
+      if (good && tid == 0) first = entry - org;
+    } else {
+      for (uint32_t q = S.block_entry[warp]; q < 1024u * warp + 1024u;) {
+        if (static_cast<uint32_t>(lane) == ((q >> 5) & 31u)) first = q;
+        q = S.run[sc_slot(q)];
       }
-      if (q < L1 || n_el > SC_MAX_EL) good = false;
     }
-    good = !__syncthreads_or(!good);
-    if (tid == 0) *reinterpret_cast<volatile unsigned long long*>(ss.len + g) = SN_SET | (good ? total : 0u);
-    // output of the segments before this one
+    end = end < L ? end : L;
     uint64_t mine = 0;
+    for (uint32_t q = first; q < end;) {
+      uint32_t tag, x, kind, len, arg, nx;
+      sn_bytes5(smem_u32(S.stage) + q, &tag, &x);
+      if (!sn_hdr(tag, x, org + q, in_len, &kind, &len, &arg, &nx)) {
+        good = false;
+        break;
+      }
+      mine += len;
+      q = nx - org;
+    }
+    uint64_t total;
+    const uint64_t o_at = block_exclusive_sum<uint64_t>(mine, S.tmp, &total);
+    if (total > out_len) good = false;
+    good = !__syncthreads_or(!good);
+    if (tid == 0)
+      *reinterpret_cast<volatile unsigned long long*>(ss.len + g) = SN_SET | (good ? total : 0u);
+    // output of the segments before this one
+    uint64_t part = 0;
     for (uint32_t i = tid; i < k; i += SC_THREADS) {
       const unsigned long long v = sn_await(ss.len + jb.seg + i);
       if (!v) good = false;
-      mine += static_cast<uint32_t>(v);
+      part += static_cast<uint32_t>(v);
     }
     uint64_t base;
-    block_exclusive_sum<uint64_t>(mine, reinterpret_cast<uint64_t*>(S.el.h.j1), &base);
+    block_exclusive_sum<uint64_t>(part, S.tmp, &base);
     if (base > out_len || total > out_len - base) good = false;
     if (good) {
-      for (uint32_t i = tid; i < n_el; i += SC_THREADS) {
-        const uint32_t p = S.el.pos[i], o = static_cast<uint32_t>(base) + S.el.at[i];
+      uint32_t o = static_cast<uint32_t>(base + o_at);
+      for (uint32_t q = first; q < end;) {
         uint32_t tag, x, kind, len, arg, nx;
-        sn_bytes5(smem_u32(S.stage) + p, &tag, &x);
-        sn_hdr(tag, x, p - shift + s0, in_len, &kind, &len, &arg, &nx);
+        sn_bytes5(smem_u32(S.stage) + q, &tag, &x);
+        sn_hdr(tag, x, org + q, in_len, &kind, &len, &arg, &nx);
         const uint32_t in_frag = o & (SNAPPY_FRAGMENT - 1);
         if (in_frag + len > SNAPPY_FRAGMENT || (kind != 0 && (arg == 0 || arg > in_frag))) good = false;
-        if (in_frag == 0 && o / SNAPPY_FRAGMENT < jb.nsub) ss.start[jb.sub + o / SNAPPY_FRAGMENT] = p - shift + s0;
+        if (in_frag == 0 && o / SNAPPY_FRAGMENT < jb.nsub) ss.start[jb.sub + o / SNAPPY_FRAGMENT] = org + q;
+        o += len;
+        q = nx - org;
       }
       if (k + 1 == jb.nseg && (exit != in_len || base + total != out_len)) good = false;
     }
