@@ -139,11 +139,12 @@ int walk_blocks_per_sm();
 // One block per page; wide: 16 warps each (large pages), else 4.  Pages with
 // nsub > 1 are skipped: launch_snappy_scan locates their fragments (segments
 // [seg_begin, seg_begin + n_segs) of the list's jobs, handed out through
-// SNAPPY_RUNS counters, zero before the launch) and launch_snappy_fragments decompresses
+// SNAPPY_RUNS counters, zero before the launch; long_first: pages of long elements
+// are stepped along beforehand) and launch_snappy_fragments decompresses
 // fragments [first, first + n).
 void launch_snappy(const SnappyJob* jobs, int n_jobs, int n_sms, DevStatus* st, cudaStream_t s, bool wide);
 void launch_snappy_scan(const SnappyJob* jobs, int n_jobs, uint32_t seg_begin, uint32_t n_segs, SnapState ss,
-                        uint32_t* tickets, int n_sms, DevStatus* st, cudaStream_t s);
+                        uint32_t* tickets, bool long_first, int n_sms, DevStatus* st, cudaStream_t s);
 void launch_snappy_fragments(const SnappyJob* jobs, int first, int n, SnapState ss, int n_sms, DevStatus* st,
                              cudaStream_t s);
 // Zstandard pages of jobs [0, n_jobs) (the others are skipped)

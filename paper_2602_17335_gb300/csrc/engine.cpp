@@ -1378,7 +1378,7 @@ pq_status plan_upload(pq_plan* plan, cudaStream_t s) {
         fixed |= cw.dict_n && plan->outcols[oc].ptype != pqi::T_BYTE_ARRAY;
         bss += cw.tc_bss;
       }
-      n += (plan->snappy_data.empty() ? 0 : dk + 2 * split[0]) + (plan->snappy_dict.empty() ? 0 : dk + 2 * split[1]) +
+      n += (plan->snappy_data.empty() ? 0 : dk + 3 * split[0]) + (plan->snappy_dict.empty() ? 0 : dk + 2 * split[1]) +
            fixed + 3 * strs + (bss ? 1 : 0) + (static_cast<int>(plan->tc_jobs.size()) > bss ? 1 : 0) +
            (plan->walk_pps.empty() ? 0 : 1) + (plan->delta_pps.empty() ? 0 : 4) + (nit ? 1 : 0);
     } else {
@@ -1387,7 +1387,7 @@ pq_status plan_upload(pq_plan* plan, cudaStream_t s) {
         const int dk = plan->zstd_jobs ? 2 : 1;  // decompression kernels per job list
         // (+2 per job list with split pages: the element scan and the fragments)
         n += (cw.snap_dict_n ? dk + (cw.blk_dict_n ? 2 : 0) : 0) + (cw.dict_n ? 2 : 0) +
-             (cw.snap_data_n ? dk + (cw.blk_data_n ? 2 : 0) : 0) + (cw.walk_n ? 1 : 0) +
+             (cw.snap_data_n ? dk + (cw.blk_data_n ? 3 : 0) : 0) + (cw.walk_n ? 1 : 0) +
              (cw.delta_n ? 4 : 0) + (cw.tc_bss ? 1 : 0) + (cw.tc_n > cw.tc_bss ? 1 : 0) + (plan->outcols[oc].item_count ? 1 : 0);
       }
     }
@@ -1600,6 +1600,7 @@ struct SnapRange {
   int n;
   uint32_t blk0, nblk, seg0, nseg, data_max;
   uint32_t* tickets;
+  bool dicts;
 };
 
 static uint32_t* snap_tickets(const pq_plan* plan, size_t oc, bool dicts) {
@@ -1612,9 +1613,9 @@ static SnapRange column_range(const pq_plan* plan, size_t oc, bool dicts) {
   const auto& cw = plan->colwork[oc];
   if (dicts)
     return {plan->d_snappy + plan->snappy_data.size() + cw.snap_dict_begin, cw.snap_dict_n, cw.blk_dict_begin,
-            cw.blk_dict_n, cw.seg_dict_begin, cw.seg_dict_n, ~0u, snap_tickets(plan, oc, true)};
+            cw.blk_dict_n, cw.seg_dict_begin, cw.seg_dict_n, ~0u, snap_tickets(plan, oc, true), true};
   return {plan->d_snappy + cw.snap_data_begin, cw.snap_data_n, cw.blk_data_begin, cw.blk_data_n, cw.seg_data_begin,
-          cw.seg_data_n, cw.snap_data_max, snap_tickets(plan, oc, false)};
+          cw.seg_data_n, cw.snap_data_max, snap_tickets(plan, oc, false), false};
 }
 
 // Those of all columns (the lists hold them one column after another).
@@ -1639,7 +1640,7 @@ static void launch_range(pq_plan* plan, const SnapRange& r, pqi::DevStatus* st, 
   if (r.nblk) {
     const int n_sms = plan->ctx->n_sms;
     const pqi::SnapState ss = pqi::snap_state(plan->d_snap_state, plan->snap_blocks, plan->snap_segs);
-    pqi::launch_snappy_scan(r.jobs, r.n, r.seg0, r.nseg, ss, r.tickets, n_sms, st, s);
+    pqi::launch_snappy_scan(r.jobs, r.n, r.seg0, r.nseg, ss, r.tickets, !r.dicts, n_sms, st, s);
     pqi::launch_snappy_fragments(r.jobs, static_cast<int>(r.blk0), static_cast<int>(r.nblk), ss, n_sms, st, s);
   }
   launch_decompress(plan, r.jobs, r.n, r.data_max >= wide_snappy_bytes(plan), st, s);

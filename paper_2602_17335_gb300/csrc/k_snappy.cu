@@ -656,6 +656,38 @@ __device__ __forceinline__ int sc_job(const SnappyJob* jobs, int n, uint32_t g, 
   return lo;
 }
 
+// Split pages whose elements are long (incompressible values: a literal per
+// fragment and a few copies): one thread steps along the page, straight from
+// the input, and records its fragments; the scan then leaves the page out.  It
+// gives up, and leaves the page to the scan, once elements are shorter than
+// SC_LONG bytes on average, or at anything the scan would mark the page for.
+// Bound by the latency of a load an element: 64 1 MiB pages of doubles (5
+// elements per 32 KB) 89 us and the scan 35, where the scan's maps took 300.
+// Data pages only: dictionary pages are few, mostly dense, and waited for
+// (giving up on four of them took 24 us of their column's 250).
+constexpr uint32_t SC_LONG = 1024;
+__global__ void __launch_bounds__(32) k_snappy_long(const SnappyJob* __restrict__ jobs, SnapState ss) {
+  if (threadIdx.x != 0) return;
+  const SnappyJob jb = jobs[blockIdx.x];
+  if (jb.nsub <= 1) return;
+  const uint8_t* in = jb.src + jb.prefix;
+  const uint32_t in_len = jb.src_len - jb.prefix, out_len = jb.dst_len - jb.prefix;
+  uint32_t q = sn_preamble(in, in_len, out_len), o = 0;
+  if (q == 0) return;
+  for (uint32_t n = 0; q < in_len; ++n) {
+    if (n > 16 + q / SC_LONG) return;
+    const uint64_t h = ld_unaligned_g(in + q, 8);
+    uint32_t kind, len, arg, nx;
+    if (!sn_hdr(static_cast<uint32_t>(h) & 0xffu, static_cast<uint32_t>(h >> 8), q, in_len, &kind, &len, &arg, &nx)) return;
+    const uint32_t in_frag = o & (SNAPPY_FRAGMENT - 1);
+    if (len > SNAPPY_FRAGMENT - in_frag || len > out_len - o || (kind != 0 && (arg == 0 || arg > in_frag))) return;
+    if (in_frag == 0) ss.start[jb.sub + o / SNAPPY_FRAGMENT] = q;
+    o += len;
+    q = nx;
+  }
+  if (q == in_len && o == out_len) ss.bad[jb.sub + 1] = 1;  // (a split page has three fragments or more)
+}
+
 __global__ void __launch_bounds__(SC_THREADS, 1) k_snappy_scan(const SnappyJob* __restrict__ jobs, int n_jobs,
                                                                uint32_t seg_begin, uint32_t n_segs, SnapState ss,
                                                                uint32_t* tickets, DevStatus* st) {
@@ -694,16 +726,18 @@ __global__ void __launch_bounds__(SC_THREADS, 1) k_snappy_scan(const SnappyJob* 
         }
         if (lane == 0 && S.from < S.to) t = S.from + atomicAdd(tickets + run, 1u);
         t = __shfl_sync(0xffffffffu, t, 0);
-        if (t < S.to) break;
+        if (t < S.to) {
+          const int j = sc_job(jobs, n_jobs, t, lane);
+          // of a page that k_snappy_long has done, the first segment only
+          if (t != jobs[j].seg && ss.bad[jobs[j].sub + 1]) continue;
+          if (lane == 0) S.job = j;
+          break;
+        }
         t = 0xffffffffu;
         run = (run + 1) % SNAPPY_RUNS;
         bounded = false;
         ++used;
         __syncwarp();
-      }
-      if (t != 0xffffffffu) {
-        const int j = sc_job(jobs, n_jobs, t, lane);
-        if (lane == 0) S.job = j;
       }
       if (lane == 0) S.ticket = t;
     }
@@ -714,6 +748,14 @@ __global__ void __launch_bounds__(SC_THREADS, 1) k_snappy_scan(const SnappyJob* 
     const uint32_t k = g - jb.seg;  // segment of the page
     const uint8_t* in = jb.src + jb.prefix;
     const uint32_t in_len = jb.src_len - jb.prefix, out_len = jb.dst_len - jb.prefix;
+    if (k == 0) {
+      lz_block_copy<SC_THREADS>(jb.dst, jb.src, jb.prefix);  // V2 level bytes, never compressed
+      for (uint32_t f = tid; f < jb.nsub; f += SC_THREADS) ss.owner[jb.sub + f] = static_cast<uint32_t>(S.job);
+    }
+    if (ss.bad[jb.sub + 1]) {
+      __syncthreads();
+      continue;
+    }
     // segment byte p is input byte org + p (the first segment starts at the
     // 16-byte boundary before the input)
     const uint32_t lead = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(in) & 15);
@@ -729,10 +771,6 @@ __global__ void __launch_bounds__(SC_THREADS, 1) k_snappy_scan(const SnappyJob* 
       fence_proxy_async_smem();
       mbar_arrive_expect_tx(&S.bar, static_cast<uint32_t>(bytes));
       bulk_g2s(S.stage, reinterpret_cast<const void*>(a0), static_cast<uint32_t>(bytes), &S.bar);
-    }
-    if (k == 0) {
-      lz_block_copy<SC_THREADS>(jb.dst, jb.src, jb.prefix);  // V2 level bytes, never compressed
-      for (uint32_t f = tid; f < jb.nsub; f += SC_THREADS) ss.owner[jb.sub + f] = static_cast<uint32_t>(S.job);
     }
     bool staged = mbar_wait(&S.bar, parity);
     if (!staged) staged = mbar_wait(&S.bar, parity) && false;  // (the copy may not outlive its buffer)
@@ -917,7 +955,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) k_snappy_scan(const SnappyJob* 
 }
 
 void launch_snappy_scan(const SnappyJob* jobs, int n_jobs, uint32_t seg_begin, uint32_t n_segs, SnapState ss,
-                        uint32_t* tickets, int n_sms, DevStatus* st, cudaStream_t s) {
+                        uint32_t* tickets, bool long_first, int n_sms, DevStatus* st, cudaStream_t s) {
   if (n_jobs <= 0 || n_segs == 0) return;
   static bool attr = false;
   if (!attr) {
@@ -925,6 +963,7 @@ void launch_snappy_scan(const SnappyJob* jobs, int n_jobs, uint32_t seg_begin, u
     attr = true;
   }
   const unsigned blocks = n_segs < static_cast<uint32_t>(n_sms) ? n_segs : n_sms;
+  if (long_first) k_snappy_long<<<n_jobs, 32, 0, s>>>(jobs, ss);
   k_snappy_scan<<<blocks, SC_THREADS, sizeof(SnScan), s>>>(jobs, n_jobs, seg_begin, n_segs, ss, tickets, st);
 }
 

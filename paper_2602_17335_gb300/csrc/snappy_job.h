@@ -36,7 +36,8 @@ struct SnappyJob {
 struct SnapState {
   uint32_t* owner;     // fragment: its job's index in the job list, written by the scan
   uint32_t* start;     // fragment: input offset of its first element
-  uint32_t* bad;       // first fragment of a job: the page is not framed, decompress it whole
+  uint32_t* bad;       // first fragment of a job: the page is not framed, decompress it whole;
+                       // second: k_snappy_long has recorded its fragments
   unsigned long long* exit;  // segment: SN_SET | input offset of the first element past it
   unsigned long long* len;   // segment: SN_SET | output bytes of the elements that start in it
 };
