@@ -29,6 +29,8 @@
 // Huffman and RLE literals are kept in the page's own output tail until the
 // sequences use them (the output never passes the unread ones: what is still
 // to be written is at least what is unread); raw literals stay in the input.
+#include <stddef.h>
+
 #include "dev_util.cuh"
 #include "lz_exec.cuh"
 #include "snappy_job.h"
@@ -421,91 +423,157 @@ __device__ void z_huffman_tree(ZBlock& S, const uint8_t* p, uint32_t len) {
 
 // ------------------------------------------------------------------ Huffman literals
 
-// Symbols of one stream whose codes start at bits (lim, pos]: each is given
-// to put; returns the position after the last.  A window holds 57 bits, so it
-// is reloaded every 57 / mb symbols, by all lanes of a warp at once (reloading
-// where each lane runs dry made every symbol wait for some lane's load: 570
-// cycles a symbol).
+// Symbols of one stream whose codes start at staged bits (lim, pos]: each is
+// given to put(symbol, true); returns the position after the last.  A window
+// holds 64 bits, enough for five codes of at most 12, and is reloaded by all
+// lanes of a warp at once (where each lane ran dry, every symbol waited for
+// some lane's load: 570 cycles a symbol); past lim a lane decodes on without
+// moving, as a branch a symbol cost more than that.
 template <typename Put>
-__device__ __forceinline__ int32_t z_huf_share(const uint16_t* huf, int mb, const uint8_t* p, int32_t pos, int32_t lim,
-                                               Put put) {
-  const int per = 57 / mb;
+__device__ __forceinline__ int32_t z_huf_share(const uint16_t* huf, int mb, const uint32_t* words, int32_t pos,
+                                               int32_t lim, Put put) {
+  const int drop = 32 - mb;
   while (pos > lim) {
-    uint64_t w = z_top(ZRead{p, pos});
-    for (int i = 0; i < per; ++i) {
-      if (pos > lim) {
-        const uint32_t e = huf[static_cast<uint32_t>(w >> (64 - mb))];
-        const int32_t n = static_cast<int32_t>(e >> 8);
-        put(e & 0xffu);
-        w <<= n;
-        pos -= n;
-      }
+    const uint32_t* q = words + (pos >> 5);
+    const uint32_t q0 = q[0], q1 = q[-1], q2 = q[-2];
+    uint32_t hi = __funnelshift_r(q1, q0, pos), lo = __funnelshift_r(q2, q1, pos);
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+      const uint32_t e = huf[hi >> drop];
+      const bool live = pos > lim;
+      const uint32_t n = live ? e >> 8 : 0u;
+      put(e & 0xffu, live);
+      hi = __funnelshift_l(lo, hi, n);
+      lo <<= n;
+      pos -= static_cast<int32_t>(n);
     }
   }
   return pos;
 }
 
-// The literal streams into out.  Block-collective; errors in S.err.
+// The same, only counted: (position after the last, symbols).  (Not inlined:
+// three copies of it cost the kernel registers.)
+__device__ __noinline__ int2 z_huf_count(const uint16_t* huf, int mb, const uint32_t* words, int32_t pos, int32_t lim) {
+  int32_t m = 0;
+  const int32_t end = z_huf_share(huf, mb, words, pos, lim, [&](uint32_t, bool live) { m += live; });
+  return make_int2(end, m);
+}
+
+// The literal streams into out.  The streams are decoded from the top, a part
+// at a time that fits the idle workspace of lz_pairs (gathered from the input
+// by 32 lanes in 32 lines, a window of a warp took 64 L1 wavefronts: 205,000
+// cycles a block of 112,000 literals, now 130,000, a third of them the
+// scattered stores), every thread a share of a part.
+// A share is decoded in three pieces, so that a thread whose start moves need
+// only decode until it meets a piece's end that it had reached before.
+// Block-collective; errors in S.err.
 __device__ void z_huffman_literals(ZBlock& S, const ZHufStreams& hs, uint8_t* out) {
   const int tid = threadIdx.x;
   const int per = ZT / hs.n, k = tid / per, i = tid % per;
   const int mb = S.huf_bits;
+  constexpr uint32_t kPad = 4;  // words of padding below a stream's bytes
+  uint32_t* const work = reinterpret_cast<uint32_t*>(S.lz.rec);
+  constexpr uint32_t kWork = (sizeof(S.lz) - offsetof(decltype(S.lz), rec)) / 64 * 16;  // words
+  const uint32_t room = kWork / hs.n / 4 * 4;  // words of a stream (16-byte aligned)
+  uint32_t* const words = work + room * k;
+  const int32_t most = static_cast<int32_t>((room - kPad - 16) * 32 / per);  // bits of a share
   ZRead r{nullptr, 0};
   const bool ok = z_open(r, hs.p[k], hs.len[k]);
   if (!ok && i == 0) S.err = ZE_STREAM;
-  const int32_t bits = ok ? r.pos : 0;
-  const int32_t share = (bits + per - 1) / per > 128 ? (bits + per - 1) / per : 128;
-  const int64_t hi64 = static_cast<int64_t>(bits) - static_cast<int64_t>(i) * share;
-  int32_t start = hi64 > 0 ? static_cast<int32_t>(hi64) : 0;
-  const int32_t lim = hi64 - share > 0 ? static_cast<int32_t>(hi64 - share) : 0;
-  int32_t end = start;
-  uint32_t count = 0;
-  bool todo = true;
-  // a round fixes at least one more share of every stream
-  for (int round = 0; round <= per; ++round) {
-    if (todo) {
-      count = 0;
-      end = z_huf_share(S.huf, mb, r.p, start, lim, [&](uint32_t) { ++count; });
-      S.end[tid] = end;
-    }
-    __syncthreads();
-    const int32_t s = i == 0 ? start : S.end[tid - 1];
-    todo = s != start;
-    start = s;
-    if (!__syncthreads_or(todo)) break;
-  }
-  // each share's place among its stream's symbols
-  const int lane = tid & 31, warp = tid >> 5;
-  uint32_t incl = count;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += y;
-  }
-  if (lane == 31) S.tmp[warp] = incl;
-  __syncthreads();
-  uint32_t before = incl - count;
-  for (int w = k * per / 32; w < warp; ++w) before += S.tmp[w];
+  int32_t top = ok ? r.pos : 0;  // bits left
+  uint32_t written = 0;          // symbols of the stream before the part
   const uint32_t want = hs.cnt[k];
-  if (i == per - 1 && (end != 0 || before + count != want)) S.err = ZE_STREAM;
-  __syncthreads();
-  if (S.err) return;
-  uint8_t* o = out + hs.out[k] + before;
-  uint32_t word = 0, fill = 0;
-  z_huf_share(S.huf, mb, r.p, start, lim, [&](uint32_t b) {
-    if (fill == 0 && (reinterpret_cast<uintptr_t>(o) & 3)) {
-      *o++ = static_cast<uint8_t>(b);
-      return;
+  const int lane = tid & 31, warp = tid >> 5;
+  for (;;) {
+    int32_t share = (top + per - 1) / per > 128 ? (top + per - 1) / per : 128;
+    share = share < most ? share : most;
+    const int32_t low = top - share * per > 0 ? top - share * per : 0;
+    // bytes [from, (top + 7) / 8): the part's and, below it, those its last codes reach into
+    const int32_t from = low / 8 > 16 ? low / 8 - 16 : 0;
+    const uintptr_t a = reinterpret_cast<uintptr_t>(r.p + from) & ~uintptr_t(15);
+    if (top > 0) {
+      const uint32_t n16 = static_cast<uint32_t>((reinterpret_cast<uintptr_t>(r.p) + (top + 7) / 8 + 15 - a) / 16);
+      uint4* d = reinterpret_cast<uint4*>(words + kPad);
+      for (uint32_t q = i; q < n16; q += per) d[q] = __ldg(reinterpret_cast<const uint4*>(a) + q);
     }
-    word |= b << (8 * fill);
-    if (++fill == 4) {
-      *reinterpret_cast<uint32_t*>(o) = word;
-      o += 4;
-      word = fill = 0;
+    // stream bit b is staged bit b + base
+    const int32_t base = static_cast<int32_t>(8 * (reinterpret_cast<intptr_t>(r.p) - static_cast<intptr_t>(a))) + 32 * kPad;
+    __syncthreads();
+    const int32_t hi = top - i * share > 0 ? top - i * share : 0;
+    int32_t start = hi;
+    const int32_t lim = hi - share > low ? hi - share : low;
+    int32_t met[3] = {-1, -1, -1};  // where each piece ended, and its symbols
+    uint32_t cnt[3] = {0, 0, 0};
+    const int32_t cut[3] = {hi - (hi - lim) / 4, hi - (hi - lim) / 2, lim};
+    int32_t end = start;
+    bool todo = true;
+    // a round fixes at least one more share of every stream
+    for (int round = 0; round <= per; ++round) {
+      if (todo) {
+        int32_t q = start;
+        bool same = false;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          if (!same) {
+            const int2 r2 = z_huf_count(S.huf, mb, words, q + base, cut[c] + base);
+            q = r2.x - base;
+            cnt[c] = static_cast<uint32_t>(r2.y);
+            same = q == met[c];
+            met[c] = q;
+          }
+        }
+        end = met[2];
+        S.end[tid] = end;
+      }
+      __syncthreads();
+      const int32_t s = i == 0 ? start : S.end[tid - 1];
+      todo = s != start;
+      start = s;
+      if (!__syncthreads_or(todo)) break;
     }
-  });
-  for (uint32_t q = 0; q < fill; ++q) o[q] = static_cast<uint8_t>(word >> (8 * q));
-  __syncthreads();
+    const uint32_t count = cnt[0] + cnt[1] + cnt[2];
+    // each share's place among its stream's symbols
+    uint32_t incl = count;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += y;
+    }
+    if (lane == 31) S.tmp[warp] = incl;
+    __syncthreads();
+    uint32_t before = written + incl - count, total = 0;
+    for (int w = k * per / 32; w < (k + 1) * per / 32; ++w) {
+      before += w < warp ? S.tmp[w] : 0u;
+      total += S.tmp[w];
+    }
+    const int32_t next = S.end[k * per + per - 1];  // where the part's codes end
+    if (i == 0 && (total > want - written || (low == 0 && (next != 0 || written + total != want)))) S.err = ZE_STREAM;
+    __syncthreads();
+    if (S.err) return;
+    // bytes up to the first 4-byte boundary, words, bytes
+    uint8_t* o = out + hs.out[k] + before;
+    uint32_t skip = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(o) & 3), fill = skip, word = 0;
+    o -= skip;
+    z_huf_share(S.huf, mb, words, start + base, lim + base, [&](uint32_t b, bool live) {
+      word |= (live ? b : 0u) << (8 * fill);
+      fill += live;
+      if (fill == 4) {
+        if (skip) {
+          for (uint32_t q = skip; q < 4; ++q) o[q] = static_cast<uint8_t>(word >> (8 * q));
+          skip = 0;
+        } else {
+          *reinterpret_cast<uint32_t*>(o) = word;
+        }
+        o += 4;
+        word = fill = 0;
+      }
+    });
+    for (uint32_t q = skip; q < fill; ++q) o[q] = static_cast<uint8_t>(word >> (8 * q));
+    written += total;
+    top = low > 0 && next > 0 ? next : 0;
+    if (i == 0 && low > 0 && next <= 0 && (next != 0 || written != want)) S.err = ZE_STREAM;
+    if (!__syncthreads_or(top > 0)) break;
+  }
 }
 
 // ------------------------------------------------------------------ a compressed block
