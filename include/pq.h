@@ -229,9 +229,9 @@ void pq_free_plan(pq_plan* plan);
 
 /* Stages of a scan, in order, for pq_plan_stage_ms. */
 #define PQ_STAGE_PREPARE 0     /* reset of bitmaps, counters, error word */
-#define PQ_STAGE_SNAPPY 1      /* page decompression (K1), then the rewrite of
-                                  BYTE_STREAM_SPLIT / DELTA_(LENGTH_)BYTE_ARRAY
-                                  pages into PLAIN bodies */
+#define PQ_STAGE_SNAPPY 1      /* page decompression (K1), then PLAIN bodies of
+                                  BYTE_STREAM_SPLIT pages and entry tables of
+                                  DELTA_(LENGTH_)BYTE_ARRAY pages */
 #define PQ_STAGE_DICT 2        /* dictionary decode (K6) */
 #define PQ_STAGE_WALK 3        /* page walk: levels, stream checkpoints */
 #define PQ_STAGE_EXPAND 4      /* value expansion of the work items */
@@ -419,9 +419,9 @@ typedef struct pq_tuning {
                                  page through; 0 = chosen by page count (default), else a
                                  power of two in 4096..65536 */
   int32_t snappy_block_kib;   /* compressed data pages of at least this many KiB are
-                                 decompressed by a block of 8 warps each, smaller ones by one
-                                 warp (dictionary pages always by a block); 1..1048576
-                                 (default 256) */
+                                 decompressed by blocks of 16 warps, smaller ones by blocks
+                                 of 4 (dictionary pages and short lists of pages always by
+                                 16); 1..1048576 (default 256) */
   int32_t staged_expand;      /* 1: REQUIRED fixed-width dictionary columns take the staged
                                  expansion (index bytes bulk-copied to shared memory); 0: the
                                  general warp decode (default 1) */

@@ -7,8 +7,8 @@ The knobs set scheduling granularity, block sizes and staging depth:
 - how many streams one scan's columns are forked onto;
 - the staging depth of the page walks (bytes per shared-memory chain
   window);
-- the compressed page size from which a block of 8 warps, rather than one
-  warp, decompresses a Snappy page;
+- the compressed page size from which a block of 16 warps, rather than 4,
+  decompresses a Snappy page;
 - whether dictionary columns take the staged (shared-memory) expansion.
 
 The paper's Section 3 (Insight 1) ties a GPU reader's parallelism to its

@@ -143,8 +143,9 @@ struct pq_plan {
   std::vector<int32_t> str_cols;             // output columns of type BYTE_ARRAY
   std::vector<uint32_t> walk_pps;            // plan pages that need the walk, longest first
   std::vector<uint32_t> delta_pps;           // DELTA plan pages
-  // V2 pages rewritten into PLAIN bodies (plan page order); host side: where
-  // each job's source and destination lie (scratch offset, or -1: `src` is
+  // V2 pages transcoded (plan page order): PLAIN bodies of BYTE_STREAM_SPLIT,
+  // entry tables of the delta string encodings; host side: where each job's
+  // source and destination lie (scratch offset, or -1: `src` is
   // the stored page / the destination is the pool)
   std::vector<pqi::TranscodeJob> tc_jobs;
   std::vector<int64_t> tc_src_off, tc_dst_off;
