@@ -92,6 +92,14 @@ struct DecodeArgs {
   int n_delta;
 };
 
+// Jobs [0, n) in launches of as many as a grid's y dimension holds (a column of
+// 2^26 DOUBLE rows in 8 KiB pages is 65,536 of them): launch(first, jobs).
+constexpr int GRID_Y_MAX = 65535;
+template <typename Launch>
+inline void launch_slices(int n, Launch launch) {
+  for (int at = 0; at < n; at += GRID_Y_MAX) launch(at, n - at < GRID_Y_MAX ? n - at : GRID_Y_MAX);
+}
+
 // The transcode of jobs [0, n), n_bss of them BYTE_STREAM_SPLIT pages;
 // `counters` is the plan's item_counter array (its pool word); `pool` holds
 // `pool_cap` bytes for DELTA_BYTE_ARRAY bodies; string pages get their entry

@@ -567,16 +567,18 @@ void launch_dict(const DictJob* jobs, int n_jobs, bool fixed, int max_fixed_byte
   if (gx < 1) gx = 1;
   if (gx > 4 * n_sms) gx = 4 * n_sms;
   if (fixed)
-    k_dict_fixed<<<dim3(gx, n_jobs), 256, 0, s>>>(jobs, dicts, st);
+    launch_slices(n_jobs, [&](int at, int m) { k_dict_fixed<<<dim3(gx, m), 256, 0, s>>>(jobs + at, dicts, st); });
   if (max_str_regions > 0) {
     static bool attr = false;
     if (!attr) {
       cudaFuncSetAttribute(k_sreg, cudaFuncAttributeMaxDynamicSharedMemorySize, SREG_SMEM);
       attr = true;
     }
-    k_sreg<<<dim3(max_str_regions, n_jobs), 32, SREG_SMEM, s>>>(jobs, ds, st);
+    launch_slices(n_jobs, [&](int at, int m) {
+      k_sreg<<<dim3(max_str_regions, m), 32, SREG_SMEM, s>>>(jobs + at, ds, st);
+    });
     k_sfix<<<n_jobs, SFIX_THREADS, 0, s>>>(jobs, ds, dicts, st);
-    k_dict_pad<<<dim3(32, n_jobs), 256, 0, s>>>(jobs, dicts);
+    launch_slices(n_jobs, [&](int at, int m) { k_dict_pad<<<dim3(32, m), 256, 0, s>>>(jobs + at, dicts); });
   }
 }
 
@@ -3825,10 +3827,10 @@ void launch_delta_bases(const DecodeArgs& a, int dbegin, int n, int max_regions,
     attr = true;
   }
   if (max_regions > 0) {
-    k_dreg<<<dim3(max_regions, n), 32, dreg_smem, s>>>(a, dbegin);
+    launch_slices(n, [&](int at, int m) { k_dreg<<<dim3(max_regions, m), 32, dreg_smem, s>>>(a, dbegin + at); });
     k_dfix<<<n, DFIX_THREADS, 0, s>>>(a, dbegin);
   }
-  k_delta_sums<<<dim3(64, n), 256, 0, s>>>(a, dbegin);
+  launch_slices(n, [&](int at, int m) { k_delta_sums<<<dim3(64, m), 256, 0, s>>>(a, dbegin + at); });
   k_delta_scan<<<n, 1024, 0, s>>>(a, dbegin);
 }
 

@@ -681,7 +681,8 @@ __global__ void __launch_bounds__(256) k_bss(const TranscodeJob* jobs, PlanPage*
 void launch_transcode(const TranscodeJob* jobs, int n, int n_bss, PlanPage* pps, uint8_t* pool, uint64_t pool_cap,
                       uint32_t* counters, uint64_t* vpos, DevStatus* st, cudaStream_t s) {
   if (n <= 0) return;
-  if (n_bss > 0) k_bss<<<dim3(BSS_BLOCKS, n), 256, 0, s>>>(jobs, pps, st);
+  if (n_bss > 0)
+    launch_slices(n, [&](int at, int m) { k_bss<<<dim3(BSS_BLOCKS, m), 256, 0, s>>>(jobs + at, pps, st); });
   if (n_bss == n) return;
   static bool attr = false;
   if (!attr) {
