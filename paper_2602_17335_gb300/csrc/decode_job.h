@@ -92,6 +92,9 @@ struct DecodeArgs {
   int n_delta;
 };
 
+// No launch of this thread has failed since its last error was taken.
+inline bool launched() { return cudaPeekAtLastError() == cudaSuccess; }
+
 // Jobs [0, n) in launches of as many as a grid's y dimension holds (a column of
 // 2^26 DOUBLE rows in 8 KiB pages is 65,536 of them): launch(first, jobs).
 constexpr int GRID_Y_MAX = 65535;

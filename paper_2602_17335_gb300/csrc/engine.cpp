@@ -305,8 +305,10 @@ pq_status pq_ctx_get_tuning(const pq_ctx* ctx, pq_tuning* t) {
 // Small device-to-host reads (status words, page counts, the page table)
 // go by a copy kernel into pinned host memory rather than by the copy
 // engine, where they would wait behind bulk transfers of other streams.
+// Returns the error of a launch before it too (which its own checks clear).
 static cudaError_t d2h_small(void* pinned_dst, const void* src, size_t bytes, cudaStream_t s) {
-  if (!bytes) return cudaSuccess;
+  const cudaError_t before = cudaGetLastError();
+  if (before != cudaSuccess || !bytes) return before;
   void* dv = nullptr;
   if (bytes >= (1u << 31) || cudaHostGetDevicePointer(&dv, pinned_dst, 0) != cudaSuccess || !dv) {
     cudaGetLastError();
@@ -1331,7 +1333,14 @@ pq_status plan_upload(pq_plan* plan, cudaStream_t s) {
     CK(cudaMemcpyAsync(u.dst, plan->h_up.p + up_off, u.bytes, cudaMemcpyHostToDevice, s));
     up_off += (u.bytes + 15) & ~size_t(15);
   }
-  if (nit) pqi::launch_make_items(decode_args(plan), static_cast<int>(npp), s);
+  if (nit) {
+    pqi::launch_make_items(decode_args(plan), static_cast<int>(npp), s);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) {
+      free_plan_device(plan);
+      return cuda_fail(ctx, e, "kernel launch");
+    }
+  }
   // no host wait: a scan's stream waits on this event (the host arrays are
   // plan members, alive until the plan is freed)
   CK(ctx->events.take(&plan->ready));
@@ -1590,7 +1599,7 @@ static void launch_decompress(pq_plan* plan, const pqi::SnappyJob* jobs, int n, 
   if (n <= 0) return;
   const int n_sms = plan->ctx->n_sms;
   pqi::launch_snappy(jobs, n, n_sms, st, s, wide);
-  if (plan->zstd_jobs) pqi::launch_zstd(jobs, n, n_sms, st, s);
+  if (plan->zstd_jobs && pqi::launched()) pqi::launch_zstd(jobs, n, n_sms, st, s);
 }
 
 // A stretch of one of the plan's decompression job lists: jobs, fragments and
@@ -1641,7 +1650,9 @@ static void launch_range(pq_plan* plan, const SnapRange& r, pqi::DevStatus* st, 
     const int n_sms = plan->ctx->n_sms;
     const pqi::SnapState ss = pqi::snap_state(plan->d_snap_state, plan->snap_blocks, plan->snap_segs);
     pqi::launch_snappy_scan(r.jobs, r.n, r.seg0, r.nseg, ss, r.tickets, !r.dicts, n_sms, st, s);
+    if (!pqi::launched()) return;
     pqi::launch_snappy_fragments(r.jobs, static_cast<int>(r.blk0), static_cast<int>(r.nblk), ss, n_sms, st, s);
+    if (!pqi::launched()) return;
   }
   launch_decompress(plan, r.jobs, r.n, r.data_max >= wide_snappy_bytes(plan), st, s);
 }
@@ -1679,23 +1690,39 @@ static uint32_t* strings_left(pq_plan* plan, size_t oc) {
   return plan->d_counter + pqi::STR_COUNTER0(static_cast<uint32_t>(plan->outcols.size())) + oc;
 }
 
-// Kernels of one output column, in order, on one stream.
+// Kernels of one output column, in order, on one stream.  As everywhere in a
+// scan, a stage whose launch failed is the last: the next ones would read what
+// it never wrote.
 static void enqueue_column(pq_plan* plan, size_t oc, const pqi::DecodeArgs& a, bool with_dicts, cudaStream_t s) {
   pq_ctx* ctx = plan->ctx;
   const auto& cw = plan->colwork[oc];
   if (with_dicts) launch_range(plan, column_range(plan, oc, true), a.st, s);
+  if (!pqi::launched()) return;
   if (with_dicts && cw.dict_n)
     pqi::launch_dict(plan->d_dict_jobs + cw.dict_begin, cw.dict_n, plan->outcols[oc].ptype != pqi::T_BYTE_ARRAY, cw.max_fixed_dict, cw.max_str_regions,
                      pqi::DictScratch{plan->d_sregs, plan->d_slists}, plan->idx->d_dicts, ctx->n_sms, a.st, s);
+  if (!pqi::launched()) return;
   launch_range(plan, column_range(plan, oc, false), a.st, s);
+  if (!pqi::launched()) return;
   enqueue_transcode(plan, cw.tc_begin, cw.tc_n, cw.tc_bss, a, s);
+  if (!pqi::launched()) return;
   const auto& col = plan->outcols[oc];
   pqi::launch_walk(a, cw.walk_begin, cw.walk_n, ctx->n_sms, col.optional != 0, plan->tuning.walk_window, s);
+  if (!pqi::launched()) return;
   pqi::launch_delta_bases(a, cw.delta_begin, cw.delta_n, cw.max_regions, s);
+  if (!pqi::launched()) return;
   launch_column_expand(plan, oc, a, s);
-  if (col.ptype == pqi::T_BYTE_ARRAY)
+  if (col.ptype == pqi::T_BYTE_ARRAY && pqi::launched())
     pqi::launch_strings(a, static_cast<int>(oc), static_cast<int>(col.item_count), ctx->n_sms, !plan->sizing,
                         strings_left(plan, oc), s);
+}
+
+// The string columns' offsets and characters, all on one stream.
+static void enqueue_strings(pq_plan* plan, const pqi::DecodeArgs& a, cudaStream_t s) {
+  for (int32_t sc : plan->str_cols)
+    if (pqi::launched())
+      pqi::launch_strings(a, sc, static_cast<int>(plan->outcols[sc].item_count), plan->ctx->n_sms, !plan->sizing,
+                          strings_left(plan, sc), s);
 }
 
 // The stages of all output columns, each launched once: dictionaries beside
@@ -1715,22 +1742,23 @@ static void enqueue_merged(pq_plan* plan, const pqi::DecodeArgs& a, bool with_di
   if (dicts) {
     cudaEventRecord(plan->fork, s);
     cudaStreamWaitEvent(side, plan->fork, 0);
-    launch_range(plan, plan_range(plan, true), a.st, side);
-    pqi::launch_dict(plan->d_dict_jobs, static_cast<int>(plan->dict_jobs.size()), fixed, plan->max_fixed_dict_bytes,
-                     max_str_regions_all(plan), pqi::DictScratch{plan->d_sregs, plan->d_slists}, plan->idx->d_dicts,
-                     ctx->n_sms, a.st, side);
+    if (pqi::launched()) launch_range(plan, plan_range(plan, true), a.st, side);
+    if (pqi::launched())
+      pqi::launch_dict(plan->d_dict_jobs, static_cast<int>(plan->dict_jobs.size()), fixed, plan->max_fixed_dict_bytes,
+                       max_str_regions_all(plan), pqi::DictScratch{plan->d_sregs, plan->d_slists}, plan->idx->d_dicts,
+                       ctx->n_sms, a.st, side);
     cudaEventRecord(plan->join[0], side);
   }
-  launch_range(plan, plan_range(plan, false), a.st, s);
-  enqueue_transcode(plan, 0, static_cast<int>(plan->tc_jobs.size()), n_bss, a, s);
-  pqi::launch_walk(a, 0, static_cast<int>(plan->walk_pps.size()), ctx->n_sms, levels, plan->tuning.walk_window, s);
-  pqi::launch_delta_bases(a, 0, static_cast<int>(plan->delta_pps.size()), max_regions, s);
+  if (pqi::launched()) launch_range(plan, plan_range(plan, false), a.st, s);
+  if (pqi::launched()) enqueue_transcode(plan, 0, static_cast<int>(plan->tc_jobs.size()), n_bss, a, s);
+  if (pqi::launched())
+    pqi::launch_walk(a, 0, static_cast<int>(plan->walk_pps.size()), ctx->n_sms, levels, plan->tuning.walk_window, s);
+  if (pqi::launched()) pqi::launch_delta_bases(a, 0, static_cast<int>(plan->delta_pps.size()), max_regions, s);
   if (dicts) cudaStreamWaitEvent(s, plan->join[0], 0);
-  pqi::launch_expand(a, 0, static_cast<int>(plan->n_items), 0, !plan->delta_pps.empty(), ctx->n_sms,
-                     plan->tuning.expand_ctas_per_sm, s);
-  for (int32_t sc : plan->str_cols)
-    pqi::launch_strings(a, sc, static_cast<int>(plan->outcols[sc].item_count), ctx->n_sms, !plan->sizing,
-                        strings_left(plan, sc), s);
+  if (pqi::launched())
+    pqi::launch_expand(a, 0, static_cast<int>(plan->n_items), 0, !plan->delta_pps.empty(), ctx->n_sms,
+                       plan->tuning.expand_ctas_per_sm, s);
+  enqueue_strings(plan, a, s);
 }
 
 // Enqueues the kernels of one scan (no host synchronisation).  Default:
@@ -1739,7 +1767,8 @@ static void enqueue_merged(pq_plan* plan, const pqi::DecodeArgs& a, bool with_di
 // column overlap the bandwidth-bound expansion of the others.  With
 // PQ_SCAN_TIMING the stages run one after another over all columns, so that
 // each stage can be timed.  PQ_SCAN_PLAIN: per chunk, one launch per stage.
-static void enqueue_scan(pq_plan* plan, cudaStream_t s, bool with_dicts, const cudaStream_t* branches,
+// Returns the first error of its launches.
+static cudaError_t enqueue_scan(pq_plan* plan, cudaStream_t s, bool with_dicts, const cudaStream_t* branches,
                          int n_branches) {
   pq_ctx* ctx = plan->ctx;
   pqi::DecodeArgs a = decode_args(plan);
@@ -1755,22 +1784,23 @@ static void enqueue_scan(pq_plan* plan, cudaStream_t s, bool with_dicts, const c
   const int n_dict_jobs = static_cast<int>(plan->snappy_dict.size());
   if (plan->flags & PQ_SCAN_PLAIN) {
     // baseline: per chunk, one launch per stage; one page per thread block
-    if (with_dicts && n_dict_jobs)
+    if (with_dicts && n_dict_jobs && pqi::launched())
       launch_decompress(plan, plan->d_snappy + n_data_jobs, n_dict_jobs, true, a.st, s);
     mark(2);
-    if (with_dicts && !plan->dict_jobs.empty())
+    if (with_dicts && !plan->dict_jobs.empty() && pqi::launched())
       pqi::launch_dict(plan->d_dict_jobs, static_cast<int>(plan->dict_jobs.size()), true, plan->max_fixed_dict_bytes,
                        max_str_regions_all(plan), pqi::DictScratch{plan->d_sregs, plan->d_slists}, plan->idx->d_dicts,
                        ctx->n_sms, a.st, s);
     mark(3);
     size_t job = 0, tcj = 0;
-    for (size_t k = 0; k < plan->chunk_pp.size(); ++k) {
+    for (size_t k = 0; k < plan->chunk_pp.size() && pqi::launched(); ++k) {
       const int first = plan->chunk_pp[k].first, n = plan->chunk_pp[k].second;
       int nj = 0;
       for (int p = first; p < first + n; ++p)
         if (job + nj < plan->snappy_data.size() && plan->snappy_data[job + nj].page == static_cast<int32_t>(plan->pps[p].page))
           ++nj;
       if (nj) launch_decompress(plan, plan->d_snappy + job, nj, plan->snap_data_max >= wide_snappy_bytes(plan), a.st, s);
+      if (!pqi::launched()) break;
       job += nj;
       int ntc = 0;
       while (tcj + ntc < plan->tc_jobs.size() && plan->tc_jobs[tcj + ntc].pp < static_cast<uint32_t>(first + n)) ++ntc;
@@ -1778,60 +1808,57 @@ static void enqueue_scan(pq_plan* plan, cudaStream_t s, bool with_dicts, const c
       for (int q = 0; q < ntc; ++q) nbss += plan->tc_jobs[tcj + q].enc == pqi::ENC_BSS;
       enqueue_transcode(plan, static_cast<int>(tcj), ntc, nbss, a, s);
       tcj += ntc;
-      pqi::launch_plain_pages(a, first, n, s);
+      if (pqi::launched()) pqi::launch_plain_pages(a, first, n, s);
     }
     mark(4);
     mark(5);
-    for (int32_t sc : plan->str_cols)
-      pqi::launch_strings(a, sc, static_cast<int>(plan->outcols[sc].item_count), ctx->n_sms, !plan->sizing,
-                          strings_left(plan, sc), s);
+    enqueue_strings(plan, a, s);
   } else if (timing) {
-    for (int oc = 0; oc < ncols; ++oc) {
+    for (int oc = 0; oc < ncols && pqi::launched(); ++oc) {
       const auto& cw = plan->colwork[oc];
       if (with_dicts) launch_range(plan, column_range(plan, oc, true), a.st, s);
-      launch_range(plan, column_range(plan, oc, false), a.st, s);
-      enqueue_transcode(plan, cw.tc_begin, cw.tc_n, cw.tc_bss, a, s);
+      if (pqi::launched()) launch_range(plan, column_range(plan, oc, false), a.st, s);
+      if (pqi::launched()) enqueue_transcode(plan, cw.tc_begin, cw.tc_n, cw.tc_bss, a, s);
     }
     mark(2);
-    for (int oc = 0; oc < ncols; ++oc) {
+    for (int oc = 0; oc < ncols && pqi::launched(); ++oc) {
       const auto& cw = plan->colwork[oc];
       if (with_dicts && cw.dict_n)
         pqi::launch_dict(plan->d_dict_jobs + cw.dict_begin, cw.dict_n, plan->outcols[oc].ptype != pqi::T_BYTE_ARRAY, cw.max_fixed_dict, cw.max_str_regions,
                          pqi::DictScratch{plan->d_sregs, plan->d_slists}, plan->idx->d_dicts, ctx->n_sms, a.st, s);
     }
     mark(3);
-    for (int oc = 0; oc < ncols; ++oc) {
+    for (int oc = 0; oc < ncols && pqi::launched(); ++oc) {
       const auto& cw = plan->colwork[oc];
       pqi::launch_walk(a, cw.walk_begin, cw.walk_n, ctx->n_sms, plan->outcols[oc].optional != 0,
                        plan->tuning.walk_window, s);
-      pqi::launch_delta_bases(a, cw.delta_begin, cw.delta_n, cw.max_regions, s);
+      if (pqi::launched()) pqi::launch_delta_bases(a, cw.delta_begin, cw.delta_n, cw.max_regions, s);
     }
     mark(4);
-    for (int oc = 0; oc < ncols; ++oc) launch_column_expand(plan, oc, a, s);
+    for (int oc = 0; oc < ncols && pqi::launched(); ++oc) launch_column_expand(plan, oc, a, s);
     mark(5);
-    for (int32_t sc : plan->str_cols)
-      pqi::launch_strings(a, sc, static_cast<int>(plan->outcols[sc].item_count), ctx->n_sms, !plan->sizing,
-                          strings_left(plan, sc), s);
+    enqueue_strings(plan, a, s);
   } else if (merged_scan(plan)) {
     enqueue_merged(plan, a, with_dicts, branches[0], s);
   } else {
     cudaEventRecord(plan->fork, s);
-    for (int oc = 0; oc < ncols; ++oc) {
+    for (int oc = 0; oc < ncols; ++oc) {  // (a failed launch leaves the branches joined all the same)
       cudaStream_t b = branches[oc % n_branches];
       cudaStreamWaitEvent(b, plan->fork, 0);
-      enqueue_column(plan, oc, a, with_dicts, b);
+      if (pqi::launched()) enqueue_column(plan, oc, a, with_dicts, b);
       cudaEventRecord(plan->join[oc], b);
     }
     for (int oc = 0; oc < ncols; ++oc) cudaStreamWaitEvent(s, plan->join[oc], 0);
   }
   mark(6);
   // status and string totals back to pinned host memory
-  d2h_small(plan->h_out.p, plan->d_status, sizeof(pqi::DevStatus), s);
-  for (size_t i = 0; i < plan->str_cols.size(); ++i) {
+  cudaError_t e = d2h_small(plan->h_out.p, plan->d_status, sizeof(pqi::DevStatus), s);
+  for (size_t i = 0; i < plan->str_cols.size() && e == cudaSuccess; ++i) {
     const auto& col = plan->outcols[plan->str_cols[i]];
-    d2h_small(plan->h_out.p + sizeof(pqi::DevStatus) + 8 * i, reinterpret_cast<int64_t*>(col.values) + plan->n_rows,
-              8, s);
+    e = d2h_small(plan->h_out.p + sizeof(pqi::DevStatus) + 8 * i,
+                  reinterpret_cast<int64_t*>(col.values) + plan->n_rows, 8, s);
   }
+  return e;
 }
 
 }  // extern "C"
@@ -1899,12 +1926,16 @@ pq_status scan_enqueue(pq_plan* plan, const pq_column* outs, cudaStream_t s, con
         own = true;
       }
       CK(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
-      enqueue_scan(plan, cs, with_dicts, branches, n_branches);
+      const cudaError_t launch = enqueue_scan(plan, cs, with_dicts, branches, n_branches);
       cudaGraph_t g = nullptr;
       cudaError_t e = cudaStreamEndCapture(cs, &g);
       if (own) {
         cudaStreamSynchronize(cs);
         cudaStreamDestroy(cs);
+      }
+      if (launch != cudaSuccess) {
+        if (g) cudaGraphDestroy(g);
+        return cuda_fail(ctx, launch, "kernel launch");
       }
       if (e != cudaSuccess) return cuda_fail(ctx, e, "graph capture");
       e = cudaGraphInstantiate(&plan->graph, g, 0);
@@ -1914,7 +1945,12 @@ pq_status scan_enqueue(pq_plan* plan, const pq_column* outs, cudaStream_t s, con
     }
     CK(cudaGraphLaunch(plan->graph, s));
   } else {
-    enqueue_scan(plan, s, with_dicts, branches, n_branches);
+    const cudaError_t launch = enqueue_scan(plan, s, with_dicts, branches, n_branches);
+    if (launch != cudaSuccess) {
+      // (what was launched before uses the plan's memory until `done`)
+      cudaEventRecord(plan->done, s);
+      return cuda_fail(ctx, launch, "kernel launch");
+    }
   }
   CK(cudaGetLastError());
   CK(cudaEventRecord(plan->done, s));

@@ -327,7 +327,8 @@ pq_status scan_pipelined(pq_ctx* ctx, const pq_file* host_files, int n_files, co
     for (size_t c = 0; c < cols.size(); ++c)
       if (sl.sz[c].type == PQ_TYPE_BYTE_ARRAY)
         pqi::launch_add_offsets(static_cast<int64_t*>(sl.outs[c].values), n + 1, chars_base[c], sl.sc);
-    if (cudaEventRecord(sl.scanned, sl.sc) != cudaSuccess || cudaStreamWaitEvent(g.sd, sl.scanned, 0) != cudaSuccess)
+    if (cudaGetLastError() != cudaSuccess || cudaEventRecord(sl.scanned, sl.sc) != cudaSuccess ||
+        cudaStreamWaitEvent(g.sd, sl.scanned, 0) != cudaSuccess)
       return fail(ctx, PQ_ERR_CUDA, "event");
     for (size_t c = 0; c < cols.size(); ++c) {
       const pq_out_size& z = sl.sz[c];

@@ -577,7 +577,9 @@ void launch_dict(const DictJob* jobs, int n_jobs, bool fixed, int max_fixed_byte
     launch_slices(n_jobs, [&](int at, int m) {
       k_sreg<<<dim3(max_str_regions, m), 32, SREG_SMEM, s>>>(jobs + at, ds, st);
     });
+    if (!launched()) return;
     k_sfix<<<n_jobs, SFIX_THREADS, 0, s>>>(jobs, ds, dicts, st);
+    if (!launched()) return;
     launch_slices(n_jobs, [&](int at, int m) { k_dict_pad<<<dim3(32, m), 256, 0, s>>>(jobs + at, dicts); });
   }
 }
@@ -3775,8 +3777,9 @@ void launch_delta_static(uint8_t* scratch, const uint8_t* stream, uint32_t len, 
   a.n_delta = 1;
   k_dstatic_init<<<1, 32, 0, s>>>(a, reinterpret_cast<ChunkDev*>(scratch + DS_OFF_CHUNK),
                                   reinterpret_cast<uint32_t*>(scratch + DS_OFF_PPS), stream, len, ptype, n);
+  if (!launched()) return;
   launch_delta_bases(a, 0, 1, static_cast<int>(len / DELTA_REGION + 2), s);
-  if (n > 0) {
+  if (n > 0 && launched()) {
     const int64_t warps = (static_cast<int64_t>(n) + DS_WARP_VALUES - 1) / DS_WARP_VALUES;
     k_dstatic_expand<<<static_cast<unsigned>((warps + 7) / 8), 256, 0, s>>>(a, static_cast<uint8_t*>(out), n);
   }
@@ -3828,9 +3831,12 @@ void launch_delta_bases(const DecodeArgs& a, int dbegin, int n, int max_regions,
   }
   if (max_regions > 0) {
     launch_slices(n, [&](int at, int m) { k_dreg<<<dim3(max_regions, m), 32, dreg_smem, s>>>(a, dbegin + at); });
+    if (!launched()) return;
     k_dfix<<<n, DFIX_THREADS, 0, s>>>(a, dbegin);
   }
+  if (!launched()) return;
   launch_slices(n, [&](int at, int m) { k_delta_sums<<<dim3(64, m), 256, 0, s>>>(a, dbegin + at); });
+  if (!launched()) return;
   k_delta_scan<<<n, 1024, 0, s>>>(a, dbegin);
 }
 

@@ -1,0 +1,91 @@
+"""Planning and scan enqueueing (csrc/engine.cpp) compiled for the CPU with g++
+over a CUDA runtime of the test's own: device memory is host memory and a kernel
+is an entry in a log.  A launch that the runtime refuses has to come back as an
+error from the scan, whichever it is.  No GPU needed."""
+import ctypes
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+import synth
+from oracle import writer as W
+from paper_2602_17335_gb300 import native as N
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+HERE = os.path.dirname(os.path.abspath(__file__))
+CSRC = os.path.join(ROOT, "paper_2602_17335_gb300", "csrc")
+CUDA_INC = "/usr/local/cuda/include"
+
+
+@pytest.fixture(scope="module")
+def scan(tmp_path_factory):
+    """scan(file, flags, n_sms, fail_at) -> (status, {what: text})."""
+    if shutil.which("g++") is None or not os.path.exists(os.path.join(CUDA_INC, "cuda_runtime.h")):
+        pytest.skip("no g++ or CUDA headers")
+    out = str(tmp_path_factory.mktemp("scan_host") / "scan_host.so")
+    # (-Bsymbolic: the runtime of this library, whatever else the process has loaded)
+    subprocess.run(["g++", "-O1", "-std=c++17", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-I", CSRC, "-I",
+                    os.path.join(ROOT, "include"), "-I", CUDA_INC, os.path.join(HERE, "scan_host_harness.cpp"),
+                    *(os.path.join(CSRC, f) for f in ("engine.cpp", "host_meta.cpp", "host_pages.cpp")), "-o", out],
+                   check=True)
+    lib = ctypes.CDLL(out)
+    lib.scan_with_fake_cuda.argtypes = [ctypes.c_char_p, ctypes.c_uint64, ctypes.c_uint32, ctypes.c_int, ctypes.c_int,
+                                        ctypes.c_char_p, ctypes.c_uint64]
+
+    def run(data, flags=0, n_sms=152, fail_at=-1):
+        text = ctypes.create_string_buffer(1 << 16)
+        st = lib.scan_with_fake_cuda(data, len(data), flags, n_sms, fail_at, text, len(text))
+        return st, dict(line.split(" ", 1) for line in text.value.decode().splitlines())
+    return run
+
+
+def _eight(codec):
+    spec = synth.config2_spec(2500, 4096, codec, 1)
+    for c in spec.columns:
+        c.compress_threshold = -1.0
+    return W.write_file(synth.config2_table(6000, 2500, string_pool_size=200, zipf_k=300), spec)
+
+
+def _split():
+    """Snappy pages long enough to be decompressed by fragments."""
+    from paper_2602_17335_gb300.tables import write_table
+    from test_native_writer import _native
+    _native()
+    rng = np.random.default_rng(1)
+    cols = [synth.ColumnData(f"x{k}", "INT64", rng.integers(0, 50_000, 60_000)) for k in range(3)]
+    spec = synth.TableSpec(60_000, 1 << 20, [synth.ColumnSpec(e, "SNAPPY") for e in ("PLAIN", "RLE_DICTIONARY", "PLAIN")])
+    for c in spec.columns:
+        c.compress_threshold = -1.0
+    return write_table(synth.Table(cols), spec).tobytes()
+
+
+def _v2():
+    return W.write_file(synth.v2_encodings_table(4000, 2000), synth.v2_encodings_spec(2000, 1500))
+
+
+@pytest.mark.parametrize("flags", ["BATCHED", "PLAIN", "GRAPH", "TIMING"])
+@pytest.mark.parametrize("n_sms", [1, 152])  # one: launched column by column, many: all columns together
+@pytest.mark.parametrize("table", ["none", "snappy", "zstd", "split", "v2"])
+def test_refused_launches_are_errors(scan, flags, n_sms, table):
+    """Each launch of a scan refused in turn: the scan reports it, launches
+    nothing after it, leaves no stream unjoined, records the plan's end (which
+    freeing the plan waits for) and no error stays behind."""
+    data = {"none": lambda: _eight("UNCOMPRESSED"), "snappy": lambda: _eight("SNAPPY"), "zstd": lambda: _eight("ZSTD"),
+            "split": _split, "v2": _v2}[table]()
+    fl = getattr(N, "PQ_SCAN_" + flags)
+    st, good = scan(data, fl, n_sms)
+    assert st == N.PQ_OK and good["done"] == "1" and good["last_error"] == "0"
+    kernels = [k for k in good["launches"].split() if k != "graph"]
+    assert "prepare" == kernels[0] and "copy_small" == kernels[-1]
+    if table == "split" and flags != "PLAIN":
+        assert "snappy_fragments" in kernels
+    for k in range(len(kernels)):
+        st, got = scan(data, fl, n_sms, k)
+        assert st == N.PQ_ERR_CUDA, (k, kernels[k])
+        assert got["launches"].split() == kernels[:k + 1], kernels[k]
+        assert got["joins"] == good["joins"] and got["forks"] == good["forks"]
+        assert got["last_error"] == "0"
+        assert got["done"] == ("0" if flags == "GRAPH" else "1")  # (a graph that was not made has not run)
