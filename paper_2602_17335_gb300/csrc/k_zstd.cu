@@ -81,6 +81,13 @@ struct __align__(16) ZBlock {
   uint32_t sl, so, sm, pos;            // the chain between groups
 };
 
+// The error any thread has noted in S.err by now, the same for all threads.
+// Block-collective, with a barrier: the word is read on one side of it and
+// decided on by all threads at once.  (Read by each thread after a plain
+// barrier, a slow warp could see a later error than the others, return where
+// they went on, and leave the block's barriers out of step for its next pages.)
+__device__ __forceinline__ int z_error(const ZBlock& S) { return __syncthreads_or(S.err) ? S.err : 0; }
+
 __device__ __forceinline__ uint64_t z_load8(const uint8_t* p) { return ld_unaligned_g(p, 8); }
 
 // A backward bit stream read through 64-bit windows: p's bits [0, pos) are
@@ -279,8 +286,8 @@ __device__ __forceinline__ void z_entry(ZBlock& S, int which, int state, uint32_
 }
 
 // The Huffman tree description at p[0, len): S.huf, S.huf_bits; S.used bytes.
-// Block-collective; errors in S.err.
-__device__ void z_huffman_tree(ZBlock& S, const uint8_t* p, uint32_t len) {
+// Returns 0 or an error.  Block-collective.
+__device__ int z_huffman_tree(ZBlock& S, const uint8_t* p, uint32_t len) {
   const int tid = threadIdx.x;
   if (tid < 16) S.wcount[tid] = 0;
   for (int i = tid; i < 256; i += ZT) S.weights[i] = 0;
@@ -359,8 +366,7 @@ __device__ void z_huffman_tree(ZBlock& S, const uint8_t* p, uint32_t len) {
     }
     if (bad) S.err = ZE_HUF;
   }
-  __syncthreads();
-  if (S.err) return;
+  if (const int e = z_error(S)) return e;
   // the last symbol's weight is what is left to the next power of two
   const int n = S.n_weights;
   if (tid < 32) {
@@ -388,8 +394,7 @@ __device__ void z_huffman_tree(ZBlock& S, const uint8_t* p, uint32_t len) {
       if (bad) S.err = ZE_HUF;
     }
   }
-  __syncthreads();
-  if (S.err) return;
+  if (const int e = z_error(S)) return e;
   const int ns = n + 1, mb = S.huf_bits;
   if (tid < ns && S.weights[tid]) atomicAdd(&S.wcount[S.weights[tid]], 1u);
   __syncthreads();
@@ -403,8 +408,7 @@ __device__ void z_huffman_tree(ZBlock& S, const uint8_t* p, uint32_t len) {
     }
     if (at != (1u << mb)) S.err = ZE_HUF;  // (a weight above mb would be left out)
   }
-  __syncthreads();
-  if (S.err) return;
+  if (const int e = z_error(S)) return e;
   if (tid < ns && S.weights[tid]) {
     // its place among the symbols of its weight
     const uint32_t w = S.weights[tid], same = w * 0x01010101u;
@@ -422,6 +426,7 @@ __device__ void z_huffman_tree(ZBlock& S, const uint8_t* p, uint32_t len) {
     S.huf[i] = static_cast<uint16_t>(((mb + 1 - w) << 8) | sym);
   }
   __syncthreads();
+  return ZE_OK;
 }
 
 // ------------------------------------------------------------------ Huffman literals
@@ -469,8 +474,8 @@ __device__ __noinline__ int2 z_huf_count(const uint16_t* huf, int mb, const uint
 // scattered stores), every thread a share of a part.
 // A share is decoded in three pieces, so that a thread whose start moves need
 // only decode until it meets a piece's end that it had reached before.
-// Block-collective; errors in S.err.
-__device__ void z_huffman_literals(ZBlock& S, const ZHufStreams& hs, uint8_t* out) {
+// Returns 0 or an error.  Block-collective.
+__device__ int z_huffman_literals(ZBlock& S, const ZHufStreams& hs, uint8_t* out) {
   const int tid = threadIdx.x;
   const int per = ZT / hs.n, k = tid / per, i = tid % per;
   const int mb = S.huf_bits;
@@ -551,8 +556,7 @@ __device__ void z_huffman_literals(ZBlock& S, const ZHufStreams& hs, uint8_t* ou
     }
     const int32_t next = S.end[k * per + per - 1];  // where the part's codes end
     if (i == 0 && (total > want - written || (low == 0 && (next != 0 || written + total != want)))) S.err = ZE_STREAM;
-    __syncthreads();
-    if (S.err) return;
+    if (const int e = z_error(S)) return e;
     // bytes up to the first 4-byte boundary, words, bytes
     uint8_t* o = out + hs.out[k] + before;
     uint32_t skip = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(o) & 3), fill = skip, word = 0;
@@ -577,81 +581,75 @@ __device__ void z_huffman_literals(ZBlock& S, const ZHufStreams& hs, uint8_t* ou
     if (i == 0 && low > 0 && next <= 0 && (next != 0 || written != want)) S.err = ZE_STREAM;
     if (!__syncthreads_or(top > 0)) break;
   }
+  return z_error(S);
 }
 
 // ------------------------------------------------------------------ a compressed block
 
 // Compressed block src[0, len): its output from `out` on (frame output starts
 // at out0) into dst[0, dst_len).  The ring holds nothing below vfloor.
-// Returns the output position after it; errors in S.err.  Block-collective.
-__device__ __forceinline__ uint64_t z_block(ZBlock& S, const uint8_t* src, uint32_t len, uint8_t* dst, uint64_t out, uint64_t out0,
-                            uint64_t dst_len, uint32_t& vfloor) {
+// Moves out past the block's output; returns 0 or an error.  Block-collective.
+__device__ __forceinline__ int z_block(ZBlock& S, const uint8_t* src, uint32_t len, uint8_t* dst, uint64_t& out,
+                                       uint64_t out0, uint64_t dst_len, uint32_t& vfloor) {
   const int tid = threadIdx.x;
-  auto fail = [&](int e) {
-    if (tid == 0 && !S.err) S.err = e;
-    __syncthreads();
-    return out;
-  };
   // literals section
-  if (len == 0) return fail(ZE_LIT);
+  if (len == 0) return ZE_LIT;
   const uint32_t b0 = __ldg(src), type = b0 & 3, sf = (b0 >> 2) & 3;
   uint32_t hlen, regen, csize = 0;
   if (type < 2) {
     hlen = (sf & 1) == 0 ? 1 : (sf == 1 ? 2 : 3);
-    if (len < hlen) return fail(ZE_LIT);
+    if (len < hlen) return ZE_LIT;
     const uint32_t h = z_le(src, static_cast<int>(hlen));
     regen = hlen == 1 ? b0 >> 3 : h >> 4;
   } else {
     const uint32_t bits = sf < 2 ? 10 : sf == 2 ? 14 : 18;
     hlen = sf < 2 ? 3 : sf == 2 ? 4 : 5;
-    if (len < hlen) return fail(ZE_LIT);
+    if (len < hlen) return ZE_LIT;
     uint64_t h = 0;
     for (int i = static_cast<int>(hlen) - 1; i >= 0; --i) h = (h << 8) | __ldg(src + i);
     regen = static_cast<uint32_t>((h >> 4) & ((1u << bits) - 1));
     csize = static_cast<uint32_t>((h >> (4 + bits)) & ((1u << bits) - 1));
   }
-  if (regen > dst_len - out) return fail(ZE_SIZE);
+  if (regen > dst_len - out) return ZE_SIZE;
   const uint8_t* lit = dst + (dst_len - regen);  // Huffman literals: in the output's tail
   uint32_t lit_step = 1, used = hlen;
   bool lit_ro = false;
   if (type == 0) {
-    if (hlen + regen > len) return fail(ZE_LIT);
+    if (hlen + regen > len) return ZE_LIT;
     lit = src + hlen;
     lit_ro = true;
     used += regen;
   } else if (type == 1) {
-    if (hlen + 1 > len) return fail(ZE_LIT);
+    if (hlen + 1 > len) return ZE_LIT;
     lit = src + hlen;
     lit_step = 0;
     used += 1;
   } else {
-    if (hlen + csize > len) return fail(ZE_LIT);
+    if (hlen + csize > len) return ZE_LIT;
     const uint8_t* q = src + hlen;
     uint32_t qlen = csize;
     if (type == 2) {
-      z_huffman_tree(S, q, qlen);
-      if (S.err) return out;
+      if (const int e = z_huffman_tree(S, q, qlen)) return e;
       q += S.used;
       qlen -= S.used;
     } else if (S.huf_bits == 0) {
-      return fail(ZE_HUF);
+      return ZE_HUF;
     }
     ZHufStreams hs;
     const int e = z_huf_split(q, qlen, regen, sf == 0 ? 1 : 4, &hs);
-    if (e) return fail(e);
-    z_huffman_literals(S, hs, dst + (dst_len - regen));
-    if (S.err) return out;
+    if (e) return e;
+    if (const int e = z_huffman_literals(S, hs, dst + (dst_len - regen))) return e;
     used += csize;
   }
   // sequences section: header and tables
   const uint8_t* p = src + used;
   const uint32_t plen = len - used;
-  if (plen == 0) return fail(ZE_SEQ);
+  if (plen == 0) return ZE_SEQ;
   uint32_t nseq = __ldg(p), q = 1;
-  if (nseq == 0 && plen != 1) return fail(ZE_SEQ);
+  if (nseq == 0 && plen != 1) return ZE_SEQ;
   if (nseq >= 128) {
     const bool big = nseq == 255;
-    if (plen < (big ? 3u : 2u)) return fail(ZE_SEQ);
+    if (plen < (big ? 3u : 2u)) return ZE_SEQ;
     nseq = big ? __ldg(p + 1) + (static_cast<uint32_t>(__ldg(p + 2)) << 8) + 0x7F00 : ((nseq - 128) << 8) + __ldg(p + 1);
     q = big ? 3 : 2;
   }
@@ -691,8 +689,7 @@ __device__ __forceinline__ uint64_t z_block(ZBlock& S, const uint8_t* src, uint3
       S.used = at;
       S.err = e;
     }
-    __syncthreads();
-    if (S.err) return out;
+    if (const int e = z_error(S)) return e;
     const int w = tid >> 5;
     if (w < 3 && (S.mode[w] == 0 || S.mode[w] == 2)) {
       const int e = z_fse_table(S, w, 9, [&](int st, int s, int nb, uint32_t base) {
@@ -700,8 +697,7 @@ __device__ __forceinline__ uint64_t z_block(ZBlock& S, const uint8_t* src, uint3
       });
       if (e) S.err = e;
     }
-    __syncthreads();
-    if (S.err) return out;
+    if (const int e = z_error(S)) return e;
     if (tid == 0) {
       ZRead r{nullptr, 0};
       const uint32_t at = S.used;
@@ -715,8 +711,7 @@ __device__ __forceinline__ uint64_t z_block(ZBlock& S, const uint8_t* src, uint3
         S.pos = static_cast<uint32_t>(r.pos);
       }
     }
-    __syncthreads();
-    if (S.err) return out;
+    if (const int e = z_error(S)) return e;
   }
   const uint8_t* bs = p + (nseq ? S.used : 0u);  // the sequence bits
   const uint32_t va = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(dst) & 31);
@@ -784,8 +779,7 @@ __device__ __forceinline__ uint64_t z_block(ZBlock& S, const uint8_t* src, uint3
       S.err = e;
       S.bad = ZE_OK;
     }
-    __syncthreads();
-    if (S.err) return out;
+    if (const int e = z_error(S)) return e;
     // a sequence a thread: its values, and what it does to the last three offsets
     const int lane = tid & 31, warp = tid >> 5;
     uint32_t ll = 0, ml = 0, ov = 0;
@@ -872,7 +866,7 @@ __device__ __forceinline__ uint64_t z_block(ZBlock& S, const uint8_t* src, uint3
       if (e) atomicMax(&S.bad, e);
     }
     __syncthreads();
-    if (S.bad) return fail(S.bad);
+    if (const int e = S.bad) return e;
     if (lit_ro)
       lz_pairs<true>(S.lz, nb, vout, v, vfloor, ll, LZ_LIT | (lits + l_at), ml, off, lit_byte, plain);
     else
@@ -883,7 +877,8 @@ __device__ __forceinline__ uint64_t z_block(ZBlock& S, const uint8_t* src, uint3
   // the literals after the last sequence
   if (lit_ro) lz_one<true>(S.lz, vout, v, vfloor, LZ_LIT | lits, regen - lits, lit_byte, plain);
   else lz_one<false>(S.lz, vout, v, vfloor, LZ_LIT | lits, regen - lits, lit_byte, plain);
-  return v - va;
+  out = v - va;
+  return ZE_OK;
 }
 
 // Every frame of src[0, src_len) into dst[0, dst_len); returns 0 or an error.
@@ -958,8 +953,7 @@ __device__ __forceinline__ int z_frames(ZBlock& S, const uint8_t* src, uint32_t 
         __syncthreads();
       } else if (type == 2) {
         if (bsize > (128u << 10) || bsize > src_len - pos) return ZE_BLOCK;
-        out = z_block(S, src + pos, bsize, dst, out, out0, dst_len, vfloor);
-        if (S.err) return S.err;
+        if (const int e = z_block(S, src + pos, bsize, dst, out, out0, dst_len, vfloor)) return e;
         pos += bsize;
       } else {
         return ZE_BLOCK;
