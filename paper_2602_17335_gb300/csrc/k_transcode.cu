@@ -85,6 +85,12 @@ __device__ __forceinline__ void tc_fail(TcSmem& sm, uint32_t flag, int detail) {
   }
 }
 
+// Whether any thread has failed by now, the same answer for all threads.
+// Block-collective, with a barrier: the word is read on one side of it and
+// decided on by all threads at once (a warp that read it by itself could see a
+// later failure than the others and leave their next barriers to them).
+__device__ __forceinline__ bool tc_error(const TcSmem& sm) { return __syncthreads_or(sm.err) != 0; }
+
 // Moves the cursor's window to source offset `from` (block-collective, a
 // barrier on each side).  Reads up to 15 bytes on either side of the source.
 __device__ void tc_stage(const uint8_t* b, DCursor& c, uint32_t from) {
@@ -143,8 +149,8 @@ __device__ int tc_block(const DCursor& c, uint32_t q, uint32_t need, bool header
 
 // Parses the stream header at `p` and walks the block headers to the stream
 // end (after the last miniblock that holds values).  Records the result in
-// `c`; errors go to sm.  Block-collective.
-__device__ void dstream_open(const uint8_t* b, uint32_t p, uint32_t end, DCursor& c, TcSmem& sm) {
+// `c`; false, with the error in sm, when it is malformed.  Block-collective.
+__device__ bool dstream_open(const uint8_t* b, uint32_t p, uint32_t end, DCursor& c, TcSmem& sm) {
   if (threadIdx.x == 0) {
     auto get = [b](uint32_t i) { return ld_u8(b + i); };
     uint64_t v[4];
@@ -173,8 +179,7 @@ __device__ void dstream_open(const uint8_t* b, uint32_t p, uint32_t end, DCursor
       c.wn = 0;
     }
   }
-  __syncthreads();
-  if (sm.err) return;
+  if (tc_error(sm)) return false;
   while (c.left) {  // each window holds one header at least
     tc_stage(b, c, c.pos);
     if (threadIdx.x == 0) {
@@ -209,6 +214,7 @@ __device__ void dstream_open(const uint8_t* b, uint32_t p, uint32_t end, DCursor
     }
     __syncthreads();
   }
+  return !tc_error(sm);
 }
 
 __device__ __forceinline__ void dstream_rewind(DCursor& c) {
@@ -282,8 +288,7 @@ __device__ bool dstream_refill(const uint8_t* b, DCursor& c, TcSmem& sm) {
         tc_fail(sm, DERR_CORRUPT, 9);  // more values asked for than the stream holds
       }
     }
-    __syncthreads();
-    if (sm.err) return false;
+    if (tc_error(sm)) return false;
     if (!sm.more) break;
     tc_stage(b, c, c.pos);
   }
@@ -334,8 +339,7 @@ __device__ bool dstream_refill(const uint8_t* b, DCursor& c, TcSmem& sm) {
 // offsets from v0, into tab.  Returns the values, or -1 on an error.
 __device__ int64_t tc_dlba(const TranscodeJob& j, TcSmem& sm, uint32_t v0, uint64_t* tab) {
   DCursor& c = sm.c[0];
-  dstream_open(j.src, v0, j.src_len, c, sm);
-  if (sm.err) return -1;
+  if (!dstream_open(j.src, v0, j.src_len, c, sm)) return -1;
   const uint32_t M = c.total;
   const uint32_t cstart = c.pos;
   if (M > static_cast<uint32_t>(j.num_values) || (j.required && M != static_cast<uint32_t>(j.num_values))) {
@@ -359,7 +363,7 @@ __device__ int64_t tc_dlba(const TranscodeJob& j, TcSmem& sm, uint32_t v0, uint6
     }
     int64_t tot;
     int64_t at = C + block_exclusive_sum<int64_t>(mine, sm.tmp, &tot);
-    if (sm.err) return -1;
+    if (tc_error(sm)) return -1;
     if (C + tot > room) {
       if (threadIdx.x == 0) tc_fail(sm, DERR_CORRUPT, 22);
       return -1;
@@ -388,10 +392,8 @@ __device__ int64_t tc_dba(const TranscodeJob& j, TcSmem& sm, uint32_t v0, uint8_
   DCursor& cp = sm.c[0];
   DCursor& cs = sm.c[1];
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  dstream_open(j.src, v0, j.src_len, cp, sm);
-  if (sm.err) return -1;
-  dstream_open(j.src, cp.pos, j.src_len, cs, sm);
-  if (sm.err) return -1;
+  if (!dstream_open(j.src, v0, j.src_len, cp, sm)) return -1;
+  if (!dstream_open(j.src, cp.pos, j.src_len, cs, sm)) return -1;
   const uint32_t M = cp.total;
   const uint32_t cstart = cs.pos;
   if (cs.total != M || M > static_cast<uint32_t>(j.num_values) ||
@@ -438,7 +440,7 @@ __device__ int64_t tc_dba(const TranscodeJob& j, TcSmem& sm, uint32_t v0, uint8_
     int64_t totL, totS;
     block_exclusive_sum<int64_t>(sumL, sm.tmp, &totL);
     block_exclusive_sum<int64_t>(sumS, sm.tmp, &totS);
-    if (sm.err) return -1;
+    if (tc_error(sm)) return -1;
     if (S + totS > room) {
       if (t == 0) tc_fail(sm, DERR_CORRUPT, 32);
       return -1;
@@ -463,8 +465,7 @@ __device__ int64_t tc_dba(const TranscodeJob& j, TcSmem& sm, uint32_t v0, uint8_
       else sm.dst_off = off;
     }
   }
-  __syncthreads();
-  if (sm.err) return -1;
+  if (tc_error(sm)) return -1;
   // body: levels, the S suffix bytes, the values put together (offsets below
   // count from behind the levels)
   uint8_t* body = pool + sm.dst_off + v0;
@@ -566,9 +567,10 @@ __global__ void __launch_bounds__(TC_THREADS, 2) k_transcode(const TranscodeJob*
     sm.v0 = v0;
   }
   __syncthreads();
+  const bool failed = tc_error(sm);
   const uint32_t v0 = sm.v0;
   int64_t values = -1, bytes = -1;
-  if (!sm.err) {
+  if (!failed) {
     if (j.enc == ENC_DELTA_LBA) {
       values = tc_dlba(j, sm, v0, tab);
     } else if (j.enc == ENC_DELTA_BA) {
