@@ -1151,12 +1151,10 @@ pq_status plan_build(pq_ctx* ctx, pq_index* idx, const std::vector<int32_t>& col
         // pages with definition levels take the short items (their walks and
         // expands carry a bitmap per item; measured faster for PLAIN too)
         const uint32_t per = static_cast<uint32_t>(cd.max_def ? item_rows_opt : item_rows_max);
-        const uint32_t full = static_cast<uint32_t>(cd.max_def ? plan->tuning.item_rows_opt : plan->tuning.item_rows);
         const uint32_t n_it = span / per + (span % per ? 1 : 0);
         pp.item_rows = static_cast<int32_t>(per);
         pp.item_count = n_it;
         plan->n_items += n_it;
-        plan->budget_items += span / full + (span % full ? 1 : 0);
         plan->pps.push_back(pp);
       }
       const int32_t n_pp = static_cast<int32_t>(plan->pps.size()) - pp_first;
@@ -1480,9 +1478,7 @@ static pq_status plan_size_strings(pq_plan* plan) {
 }
 
 uint64_t plan_device_bytes(const pq_plan* plan, uint64_t scratch) {
-  // (items counted at the tuning's size: the smaller ones of small scans add
-  // less than the pool's rounding)
-  const uint64_t npp = plan->pps.size(), nit = plan->budget_items;
+  const uint64_t npp = plan->pps.size(), nit = plan->n_items;
   const uint64_t str_rows = static_cast<uint64_t>(plan->n_rows) * plan->str_cols.size();
   return npp * sizeof(pqi::PlanPage) + nit * sizeof(pqi::Item) + plan->outcols.size() * sizeof(pqi::OutCol) +
          (plan->snappy_data.size() + plan->snappy_dict.size()) * sizeof(pqi::SnappyJob) + 56ull * plan->snap_blocks +

@@ -128,7 +128,6 @@ struct pq_plan {
   std::vector<pqi::PlanPage> pps;
   uint64_t n_items = 0;                      // work items (built on the device)
   int32_t item_rows = 0;                     // rows per item of pages without definition levels
-  uint64_t budget_items = 0;                 // the same at the tuning's item sizes (plan_device_bytes)
   std::vector<pqi::OutCol> outcols;
   std::vector<pqi::SnappyJob> snappy_data;   // data pages
   std::vector<pqi::SnappyJob> snappy_dict;   // dictionary pages (into index buffers)

@@ -26,6 +26,8 @@ struct World {
   cudaStream_t main = nullptr;
   std::vector<cudaEvent_t> recorded;
   bool capturing = false;
+  uint64_t device_bytes = 0;        // asked of cudaMalloc, in
+  int mallocs = 0;                  // so many calls
 } W;
 
 uintptr_t handles = 0x1000;
@@ -56,7 +58,11 @@ cudaError_t cudaGetDeviceCount(int* n) { return *n = 1, cudaSuccess; }
 cudaError_t cudaSetDevice(int) { return cudaSuccess; }
 cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr, int) { return *v = W.n_sms, cudaSuccess; }
 cudaError_t cudaDeviceSynchronize() { return cudaSuccess; }
-cudaError_t cudaMalloc(void** p, size_t n) { return *p = calloc(n, 1), cudaSuccess; }
+cudaError_t cudaMalloc(void** p, size_t n) {
+  W.device_bytes += n;
+  ++W.mallocs;
+  return *p = calloc(n, 1), cudaSuccess;
+}
 cudaError_t cudaFree(void* p) { return free(p), cudaSuccess; }
 cudaError_t cudaHostAlloc(void** p, size_t n, unsigned) { return *p = calloc(n, 1), cudaSuccess; }
 cudaError_t cudaFreeHost(void* p) { return free(p), cudaSuccess; }
@@ -184,7 +190,11 @@ extern "C" int scan_with_fake_cuda(const uint8_t* file, uint64_t size, uint32_t 
   req.row_count = -1;
   pq_plan* plan = nullptr;
   std::vector<pq_out_size> sizes(static_cast<size_t>(idx->n_columns));
+  const uint64_t bytes_before = W.device_bytes;
+  const int mallocs_before = W.mallocs;
   if (pq_plan_scan(ctx, idx, &req, &plan, sizes.data()) != PQ_OK) return -1;
+  const uint64_t bytes = W.device_bytes - bytes_before;
+  const int mallocs = W.mallocs - mallocs_before;
   std::vector<pq_column> outs;
   std::vector<std::vector<uint8_t>> mem;
   const auto buffer = [&](uint64_t n) {
@@ -206,7 +216,8 @@ extern "C" int scan_with_fake_cuda(const uint8_t* file, uint64_t size, uint32_t 
   W.scanning = false;
   bool done = false;
   for (cudaEvent_t e : W.recorded) done |= e == plan->done;
-  std::string t = "done " + std::to_string(done) + "\nforks " + std::to_string(W.forks) + "\njoins " +
+  std::string t = "plan_bytes " + std::to_string(bytes) + "\nplan_mallocs " + std::to_string(mallocs) + "\nbudget " +
+                  std::to_string(plan->device_bytes) + "\ndone " + std::to_string(done) + "\nforks " + std::to_string(W.forks) + "\njoins " +
                   std::to_string(W.joins) + "\nlast_error " + std::to_string(static_cast<int>(W.last)) + "\nlaunches";
   for (const auto& l : W.log) t += " " + l;
   snprintf(text, cap, "%s", t.c_str());

@@ -89,3 +89,19 @@ def test_refused_launches_are_errors(scan, flags, n_sms, table):
         assert got["joins"] == good["joins"] and got["forks"] == good["forks"]
         assert got["last_error"] == "0"
         assert got["done"] == ("0" if flags == "GRAPH" else "1")  # (a graph that was not made has not run)
+
+
+def test_plan_budget_covers_its_memory(scan):
+    """What serving admits a request by is no less than what its plan takes (up to
+    the allocator's rounding, less than 64 KiB an allocation): twelve columns of
+    so few rows that they are cut into small work items."""
+    from paper_2602_17335_gb300.tables import write_table
+    from test_native_writer import _native
+    _native()
+    rows = 1_200_000
+    v = np.random.default_rng(1).integers(0, 1000, rows).astype(np.int32)
+    data = write_table(synth.Table([synth.ColumnData(f"x{k}", "INT32", v) for k in range(12)]),
+                       synth.TableSpec(rows, 1 << 20, [synth.ColumnSpec("RLE_DICTIONARY") for _ in range(12)])).tobytes()
+    st, got = scan(data)
+    assert st == N.PQ_OK
+    assert int(got["budget"]) >= int(got["plan_bytes"]) - 65536 * int(got["plan_mallocs"])
