@@ -102,6 +102,25 @@ template <typename Launch>
 inline void launch_slices(int n, Launch launch) {
   for (int at = 0; at < n; at += GRID_Y_MAX) launch(at, n - at < GRID_Y_MAX ? n - at : GRID_Y_MAX);
 }
+inline int n_slices(int n) { return (n + GRID_Y_MAX - 1) / GRID_Y_MAX; }
+
+// Kernels that the launchers below launch for the same arguments (the others
+// launch one each).
+inline int transcode_kernels(int n, int n_bss) {
+  return n <= 0 ? 0 : (n_bss > 0 ? n_slices(n) : 0) + (n_bss < n ? 1 : 0);
+}
+inline int dict_kernels(int n_jobs, bool fixed, int max_str_regions) {
+  return n_jobs <= 0 ? 0 : (fixed ? n_slices(n_jobs) : 0) + (max_str_regions > 0 ? 2 * n_slices(n_jobs) + 1 : 0);
+}
+inline int delta_kernels(int n, int max_regions) {
+  return n <= 0 ? 0 : (max_regions > 0 ? n_slices(n) + 1 : 0) + n_slices(n) + 1;
+}
+inline int strings_kernels(int n_items, bool copy_chars, bool left) {
+  return n_items <= 0 ? 0 : 1 + (copy_chars ? 1 + (left ? 1 : 0) : 0);
+}
+inline int snappy_scan_kernels(int n_jobs, uint32_t n_segs, bool long_first) {
+  return n_jobs <= 0 || n_segs == 0 ? 0 : 1 + (long_first ? 1 : 0);
+}
 
 // The transcode of jobs [0, n), n_bss of them BYTE_STREAM_SPLIT pages;
 // `counters` is the plan's item_counter array (its pool word); `pool` holds

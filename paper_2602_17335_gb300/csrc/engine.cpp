@@ -851,6 +851,8 @@ static void* plan_alloc_bytes(pq_plan* plan, size_t bytes) {
 }
 #define plan_alloc(T, plan, count) static_cast<T*>(plan_alloc_bytes(plan, std::max<size_t>(count, 1) * sizeof(T)))
 
+static int scan_kernels(const pq_plan* plan);
+
 }  // extern "C"
 
 namespace pqe {
@@ -1349,59 +1351,7 @@ pq_status plan_upload(pq_plan* plan, cudaStream_t s) {
   CK(ctx->events.take(&plan->fork));
   plan->join.assign(plan->outcols.size(), nullptr);
   for (auto& e : plan->join) CK(ctx->events.take(&e));
-  {
-    // kernels per scan: prepare, snappy, dictionary (2), walk + expand or one
-    // plain launch (+ its snappy) per chunk, strings (2)
-    int n = 1;
-    const bool any_dict = !plan->dict_jobs.empty();
-    if (plain) {
-      n += (plan->snappy_dict.empty() ? 0 : (plan->zstd_jobs ? 2 : 1)) + (any_dict ? 2 : 0);
-      size_t job = 0;
-      for (auto& cp : plan->chunk_pp) {
-        int nj = 0;
-        for (int q = cp.first; q < cp.first + cp.second; ++q)
-          if (job + nj < plan->snappy_data.size() && plan->snappy_data[job + nj].page == static_cast<int32_t>(plan->pps[q].page))
-            ++nj;
-        n += (nj ? (plan->zstd_jobs ? 2 : 1) : 0) + 1;
-        job += nj;
-      }
-      size_t tcj = 0;
-      for (auto& cp : plan->chunk_pp) {
-        int ntc = 0, nbss = 0;
-        while (tcj + ntc < plan->tc_jobs.size() &&
-               plan->tc_jobs[tcj + ntc].pp < static_cast<uint32_t>(cp.first + cp.second))
-          nbss += plan->tc_jobs[tcj + ntc++].enc == pqi::ENC_BSS;
-        n += (nbss ? 1 : 0) + (ntc > nbss ? 1 : 0);
-        tcj += ntc;
-      }
-    } else if (merged_scan(plan)) {
-      const int dk = plan->zstd_jobs ? 2 : 1;
-      int split[2] = {0, 0}, strs = 0, fixed = 0, bss = 0;
-      for (size_t oc = 0; oc < plan->colwork.size(); ++oc) {
-        const auto& cw = plan->colwork[oc];
-        split[0] |= cw.blk_data_n != 0;
-        split[1] |= cw.blk_dict_n != 0;
-        strs |= cw.max_str_regions > 0;
-        fixed |= cw.dict_n && plan->outcols[oc].ptype != pqi::T_BYTE_ARRAY;
-        bss += cw.tc_bss;
-      }
-      n += (plan->snappy_data.empty() ? 0 : dk + 3 * split[0]) + (plan->snappy_dict.empty() ? 0 : dk + 2 * split[1]) +
-           fixed + 3 * strs + (bss ? 1 : 0) + (static_cast<int>(plan->tc_jobs.size()) > bss ? 1 : 0) +
-           (plan->walk_pps.empty() ? 0 : 1) + (plan->delta_pps.empty() ? 0 : 4) + (nit ? 1 : 0);
-    } else {
-      for (size_t oc = 0; oc < plan->colwork.size(); ++oc) {
-        const auto& cw = plan->colwork[oc];
-        const int dk = plan->zstd_jobs ? 2 : 1;  // decompression kernels per job list
-        // (+2 per job list with split pages: the element scan and the fragments)
-        n += (cw.snap_dict_n ? dk + (cw.blk_dict_n ? 2 : 0) : 0) + (cw.dict_n ? 2 : 0) +
-             (cw.snap_data_n ? dk + (cw.blk_data_n ? 3 : 0) : 0) + (cw.walk_n ? 1 : 0) +
-             (cw.delta_n ? 4 : 0) + (cw.tc_bss ? 1 : 0) + (cw.tc_n > cw.tc_bss ? 1 : 0) + (plan->outcols[oc].item_count ? 1 : 0);
-      }
-    }
-    for (int32_t sc : plan->str_cols)
-      n += plan->outcols[sc].item_count ? (plan->colwork[sc].dict_pages ? 3 : 2) : 0;
-    plan->launches = n;
-  }
+  plan->launches = scan_kernels(plan);
   const int wbps = pqi::walk_blocks_per_sm(), ebps = pqi::expand_blocks_per_sm();
   plan->walk_grid =
       static_cast<int>(std::min<size_t>(std::max<size_t>(plan->walk_pps.size(), 1), size_t(ctx->n_sms) * wbps));
@@ -1721,19 +1671,28 @@ static void enqueue_strings(pq_plan* plan, const pqi::DecodeArgs& a, cudaStream_
                           strings_left(plan, sc), s);
 }
 
+// What the stages of all columns are launched with.
+struct AllColumns {
+  int max_regions, n_bss;
+  bool fixed, levels;
+};
+static AllColumns all_columns(const pq_plan* plan) {
+  AllColumns r{};
+  for (size_t oc = 0; oc < plan->colwork.size(); ++oc) {
+    const auto& cw = plan->colwork[oc];
+    r.max_regions = std::max(r.max_regions, cw.max_regions);
+    r.n_bss += cw.tc_bss;
+    r.fixed |= cw.dict_n && plan->outcols[oc].ptype != pqi::T_BYTE_ARRAY;
+    r.levels |= plan->outcols[oc].optional != 0;
+  }
+  return r;
+}
+
 // The stages of all output columns, each launched once: dictionaries beside
 // the walks of the data pages on a branch stream, then expansion and strings.
 static void enqueue_merged(pq_plan* plan, const pqi::DecodeArgs& a, bool with_dicts, cudaStream_t side, cudaStream_t s) {
   pq_ctx* ctx = plan->ctx;
-  int max_regions = 0, n_bss = 0;
-  bool fixed = false, levels = false;
-  for (size_t oc = 0; oc < plan->colwork.size(); ++oc) {
-    const auto& cw = plan->colwork[oc];
-    max_regions = std::max(max_regions, cw.max_regions);
-    n_bss += cw.tc_bss;
-    fixed |= cw.dict_n && plan->outcols[oc].ptype != pqi::T_BYTE_ARRAY;
-    levels |= plan->outcols[oc].optional != 0;
-  }
+  const auto [max_regions, n_bss, fixed, levels] = all_columns(plan);
   const bool dicts = with_dicts && !plan->dict_jobs.empty();
   if (dicts) {
     cudaEventRecord(plan->fork, s);
@@ -1755,6 +1714,50 @@ static void enqueue_merged(pq_plan* plan, const pqi::DecodeArgs& a, bool with_di
     pqi::launch_expand(a, 0, static_cast<int>(plan->n_items), 0, !plan->delta_pps.empty(), ctx->n_sms,
                        plan->tuning.expand_ctas_per_sm, s);
   enqueue_strings(plan, a, s);
+}
+
+static int range_kernels(const pq_plan* plan, const SnapRange& r) {
+  if (r.n <= 0) return 0;
+  return (r.nblk ? pqi::snappy_scan_kernels(r.n, r.nseg, !r.dicts) + 1 : 0) + 1 + (plan->zstd_jobs ? 1 : 0);
+}
+
+// Kernels that enqueue_scan launches (dictionaries included).
+static int scan_kernels(const pq_plan* plan) {
+  int n = 2 + static_cast<int>(plan->str_cols.size());  // prepare, the status word and string totals to the host
+  for (int32_t sc : plan->str_cols)
+    n += pqi::strings_kernels(static_cast<int>(plan->outcols[sc].item_count), true, plan->colwork[sc].dict_pages > 0);
+  if (plan->flags & PQ_SCAN_PLAIN) {
+    const int dk = plan->zstd_jobs ? 2 : 1;  // decompression kernels of a job list
+    n += (plan->snappy_dict.empty() ? 0 : dk) +
+         pqi::dict_kernels(static_cast<int>(plan->dict_jobs.size()), true, max_str_regions_all(plan));
+    size_t job = 0, tcj = 0;
+    for (const auto& cp : plan->chunk_pp) {
+      int nj = 0, ntc = 0, nbss = 0;
+      for (int q = cp.first; q < cp.first + cp.second; ++q)
+        if (job + nj < plan->snappy_data.size() && plan->snappy_data[job + nj].page == static_cast<int32_t>(plan->pps[q].page))
+          ++nj;
+      job += nj;
+      while (tcj + ntc < plan->tc_jobs.size() && plan->tc_jobs[tcj + ntc].pp < static_cast<uint32_t>(cp.first + cp.second))
+        nbss += plan->tc_jobs[tcj + ntc++].enc == pqi::ENC_BSS;
+      tcj += ntc;
+      n += (nj ? dk : 0) + pqi::transcode_kernels(ntc, nbss) + 1;
+    }
+  } else if (merged_scan(plan)) {
+    const auto [max_regions, n_bss, fixed, levels] = all_columns(plan);
+    n += range_kernels(plan, plan_range(plan, true)) + range_kernels(plan, plan_range(plan, false)) +
+         pqi::dict_kernels(static_cast<int>(plan->dict_jobs.size()), fixed, max_str_regions_all(plan)) +
+         pqi::transcode_kernels(static_cast<int>(plan->tc_jobs.size()), n_bss) + (plan->walk_pps.empty() ? 0 : 1) +
+         pqi::delta_kernels(static_cast<int>(plan->delta_pps.size()), max_regions) + (plan->n_items ? 1 : 0);
+  } else {
+    for (size_t oc = 0; oc < plan->colwork.size(); ++oc) {
+      const auto& cw = plan->colwork[oc];
+      n += range_kernels(plan, column_range(plan, oc, true)) + range_kernels(plan, column_range(plan, oc, false)) +
+           pqi::dict_kernels(cw.dict_n, plan->outcols[oc].ptype != pqi::T_BYTE_ARRAY, cw.max_str_regions) +
+           pqi::transcode_kernels(cw.tc_n, cw.tc_bss) + (cw.walk_n ? 1 : 0) +
+           pqi::delta_kernels(cw.delta_n, cw.max_regions) + (plan->outcols[oc].item_count ? 1 : 0);
+    }
+  }
+  return n;
 }
 
 // Enqueues the kernels of one scan (no host synchronisation).  Default:

@@ -28,6 +28,7 @@ struct World {
   bool capturing = false;
   uint64_t device_bytes = 0;        // asked of cudaMalloc, in
   int mallocs = 0;                  // so many calls
+  int kernels = 0;                  // of the scan's launches
 } W;
 
 uintptr_t handles = 0x1000;
@@ -36,8 +37,9 @@ T handle() {
   return reinterpret_cast<T>(handles += 16);
 }
 
-bool launch(const char* name) {
+bool launch(const char* name, int kernels = 1) {
   if (!W.scanning) return true;
+  W.kernels += kernels;
   const bool fails = static_cast<int>(W.log.size()) == W.fail_at;
   W.log.push_back(name);
   if (fails) W.last = cudaErrorInvalidConfiguration;
@@ -106,18 +108,19 @@ cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t) { return W.recorded.pus
 }
 
 namespace pqi {
-void launch_transcode(const TranscodeJob*, int n, int, PlanPage*, uint8_t*, uint64_t, uint32_t*, uint64_t*, DevStatus*,
+void launch_transcode(const TranscodeJob*, int n, int n_bss, PlanPage*, uint8_t*, uint64_t, uint32_t*, uint64_t*, DevStatus*,
                       cudaStream_t) {
-  if (n > 0) launch("transcode");
+  if (n > 0) launch("transcode", transcode_kernels(n, n_bss));
 }
-void launch_dict(const DictJob*, int, bool, int, int, DictScratch, DictDev*, int, DevStatus*, cudaStream_t) {
-  launch("dict");
+void launch_dict(const DictJob*, int n, bool fixed, int, int regions, DictScratch, DictDev*, int, DevStatus*,
+                 cudaStream_t) {
+  launch("dict", dict_kernels(n, fixed, regions));
 }
 void launch_walk(const DecodeArgs&, int, int n, int, bool, uint32_t, cudaStream_t) {
   if (n > 0) launch("walk");
 }
-void launch_delta_bases(const DecodeArgs&, int, int n, int, cudaStream_t) {
-  if (n > 0) launch("delta");
+void launch_delta_bases(const DecodeArgs&, int, int n, int regions, cudaStream_t) {
+  if (n > 0) launch("delta", delta_kernels(n, regions));
 }
 void launch_expand(const DecodeArgs&, int, int n, int, bool, int, int, cudaStream_t) {
   if (n > 0) launch("expand");
@@ -128,7 +131,9 @@ void launch_dict_expand(const DecodeArgs&, int, int, int, int, int, uint32_t, ui
   launch("dict_expand");
 }
 void launch_copy_items(const DecodeArgs&, int, int, int, int, int, cudaStream_t) { launch("copy"); }
-void launch_strings(const DecodeArgs&, int, int, int, bool, uint32_t*, cudaStream_t) { launch("strings"); }
+void launch_strings(const DecodeArgs&, int, int n, int, bool copy, uint32_t* left, cudaStream_t) {
+  if (n > 0) launch("strings", strings_kernels(n, copy, left != nullptr));
+}
 void launch_plain_pages(const DecodeArgs&, int, int, cudaStream_t) { launch("plain"); }
 void launch_prepare(const DecodeArgs& a, int, int, cudaStream_t) {
   if (launch("prepare")) *a.st = DevStatus{0, -1, 0, 0};
@@ -140,9 +145,9 @@ void launch_make_items(const DecodeArgs&, int, cudaStream_t) {}
 int expand_blocks_per_sm() { return 4; }
 int walk_blocks_per_sm() { return 4; }
 void launch_snappy(const SnappyJob*, int, int, DevStatus*, cudaStream_t, bool) { launch("snappy"); }
-void launch_snappy_scan(const SnappyJob*, int, uint32_t, uint32_t, SnapState, uint32_t*, bool, int, DevStatus*,
-                        cudaStream_t) {
-  launch("snappy_scan");
+void launch_snappy_scan(const SnappyJob*, int n, uint32_t, uint32_t segs, SnapState, uint32_t*, bool long_first, int,
+                        DevStatus*, cudaStream_t) {
+  launch("snappy_scan", snappy_scan_kernels(n, segs, long_first));
 }
 void launch_snappy_fragments(const SnappyJob*, int, int, SnapState, int, DevStatus*, cudaStream_t) {
   launch("snappy_fragments");
@@ -217,7 +222,7 @@ extern "C" int scan_with_fake_cuda(const uint8_t* file, uint64_t size, uint32_t 
   bool done = false;
   for (cudaEvent_t e : W.recorded) done |= e == plan->done;
   std::string t = "plan_bytes " + std::to_string(bytes) + "\nplan_mallocs " + std::to_string(mallocs) + "\nbudget " +
-                  std::to_string(plan->device_bytes) + "\ndone " + std::to_string(done) + "\nforks " + std::to_string(W.forks) + "\njoins " +
+                  std::to_string(plan->device_bytes) + "\nplanned_kernels " + std::to_string(plan->launches) + "\nkernels " + std::to_string(W.kernels) + "\ndone " + std::to_string(done) + "\nforks " + std::to_string(W.forks) + "\njoins " +
                   std::to_string(W.joins) + "\nlast_error " + std::to_string(static_cast<int>(W.last)) + "\nlaunches";
   for (const auto& l : W.log) t += " " + l;
   snprintf(text, cap, "%s", t.c_str());

@@ -80,6 +80,8 @@ def test_refused_launches_are_errors(scan, flags, n_sms, table):
     assert st == N.PQ_OK and good["done"] == "1" and good["last_error"] == "0"
     kernels = [k for k in good["launches"].split() if k != "graph"]
     assert "prepare" == kernels[0] and "copy_small" == kernels[-1]
+    # (the count of kernels that a plan tells is the one that a scan launches)
+    assert int(good["planned_kernels"]) == int(good["kernels"]) >= len(kernels)
     if table == "split" and flags != "PLAIN":
         assert "snappy_fragments" in kernels
     for k in range(len(kernels)):
