@@ -119,6 +119,7 @@ pq_status pq_batch_launch(pq_batch* b, void* stream) {
     for (pq_plan* p : b->plans) {
       e = cudaEventRecord(p->done, s);
       if (e != cudaSuccess) return cuda_fail(ctx, e, "plan done event");
+      p->scanned = true;
     }
   } else {
     const pq_status st = enqueue_batch(b, s);

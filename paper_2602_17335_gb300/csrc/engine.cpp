@@ -829,7 +829,7 @@ void pq_free_plan(pq_plan* plan) {
   cudaSetDevice(plan->ctx->device);
   // once `done` (recorded after the scan's last work) and `ready` have
   // completed, so have the fork and join records: all go back to the cache
-  if (plan->done) cudaEventSynchronize(plan->done);
+  if (plan->scanned) cudaEventSynchronize(plan->done);
   if (plan->ready) cudaEventSynchronize(plan->ready);
   if (plan->graph) cudaGraphExecDestroy(plan->graph);
   for (auto& e : plan->stage_ev)
@@ -1896,11 +1896,10 @@ pq_status scan_enqueue(pq_plan* plan, const pq_column* outs, cudaStream_t s, con
   // the plan's uploads (legacy stream) come before anything of the scan.  A
   // captured stream may not wait on an event recorded outside the capture:
   // callers that capture wait for `ready` before the capture begins.
-  if (plan->ready) {
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    CK(cudaStreamIsCapturing(s, &cap));
-    if (cap == cudaStreamCaptureStatusNone) CK(cudaStreamWaitEvent(s, plan->ready, 0));
-  }
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  CK(cudaStreamIsCapturing(s, &cap));
+  const bool capturing = cap != cudaStreamCaptureStatusNone;
+  if (plan->ready && !capturing) CK(cudaStreamWaitEvent(s, plan->ready, 0));
   memcpy(plan->h_cols.p, plan->outcols.data(), sizeof(pqi::OutCol) * plan->outcols.size());
   if (!plan->outcols.empty())
     CK(cudaMemcpyAsync(plan->d_cols, plan->h_cols.p, sizeof(pqi::OutCol) * plan->outcols.size(),
@@ -1947,12 +1946,13 @@ pq_status scan_enqueue(pq_plan* plan, const pq_column* outs, cudaStream_t s, con
     const cudaError_t launch = enqueue_scan(plan, s, with_dicts, branches, n_branches);
     if (launch != cudaSuccess) {
       // (what was launched before uses the plan's memory until `done`)
-      cudaEventRecord(plan->done, s);
+      if (cudaEventRecord(plan->done, s) == cudaSuccess && !capturing) plan->scanned = true;
       return cuda_fail(ctx, launch, "kernel launch");
     }
   }
   CK(cudaGetLastError());
   CK(cudaEventRecord(plan->done, s));
+  if (!capturing) plan->scanned = true;
   if (plan->flags & PQ_SCAN_RESIDENT_DICT)
     for (int32_t ch : plan->dict_chunks) plan->idx->dict_resident[ch] = 1;
   return PQ_OK;
@@ -1973,7 +1973,7 @@ pq_status pq_scan_wait(pq_ctx* ctx, pq_plan* plan, void* stream, uint64_t* chars
   if (!ctx || !plan) return fail(ctx, PQ_ERR_INVALID_ARG, "pq_scan_wait");
   (void)stream;
   CK(cudaSetDevice(ctx->device));
-  CK(cudaEventSynchronize(plan->done));
+  if (plan->scanned) CK(cudaEventSynchronize(plan->done));
   pqi::DevStatus st;
   memcpy(&st, plan->h_out.p, sizeof st);
   if (chars_bytes) {

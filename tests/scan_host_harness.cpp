@@ -7,6 +7,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <set>
 #include <string>
 #include <vector>
 
@@ -25,6 +26,7 @@ struct World {
   int forks = 0, joins = 0;         // waits of other streams for the scan's, and back
   cudaStream_t main = nullptr;
   std::vector<cudaEvent_t> recorded;
+  std::set<cudaEvent_t> captured;   // of them, those last recorded inside a capture
   bool capturing = false;
   uint64_t device_bytes = 0;        // asked of cudaMalloc, in
   int mallocs = 0;                  // so many calls
@@ -102,9 +104,16 @@ cudaError_t cudaGraphLaunch(cudaGraphExec_t, cudaStream_t) {
 cudaError_t cudaEventCreate(cudaEvent_t* e) { return *e = handle<cudaEvent_t>(), cudaSuccess; }
 cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned) { return *e = handle<cudaEvent_t>(), cudaSuccess; }
 cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
-cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
+cudaError_t cudaEventSynchronize(cudaEvent_t e) {  // (refused for an event last recorded inside a capture)
+  return W.captured.count(e) ? W.last = cudaErrorInvalidValue : cudaSuccess;
+}
 cudaError_t cudaEventElapsedTime(float* ms, cudaEvent_t, cudaEvent_t) { return *ms = 0, cudaSuccess; }
-cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t) { return W.recorded.push_back(e), cudaSuccess; }
+cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t) {
+  W.recorded.push_back(e);
+  if (W.capturing) W.captured.insert(e);
+  else W.captured.erase(e);
+  return cudaSuccess;
+}
 }
 
 namespace pqi {
@@ -225,8 +234,14 @@ extern "C" int scan_with_fake_cuda(const uint8_t* file, uint64_t size, uint32_t 
                   std::to_string(plan->device_bytes) + "\nplanned_kernels " + std::to_string(plan->launches) + "\nkernels " + std::to_string(W.kernels) + "\ndone " + std::to_string(done) + "\nforks " + std::to_string(W.forks) + "\njoins " +
                   std::to_string(W.joins) + "\nlast_error " + std::to_string(static_cast<int>(W.last)) + "\nlaunches";
   for (const auto& l : W.log) t += " " + l;
-  snprintf(text, cap, "%s", t.c_str());
   pq_free_plan(plan);
+  // another plan, with the first one's events, that is never scanned
+  W.last = cudaSuccess;
+  pq_plan* unscanned = nullptr;
+  if (pq_plan_scan(ctx, idx, &req, &unscanned, sizes.data()) != PQ_OK) return -1;
+  pq_free_plan(unscanned);
+  t += "\nlast_error_unscanned " + std::to_string(static_cast<int>(W.last));
+  snprintf(text, cap, "%s", t.c_str());
   pq_free_index(idx);
   pq_ctx_destroy(ctx);
   return st;

@@ -107,3 +107,12 @@ def test_plan_budget_covers_its_memory(scan):
     st, got = scan(data)
     assert st == N.PQ_OK
     assert int(got["budget"]) >= int(got["plan_bytes"]) - 65536 * int(got["plan_mallocs"])
+
+
+@pytest.mark.parametrize("flags", ["BATCHED", "GRAPH"])
+@pytest.mark.parametrize("n_sms", [1, 152])
+def test_unscanned_plan_after_a_graph(scan, flags, n_sms):
+    """A plan that is freed without a scan waits for none of the events it was
+    given, which an earlier plan may have recorded inside its graph."""
+    st, got = scan(_eight("UNCOMPRESSED"), getattr(N, "PQ_SCAN_" + flags), n_sms)
+    assert st == N.PQ_OK and got["last_error_unscanned"] == "0"
