@@ -155,6 +155,7 @@ EventPool::~EventPool() {
 
 pq_status fail(pq_ctx* ctx, pq_status s, const std::string& msg) {
   if (ctx) ctx->last_error = msg;
+  if (s == PQ_ERR_CUDA) cudaGetLastError();  // reported here: the next call is not to report it again
   return s;
 }
 

@@ -20,7 +20,7 @@ namespace {
 struct World {
   cudaError_t last = cudaSuccess;
   int n_sms = 152;
-  int fail_at = -1;                 // the launch that fails, counted from the scan on
+  int fail_at = -1;                 // the launch that fails, counted from the scan on (-2: its copies)
   bool scanning = false;
   std::vector<std::string> log;     // the scan's launches, the failing one among them
   int forks = 0, joins = 0;         // waits of other streams for the scan's, and back
@@ -73,6 +73,7 @@ cudaError_t cudaFreeHost(void* p) { return free(p), cudaSuccess; }
 cudaError_t cudaHostGetDevicePointer(void** d, void* h, unsigned) { return *d = h, cudaSuccess; }
 cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) { return memmove(d, s, n), cudaSuccess; }
 cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t) {
+  if (W.scanning && W.fail_at == -2) return W.last = cudaErrorInvalidValue;
   return memmove(d, s, n), cudaSuccess;
 }
 cudaError_t cudaMemsetAsync(void* d, int v, size_t n, cudaStream_t) { return memset(d, v, n), cudaSuccess; }
@@ -168,7 +169,7 @@ void launch_index_oi(const ChunkDev*, int, const int64_t*, PageDev*, int, DevSta
 }  // namespace pqi
 
 // Plans and scans all columns of the file on a GPU of n_sms multiprocessors,
-// with launch `fail_at` of the scan failing (-1: none).  Returns the scan's
+// with launch `fail_at` of the scan failing (-1: none, -2: its copies to the GPU).  Returns the scan's
 // status, -1 when it did not get that far; `text` gets what there is to see.
 extern "C" int scan_with_fake_cuda(const uint8_t* file, uint64_t size, uint32_t flags, int n_sms, int fail_at, char* text,
                                    uint64_t cap) {

@@ -38,7 +38,7 @@ def scan(tmp_path_factory):
     def run(data, flags=0, n_sms=152, fail_at=-1):
         text = ctypes.create_string_buffer(1 << 16)
         st = lib.scan_with_fake_cuda(data, len(data), flags, n_sms, fail_at, text, len(text))
-        return st, dict(line.split(" ", 1) for line in text.value.decode().splitlines())
+        return st, {k: v for k, _, v in (line.partition(" ") for line in text.value.decode().splitlines())}
     return run
 
 
@@ -116,3 +116,8 @@ def test_unscanned_plan_after_a_graph(scan, flags, n_sms):
     given, which an earlier plan may have recorded inside its graph."""
     st, got = scan(_eight("UNCOMPRESSED"), getattr(N, "PQ_SCAN_" + flags), n_sms)
     assert st == N.PQ_OK and got["last_error_unscanned"] == "0"
+
+
+def test_a_reported_error_is_not_reported_again(scan):
+    st, got = scan(_eight("UNCOMPRESSED"), fail_at=-2)
+    assert st == N.PQ_ERR_CUDA and got["last_error"] == "0" and got["launches"] == ""
