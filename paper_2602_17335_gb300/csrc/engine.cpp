@@ -1034,8 +1034,8 @@ pq_status plan_build(pq_ctx* ctx, pq_index* idx, const std::vector<int32_t>& col
         const int64_t p0 = c0 + pg.first_row;
         const int64_t p1 = p0 + pg.num_values;
         if (p1 <= rb || p0 >= re || pg.num_values == 0) continue;
-        // BYTE_STREAM_SPLIT and the delta string encodings are rewritten into
-        // PLAIN bodies first; the decode kernels then read them as PLAIN
+        // the decode kernels read BYTE_STREAM_SPLIT pages as the PLAIN bodies and
+        // delta string pages by the entry tables that k_transcode.cu makes first
         const int32_t enc = pg.encoding;
         const bool tc = enc == pqi::ENC_BSS || enc == pqi::ENC_DELTA_LBA || enc == pqi::ENC_DELTA_BA;
         if (tc && (enc == pqi::ENC_BSS) == (cd.ptype == pqi::T_BYTE_ARRAY))

@@ -15,8 +15,8 @@
 // from host memory (host_page_walk): the device indexes nothing and reads
 // nothing back, so no row group waits for SMs held by an earlier one's
 // scan or for a page-table readback queued behind the copy-out.  Files
-// with compressed pages of 512 KiB or more take the whole-file path (their
-// scans are latency-bound; see scan_pipelined).
+// with compressed pages of 512 KiB or more take the whole-file path (see
+// scan_pipelined).
 #include <stdlib.h>
 #include <string.h>
 
@@ -161,10 +161,12 @@ pq_status scan_pipelined(pq_ctx* ctx, const pq_file* host_files, int n_files, co
   }
   if (units.size() < 2) return PQ_ERR_UNSUPPORTED;
   {
-    // Compressed pages of kLongPage or more: one row group's scan then takes
-    // as long as its longest page's element chain (about 17 ms at 1 MiB
-    // Snappy pages), which the pipeline would pay per row group and the
-    // whole-file path pays once; the first row group's pages decide.
+    // Compressed pages of kLongPage or more take the whole-file path; the first
+    // row group's pages decide.  The line was drawn when a row group of 1 MiB
+    // Snappy pages took as long as its longest page's element chain, 17 ms, which
+    // the pipeline paid per row group (98 ms against 52 for 2^26 rows of eight
+    // columns).  Since pages are decompressed by fragments the whole-file path
+    // takes 40.9 ms there, and the pipeline, with the rule off, 30.8.
     constexpr int32_t kLongPage = 512 * 1024;
     const Unit& u = units[0];
     const uint8_t* hb = static_cast<const uint8_t*>(host_files[u.file].data);

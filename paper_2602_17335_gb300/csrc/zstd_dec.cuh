@@ -1,7 +1,10 @@
-// Zstandard frame decoding core (the codec the paper's Section 2 lists
-// beside Snappy for Parquet column chunks), written as host/device
-// functions over plain pointers so that the same code runs in a kernel and
-// in a host test harness.
+// Zstandard frame decoding (the codec the paper's Section 2 lists beside
+// Snappy for Parquet column chunks) on one thread, as host/device functions
+// over plain pointers.  The kernel (k_zstd.cu) divides a page among a thread
+// block and takes from here the format's constants and header arithmetic:
+// error codes, z_le, z_hb, z_huf_split, z_default_norm, z_ll and z_ml.
+// zstd_decode and what it alone calls (z_literals, z_sequences and the readers
+// below them) run in host tests, as a second decoder beside the oracle.
 //
 // Format steps, in order: frame header (magic 0xFD2FB528; descriptor with
 // content-size, single-segment, checksum and dictionary flags; window
