@@ -1335,6 +1335,7 @@ pq_status plan_upload(pq_plan* plan, cudaStream_t s) {
     up_off += (u.bytes + 15) & ~size_t(15);
   }
   if (nit) {
+    cudaGetLastError();  // (an earlier call's)
     pqi::launch_make_items(decode_args(plan), static_cast<int>(npp), s);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
@@ -1868,6 +1869,7 @@ namespace pqe {
 pq_status scan_enqueue(pq_plan* plan, const pq_column* outs, cudaStream_t s, const cudaStream_t* branches,
                        int n_branches, bool allow_graph) {
   pq_ctx* ctx = plan->ctx;
+  cudaGetLastError();  // (what an earlier call left is not this scan's)
   // output descriptors
   bool changed = false;
   for (size_t i = 0; i < plan->outcols.size(); ++i) {

@@ -169,10 +169,11 @@ void launch_index_oi(const ChunkDev*, int, const int64_t*, PageDev*, int, DevSta
 }  // namespace pqi
 
 // Plans and scans all columns of the file on a GPU of n_sms multiprocessors,
-// with launch `fail_at` of the scan failing (-1: none, -2: its copies to the GPU).  Returns the scan's
+// with launch `fail_at` of the scan failing (-1: none, -2: its copies to the GPU),
+// on a thread whose last error is stale_error.  Returns the scan's
 // status, -1 when it did not get that far; `text` gets what there is to see.
-extern "C" int scan_with_fake_cuda(const uint8_t* file, uint64_t size, uint32_t flags, int n_sms, int fail_at, char* text,
-                                   uint64_t cap) {
+extern "C" int scan_with_fake_cuda(const uint8_t* file, uint64_t size, uint32_t flags, int n_sms, int fail_at,
+                                   int stale_error, char* text, uint64_t cap) {
   W = World{};
   W.n_sms = n_sms;
   W.fail_at = fail_at;
@@ -205,6 +206,7 @@ extern "C" int scan_with_fake_cuda(const uint8_t* file, uint64_t size, uint32_t 
   req.row_count = -1;
   pq_plan* plan = nullptr;
   std::vector<pq_out_size> sizes(static_cast<size_t>(idx->n_columns));
+  W.last = static_cast<cudaError_t>(stale_error);
   const uint64_t bytes_before = W.device_bytes;
   const int mallocs_before = W.mallocs;
   if (pq_plan_scan(ctx, idx, &req, &plan, sizes.data()) != PQ_OK) return -1;
@@ -227,6 +229,7 @@ extern "C" int scan_with_fake_cuda(const uint8_t* file, uint64_t size, uint32_t 
   W.main = handle<cudaStream_t>();
   W.scanning = true;
   W.recorded.clear();
+  W.last = static_cast<cudaError_t>(stale_error);
   const pq_status st = pqe::scan_enqueue(plan, outs.data(), W.main, ctx->branch, pq_ctx::kBranches, true);
   W.scanning = false;
   bool done = false;

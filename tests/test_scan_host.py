@@ -33,11 +33,11 @@ def scan(tmp_path_factory):
                    check=True)
     lib = ctypes.CDLL(out)
     lib.scan_with_fake_cuda.argtypes = [ctypes.c_char_p, ctypes.c_uint64, ctypes.c_uint32, ctypes.c_int, ctypes.c_int,
-                                        ctypes.c_char_p, ctypes.c_uint64]
+                                        ctypes.c_int, ctypes.c_char_p, ctypes.c_uint64]
 
-    def run(data, flags=0, n_sms=152, fail_at=-1):
+    def run(data, flags=0, n_sms=152, fail_at=-1, stale_error=0):
         text = ctypes.create_string_buffer(1 << 16)
-        st = lib.scan_with_fake_cuda(data, len(data), flags, n_sms, fail_at, text, len(text))
+        st = lib.scan_with_fake_cuda(data, len(data), flags, n_sms, fail_at, stale_error, text, len(text))
         return st, {k: v for k, _, v in (line.partition(" ") for line in text.value.decode().splitlines())}
     return run
 
@@ -116,6 +116,12 @@ def test_unscanned_plan_after_a_graph(scan, flags, n_sms):
     given, which an earlier plan may have recorded inside its graph."""
     st, got = scan(_eight("UNCOMPRESSED"), getattr(N, "PQ_SCAN_" + flags), n_sms)
     assert st == N.PQ_OK and got["last_error_unscanned"] == "0"
+
+
+@pytest.mark.parametrize("flags", ["BATCHED", "GRAPH"])
+def test_an_earlier_error_is_not_the_scans(scan, flags):
+    st, got = scan(_eight("UNCOMPRESSED"), getattr(N, "PQ_SCAN_" + flags), stale_error=1)
+    assert st == N.PQ_OK and got["kernels"] == got["planned_kernels"]
 
 
 def test_a_reported_error_is_not_reported_again(scan):
