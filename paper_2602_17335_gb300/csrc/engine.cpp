@@ -883,11 +883,15 @@ static void plan_split(pqi::SnappyJob& sj, bool plain, uint32_t* frags, uint32_t
 // Rows per work item: the tuning's, halved down to `least` while a column of
 // n_rows rows has fewer items than the GPU has expansion warps (32 a
 // multiprocessor).  2^20 dictionary rows in 512 items of 2048 occupied 16
-// thread blocks.
-static int64_t plan_item_rows(int64_t rows, int64_t least, int64_t n_rows, int n_sms) {
-  while (rows / 2 >= least && n_rows / rows < 32 * static_cast<int64_t>(n_sms)) rows = rows / 2 / 32 * 32;
+// thread blocks.  With a block per page (PQ_SCAN_PLAIN) the same holds for the
+// block's 8 warps and a page's rows, at two items a warp: smaller items than
+// that only cost their overhead (two pages of 2^19 rows 0.80 ms, all cut into
+// items of 256 1.26).
+static int64_t plan_item_rows(int64_t rows, int64_t least, int64_t n_rows, int64_t items) {
+  while (rows / 2 >= least && n_rows / rows < items) rows = rows / 2 / 32 * 32;
   return rows;
 }
+constexpr int64_t ITEM_ROWS_LEAST = 256, ITEM_ROWS_OPT_LEAST = 128, PLAIN_PAGE_ITEMS = 16;
 
 pq_status plan_build(pq_ctx* ctx, pq_index* idx, const std::vector<int32_t>& cols, const std::vector<RowSeg>& segs,
                      int64_t n_rows, uint32_t flags, std::unique_ptr<pq_plan>* out) {
@@ -903,9 +907,10 @@ pq_status plan_build(pq_ctx* ctx, pq_index* idx, const std::vector<int32_t>& col
   const bool plain = (flags & PQ_SCAN_PLAIN) != 0;
   plan->tuning = ctx->tuning;
   plan->staged_expand = plan->tuning.staged_expand && !env_flag("PQ_NO_STAGED_EXPAND");
-  const int64_t item_rows_max = plan_item_rows(plan->tuning.item_rows, 256, n_rows, ctx->n_sms);
+  const int64_t item_rows_max = plan_item_rows(plan->tuning.item_rows, ITEM_ROWS_LEAST, n_rows, 32ll * ctx->n_sms);
   plan->item_rows = static_cast<int32_t>(item_rows_max);
-  const int64_t item_rows_opt = plan_item_rows(plan->tuning.item_rows_opt, 128, n_rows, ctx->n_sms);
+  const int64_t item_rows_opt =
+      plan_item_rows(plan->tuning.item_rows_opt, ITEM_ROWS_OPT_LEAST, n_rows, 32ll * ctx->n_sms);
   uint64_t scratch = 0;
   uint64_t tc_pool = 0;               // DELTA_BYTE_ARRAY pool bytes
   std::vector<int64_t> data_job_off;  // scratch offset per data snappy job
@@ -1153,7 +1158,10 @@ pq_status plan_build(pq_ctx* ctx, pq_index* idx, const std::vector<int32_t>& col
         const uint32_t span = pp.row_hi > pp.row_lo ? static_cast<uint32_t>(pp.row_hi - pp.row_lo) : 0u;
         // pages with definition levels take the short items (their walks and
         // expands carry a bitmap per item; measured faster for PLAIN too)
-        const uint32_t per = static_cast<uint32_t>(cd.max_def ? item_rows_opt : item_rows_max);
+        const uint32_t per = static_cast<uint32_t>(
+            !plain       ? (cd.max_def ? item_rows_opt : item_rows_max)
+            : cd.max_def ? plan_item_rows(plan->tuning.item_rows_opt, ITEM_ROWS_OPT_LEAST, span, PLAIN_PAGE_ITEMS)
+                         : plan_item_rows(plan->tuning.item_rows, ITEM_ROWS_LEAST, span, PLAIN_PAGE_ITEMS));
         const uint32_t n_it = span / per + (span % per ? 1 : 0);
         pp.item_rows = static_cast<int32_t>(per);
         pp.item_count = n_it;

@@ -234,7 +234,7 @@ extern "C" int scan_with_fake_cuda(const uint8_t* file, uint64_t size, uint32_t 
   W.scanning = false;
   bool done = false;
   for (cudaEvent_t e : W.recorded) done |= e == plan->done;
-  std::string t = "plan_bytes " + std::to_string(bytes) + "\nplan_mallocs " + std::to_string(mallocs) + "\nbudget " +
+  std::string t = "items " + std::to_string(plan->n_items) + "\nplan_bytes " + std::to_string(bytes) + "\nplan_mallocs " + std::to_string(mallocs) + "\nbudget " +
                   std::to_string(plan->device_bytes) + "\nplanned_kernels " + std::to_string(plan->launches) + "\nkernels " + std::to_string(W.kernels) + "\ndone " + std::to_string(done) + "\nforks " + std::to_string(W.forks) + "\njoins " +
                   std::to_string(W.joins) + "\nlast_error " + std::to_string(static_cast<int>(W.last)) + "\nlaunches";
   for (const auto& l : W.log) t += " " + l;

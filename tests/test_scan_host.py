@@ -127,3 +127,15 @@ def test_an_earlier_error_is_not_the_scans(scan, flags):
 def test_a_reported_error_is_not_reported_again(scan):
     st, got = scan(_eight("UNCOMPRESSED"), fail_at=-2)
     assert st == N.PQ_ERR_CUDA and got["last_error"] == "0" and got["launches"] == ""
+
+
+@pytest.mark.parametrize("flags,rows,rows_per_item", [
+    ("BATCHED", 6000, 256), ("BATCHED", 40_000, 256),
+    ("PLAIN", 6000, 256), ("PLAIN", 16 * 512 + 40, 512), ("PLAIN", 40_000, 2048)])
+def test_items_of_few_rows(scan, flags, rows, rows_per_item):
+    """Few rows are cut into small work items, so that there are some for every
+    warp: of the GPU, or of a page's thread block where that takes a whole page."""
+    col = synth.ColumnData("x", "INT32", np.arange(rows, dtype=np.int32) % 7)
+    data = W.write_file(synth.Table([col]), synth.TableSpec(rows, 1 << 20, [synth.ColumnSpec("RLE_DICTIONARY")]))
+    st, got = scan(data, getattr(N, "PQ_SCAN_" + flags))
+    assert st == N.PQ_OK and int(got["items"]) == -(-rows // rows_per_item)
