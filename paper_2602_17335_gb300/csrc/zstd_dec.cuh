@@ -3,8 +3,8 @@
 // over plain pointers.  The kernel (k_zstd.cu) divides a page among a thread
 // block and takes from here the format's constants and header arithmetic:
 // error codes, z_le, z_hb, z_huf_split, z_default_norm, z_ll and z_ml.
-// zstd_decode and what it alone calls (z_literals, z_sequences and the readers
-// below them) run in host tests, as a second decoder beside the oracle.
+// The rest, up to zstd_decode, runs on the host: in tests, as a second decoder
+// beside the oracle, and (z_read_huf) where the writer checks a tree it wrote.
 //
 // Format steps, in order: frame header (magic 0xFD2FB528; descriptor with
 // content-size, single-segment, checksum and dictionary flags; window
