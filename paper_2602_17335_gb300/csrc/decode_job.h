@@ -122,12 +122,13 @@ inline int snappy_scan_kernels(int n_jobs, uint32_t n_segs, bool long_first) {
   return n_jobs <= 0 || n_segs == 0 ? 0 : 1 + (long_first ? 1 : 0);
 }
 
-// The transcode of jobs [0, n), n_bss of them BYTE_STREAM_SPLIT pages;
+// The transcode of jobs [0, n), n_bss of them BYTE_STREAM_SPLIT pages, of
+// max_bss bytes at most;
 // `counters` is the plan's item_counter array (its pool word); `pool` holds
 // `pool_cap` bytes for DELTA_BYTE_ARRAY bodies; string pages get their entry
 // table (PlanPage::vtab) filled in `vpos`.
-void launch_transcode(const TranscodeJob* jobs, int n, int n_bss, PlanPage* pps, uint8_t* pool, uint64_t pool_cap,
-                      uint32_t* counters, uint64_t* vpos, DevStatus* st, cudaStream_t s);
+void launch_transcode(const TranscodeJob* jobs, int n, int n_bss, uint32_t max_bss, PlanPage* pps, uint8_t* pool,
+                      uint64_t pool_cap, uint32_t* counters, uint64_t* vpos, DevStatus* st, cudaStream_t s);
 // fixed: the list has fixed-width dictionaries
 void launch_dict(const DictJob* jobs, int n_jobs, bool fixed, int max_fixed_bytes, int max_str_regions, DictScratch ds,
                  DictDev* dicts, int n_sms, DevStatus* st, cudaStream_t s);

@@ -1113,6 +1113,7 @@ pq_status plan_build(pq_ctx* ctx, pq_index* idx, const std::vector<int32_t>& col
             plan->tc_dst_off.push_back(-1);  // the strings stay in the page
           } else {
             cw.tc_bss++;
+            cw.max_bss = std::max(cw.max_bss, static_cast<uint32_t>(pg.uncompressed));
             j.dst_cap = static_cast<uint32_t>(pg.uncompressed);
             plan->tc_dst_off.push_back(static_cast<int64_t>(scratch));
             scratch += (static_cast<uint64_t>(pg.uncompressed) + 32 + 15) & ~uint64_t(15);
@@ -1534,9 +1535,10 @@ static int max_str_regions_all(const pq_plan* plan) {
   return m;
 }
 
-static void enqueue_transcode(pq_plan* plan, int begin, int n, int n_bss, const pqi::DecodeArgs& a, cudaStream_t s) {
+static void enqueue_transcode(pq_plan* plan, int begin, int n, int n_bss, uint32_t max_bss, const pqi::DecodeArgs& a,
+                              cudaStream_t s) {
   if (n <= 0) return;
-  pqi::launch_transcode(plan->d_tc_jobs + begin, n, n_bss, plan->d_pps, plan->d_scratch + plan->tc_pool_off,
+  pqi::launch_transcode(plan->d_tc_jobs + begin, n, n_bss, max_bss, plan->d_pps, plan->d_scratch + plan->tc_pool_off,
                         plan->tc_pool_bytes, plan->d_counter, plan->d_vpos, a.st, s);
 }
 
@@ -1660,7 +1662,7 @@ static void enqueue_column(pq_plan* plan, size_t oc, const pqi::DecodeArgs& a, b
   if (!pqi::launched()) return;
   launch_range(plan, column_range(plan, oc, false), a.st, s);
   if (!pqi::launched()) return;
-  enqueue_transcode(plan, cw.tc_begin, cw.tc_n, cw.tc_bss, a, s);
+  enqueue_transcode(plan, cw.tc_begin, cw.tc_n, cw.tc_bss, cw.max_bss, a, s);
   if (!pqi::launched()) return;
   const auto& col = plan->outcols[oc];
   pqi::launch_walk(a, cw.walk_begin, cw.walk_n, ctx->n_sms, col.optional != 0, plan->tuning.walk_window, s);
@@ -1684,6 +1686,7 @@ static void enqueue_strings(pq_plan* plan, const pqi::DecodeArgs& a, cudaStream_
 // What the stages of all columns are launched with.
 struct AllColumns {
   int max_regions, n_bss;
+  uint32_t max_bss;
   bool fixed, levels;
 };
 static AllColumns all_columns(const pq_plan* plan) {
@@ -1692,6 +1695,7 @@ static AllColumns all_columns(const pq_plan* plan) {
     const auto& cw = plan->colwork[oc];
     r.max_regions = std::max(r.max_regions, cw.max_regions);
     r.n_bss += cw.tc_bss;
+    r.max_bss = std::max(r.max_bss, cw.max_bss);
     r.fixed |= cw.dict_n && plan->outcols[oc].ptype != pqi::T_BYTE_ARRAY;
     r.levels |= plan->outcols[oc].optional != 0;
   }
@@ -1702,7 +1706,7 @@ static AllColumns all_columns(const pq_plan* plan) {
 // the walks of the data pages on a branch stream, then expansion and strings.
 static void enqueue_merged(pq_plan* plan, const pqi::DecodeArgs& a, bool with_dicts, cudaStream_t side, cudaStream_t s) {
   pq_ctx* ctx = plan->ctx;
-  const auto [max_regions, n_bss, fixed, levels] = all_columns(plan);
+  const auto [max_regions, n_bss, max_bss, fixed, levels] = all_columns(plan);
   const bool dicts = with_dicts && !plan->dict_jobs.empty();
   if (dicts) {
     cudaEventRecord(plan->fork, s);
@@ -1715,7 +1719,7 @@ static void enqueue_merged(pq_plan* plan, const pqi::DecodeArgs& a, bool with_di
     cudaEventRecord(plan->join[0], side);
   }
   if (pqi::launched()) launch_range(plan, plan_range(plan, false), a.st, s);
-  if (pqi::launched()) enqueue_transcode(plan, 0, static_cast<int>(plan->tc_jobs.size()), n_bss, a, s);
+  if (pqi::launched()) enqueue_transcode(plan, 0, static_cast<int>(plan->tc_jobs.size()), n_bss, max_bss, a, s);
   if (pqi::launched())
     pqi::launch_walk(a, 0, static_cast<int>(plan->walk_pps.size()), ctx->n_sms, levels, plan->tuning.walk_window, s);
   if (pqi::launched()) pqi::launch_delta_bases(a, 0, static_cast<int>(plan->delta_pps.size()), max_regions, s);
@@ -1753,7 +1757,7 @@ static int scan_kernels(const pq_plan* plan) {
       n += (nj ? dk : 0) + pqi::transcode_kernels(ntc, nbss) + 1;
     }
   } else if (merged_scan(plan)) {
-    const auto [max_regions, n_bss, fixed, levels] = all_columns(plan);
+    const auto [max_regions, n_bss, max_bss, fixed, levels] = all_columns(plan);
     n += range_kernels(plan, plan_range(plan, true)) + range_kernels(plan, plan_range(plan, false)) +
          pqi::dict_kernels(static_cast<int>(plan->dict_jobs.size()), fixed, max_str_regions_all(plan)) +
          pqi::transcode_kernels(static_cast<int>(plan->tc_jobs.size()), n_bss) + (plan->walk_pps.empty() ? 0 : 1) +
@@ -1814,8 +1818,13 @@ static cudaError_t enqueue_scan(pq_plan* plan, cudaStream_t s, bool with_dicts, 
       int ntc = 0;
       while (tcj + ntc < plan->tc_jobs.size() && plan->tc_jobs[tcj + ntc].pp < static_cast<uint32_t>(first + n)) ++ntc;
       int nbss = 0;
-      for (int q = 0; q < ntc; ++q) nbss += plan->tc_jobs[tcj + q].enc == pqi::ENC_BSS;
-      enqueue_transcode(plan, static_cast<int>(tcj), ntc, nbss, a, s);
+      uint32_t max_bss = 0;
+      for (int q = 0; q < ntc; ++q)
+        if (plan->tc_jobs[tcj + q].enc == pqi::ENC_BSS) {
+          nbss++;
+          max_bss = std::max(max_bss, plan->tc_jobs[tcj + q].src_len);
+        }
+      enqueue_transcode(plan, static_cast<int>(tcj), ntc, nbss, max_bss, a, s);
       tcj += ntc;
       if (pqi::launched()) pqi::launch_plain_pages(a, first, n, s);
     }
@@ -1827,7 +1836,7 @@ static cudaError_t enqueue_scan(pq_plan* plan, cudaStream_t s, bool with_dicts, 
       const auto& cw = plan->colwork[oc];
       if (with_dicts) launch_range(plan, column_range(plan, oc, true), a.st, s);
       if (pqi::launched()) launch_range(plan, column_range(plan, oc, false), a.st, s);
-      if (pqi::launched()) enqueue_transcode(plan, cw.tc_begin, cw.tc_n, cw.tc_bss, a, s);
+      if (pqi::launched()) enqueue_transcode(plan, cw.tc_begin, cw.tc_n, cw.tc_bss, cw.max_bss, a, s);
     }
     mark(2);
     for (int oc = 0; oc < ncols && pqi::launched(); ++oc) {

@@ -217,6 +217,7 @@ struct pq_plan {
     int walk_begin = 0, walk_n = 0;            // into walk_pps
     int delta_begin = 0, delta_n = 0;          // into delta_pps
     int tc_begin = 0, tc_n = 0, tc_bss = 0;    // into tc_jobs; BYTE_STREAM_SPLIT pages among them
+    uint32_t max_bss = 0;                      // and the largest of these (bytes)
     int max_regions = 0;                       // most DELTA regions of one page
     int max_str_regions = 0;                   // most chain regions of one string dictionary
     bool copy_only = false;                    // every page REQUIRED PLAIN fixed-width

@@ -627,7 +627,10 @@ __device__ __forceinline__ void bss_transpose(uint32_t (&w)[4]) {
 // one aligned word of each stream, 16-byte stores.  The new body starts where
 // its values fall on a 16-byte boundary.  Every whole value of the streams is
 // written.
-constexpr int BSS_BLOCKS = 32;  // per page: 1 MiB pages in 2 steps of every thread
+// A block for every 8 KiB of the largest page (a step of its threads, at 8-byte
+// values), at most 32: with 32 for any page, 8192 pages of 2 KiB took 974 us a
+// read, so 714 (and 64 KiB pages, 2^23 rows, 319 instead of 356).
+constexpr uint32_t BSS_BLOCK_BYTES = 8 << 10;
 __global__ void __launch_bounds__(256) k_bss(const TranscodeJob* jobs, PlanPage* pps, DevStatus* st) {
   const TranscodeJob j = jobs[blockIdx.y];
   if (j.enc != ENC_BSS) return;
@@ -680,11 +683,13 @@ __global__ void __launch_bounds__(256) k_bss(const TranscodeJob* jobs, PlanPage*
 
 }  // namespace
 
-void launch_transcode(const TranscodeJob* jobs, int n, int n_bss, PlanPage* pps, uint8_t* pool, uint64_t pool_cap,
-                      uint32_t* counters, uint64_t* vpos, DevStatus* st, cudaStream_t s) {
+void launch_transcode(const TranscodeJob* jobs, int n, int n_bss, uint32_t max_bss, PlanPage* pps, uint8_t* pool,
+                      uint64_t pool_cap, uint32_t* counters, uint64_t* vpos, DevStatus* st, cudaStream_t s) {
   if (n <= 0) return;
-  if (n_bss > 0)
-    launch_slices(n, [&](int at, int m) { k_bss<<<dim3(BSS_BLOCKS, m), 256, 0, s>>>(jobs + at, pps, st); });
+  if (n_bss > 0) {
+    const unsigned want = max_bss / BSS_BLOCK_BYTES + 1, blocks = want < 32 ? want : 32;
+    launch_slices(n, [&](int at, int m) { k_bss<<<dim3(blocks, m), 256, 0, s>>>(jobs + at, pps, st); });
+  }
   if (n_bss == n) return;
   static bool attr = false;
   if (!attr) {

@@ -118,7 +118,7 @@ cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t) {
 }
 
 namespace pqi {
-void launch_transcode(const TranscodeJob*, int n, int n_bss, PlanPage*, uint8_t*, uint64_t, uint32_t*, uint64_t*, DevStatus*,
+void launch_transcode(const TranscodeJob*, int n, int n_bss, uint32_t, PlanPage*, uint8_t*, uint64_t, uint32_t*, uint64_t*, DevStatus*,
                       cudaStream_t) {
   if (n > 0) launch("transcode", transcode_kernels(n, n_bss));
 }

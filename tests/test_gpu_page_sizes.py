@@ -1,0 +1,44 @@
+"""GPU decode where the launch follows the size of a page: thread blocks and
+threads a page, and the work items that a batch of its runs covers.  Bit for bit
+against the CPU oracle."""
+import numpy as np
+import pytest
+
+import synth
+from oracle import reader as R
+
+from gpu_util import assert_columns_equal, engine, slice_result, to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def eng():
+    e = engine()
+    yield e
+    e.close()
+
+
+def _check(eng, columns, spec, ranges=()):
+    from paper_2602_17335_gb300.tables import write_table
+    data = write_table(synth.Table(columns), spec).tobytes()
+    expect = R.read_file(data)
+    dev = to_dev(data)
+    assert_columns_equal(eng.read([dev]), expect)
+    for lo, hi in ranges:
+        assert_columns_equal(eng.read([dev], row_begin=lo, row_count=hi - lo), [slice_result(e, lo, hi) for e in expect])
+
+
+@pytest.mark.parametrize("page", [64, 8 << 10, (8 << 10) + 64, 64 << 10, 248 << 10, 300_000, 1 << 20])
+def test_byte_stream_split(eng, page):
+    """Around a block's 8 KiB and the most blocks of a page, with a short last page."""
+    rng = np.random.default_rng(page)
+    rows = 90_001 if page > 64 else 5_003
+    valid = rng.random(rows) > 0.2
+    ints = rng.integers(-2**62, 2**62, rows)
+    ints[~valid] = 0
+    cols = [synth.ColumnData("d", "DOUBLE", rng.standard_normal(rows)),
+            synth.ColumnData("i", "INT32", rng.integers(-2**31, 2**31, rows).astype(np.int32)),
+            synth.ColumnData("o", "INT64", ints, valid)]
+    _check(eng, cols, synth.TableSpec(70_000, page, [synth.ColumnSpec("BYTE_STREAM_SPLIT") for _ in cols]),
+           [(1234, rows - 7)])

@@ -43,7 +43,7 @@ extern "C" int transcode_pages(const uint8_t* src, const uint32_t* at, const int
   uint8_t* pool = static_cast<uint8_t*>(malloc(pool_cap + 64));
   uint32_t counters[8] = {};
   DevStatus st{0, -1, 0, 0};
-  launch_transcode(jobs.data(), n, 0, pps.data(), pool, pool_cap, counters, tab, &st, nullptr);
+  launch_transcode(jobs.data(), n, 0, 0, pps.data(), pool, pool_cap, counters, tab, &st, nullptr);
   uint64_t w = 0, o = 0;
   for (int i = 0; i < n && !emu::fault(); ++i) {
     const PlanPage& pp = pps[i];
