@@ -79,6 +79,13 @@ __device__ __forceinline__ uint64_t gwin64(const uint8_t* base, uint64_t b) {
   return (static_cast<uint64_t>(__funnelshift_r(r1, r2, sh)) << 32) | __funnelshift_r(r0, r1, sh);
 }
 
+// Threads of the blocks that stitch a page's regions (k_sfix, k_dfix): a warp
+// copies a region's list, so as many warps as the largest page has regions, 8
+// to 32.  (32 for pages of any size: 2^21 INT64 rows in 2 KiB DELTA pages 2259 us
+// a read, so 2030.)
+constexpr int FIX_THREADS = 1024;
+static int fix_threads(int regions) { return 32 * (regions < 8 ? 8 : regions < 32 ? regions : 32); }
+
 // ------------------------------------------------------------------ K6 dictionaries
 
 // Fixed-width dictionary: an aligned copy of the PLAIN page body.
@@ -389,8 +396,7 @@ __global__ void __launch_bounds__(32) k_sreg(const DictJob* __restrict__ jobs, D
 // A region whose found start is not the true entry is walked again from the
 // true entry, in shared memory (the region is staged by one bulk copy), its
 // entries written directly.
-constexpr int SFIX_THREADS = 1024;
-__global__ void __launch_bounds__(SFIX_THREADS) k_sfix(const DictJob* __restrict__ jobs, DictScratch ds, DictDev* dicts,
+__global__ void __launch_bounds__(FIX_THREADS) k_sfix(const DictJob* __restrict__ jobs, DictScratch ds, DictDev* dicts,
                                               DevStatus* st) {
   constexpr int MAXR = 2048;
   __shared__ int32_t s_q[MAXR], s_x[MAXR], s_c[MAXR];
@@ -578,7 +584,7 @@ void launch_dict(const DictJob* jobs, int n_jobs, bool fixed, int max_fixed_byte
       k_sreg<<<dim3(max_str_regions, m), 32, SREG_SMEM, s>>>(jobs + at, ds, st);
     });
     if (!launched()) return;
-    k_sfix<<<n_jobs, SFIX_THREADS, 0, s>>>(jobs, ds, dicts, st);
+    k_sfix<<<n_jobs, fix_threads(max_str_regions), 0, s>>>(jobs, ds, dicts, st);
     if (!launched()) return;
     launch_slices(n_jobs, [&](int at, int m) { k_dict_pad<<<dim3(32, m), 256, 0, s>>>(jobs + at, dicts); });
   }
@@ -1748,8 +1754,7 @@ __device__ int32_t dwalk_join(const uint8_t* sb, uint32_t slen, uint32_t pos, ui
 // entry until it joins the list.  The lists are then copied to the page's
 // block table in parallel and the last block is checked against the
 // stream's end.
-constexpr int DFIX_THREADS = 1024;
-__global__ void __launch_bounds__(DFIX_THREADS) k_dfix(DecodeArgs a, int dbegin) {
+__global__ void __launch_bounds__(FIX_THREADS) k_dfix(DecodeArgs a, int dbegin) {
   constexpr int MAXR = 1024;
   __shared__ int32_t s_q[MAXR], s_x[MAXR], s_c[MAXR];
   __shared__ int32_t s_skip[MAXR], s_cnt[MAXR], s_base[MAXR];
@@ -3832,7 +3837,7 @@ void launch_delta_bases(const DecodeArgs& a, int dbegin, int n, int max_regions,
   if (max_regions > 0) {
     launch_slices(n, [&](int at, int m) { k_dreg<<<dim3(max_regions, m), 32, dreg_smem, s>>>(a, dbegin + at); });
     if (!launched()) return;
-    k_dfix<<<n, DFIX_THREADS, 0, s>>>(a, dbegin);
+    k_dfix<<<n, fix_threads(max_regions), 0, s>>>(a, dbegin);
   }
   if (!launched()) return;
   launch_slices(n, [&](int at, int m) { k_delta_sums<<<dim3(64, m), 256, 0, s>>>(a, dbegin + at); });

@@ -42,3 +42,22 @@ def test_byte_stream_split(eng, page):
             synth.ColumnData("o", "INT64", ints, valid)]
     _check(eng, cols, synth.TableSpec(70_000, page, [synth.ColumnSpec("BYTE_STREAM_SPLIT") for _ in cols]),
            [(1234, rows - 7)])
+
+
+@pytest.mark.parametrize("kib", [2, 56, 64, 96, 256, 280, 600])
+def test_regions_of_a_page(eng, kib):
+    """DELTA pages and string dictionaries of a few regions (8 KiB, 4 KiB) up to
+    more than the block that stitches them has warps."""
+    rng = np.random.default_rng(kib)
+    rows = 140 * kib + 77
+    n = 60 * kib + 3
+    lens = rng.integers(0, 24, n)
+    off = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    strings = synth.StringData(off, rng.integers(33, 127, int(off[-1])).astype(np.uint8),
+                               rng.integers(0, n, rows).astype(np.int32))
+    cols = [synth.ColumnData("d", "INT64", rng.integers(-2**62, 2**62, rows)),
+            synth.ColumnData("k", "INT32", np.cumsum(rng.integers(0, 8, rows)).astype(np.int32)),
+            synth.ColumnData("s", "BYTE_ARRAY", strings)]
+    spec = synth.TableSpec(rows, kib << 10, [synth.ColumnSpec(e) for e in ("DELTA_BINARY_PACKED", "DELTA_BINARY_PACKED",
+                                                                         "RLE_DICTIONARY")])
+    _check(eng, cols, spec, [(rows // 3, rows - 5)])
