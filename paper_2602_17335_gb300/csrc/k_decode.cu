@@ -992,17 +992,24 @@ __device__ int32_t walk_levels(WalkSmem& sm, const PageCtx& pc, const PlanPage& 
         }
       }
     }
-    // dense index at each item start (and at row_hi) inside the batch
-    for (uint32_t i = tid; i <= pp.item_count; i += blockDim.x) {
-      const int32_t R = i < pp.item_count ? items[pp.item_begin + i].row0 : pp.row_hi;
-      if (nb > 0 && R >= b0 && R < b1) {
+    // dense index at each item start (and at row_hi) inside the batch: of the
+    // items that start there (every item_rows rows from row_lo on) alone: a large
+    // page has many batches and many items (2^21 OPTIONAL dictionary values in a
+    // page: with all items looked at in each batch, here and below for the
+    // indices, 3257 us a read, so 2193)
+    if (nb > 0) {
+      const auto dense = [&](int32_t R) {
         const int j = find_run(sm.rk, nb, R);
-        const int32_t kR = sm.rpre[j] + run_valid(sm, lb, lp0, j, R - sm.rk[j]);
-        if (i < pp.item_count)
-          items[pp.item_begin + i].k0 = kR;
-        else
-          sm.c64[1] = kR;
-      }
+        return sm.rpre[j] + run_valid(sm, lb, lp0, j, R - sm.rk[j]);
+      };
+      const auto items_before = [&](int32_t R) {  // items that start below row R
+        const int32_t n = R > pp.row_lo ? (R - pp.row_lo - 1) / pp.item_rows + 1 : 0;
+        return n < static_cast<int32_t>(pp.item_count) ? n : static_cast<int32_t>(pp.item_count);
+      };
+      const int32_t i1 = items_before(b1);
+      for (int32_t i = items_before(b0) + tid; i < i1; i += blockDim.x)
+        items[pp.item_begin + i].k0 = dense(pp.row_lo + i * pp.item_rows);
+      if (tid == blockDim.x - 1 && pp.row_hi >= b0 && pp.row_hi < b1) sm.c64[1] = dense(pp.row_hi);
     }
     __syncthreads();
     if (tid == 0) {
@@ -1051,6 +1058,7 @@ __device__ bool walk_hybrid(WalkSmem& sm, const uint8_t* sb, uint32_t slen, int 
     sm.ctl[1] = 0;  // dense index
     sm.ctl[5] = ch_start(c, sb, slen) ? 0 : 3;
     sm.ctl[7] = !sm.ctl[5] && slen > 0 && c.b0[0] == kMaxRun;  // next batch starts with a parallel check
+    sm.ctl[20] = sm.ctl[21] = 0;  // items whose dense range starts in earlier batches; and with this one
   }
   __syncthreads();
   for (uint32_t guard = 0; guard <= slen + 2 && !sm.ctl[5] && sm.ctl[1] < total; ++guard) {
@@ -1194,19 +1202,25 @@ __device__ bool walk_hybrid(WalkSmem& sm, const uint8_t* sb, uint32_t slen, int 
     }
     const int nb = sm.ctl[2];
     const int32_t kb0 = sm.ctl[1], kb1 = sm.ctl[3];
-    for (uint32_t i = tid; i < pp.item_count; i += blockDim.x) {
+    // (dense ranges follow one another: a batch's items come after the last one's)
+    int32_t seen = 0;
+    for (uint32_t i = static_cast<uint32_t>(sm.ctl[20]) + tid; nb > 0 && i < pp.item_count; i += blockDim.x) {
       Item& it = items[pp.item_begin + i];
       const int32_t ik = it.k0;
-      if (nb > 0 && it.nn > 0 && ik >= kb0 && ik < kb1) {
+      if (ik >= kb1) break;
+      if (it.nn > 0 && ik >= kb0) {
         const int j = find_run(sm.rk, nb, ik);
         it.pos = static_cast<int32_t>(sm.rpos[j]);
         it.run_k0 = sm.rk[j];
         it.base = 0;
       }
+      seen = static_cast<int32_t>(i) + 1;
     }
+    if (seen) atomicMax(&sm.ctl[21], seen);
     __syncthreads();
     if (tid == 0) {
       sm.ctl[1] = kb1;
+      sm.ctl[20] = sm.ctl[21];
       if (nb == 0 && kb1 < total) sm.ctl[5] = 1;
     }
     __syncthreads();

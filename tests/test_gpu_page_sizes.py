@@ -61,3 +61,31 @@ def test_regions_of_a_page(eng, kib):
     spec = synth.TableSpec(rows, kib << 10, [synth.ColumnSpec(e) for e in ("DELTA_BINARY_PACKED", "DELTA_BINARY_PACKED",
                                                                          "RLE_DICTIONARY")])
     _check(eng, cols, spec, [(rows // 3, rows - 5)])
+
+
+@pytest.mark.parametrize("nulls", ["random", "runs", "ends", "none"])
+@pytest.mark.parametrize("mode", ["BATCHED", "PLAIN"])
+def test_items_of_a_large_page(eng, nulls, mode):
+    """One page of many items and many batches of runs: definition levels and
+    dictionary indices, whole and from rows inside items on."""
+    from paper_2602_17335_gb300 import native as N
+    from paper_2602_17335_gb300.tables import write_table
+    rng = np.random.default_rng(len(nulls))
+    rows = 300_017
+    valid = {"random": rng.random(rows) > 0.3, "none": np.ones(rows, bool),
+             "runs": np.repeat(rng.random(rows // 700 + 1) > 0.5, 700)[:rows],
+             "ends": (np.arange(rows) > 70_001) & (np.arange(rows) < 240_003)}[nulls]
+    few, many = rng.integers(0, 5, rows), rng.integers(0, 3000, rows)
+    runs = np.repeat(rng.integers(0, 9, rows // 50 + 1), 50)[:rows]
+    cols = [synth.ColumnData(f"r{k}", "INT32", v.astype(np.int32)) for k, v in enumerate((few, many, runs))]
+    for k, v in enumerate((few, many, runs)):
+        v = v.copy()
+        v[~valid] = 0
+        cols.append(synth.ColumnData(f"o{k}", "INT64", v, valid))
+    data = write_table(synth.Table(cols), synth.TableSpec(rows, 8 << 20, [synth.ColumnSpec("RLE_DICTIONARY") for _ in cols]))
+    data = data.tobytes()
+    expect, dev = R.read_file(data), to_dev(data)
+    flags = getattr(N, "PQ_SCAN_" + mode)
+    for lo, hi in ((0, rows), (1, rows), (127, 128), (70_000, 240_000), (299_001, rows)):
+        outs = eng.read([dev], row_begin=lo, row_count=hi - lo, flags=flags)
+        assert_columns_equal(outs, [slice_result(e, lo, hi) for e in expect])
