@@ -830,7 +830,7 @@ void pq_free_plan(pq_plan* plan) {
   cudaSetDevice(plan->ctx->device);
   // once `done` (recorded after the scan's last work) and `ready` have
   // completed, so have the fork and join records: all go back to the cache
-  if (plan->scanned) cudaEventSynchronize(plan->done);
+  if (plan->scanned && cudaEventSynchronize(plan->done) != cudaSuccess) cudaGetLastError();
   if (plan->ready) cudaEventSynchronize(plan->ready);
   if (plan->graph) cudaGraphExecDestroy(plan->graph);
   for (auto& e : plan->stage_ev)
@@ -1966,13 +1966,13 @@ pq_status scan_enqueue(pq_plan* plan, const pq_column* outs, cudaStream_t s, con
     const cudaError_t launch = enqueue_scan(plan, s, with_dicts, branches, n_branches);
     if (launch != cudaSuccess) {
       // (what was launched before uses the plan's memory until `done`)
-      if (cudaEventRecord(plan->done, s) == cudaSuccess && !capturing) plan->scanned = true;
+      if (cudaEventRecord(plan->done, s) == cudaSuccess) (capturing ? plan->captured : plan->scanned) = true;
       return cuda_fail(ctx, launch, "kernel launch");
     }
   }
   CK(cudaGetLastError());
   CK(cudaEventRecord(plan->done, s));
-  if (!capturing) plan->scanned = true;
+  (capturing ? plan->captured : plan->scanned) = true;
   if (plan->flags & PQ_SCAN_RESIDENT_DICT)
     for (int32_t ch : plan->dict_chunks) plan->idx->dict_resident[ch] = 1;
   return PQ_OK;
@@ -1993,7 +1993,8 @@ pq_status pq_scan_wait(pq_ctx* ctx, pq_plan* plan, void* stream, uint64_t* chars
   if (!ctx || !plan) return fail(ctx, PQ_ERR_INVALID_ARG, "pq_scan_wait");
   (void)stream;
   CK(cudaSetDevice(ctx->device));
-  if (plan->scanned) CK(cudaEventSynchronize(plan->done));
+  // (of a scan that is part of a caller's graph the wait is refused)
+  if (plan->scanned || plan->captured) CK(cudaEventSynchronize(plan->done));
   pqi::DevStatus st;
   memcpy(&st, plan->h_out.p, sizeof st);
   if (chars_bytes) {

@@ -196,6 +196,7 @@ struct pq_plan {
   bool scanned = false;         // `done` has been recorded, outside a capture (before that it is as
                                 // the cache gave it: last recorded inside one, perhaps, where a wait
                                 // for it is an error)
+  bool captured = false;        // or inside one
   cudaEvent_t ready = nullptr;  // the plan's uploads and item table are in place
   cudaGraphExec_t graph = nullptr;
   cudaStream_t graph_stream = nullptr;

@@ -169,7 +169,8 @@ void launch_index_oi(const ChunkDev*, int, const int64_t*, PageDev*, int, DevSta
 }  // namespace pqi
 
 // Plans and scans all columns of the file on a GPU of n_sms multiprocessors,
-// with launch `fail_at` of the scan failing (-1: none, -2: its copies to the GPU),
+// with launch `fail_at` of the scan failing (-1: none, -2: its copies to the GPU,
+// -3: none, but the scan is captured by the caller),
 // on a thread whose last error is stale_error.  Returns the scan's
 // status, -1 when it did not get that far; `text` gets what there is to see.
 extern "C" int scan_with_fake_cuda(const uint8_t* file, uint64_t size, uint32_t flags, int n_sms, int fail_at,
@@ -230,13 +231,16 @@ extern "C" int scan_with_fake_cuda(const uint8_t* file, uint64_t size, uint32_t 
   W.scanning = true;
   W.recorded.clear();
   W.last = static_cast<cudaError_t>(stale_error);
+  W.capturing = fail_at == -3;
   const pq_status st = pqe::scan_enqueue(plan, outs.data(), W.main, ctx->branch, pq_ctx::kBranches, true);
-  W.scanning = false;
+  W.capturing = W.scanning = false;
+  const int last = static_cast<int>(W.last);
+  const pq_status waited = pq_scan_wait(ctx, plan, W.main, nullptr);
   bool done = false;
   for (cudaEvent_t e : W.recorded) done |= e == plan->done;
   std::string t = "items " + std::to_string(plan->n_items) + "\nplan_bytes " + std::to_string(bytes) + "\nplan_mallocs " + std::to_string(mallocs) + "\nbudget " +
                   std::to_string(plan->device_bytes) + "\nplanned_kernels " + std::to_string(plan->launches) + "\nkernels " + std::to_string(W.kernels) + "\ndone " + std::to_string(done) + "\nforks " + std::to_string(W.forks) + "\njoins " +
-                  std::to_string(W.joins) + "\nlast_error " + std::to_string(static_cast<int>(W.last)) + "\nlaunches";
+                  std::to_string(W.joins) + "\nwait " + std::to_string(static_cast<int>(waited)) + "\nlast_error " + std::to_string(last) + "\nlaunches";
   for (const auto& l : W.log) t += " " + l;
   pq_free_plan(plan);
   // another plan, with the first one's events, that is never scanned

@@ -139,3 +139,11 @@ def test_items_of_few_rows(scan, flags, rows, rows_per_item):
     data = W.write_file(synth.Table([col]), synth.TableSpec(rows, 1 << 20, [synth.ColumnSpec("RLE_DICTIONARY")]))
     st, got = scan(data, getattr(N, "PQ_SCAN_" + flags))
     assert st == N.PQ_OK and int(got["items"]) == -(-rows // rows_per_item)
+
+
+def test_wait_for_a_captured_scan_is_refused(scan):
+    data = _eight("UNCOMPRESSED")
+    st, got = scan(data, fail_at=-3)
+    assert st == N.PQ_OK and int(got["wait"]) == N.PQ_ERR_CUDA and got["last_error_unscanned"] == "0"
+    st, got = scan(data)
+    assert st == N.PQ_OK and int(got["wait"]) == N.PQ_OK
